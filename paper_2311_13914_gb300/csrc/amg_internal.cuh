@@ -36,7 +36,6 @@ struct Level {
     int N = 0;                 // nodes (unknowns 2N)
     BSR A;                     // operator
     DBuf<double> invdiag;      // 1 / A(i,i), 2N
-    DBuf<double> idc2, idt;    // FP64 sliced-ELL finest level: c2 / A(i,i) and 1 / (theta A(i,i))
     DBuf<double> B;            // near-null coefficients per field, 2N
     DBuf<unsigned char> mis;   // root flags (not on the coarsest)
     DBuf<int> agg;             // aggregate id per node
@@ -57,21 +56,19 @@ struct Level {
     SlicedOp sl[3];
 };
 
-// Finest level in sliced-ELL form (32 rows per slice, slot-major), using the
-// shared pattern of the Bidomain operator: per node pair only Ki and Ke are
-// stored, since the block is [Ki, Ki; Ki, Ki+Ke] off the diagonal and the
-// diagonal adds c M to the (v, v) entry.
-struct FineSell {
+// Finest level of an assembled slab as a layered stencil (fine_stencil.cuh):
+// one row of coefficients per plane and row type (3 (y face) + (x face), 0 low,
+// 1 interior, 2 high).  raw holds the assembled rows themselves, kFineRaw
+// doubles each: (Ki, Ke) at the 27 stencil positions 9 (dz + 1) + 3 (dy + 1) +
+// dx + 1, c M, and the inverse diagonal (v, u_e); tab is packed for the kernels.
+constexpr int kFineRaw = 58;
+struct FineStencil {
     bool valid = false;
-    int nslices = 0;
-    long long slots = 0;        // padded slots (x 32 lanes)
-    DBuf<int> sptr;             // nslices + 1, slot offset of each slice
-    DBuf<int> col;              // slots * 32 column (FP64 kernels: an index costs no FP64 time)
-    DBuf<unsigned char> code;   // slots * 32: neighbour q = p + off[code] (27-point stencil; FP32)
-    int off[27] = {};           // node-index offset of each stencil position
-    DBuf<double> kk;            // slots * 32 * 2: (Ki, Ke)
-    DBuf<double> cm;            // c M_p per node
-    DBuf<float> kk32, cm32;     // FP32 copies for the FP32 V-cycle
+    bool sym = false;           // rows symmetric under (dx, dy) -> (-dx, -dy)
+    int NX = 0, NY = 0, NZ = 0; // nodes
+    DBuf<double> raw;           // NZ x 9 x kFineRaw
+    DBuf<double> tab;           // packed rows, FP64 (always: the PCG's A p)
+    DBuf<float> tab32;          // packed rows of the FP32 V-cycle
 };
 
 }  // namespace bd
@@ -80,7 +77,7 @@ struct amg_hierarchy {
     amg_options opts{};
     int nlev = 0;
     bool prec32 = false;        // V-cycle in FP32 inside an FP64 flexible CG
-    bd::FineSell sell;
+    bd::FineStencil fine;
     bd::Level lev[bd::kMaxLevels];
     // coarsest level: dense inverse of A_c + s z z^T / z^T z, null vector z
     int nc = 0;
@@ -135,7 +132,7 @@ int prepare_solve(amg_hierarchy *h, cudaStream_t s);
 int pcg_solve_begin(amg_hierarchy *h, const double *f_dev, double *x_dev, int warm,
                     const solve_options *o, cudaStream_t s, solve_info *info, bool *pending);
 int pcg_solve_end(amg_hierarchy *h, cudaStream_t s, solve_info *info);
-int build_fine_sell(amg_hierarchy *h, const bd_system *sys, cudaStream_t s);
+int build_fine_stencil(amg_hierarchy *h, const bd_system *sys, cudaStream_t s);
 // Timed step of the solve phase (host-driven loop only).  `fine`: a
 // finest-operator application, timed at profiling level 1 and summed into
 // amg_kernel_profile; every labelled step is timed at level 2.

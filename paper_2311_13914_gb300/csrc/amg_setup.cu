@@ -1675,7 +1675,7 @@ extern "C" int amg_setup(const bd_system *sys, const amg_options *opts, void *st
         return BD_ECUDA;
     }
     h->prec32 = o.precision == 1;
-    if ((st = setup_from_level0(h, s)) || (st = build_fine_sell(h, sys, s)) ||
+    if ((st = setup_from_level0(h, s)) || (st = build_fine_stencil(h, sys, s)) ||
         (st = prepare_solve(h, s))) {
         delete h;
         return st;
@@ -1813,7 +1813,7 @@ extern "C" int amg_level_lanes(const amg_hierarchy *h, int level, int lanes[3])
     if (!h || !lanes || level < 0 || level >= h->nlev) return BD_EINVAL;
     const Level &L = h->lev[level];
     const bool last = level == h->nlev - 1;
-    lanes[0] = last || (level == 0 && h->sell.valid) ? 0 : L.lanes[0];
+    lanes[0] = last || (level == 0 && h->fine.valid) ? 0 : L.lanes[0];
     lanes[1] = last ? 0 : L.lanes[1];
     lanes[2] = last ? 0 : L.lanes[2];
     return BD_OK;

@@ -16,8 +16,9 @@
 #include <new>
 #include <type_traits>
 
-#include "amg_internal.cuh"
 #include "amg_bsr.cuh"
+#include "amg_internal.cuh"
+#include "fine_stencil.cuh"
 
 namespace bd {
 
@@ -157,17 +158,7 @@ __global__ void k_slice_warps(int nsl, long long groups, int warps, const int *_
     wsl[w] = lo;
 }
 
-// Threads per block of the FP64 finest-level kernels: one block of 32 warps
-// per SM (measured against four blocks of 8 warps: 2-4 us shorter launches,
-// with the same warps resident and a quarter of the blocks to start and end),
-// where every SM then gets at least a slice per warp.  Smaller levels keep
-// blocks of 8 warps, so that small solves running side by side (graph branches,
-// served requests) share the SMs instead of each block holding one.  The FP32
-// kernels keep 8 blocks of 8 warps per SM (two blocks of 32 measured the same).
-constexpr int kFineTPB = 1024;
-static bool fine_wide(long long N) { return (N + 31) / 32 >= (long long)kSM * (kFineTPB / 32); }
-
-// ------------------------------------------------------------------ finest level, sliced ELL
+// ------------------------------------------------------------------ vector kernels' shares
 // Block b's share [share_lo(n), share_hi(n)) of n rows or nodes: the grid
 // splits the 32-row slices in equal contiguous parts, so with one resident
 // wave of blocks every SM gets the same work (a grid-stride loop leaves the
@@ -181,82 +172,14 @@ __device__ __forceinline__ int share_hi(int n)
     return min(n, (int)((((long long)n + 31) >> 5) * (blockIdx.x + 1) / gridDim.x) * 32);
 }
 
-// Neighbour offsets of the 27-point stencil of a structured slab, passed by
-// value and staged in shared memory (a warp's lanes index it divergently).
-struct Stencil {
-    int off[27];
-};
-__device__ __forceinline__ void stage_stencil(const Stencil &st, int *off)
-{
-    if (threadIdx.x == 0) {
-#pragma unroll
-        for (int i = 0; i < 27; i++) off[i] = st.off[i];  // constant indices: no local copy
-    }
-    __syncthreads();
-}
-
-// One thread per row; slot j of slice s holds entry j of its 32 rows
-// contiguously, so every slot is one coalesced (Ki, Ke) load and one column
-// load per warp.  FP32 (HBM-bound) reads 1-byte stencil codes (the
-// neighbour's position in the 27-point stencil) instead of 4-byte columns:
-// 9 instead of 12 bytes per node pair; FP64 (bound by its FP64 pipe as much
-// as by HBM) keeps the columns, which spare it the shared-memory lookup.  Per node pair: s = v_q + u_q, a += Ki s, b += Ke u_q;
-// then y_v = c M_p v_p + a, y_u = a + b.  SU: the gathered vector is stored as
-// (v + u, u), which saves the add per node pair (two FP64 operations instead
-// of three where the FP64 pipe is the limit).
-template <class S, class G, bool SU, int UNROLL>
-__device__ __forceinline__ void sell_row(int p, int lane, const int *__restrict__ sptr,
-                                         const int *__restrict__ col, const unsigned char *__restrict__ code,
-                                         const int *off, const v2<S> *__restrict__ kk,
-                                         const S *__restrict__ cm, const G &gather, S &y0, S &y1)
-{
-    constexpr bool CODED = sizeof(S) == 4;
-    const int sl = p >> 5;
-    const int j1 = sptr[sl + 1];
-    S a = 0, b = 0;
-#pragma unroll (UNROLL)
-    for (int j = sptr[sl]; j < j1; j++) {
-        const size_t idx = (size_t)j * 32 + lane;
-        const int q = CODED ? p + off[code[idx]] : col[idx];
-        const v2<S> k = kk[idx];
-        const v2<S> x = gather(q);
-        a = fma(k.x, SU ? x.x : x.x + x.y, a);
-        b = fma(k.y, x.y, b);
-    }
-    const v2<S> xp = gather(p);
-    y0 = fma(cm[p], SU ? xp.x - xp.y : xp.x, a);
-    y1 = a + b;
-}
-
-template <class S, class G, class E, bool SU = false, int MINB = 8, int TPB = 256>
-__global__ void __launch_bounds__(TPB, MINB) k_sell(int N, const int *__restrict__ sptr,
-                                               const int *__restrict__ col,
-                                               const unsigned char *__restrict__ code, Stencil st,
-                                               const v2<S> *__restrict__ kk,
-                                               const S *__restrict__ cm, G gather, E epi)
-{
-    __shared__ int off[27];
-    if (sizeof(S) == 4) stage_stencil(st, off);
-    const int lane = threadIdx.x & 31, e = share_hi(N);
-    for (int p = share_lo(N) + threadIdx.x; p < e; p += blockDim.x) {
-        S y0, y1;
-        sell_row<S, G, SU, (MINB >= 8 ? 4 : 8)>(p, lane, sptr, col, code, off, kk, cm, gather, y0, y1);
-        epi(p, y0, y1);
-    }
-}
-
 // ------------------------------------------------------------------ fused epilogues
 template <class S> struct GatherVec {
     const v2<S> *__restrict__ x;
     __device__ __forceinline__ v2<S> operator()(int q) const { return x[q]; }
 };
 
-// Vectors a finest-level sliced-ELL operator gathers may be kept in the
-// (v + u, u) form (SU); these convert at the epilogue, once per node.
-template <class S, bool SU> __device__ __forceinline__ v2<S> from_su(v2<S> a)
-{
-    return SU ? V2<S>::mk(a.x - a.y, a.y) : a;
-}
+// Vectors the FP64 finest-level stencil gathers are kept in the (v + u, u)
+// form (SU): two operations per node pair instead of three.
 template <class S, bool SU> __device__ __forceinline__ v2<S> to_su(S v, S u)
 {
     return V2<S>::mk(SU ? v + u : v, u);
@@ -264,16 +187,16 @@ template <class S, bool SU> __device__ __forceinline__ v2<S> to_su(S v, S u)
 
 // pre-smoothing, degree 2 from zero, d0 = D^{-1} f / theta precomputed:
 // x1 = d0, r1 = f - A d0, d1 = c1 d0 + c2 D^{-1} r1, u = x1 + d1
-template <class S, bool SU = false> struct EpiPre {
+template <class S> struct EpiPre {
     const v2<S> *__restrict__ f;
     const v2<S> *__restrict__ invd;
     const v2<S> *__restrict__ d0;
     v2<S> *__restrict__ u;
     S c1, c2;
     __device__ __forceinline__ void operator()(int p, S y0, S y1) const {
-        const v2<S> fp = f[p], id = invd[p], dp = from_su<S, SU>(d0[p]);
+        const v2<S> fp = f[p], id = invd[p], dp = d0[p];
         const S r0 = fp.x - y0, r1 = fp.y - y1;
-        u[p] = to_su<S, SU>(dp.x + (c1 * dp.x + c2 * id.x * r0), dp.y + (c1 * dp.y + c2 * id.y * r1));
+        u[p] = V2<S>::mk(dp.x + (c1 * dp.x + c2 * id.x * r0), dp.y + (c1 * dp.y + c2 * id.y * r1));
     }
 };
 
@@ -308,7 +231,7 @@ template <class S, bool SU = false> struct EpiAdd {  // u += P e_c
 };
 
 // post-smoothing, first half: r0 = f - A u, d0 = D^{-1} r0 / theta, w = u + d0
-template <class S, bool SU = false> struct EpiPost1 {
+template <class S> struct EpiPost1 {
     const v2<S> *__restrict__ f;
     const v2<S> *__restrict__ invd;
     const v2<S> *__restrict__ u;
@@ -317,85 +240,28 @@ template <class S, bool SU = false> struct EpiPost1 {
     v2<S> *__restrict__ w;
     S it;
     __device__ __forceinline__ void operator()(int p, S y0, S y1) const {
-        const v2<S> fp = f[p], id = invd[p], up = from_su<S, SU>(u[p]);
+        const v2<S> fp = f[p], id = invd[p], up = u[p];
         const S r0 = fp.x - y0, r1 = fp.y - y1;
         const S d0 = r0 * id.x * it, d1 = r1 * id.y * it;
         r[p] = V2<S>::mk(r0, r1);
-        d[p] = to_su<S, SU>(d0, d1);
+        d[p] = V2<S>::mk(d0, d1);
         w[p] = V2<S>::mk(up.x + d0, up.y + d1);
     }
 };
 
 // post-smoothing, second half: r1 = r0 - A d0, d1 = c1 d0 + c2 D^{-1} r1, u = w + d1
-template <class S, bool SU = false> struct EpiPost2 {
+template <class S> struct EpiPost2 {
     const v2<S> *__restrict__ r;
     const v2<S> *__restrict__ d;
     const v2<S> *__restrict__ invd;
     const v2<S> *__restrict__ w;
     v2<S> *__restrict__ u;
     S c1, c2;
-    __device__ __forceinline__ v2<S> value(int p, S y0, S y1) const {
-        const v2<S> rp_ = r[p], dp = from_su<S, SU>(d[p]), id = invd[p], wp = w[p];
+    __device__ __forceinline__ void operator()(int p, S y0, S y1) const {
+        const v2<S> rp_ = r[p], dp = d[p], id = invd[p], wp = w[p];
         const S r0 = rp_.x - y0, r1 = rp_.y - y1;
-        return V2<S>::mk(wp.x + (c1 * dp.x + c2 * id.x * r0), wp.y + (c1 * dp.y + c2 * id.y * r1));
+        u[p] = V2<S>::mk(wp.x + (c1 * dp.x + c2 * id.x * r0), wp.y + (c1 * dp.y + c2 * id.y * r1));
     }
-    __device__ __forceinline__ void operator()(int p, S y0, S y1) const { u[p] = value(p, y0, y1); }
-};
-
-// The Chebyshev steps of the FP64 finest level written in the (v + u, u) form
-// of the vectors they gather, with the inverse diagonal scaled per level
-// (idc2 = c2 D^{-1}, idt = D^{-1}/theta): fewer FP64 operations per node on a
-// level bound by the FP64 pipe.  For u = d0 + (c1 d0 + c2 D^{-1} r) with
-// m = idc2 r: u_s = (1 + c1) d0_s + (m_v + m_u), u_u = (1 + c1) d0_u + m_u.
-struct EpiPreX {
-    const double2 *__restrict__ f;
-    const double2 *__restrict__ idc2;
-    const double2 *__restrict__ d0;  // (v + u, u)
-    double2 *__restrict__ u;         // (v + u, u)
-    double c1p;                      // 1 + c1
-    __device__ __forceinline__ void operator()(int p, double y0, double y1) const
-    {
-        const double2 fp = f[p], k = idc2[p], dp = d0[p];
-        const double m0 = k.x * (fp.x - y0), m1 = k.y * (fp.y - y1);
-        u[p] = make_double2(fma(c1p, dp.x, m0 + m1), fma(c1p, dp.y, m1));
-    }
-};
-// r = f - A u, d = D^{-1} r / theta, w = u + d: r plain, d and w in (v + u, u)
-struct EpiPost1X {
-    const double2 *__restrict__ f;
-    const double2 *__restrict__ idt;
-    const double2 *__restrict__ u;  // (v + u, u)
-    double2 *__restrict__ r;
-    double2 *__restrict__ d;
-    double2 *__restrict__ w;
-    __device__ __forceinline__ void operator()(int p, double y0, double y1) const
-    {
-        const double2 fp = f[p], k = idt[p], up = u[p];
-        const double r0 = fp.x - y0, r1 = fp.y - y1;
-        const double d1 = r1 * k.y, ds = r0 * k.x + d1;
-        r[p] = make_double2(r0, r1);
-        d[p] = make_double2(ds, d1);
-        w[p] = make_double2(up.x + ds, up.y + d1);
-    }
-};
-// u = w + (c1 d + c2 D^{-1} (r - A d)) in plain (v, u) form from w and d in
-// (v + u, u) form
-struct EpiPost2X {
-    const double2 *__restrict__ r;
-    const double2 *__restrict__ d;     // (v + u, u)
-    const double2 *__restrict__ idc2;
-    const double2 *__restrict__ w;     // (v + u, u)
-    double2 *__restrict__ u;
-    double c1;
-    __device__ __forceinline__ double2 value(int p, double y0, double y1) const
-    {
-        const double2 rp_ = r[p], dp = d[p], k = idc2[p], wp = w[p];
-        const double m0 = k.x * (rp_.x - y0), m1 = k.y * (rp_.y - y1);
-        const double uu = wp.y + fma(c1, dp.y, m1);
-        const double us = wp.x + fma(c1, dp.x, m0 + m1);
-        return make_double2(us - uu, uu);
-    }
-    __device__ __forceinline__ void operator()(int p, double y0, double y1) const { u[p] = value(p, y0, y1); }
 };
 
 // ------------------------------------------------------------------ per-level views
@@ -404,39 +270,10 @@ template <class S> struct LV {
     const S *Av, *Pv, *Rv;
     const v2<S> *invd;
     v2<S> *f, *u, *r, *d, *w;
-    const v2<S> *kk;  // finest level, sliced ELL
-    const S *cm;
 };
 
 template <class S> static LV<S> view(amg_hierarchy *h, int l);
 
-// The smoothing epilogues of a level: the (v + u, u)-form ones with scaled
-// inverse diagonals on the FP64 sliced-ELL finest level (SU), the plain ones
-// elsewhere.
-template <class S, bool SU>
-static auto epi_pre(const Level &L, const LV<S> &lv, const v2<S> *f, v2<S> *d0, v2<S> *u)
-{
-    if constexpr (SU && std::is_same<S, double>::value)
-        return EpiPreX{f, (const double2 *)L.idc2.p, d0, u, 1.0 + L.ch_c1};
-    else
-        return EpiPre<S, SU>{f, lv.invd, d0, u, (S)L.ch_c1, (S)L.ch_c2};
-}
-template <class S, bool SU>
-static auto epi_post1(const Level &L, const LV<S> &lv, const v2<S> *f, v2<S> *u)
-{
-    if constexpr (SU && std::is_same<S, double>::value)
-        return EpiPost1X{f, (const double2 *)L.idt.p, u, lv.r, lv.d, lv.w};
-    else
-        return EpiPost1<S, SU>{f, lv.invd, u, lv.r, lv.d, lv.w, (S)L.ch_inv_theta};
-}
-template <class S, bool SU>
-static auto epi_post2(const Level &L, const LV<S> &lv, v2<S> *u)
-{
-    if constexpr (SU && std::is_same<S, double>::value)
-        return EpiPost2X{lv.r, lv.d, (const double2 *)L.idc2.p, lv.w, u, L.ch_c1};
-    else
-        return EpiPost2<S, SU>{lv.r, lv.d, lv.invd, lv.w, u, (S)L.ch_c1, (S)L.ch_c2};
-}
 template <> LV<double> view<double>(amg_hierarchy *h, int l)
 {
     Level &L = h->lev[l];
@@ -450,8 +287,6 @@ template <> LV<double> view<double>(amg_hierarchy *h, int l)
     v.r = (double2 *)L.r.p;
     v.d = (double2 *)L.d.p;
     v.w = (double2 *)L.w.p;
-    v.kk = (const double2 *)h->sell.kk.p;
-    v.cm = h->sell.cm.p;
     return v;
 }
 template <> LV<float> view<float>(amg_hierarchy *h, int l)
@@ -467,8 +302,6 @@ template <> LV<float> view<float>(amg_hierarchy *h, int l)
     v.r = (float2 *)L.r32.p;
     v.d = (float2 *)L.d32.p;
     v.w = (float2 *)L.w32.p;
-    v.kk = (const float2 *)h->sell.kk32.p;
-    v.cm = h->sell.cm32.p;
     return v;
 }
 
@@ -608,121 +441,154 @@ static int lanes_rule(const BSR &A, bool fp32, bool sliced_ok)
     return lanes_for(A, fp32);
 }
 
-__global__ void k_sell_width(int N, const int *__restrict__ rp, int *__restrict__ w, int nslices)
-{
-    int sl = blockIdx.x * blockDim.x + threadIdx.x;
-    if (sl >= nslices) return;
-    int mx = 0;
-    for (int p = sl * 32; p < sl * 32 + 32 && p < N; p++) mx = max(mx, rp[p + 1] - rp[p]);
-    w[sl] = mx;
-}
+// ------------------------------------------------------------------ finest level, layered stencil
+__device__ __forceinline__ int fine_rep(int t, int n) { return t == 0 ? 0 : (t == 2 ? n - 1 : 1); }
 
-// Node k = i + X (j + Y l) (X = nx+1, Y = ny+1); the neighbour q of p sits
-// at stencil position 9 (lq - lp + 1) + 3 (jq - jp + 1) + (iq - ip + 1).
-__global__ void k_sell_fill(int N, int X, int Y, const int *__restrict__ rp, const int *__restrict__ ci,
-                            const double *__restrict__ Ki, const double *__restrict__ Ke,
-                            const double *__restrict__ M, double c, const int *__restrict__ sptr,
-                            int *__restrict__ col, unsigned char *__restrict__ code, double2 *__restrict__ kk,
-                            double *__restrict__ cm, int *__restrict__ bad)
+// Raw row of every (plane, row type), read from a node of that kind.  Types a
+// thin slab does not have (no interior with two nodes across) hold zeros.
+__global__ void k_fine_raw(int NX, int NY, int NZ, const int *__restrict__ rp, const double *__restrict__ Ki,
+                           const double *__restrict__ Ke, const double *__restrict__ M, double c,
+                           const double *__restrict__ invd, double *__restrict__ raw)
 {
-    int p = blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= N) return;
-    int sl = p >> 5, lane = p & 31;
-    int j0 = sptr[sl], width = sptr[sl + 1] - j0, b = rp[p], len = rp[p + 1] - b;
-    const int ip = p % X, jp = (p / X) % Y, lp = p / (X * Y);
-    for (int j = 0; j < width; j++) {
-        size_t idx = (size_t)(j0 + j) * 32 + lane;
-        if (j < len) {
-            const int q = ci[b + j];
-            const int di = q % X - ip, dj = (q / X) % Y - jp, dl = q / (X * Y) - lp;
-            if (di < -1 || di > 1 || dj < -1 || dj > 1 || dl < -1 || dl > 1) {
-                atomicOr(bad, 1);
-                col[idx] = p;
-                code[idx] = 13;
-                kk[idx] = make_double2(0.0, 0.0);
-                continue;
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= 9 * NZ) return;
+    const int l = t / 9, ti = t % 3, tj = (t % 9) / 3;
+    double *o = raw + (size_t)t * kFineRaw;
+    for (int k = 0; k < kFineRaw; k++) o[k] = 0.0;
+    if ((ti == 1 && NX < 3) || (tj == 1 && NY < 3)) return;
+    const int p = fine_rep(ti, NX) + NX * (fine_rep(tj, NY) + NY * l);
+    int b = rp[p];
+    for (int dz = -1; dz <= 1; dz++)
+        for (int dy = -1; dy <= 1; dy++)
+            for (int dx = -1; dx <= 1; dx++) {
+                if ((dx < 0 && ti == 0) || (dx > 0 && ti == 2) || (dy < 0 && tj == 0) || (dy > 0 && tj == 2) ||
+                    l + dz < 0 || l + dz >= NZ)
+                    continue;
+                const int k = 9 * (dz + 1) + 3 * (dy + 1) + dx + 1;
+                o[2 * k] = Ki[b];
+                o[2 * k + 1] = Ke[b];
+                b++;
             }
-            col[idx] = q;
-            code[idx] = (unsigned char)(9 * (dl + 1) + 3 * (dj + 1) + (di + 1));
-            kk[idx] = make_double2(Ki[b + j], Ke[b + j]);
-        } else {
-            col[idx] = p;
-            code[idx] = 13;  // the row itself, with zero weights
-            kk[idx] = make_double2(0.0, 0.0);
-        }
-    }
-    cm[p] = c * M[p];
+    o[54] = c * M[p];
+    o[55] = invd[2 * p];
+    o[56] = invd[2 * p + 1];
 }
 
-int build_fine_sell(amg_hierarchy *h, const bd_system *sys, cudaStream_t s)
+// bad[0]: a node whose row is not its type's (the assembled system was
+// corrupted); bad[1]: a row that is not symmetric under (dx, dy) -> (-dx, -dy)
+// beyond the rounding of its sums.
+__global__ void k_fine_check(int NX, int NY, int NZ, const int *__restrict__ rp, const int *__restrict__ ci,
+                             const double *__restrict__ Ki, const double *__restrict__ Ke,
+                             const double *__restrict__ raw, int *__restrict__ bad)
 {
-    FineSell &F = h->sell;
-    const int N = sys->N;
-    F.nslices = (N + 31) / 32;
-    DBuf<int> w;
-    BD_TRY(w.alloc((size_t)F.nslices + 1));
-    BD_TRY(F.sptr.alloc((size_t)F.nslices + 1));
-    k_sell_width<<<(F.nslices + 255) / 256, 256, 0, s>>>(N, sys->A.rp.p, w.p, F.nslices); ::bd::note_launch();
-    BD_LAUNCH_CHECK();
-    long long slots = 0;
-    BD_TRY(exclusive_scan(w.p, F.sptr.p, F.nslices, &slots, s));
-    F.slots = slots;
-    BD_TRY(F.col.alloc((size_t)slots * 32));
-    BD_TRY(F.code.alloc((size_t)slots * 32));
-    BD_TRY(F.kk.alloc((size_t)slots * 64));
-    BD_TRY(F.cm.alloc((size_t)N));
+    const int N = NX * NY * NZ;
+    for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < N; p += gridDim.x * blockDim.x) {
+        const int i = p % NX, j = (p / NX) % NY, l = p / (NX * NY);
+        const int ti = i == 0 ? 0 : (i == NX - 1 ? 2 : 1), tj = j == 0 ? 0 : (j == NY - 1 ? 2 : 1);
+        const double *o = raw + (size_t)(9 * l + 3 * tj + ti) * kFineRaw;
+        int b = rp[p];
+        bool same = true, sym = true;
+        const double tol0 = 16.0 * 0x1p-52 * fabs(o[26]), tol1 = 16.0 * 0x1p-52 * fabs(o[27]);
+        for (int k = 0; k < 27; k++) {
+            const int dx = k % 3 - 1, dy = (k / 3) % 3 - 1, dz = k / 9 - 1;
+            if (i + dx < 0 || i + dx >= NX || j + dy < 0 || j + dy >= NY || l + dz < 0 || l + dz >= NZ) continue;
+            if (b < rp[p + 1])
+                same = same && ci[b] == p + dx + NX * (dy + NY * dz) && Ki[b] == o[2 * k] && Ke[b] == o[2 * k + 1];
+            b++;
+            if (i - dx < 0 || i - dx >= NX || j - dy < 0 || j - dy >= NY) continue;
+            const int m = 9 * (dz + 1) + 3 * (1 - dy) + 1 - dx;
+            sym = sym && fabs(o[2 * k] - o[2 * m]) <= tol0 && fabs(o[2 * k + 1] - o[2 * m + 1]) <= tol1;
+        }
+        if (!same || b != rp[p + 1]) atomicOr(bad, 1);
+        if (!sym) atomicOr(bad + 1, 1);
+    }
+}
+
+int build_fine_stencil(amg_hierarchy *h, const bd_system *sys, cudaStream_t s)
+{
+    FineStencil &F = h->fine;
+    F.NX = sys->mesh.nx + 1;
+    F.NY = sys->mesh.ny + 1;
+    F.NZ = sys->mesh.nz + 1;
+    BD_TRY(F.raw.alloc((size_t)9 * F.NZ * kFineRaw));
     DBuf<int> bad;
-    BD_TRY(bad.alloc(1));
-    BD_CUDA(cudaMemsetAsync(bad.p, 0, sizeof(int), s));
-    const int X = sys->mesh.nx + 1, Y = sys->mesh.ny + 1;
-    for (int dl = 0; dl < 3; dl++)
-        for (int dj = 0; dj < 3; dj++)
-            for (int di = 0; di < 3; di++)
-                F.off[9 * dl + 3 * dj + di] = (dl - 1) * X * Y + (dj - 1) * X + (di - 1);
+    BD_TRY(bad.alloc(2));
+    BD_CUDA(cudaMemsetAsync(bad.p, 0, 2 * sizeof(int), s));
     const bd_params &P = sys->params;
-    k_sell_fill<<<(N + 255) / 256, 256, 0, s>>>(N, X, Y, sys->A.rp.p, sys->A.ci.p, sys->Ki.p, sys->Ke.p,
-                                                sys->M.p, (P.chi * P.cm) / P.dt, F.sptr.p, F.col.p, F.code.p,
-                                                (double2 *)F.kk.p, F.cm.p, bad.p); ::bd::note_launch();
+    k_fine_raw<<<(9 * F.NZ + 63) / 64, 64, 0, s>>>(F.NX, F.NY, F.NZ, sys->A.rp.p, sys->Ki.p, sys->Ke.p, sys->M.p,
+                                                   (P.chi * P.cm) / P.dt, h->lev[0].invdiag.p, F.raw.p);
+    ::bd::note_launch();
+    k_fine_check<<<grid_for(sys->N, 256), 256, 0, s>>>(F.NX, F.NY, F.NZ, sys->A.rp.p, sys->A.ci.p, sys->Ki.p,
+                                                       sys->Ke.p, F.raw.p, bad.p);
+    ::bd::note_launch();
     BD_LAUNCH_CHECK();
-    int hbad = 0;
-    BD_CUDA(cudaMemcpyAsync(&hbad, bad.p, sizeof(int), cudaMemcpyDeviceToHost, s));
+    int hbad[2] = {0, 0};
+    BD_CUDA(cudaMemcpyAsync(hbad, bad.p, sizeof(hbad), cudaMemcpyDeviceToHost, s));
     BD_CUDA(cudaStreamSynchronize(s));
-    if (hbad) return BD_EINVAL;  // not a 27-point pattern: the assembled system was corrupted
+    if (hbad[0]) return BD_EINVAL;
+    F.sym = !hbad[1];
     F.valid = true;
     return BD_OK;
 }
 
-static Stencil stencil_of(const FineSell &F)
+// Packed row from a raw one; a pair's coefficient is taken from its member
+// that exists on this row type.
+template <bool SYM>
+__global__ void k_fine_pack(int rows, const double *__restrict__ raw, double c2, double it, double *__restrict__ tab,
+                            float *__restrict__ tab32)
 {
-    Stencil st;
-    for (int i = 0; i < 27; i++) st.off[i] = F.off[i];
-    return st;
+    using Row = FineRow<SYM>;
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= rows) return;
+    const double *o = raw + (size_t)t * kFineRaw;
+    const int ti = t % 3, tj = (t % 9) / 3;
+    auto put = [&](int k, double x, double y) {
+        const size_t e = (size_t)t * Row::LEN + k;
+        if (tab) ((double2 *)tab)[e] = make_double2(x, y);
+        if (tab32) ((float2 *)tab32)[e] = make_float2((float)x, (float)y);
+    };
+    for (int z = 0; z < (SYM ? 2 : 3); z++) {
+        const int b = 9 * (z == 0 ? 1 : (z == 1 ? 2 : 0));  // dz = 0, +1, -1
+        for (int k = 0; k < Row::NP; k++) {
+            int q = k;
+            if (SYM) {
+                if (k == 0) q = 4;
+                else if (k == 1) q = ti == 2 ? 3 : 5;
+                else if (k == 2) q = tj == 2 ? 1 : 7;
+                else if (k == 3) q = (ti == 2 || tj == 2) ? 0 : 8;
+                else q = (ti == 2 || tj == 0) ? 6 : 2;
+            }
+            put(z * Row::G + k, o[2 * (b + q)], o[2 * (b + q) + 1]);
+        }
+        put(z * Row::G + Row::NP, z == 0 ? o[54] : 0.0, 0.0);
+    }
+    put(Row::IDC2, c2 * o[55], c2 * o[56]);
+    put(Row::IDT, o[55] * it, o[56] * it);
 }
 
-// operator application of level l in precision S: sliced ELL on the finest
-// level when available, 2x2-block CSR otherwise.  SU (sliced ELL only): the
-// gathered vector is in (v + u, u) form.
-template <bool SU = false, class S, class G, class E>
-static int apply_level(amg_hierarchy *h, int l, const LV<S> &lv, G g, E e, cudaStream_t s)
+int fine_pack(const FineStencil &F, bool sym, double c2, double inv_theta, double *tab, float *tab32, cudaStream_t s)
 {
-    const Level &L = h->lev[l];
-    if (l == 0 && h->sell.valid) {
-        const FineSell &F = h->sell;
-        const long long slices = ((long long)L.N + 31) / 32;
-        if (sizeof(S) == 8 && fine_wide(L.N)) {
-            k_sell<S, G, E, SU, 1, kFineTPB><<<(int)std::min<long long>(slices, kSM), kFineTPB, 0, s>>>(
-                L.N, F.sptr.p, F.col.p, F.code.p, stencil_of(F), lv.kk, lv.cm, g, e);
-        } else {
-            constexpr int MB = sizeof(S) == 8 ? 4 : 8;  // FP64: fewer, deeper-pipelined threads
-            k_sell<S, G, E, SU, MB><<<(int)std::min<long long>(slices, (long long)kSM * MB), 256, 0, s>>>(
-                L.N, F.sptr.p, F.col.p, F.code.p, stencil_of(F), lv.kk, lv.cm, g, e);
-        }
-        ::bd::note_launch();
-        BD_LAUNCH_CHECK();
-        return BD_OK;
-    }
-    if constexpr (SU) return BD_EINVAL;
-    else return apply_op<S>(L, 0, lv.Av, g, e, s);
+    const int rows = 9 * F.NZ, grid = (rows + 63) / 64;
+    if (sym) k_fine_pack<true><<<grid, 64, 0, s>>>(rows, F.raw.p, c2, inv_theta, tab, tab32);
+    else k_fine_pack<false><<<grid, 64, 0, s>>>(rows, F.raw.p, c2, inv_theta, tab, tab32);
+    ::bd::note_launch();
+    BD_LAUNCH_CHECK();
+    return BD_OK;
+}
+
+// One finest-level launch: make(SYM) gives the epilogue for the table's form.
+template <class S, bool SU, class F>
+static int fine_apply(const amg_hierarchy *h, const v2<S> *x, F make, cudaStream_t s)
+{
+    const FineGrid g = fine_grid<S>(h->fine, h->lev[0].ch_c1);
+    const long long units = (long long)g.ncb * g.NZ;
+    if (h->fine.sym)
+        k_fine<S, true, SU><<<fine_blocks<S, true>(units), kFineTPB, 0, s>>>(g, x, make(std::true_type{}));
+    else
+        k_fine<S, false, SU><<<fine_blocks<S, false>(units), kFineTPB, 0, s>>>(g, x, make(std::false_type{}));
+    ::bd::note_launch();
+    BD_LAUNCH_CHECK();
+    return BD_OK;
 }
 
 // ------------------------------------------------------------------ live kernel timing
@@ -785,45 +651,42 @@ void prof_collect(amg_hierarchy *h)
 }
 
 // Algorithmic bytes of one finest-level operator application in precision S:
-// the stored matrix once (sliced ELL: Ki, Ke and a 4-byte column (FP64) or a
-// 1-byte stencil code (FP32) per slot incl. padding, slice offsets, c M;
-// block CSR: four values and a column per block, row offsets) and `vec`
-// per-node vector streams of two S each.
+// the operator once (the stencil's table; block CSR: four values and a column
+// per block, row offsets) and `vec` per-node vector streams of two S each.
 template <class S>
 static double fine_bytes(const amg_hierarchy *h, const Level &L, int vec)
 {
     const double sz = (double)sizeof(S);
-    double mat = h->sell.valid ? (2 * sz + (sz == 4 ? 1.0 : 4.0)) * 32.0 * (double)h->sell.slots +
-                                     4.0 * (h->sell.nslices + 1) + sz * L.N
+    double mat = h->fine.valid ? 2 * sz * fine_row_len(h->fine.sym) * 9.0 * h->fine.NZ
                                : (4 * sz + 4.0) * (double)L.A.nb + 4.0 * (L.N + 1);
     return mat + 2 * sz * vec * (double)L.N;
 }
-// Flops one finest-level launch executes (an FMA counts 2): sliced ELL 2 FMA
-// per stored slot with the gathered vector in (v + u, u) form, 2 FMA and an
-// add otherwise; block CSR 4 FMA per 2x2 block.  The epilogue's few flops per
-// node are not counted.
-static double fine_flops(const amg_hierarchy *h, const Level &L, bool su)
+// FP64 pipe operations per node of the stencil (a fused multiply-add, an add
+// and a multiply count one each): two operators of 4 adds and 15 FMA in the
+// symmetric form, 27 FMA in the general one, and the row tail (c M v + a, a + b
+// and v = (v + u) - u).
+static double fine_node_ops(const amg_hierarchy *h) { return (h->fine.sym ? 38.0 : 54.0) + 3.0; }
+// Flops one finest-level launch executes (an FMA counts 2); the epilogue's few
+// per node are not counted.
+static double fine_flops(const amg_hierarchy *h, const Level &L)
 {
-    if (h->sell.valid) return (su ? 4.0 : 5.0) * 32.0 * (double)h->sell.slots;
+    if (h->fine.valid) return (h->fine.sym ? 68.0 : 108.0) * L.N;
     return 8.0 * (double)L.A.nb;
 }
-// FP64 pipe operations (a fused multiply-add, an add and a multiply count one
-// each: what the pipe issues) of one finest-level launch of the FP64 V-cycle
-// or of the PCG's A p: per stored slot the 2 FMA of the (v + u, u) form, per
-// node the row tail (c M v + a, a + b, and v = (v + u) - u) and the fused
-// step as its epilogue issues it: pre-smoother 6, residual 2, first
-// post-smoothing half 6, second half 10 (14 with the PCG's z statistics),
-// A p with p.Ap 2.  The FP32 V-cycle's launches issue FP64 operations only
-// for the z statistics (conversions and sums, 10 per node).  Block-CSR finest
-// levels: 4 FMA per 2x2 block, epilogues not counted.
+// FP64 pipe operations of one finest-level launch of the FP64 V-cycle or of the
+// PCG's A p: the stencil's per node and the fused step as its epilogue issues
+// it: pre-smoother 7, residual 2, first post-smoothing half 4, second half 11
+// (16 with the PCG's z statistics), A p with p.Ap 2.  The FP32 V-cycle's
+// launches issue none.  Block-CSR finest levels: 4 FMA per 2x2 block,
+// epilogues not counted.
 enum FineRole { FR_PRE, FR_RESID, FR_POST1, FR_POST2, FR_POST2Z, FR_AP };
 template <class S>
 static double fine_ops(const amg_hierarchy *h, const Level &L, int role)
 {
-    if (!h->sell.valid) return sizeof(S) == 8 || role == FR_AP ? 4.0 * (double)L.A.nb : 0.0;
-    if (sizeof(S) == 4 && role != FR_AP) return role == FR_POST2Z ? 10.0 * L.N : 0.0;
-    static const double epi[] = {6.0, 2.0, 6.0, 10.0, 14.0, 2.0};
-    return 2.0 * 32.0 * (double)h->sell.slots + (3.0 + epi[role]) * (double)L.N;
+    if (!h->fine.valid) return sizeof(S) == 8 || role == FR_AP ? 4.0 * (double)L.A.nb : 0.0;
+    if (sizeof(S) == 4 && role != FR_AP) return 0.0;
+    static const double epi[] = {7.0, 2.0, 4.0, 11.0, 16.0, 2.0};
+    return (fine_node_ops(h) + epi[role]) * (double)L.N;
 }
 
 // ------------------------------------------------------------------ coarsest level
@@ -934,13 +797,6 @@ __global__ void k_out64(int N, const float2 *__restrict__ u, double2 *__restrict
     }
 }
 
-__global__ void k_scale_vec(long long n, const double *__restrict__ a, double c, double *__restrict__ b)
-{
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
-         i += (long long)gridDim.x * blockDim.x)
-        b[i] = c * a[i];
-}
-
 __global__ void k_to_f32(long long n, const double *__restrict__ a, float *__restrict__ b)
 {
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
@@ -951,36 +807,41 @@ __global__ void k_to_f32(long long n, const double *__restrict__ a, float *__res
 // The PCG's z statistics computed by the V-cycle's last finest-level kernel
 // (defined with the PCG reductions below).
 struct ZOut;
-static int zo_streams(const ZOut *zo);
-template <class S, bool SU, class E2>
-static int launch_sell_z(amg_hierarchy *h, const LV<S> &lv, const E2 &epi, const ZOut &zo, cudaStream_t s);
+static int launch_fine_z(amg_hierarchy *h, const LV<double> &lv, const double2 *u, const ZOut &zo, cudaStream_t s);
 // FP32 V-cycle output to the PCG's z (FP64) with the z statistics in one pass
 static int launch_z_from32(amg_hierarchy *h, const float2 *u, const ZOut &zo, cudaStream_t s);
 
 // One V-cycle in precision S; f0/u0 are the finest level's right-hand side and
-// output (d0 of the finest level must already be in lev[0]'s d vector).  SU0:
-// the finest level's gathered vectors (d0, the iterate u until the last
-// smoothing step, the post-smoother's d) are kept in (v + u, u) form; the
+// output (d0 of the finest level must already be in lev[0]'s d vector).  On a
+// stencil finest level in FP64 its gathered vectors (d0, the iterate u until the
+// last smoothing step, the post-smoother's d) are kept in (v + u, u) form; the
 // output u0 is in (v, u) form either way.  zo (PCG only): the last
-// post-smoothing step on a sliced-ELL finest level writes the FP64 result to
-// zo->z and sums the z statistics (*zdone set); u0 is then not written.
-template <class S, bool SU0>
+// post-smoothing step on a stencil finest level writes the FP64 result to
+// zo->z and sums the z statistics (*zdone set); u0 then holds the iterate
+// before that step.
+template <class S>
 static int vcycle_impl(amg_hierarchy *h, const v2<S> *f0, v2<S> *u0, cudaStream_t s, const ZOut *zo = nullptr,
                        bool *zdone = nullptr)
 {
+    constexpr bool SU = std::is_same<S, double>::value;
     const int nl = h->nlev;
     const bool deg2 = h->opts.cheb_degree == 2;
-    auto down = [&](int l, auto su) -> int {
-        constexpr bool SU = decltype(su)::value;
+    auto down = [&](int l) -> int {
         Level &L = h->lev[l];
         const LV<S> lv = view<S>(h, l);
+        const bool fine = l == 0 && h->fine.valid;
         const v2<S> *f = l == 0 ? f0 : lv.f;
         v2<S> *u = l == 0 ? u0 : lv.u;
         v2<S> *d0 = lv.d;
         if (deg2) {
             int sl = prof_begin(h, s, 16 * l + R_PRE, l == 0);
-            BD_TRY(apply_level<SU>(h, l, lv, GatherVec<S>{d0}, epi_pre<S, SU>(L, lv, f, d0, u), s));
-            prof_end(h, sl, l == 0 ? fine_bytes<S>(h, L, 4) : 0.0, fine_flops(h, L, SU), s, fine_ops<S>(h, L, FR_PRE));
+            if (fine)
+                BD_TRY((fine_apply<S, SU>(h, d0, [&](auto sym) { return FinePre<S, sym.value, SU>{f, u}; }, s)));
+            else
+                BD_TRY(apply_op<S>(L, 0, lv.Av, GatherVec<S>{d0},
+                                   EpiPre<S>{f, lv.invd, d0, u, (S)L.ch_c1, (S)L.ch_c2}, s));
+            prof_end(h, sl, l == 0 ? fine_bytes<S>(h, L, fine ? 3 : 4) : 0.0, fine_flops(h, L), s,
+                     fine_ops<S>(h, L, FR_PRE));
         } else {
             int sl = prof_begin(h, s, 16 * l + R_PRE, false);
             k_copy2<S><<<grid_for(L.N, 256), 256, 0, s>>>(L.N, d0, u); ::bd::note_launch();
@@ -988,8 +849,11 @@ static int vcycle_impl(amg_hierarchy *h, const v2<S> *f0, v2<S> *u0, cudaStream_
             prof_end(h, sl, 0.0, 0.0, s);
         }
         int sr = prof_begin(h, s, 16 * l + R_RESID, l == 0);
-        BD_TRY(apply_level<SU>(h, l, lv, GatherVec<S>{u}, EpiResid<S>{f, lv.r}, s));
-        prof_end(h, sr, l == 0 ? fine_bytes<S>(h, L, 3) : 0.0, fine_flops(h, L, SU), s, fine_ops<S>(h, L, FR_RESID));
+        if (fine)
+            BD_TRY((fine_apply<S, SU>(h, u, [&](auto sym) { return FineResid<S, sym.value>{f, lv.r}; }, s)));
+        else
+            BD_TRY(apply_op<S>(L, 0, lv.Av, GatherVec<S>{u}, EpiResid<S>{f, lv.r}, s));
+        prof_end(h, sr, l == 0 ? fine_bytes<S>(h, L, 3) : 0.0, fine_flops(h, L), s, fine_ops<S>(h, L, FR_RESID));
         const Level &C = h->lev[l + 1];
         const LV<S> cv = view<S>(h, l + 1);
         int sx = prof_begin(h, s, 16 * l + R_RESTRICT, false);
@@ -998,38 +862,47 @@ static int vcycle_impl(amg_hierarchy *h, const v2<S> *f0, v2<S> *u0, cudaStream_
         prof_end(h, sx, 0.0, 0.0, s);
         return BD_OK;
     };
-    auto up = [&](int l, auto su) -> int {
-        constexpr bool SU = decltype(su)::value;
+    auto up = [&](int l) -> int {
         Level &L = h->lev[l];
         const LV<S> lv = view<S>(h, l);
+        const bool fine = l == 0 && h->fine.valid;
         const v2<S> *f = l == 0 ? f0 : lv.f;
         v2<S> *u = l == 0 ? u0 : lv.u;
         const LV<S> cv = view<S>(h, l + 1);
         int sp = prof_begin(h, s, 16 * l + R_PROLONG, false);
-        BD_TRY(apply_op<S>(L, 2, lv.Pv, GatherVec<S>{cv.u},
-                             EpiAdd<S, SU>{u}, s));
+        if (fine) BD_TRY(apply_op<S>(L, 2, lv.Pv, GatherVec<S>{cv.u}, EpiAdd<S, SU>{u}, s));
+        else BD_TRY(apply_op<S>(L, 2, lv.Pv, GatherVec<S>{cv.u}, EpiAdd<S>{u}, s));
         prof_end(h, sp, 0.0, 0.0, s);
         int s1 = prof_begin(h, s, 16 * l + R_POST1, l == 0);
-        BD_TRY(apply_level<SU>(h, l, lv, GatherVec<S>{u}, epi_post1<S, SU>(L, lv, f, u), s));
-        prof_end(h, s1, l == 0 ? fine_bytes<S>(h, L, 6) : 0.0, fine_flops(h, L, SU), s, fine_ops<S>(h, L, FR_POST1));
+        if (fine)
+            BD_TRY((fine_apply<S, SU>(h, u, [&](auto sym) {
+                return FinePost1<S, sym.value, SU>{f, lv.r, lv.d, deg2 ? nullptr : lv.w};
+            }, s)));
+        else
+            BD_TRY(apply_op<S>(L, 0, lv.Av, GatherVec<S>{u},
+                               EpiPost1<S>{f, lv.invd, u, lv.r, lv.d, lv.w, (S)L.ch_inv_theta}, s));
+        prof_end(h, s1, l == 0 ? fine_bytes<S>(h, L, fine ? 4 : 6) : 0.0, fine_flops(h, L), s,
+                 fine_ops<S>(h, L, FR_POST1));
         if (deg2) {
             int s2 = prof_begin(h, s, 16 * l + R_POST2, l == 0);
-            const auto epi = epi_post2<S, SU>(L, lv, u);
-            double bytes = l == 0 ? fine_bytes<S>(h, L, 5) : 0.0;
+            double bytes = l == 0 ? fine_bytes<S>(h, L, fine ? 4 : 5) : 0.0;
             // FP64: the post-smoother's last kernel carries the PCG's z statistics;
             // FP32: the plain kernel, then one pass that converts u to z and sums
-            // the statistics (faster than carrying the FP64 work in the
-            // HBM-bound FP32 kernel, measured)
-            const bool fuse_z = l == 0 && zo && h->sell.valid && sizeof(S) == 8;
+            // the statistics
+            const bool fuse_z = fine && zo && sizeof(S) == 8;
             if (fuse_z) {
-                BD_TRY((launch_sell_z<S, SU>(h, lv, epi, *zo, s)));
+                if constexpr (SU) BD_TRY(launch_fine_z(h, lv, u, *zo, s));
                 if (zdone) *zdone = true;
-                // u is not stored; z written and the PCG's r (and z_old) read in FP64
-                bytes = fine_bytes<S>(h, L, 4) + 16.0 * L.N * (zo_streams(zo));
+                bytes += 16.0 * L.N;  // u is not stored; z is, and the PCG's r is read
+            } else if (fine) {
+                BD_TRY((fine_apply<S, SU>(h, lv.d, [&](auto sym) {
+                    return FinePost2<S, sym.value, SU>{lv.r, u, u};
+                }, s)));
             } else {
-                BD_TRY(apply_level<SU>(h, l, lv, GatherVec<S>{lv.d}, epi, s));
+                BD_TRY(apply_op<S>(L, 0, lv.Av, GatherVec<S>{lv.d},
+                                   EpiPost2<S>{lv.r, lv.d, lv.invd, lv.w, u, (S)L.ch_c1, (S)L.ch_c2}, s));
             }
-            prof_end(h, s2, bytes, fine_flops(h, L, SU), s, fine_ops<S>(h, L, fuse_z ? FR_POST2Z : FR_POST2));
+            prof_end(h, s2, bytes, fine_flops(h, L), s, fine_ops<S>(h, L, fuse_z ? FR_POST2Z : FR_POST2));
             if (l == 0 && zo && sizeof(S) == 4) {
                 int sz = prof_begin(h, s, R_ZSTATS, false);
                 BD_TRY(launch_z_from32(h, (const float2 *)u, *zo, s));
@@ -1044,8 +917,7 @@ static int vcycle_impl(amg_hierarchy *h, const v2<S> *f0, v2<S> *u0, cudaStream_
         }
         return BD_OK;
     };
-    for (int l = 0; l < nl - 1; l++)
-        BD_TRY(l == 0 ? down(l, std::integral_constant<bool, SU0>{}) : down(l, std::false_type{}));
+    for (int l = 0; l < nl - 1; l++) BD_TRY(down(l));
     {
         const LV<S> cv = view<S>(h, nl - 1);
         const S *f = (const S *)(nl == 1 ? f0 : cv.f);
@@ -1061,8 +933,7 @@ static int vcycle_impl(amg_hierarchy *h, const v2<S> *f0, v2<S> *u0, cudaStream_
         BD_LAUNCH_CHECK();
         prof_end(h, sc, 0.0, 0.0, s);
     }
-    for (int l = nl - 2; l >= 0; l--)
-        BD_TRY(l == 0 ? up(l, std::integral_constant<bool, SU0>{}) : up(l, std::false_type{}));
+    for (int l = nl - 2; l >= 0; l--) BD_TRY(up(l));
     return BD_OK;
 }
 
@@ -1084,7 +955,7 @@ static int vcycle_run(amg_hierarchy *h, const double *r_dev, double *z_dev, cuda
             prof_end(h, si, 0.0, 0.0, s);
         }
         bool zd = false;
-        BD_TRY((vcycle_impl<float, false>(h, v0.f, v0.u, s, zo, &zd)));
+        BD_TRY((vcycle_impl<float>(h, v0.f, v0.u, s, zo, &zd)));
         if (!zd) {
             int so = prof_begin(h, s, R_VOUT, false);
             k_out64<<<grid_for(L0.N, 256), 256, 0, s>>>(L0.N, v0.u, (double2 *)z_dev); ::bd::note_launch();
@@ -1094,9 +965,9 @@ static int vcycle_run(amg_hierarchy *h, const double *r_dev, double *z_dev, cuda
         if (zdone) *zdone = zd;
         return BD_OK;
     }
-    // FP64 sliced ELL: the finest level's gathered vectors in (v + u, u) form
+    // FP64 stencil: the finest level's gathered vectors in (v + u, u) form
     const LV<double> v0 = view<double>(h, 0);
-    const bool su = h->sell.valid;
+    const bool su = h->fine.valid;
     if (h->nlev > 1 && !d0_ready) {
         int si = prof_begin(h, s, R_VIN, false);
         if (su)
@@ -1109,8 +980,7 @@ static int vcycle_run(amg_hierarchy *h, const double *r_dev, double *z_dev, cuda
         BD_LAUNCH_CHECK();
         prof_end(h, si, 0.0, 0.0, s);
     }
-    return su ? vcycle_impl<double, true>(h, (const double2 *)r_dev, (double2 *)z_dev, s, zo, zdone)
-              : vcycle_impl<double, false>(h, (const double2 *)r_dev, (double2 *)z_dev, s, zo, zdone);
+    return vcycle_impl<double>(h, (const double2 *)r_dev, (double2 *)z_dev, s, zo, zdone);
 }
 
 int vcycle_device(amg_hierarchy *h, const double *r_dev, double *z_dev, cudaStream_t s)
@@ -1393,66 +1263,60 @@ __global__ void __launch_bounds__(256) k_bsr_reduce(int N, const int *__restrict
     block_finish<MODE == 0 ? 1 : 2, 256>(acc, xs, 0.0, 0.0, fin);
 }
 
-// Same with the sliced-ELL finest level.  SU: x is stored as (v + u, u), so a
-// node pair costs two FP64 FMAs (a += Ki s, b += Ke u) instead of three.
-template <int MODE, bool SU, int TPB = 256>
-__global__ void __launch_bounds__(TPB, 1024 / TPB) k_sell_reduce(int N, const int *__restrict__ sptr,
-                                                      const int *__restrict__ col,
-                                                      const double2 *__restrict__ kk,
-                                                      const double *__restrict__ cm,
-                                                      const double2 *__restrict__ x,
-                                                      const double2 *__restrict__ f,
-                                                      double2 *__restrict__ out, Fin fin, D0Out d0)
-{
-    double acc = 0.0, xs = 0.0;
-    const int lane = threadIdx.x & 31, e = share_hi(N);
-    for (int p = share_lo(N) + threadIdx.x; p < e; p += blockDim.x) {
-        const int sl = p >> 5;
-        const int j1 = sptr[sl + 1];
-        double a = 0.0, b = 0.0;
-#pragma unroll 8
-        for (int j = sptr[sl]; j < j1; j++) {
-            const size_t idx = (size_t)j * 32 + lane;
-            const int q = col[idx];
-            const double2 k = kk[idx];
-            const double2 xq = x[q];
-            a = fma(k.x, SU ? xq.x : xq.x + xq.y, a);
-            b = fma(k.y, xq.y, b);
-        }
-        const double2 xs2 = x[p];
-        const double vp = SU ? xs2.x - xs2.y : xs2.x, up = xs2.y;
-        const double y0 = fma(cm[p], vp, a), y1 = a + b;
+// The same with the stencil: SU in MODE 0 (the search direction is stored as
+// (v + u, u)), plain in MODE 1.
+template <int MODE> struct FineReduce {
+    const double2 *__restrict__ f;
+    double2 *__restrict__ out;
+    D0Out d0;
+    double acc, xs;
+    __device__ __forceinline__ double2 load(int p, bool ok) const
+    {
+        return MODE == 0 ? make_double2(0.0, 0.0) : fine_ld<double>(f, p, ok);
+    }
+    __device__ __forceinline__ void operator()(int p, const double2 *, double2 fp, double2 c, double, double y0, double y1)
+    {
         if (MODE == 0) {
             out[p] = make_double2(y0, y1);
-            acc = fma(vp, y0, fma(up, y1, acc));
+            acc = fma(c.x - c.y, y0, fma(c.y, y1, acc));
         } else {
-            const double2 fp = f[p];
             const double r0 = fp.x - y0, r1 = fp.y - y1;
             if (out) out[p] = make_double2(r0, r1);
             d0(p, r0, r1);
             acc += r0 * r0 + r1 * r1;
-            xs += up;
+            xs += c.y;
         }
     }
-    block_finish<MODE == 0 ? 1 : 2, TPB>(acc, xs, 0.0, 0.0, fin);
+};
+
+template <int MODE, bool SYM>
+__global__ void __launch_bounds__(kFineTPB, FineMinB<double, SYM>::v)
+    k_fine_reduce(FineGrid g, const double2 *__restrict__ x, FineReduce<MODE> e, Fin fin)
+{
+    fine_block<double, SYM, MODE == 0>(g, x, e);
+    block_finish<MODE == 0 ? 1 : 2, kFineTPB>(e.acc, e.xs, 0.0, 0.0, fin);
+}
+
+template <int MODE, bool SYM>
+static void launch_fine_reduce(const amg_hierarchy *h, const double2 *x, const double2 *f, double2 *out,
+                               const Fin &fin, cudaStream_t s, const D0Out &d0)
+{
+    const FineGrid g = fine_grid<double>(h->fine, h->lev[0].ch_c1);
+    k_fine_reduce<MODE, SYM><<<fine_blocks<double, SYM>((long long)g.ncb * g.NZ), kFineTPB, 0, s>>>(
+        g, x, FineReduce<MODE>{f, out, d0, 0.0, 0.0}, fin);
+    ::bd::note_launch();
 }
 
 // MODE 0 applies A to the search direction (in (v+u, u) form when the finest
-// level is sliced ELL); MODE 1 forms f - A x for an iterate in (v, u) form.
+// level is a stencil); MODE 1 forms f - A x for an iterate in (v, u) form.
 template <int MODE>
 static void fine_reduce(const amg_hierarchy *h, const double2 *x, const double2 *f, double2 *out,
                         const Fin &fin, cudaStream_t s, const D0Out &d0 = D0Out{})
 {
     const Level &L0 = h->lev[0];
-    if (h->sell.valid) {
-        const FineSell &F = h->sell;
-        if (fine_wide(L0.N))
-            k_sell_reduce<MODE, MODE == 0, kFineTPB><<<kSM, kFineTPB, 0, s>>>(
-                L0.N, F.sptr.p, F.col.p, (const double2 *)F.kk.p, F.cm.p, x, f, out, fin, d0);
-        else
-            k_sell_reduce<MODE, MODE == 0><<<kSM * 4, 256, 0, s>>>(L0.N, F.sptr.p, F.col.p,
-                                                                  (const double2 *)F.kk.p, F.cm.p, x, f, out, fin, d0);
-        ::bd::note_launch();
+    if (h->fine.valid) {
+        if (h->fine.sym) launch_fine_reduce<MODE, true>(h, x, f, out, fin, s, d0);
+        else launch_fine_reduce<MODE, false>(h, x, f, out, fin, s, d0);
         return;
     }
     const BSR &A = L0.A;
@@ -1495,44 +1359,48 @@ struct ZOut {
     Fin fin;
 };
 
-// FP64: at most 64 registers (32 warps per SM, as the other FP64 finest-level
-// kernels).  FP32 V-cycle: the per-thread partial sums are FP32, the
-// precision z itself comes in (the V-cycle's output, converted exactly), with
-// r and z_old rounded to FP32 for the products; blocks and the grid add the
-// partials in FP64.  That keeps the kernel within 32 registers, so it runs 8
-// blocks per SM like the other FP32 finest-level kernels, which need every
-// resident warp to keep enough bytes in flight.
-template <class S, bool SU, int MINB, class E2, int TPB = 256>
-__global__ void __launch_bounds__(TPB, MINB) k_sell_z(int N, const int *__restrict__ sptr,
-                                                    const int *__restrict__ col,
-                                                    const unsigned char *__restrict__ code, Stencil st,
-                                                    const v2<S> *__restrict__ kk, const S *__restrict__ cm,
-                                                    GatherVec<S> gather, E2 epi, ZOut zo)
-{
-    __shared__ int off[27];
-    if (sizeof(S) == 4) stage_stencil(st, off);
-    S a = 0, b = 0, c = 0, d = 0;
-    const int lane = threadIdx.x & 31, e = share_hi(N);
-    for (int p = share_lo(N) + threadIdx.x; p < e; p += blockDim.x) {
-        S y0, y1;
-        sell_row<S, GatherVec<S>, SU, (sizeof(S) == 8 ? 8 : 4)>(p, lane, sptr, col, code, off, kk, cm, gather, y0,
-                                                                 y1);
-        const v2<S> u = epi.value(p, y0, y1);
-        const double2 z = make_double2((double)u.x, (double)u.y), r = zo.r[p];
-        zo.z[p] = z;
-        const S rx = (S)r.x, ry = (S)r.y;
+template <bool SYM> struct FineZ {
+    FinePost2<double, SYM, true> post;
+    double2 *z;  // may be the iterate's own storage
+    const double2 *__restrict__ r;
+    double a, b, c;
+    struct Pre {
+        typename FinePost2<double, SYM, true>::Pre q;
+        double2 r;
+    };
+    __device__ __forceinline__ Pre load(int p, bool ok) const { return {post.load(p, ok), fine_ld<double>(r, p, ok)}; }
+    __device__ __forceinline__ void operator()(int p, const double2 *t, const Pre &q, double2 x, double c1, double y0, double y1)
+    {
+        const double2 u = post.value(t, q.q, x, c1, y0, y1);
+        z[p] = u;
         a += u.y;
-        b += ry;
-        c = fma(rx, u.x, fma(ry, u.y, c));
-        if (zo.zold) {
-            const double2 o = zo.zold[p];
-            d = fma(rx, (S)o.x, fma(ry, (S)o.y, d));
-        }
+        b += q.r.y;
+        c = fma(q.r.x, u.x, fma(q.r.y, u.y, c));
     }
-    block_finish<4, TPB>((double)a, (double)b, (double)c, (double)d, zo.fin);
+};
+
+template <bool SYM>
+__global__ void __launch_bounds__(kFineTPB, FineMinB<double, SYM>::v)
+    k_fine_z(FineGrid g, const double2 *__restrict__ x, FineZ<SYM> e, Fin fin)
+{
+    fine_block<double, SYM, true>(g, x, e);
+    block_finish<3, kFineTPB>(e.a, e.b, e.c, 0.0, fin);
 }
 
-static int zo_streams(const ZOut *zo) { return zo->zold ? 3 : 2; }
+static int launch_fine_z(amg_hierarchy *h, const LV<double> &lv, const double2 *u, const ZOut &zo, cudaStream_t s)
+{
+    const FineGrid g = fine_grid<double>(h->fine, h->lev[0].ch_c1);
+    auto launch = [&](auto sym) {
+        constexpr bool SYM = decltype(sym)::value;
+        k_fine_z<SYM><<<fine_blocks<double, SYM>((long long)g.ncb * g.NZ), kFineTPB, 0, s>>>(
+            g, lv.d, FineZ<SYM>{{lv.r, u, nullptr}, zo.z, zo.r, 0.0, 0.0, 0.0}, zo.fin);
+    };
+    if (h->fine.sym) launch(std::true_type{});
+    else launch(std::false_type{});
+    ::bd::note_launch();
+    BD_LAUNCH_CHECK();
+    return BD_OK;
+}
 
 // z = (double) u of the FP32 V-cycle, and its statistics (z_u, r_u, r.z,
 // r.z_old) in FP64 (stage 3), in one pass
@@ -1557,25 +1425,6 @@ __global__ void k_z_from32(int N, const float2 *__restrict__ u, ZOut zo)
 static int launch_z_from32(amg_hierarchy *h, const float2 *u, const ZOut &zo, cudaStream_t s)
 {
     k_z_from32<<<kVecBlocks, kVecThreads, 0, s>>>(h->lev[0].N, u, zo);
-    ::bd::note_launch();
-    BD_LAUNCH_CHECK();
-    return BD_OK;
-}
-
-template <class S, bool SU, class E2>
-static int launch_sell_z(amg_hierarchy *h, const LV<S> &lv, const E2 &epi, const ZOut &zo, cudaStream_t s)
-{
-    const FineSell &F = h->sell;
-    const int N = h->lev[0].N;
-    const long long slices = ((long long)N + 31) / 32;
-    if (sizeof(S) == 8 && fine_wide(N)) {
-        k_sell_z<S, SU, 1, E2, kFineTPB><<<(int)std::min<long long>(slices, kSM), kFineTPB, 0, s>>>(
-            N, F.sptr.p, F.col.p, F.code.p, stencil_of(F), lv.kk, lv.cm, GatherVec<S>{lv.d}, epi, zo);
-    } else {
-        constexpr int MB = sizeof(S) == 8 ? 4 : 8;
-        k_sell_z<S, SU, MB, E2><<<(int)std::min<long long>(slices, (long long)kSM * MB), 256, 0, s>>>(
-            N, F.sptr.p, F.col.p, F.code.p, stencil_of(F), lv.kk, lv.cm, GatherVec<S>{lv.d}, epi, zo);
-    }
     ::bd::note_launch();
     BD_LAUNCH_CHECK();
     return BD_OK;
@@ -1636,7 +1485,7 @@ __global__ void k_project_x(int N, double2 *__restrict__ x, const double *__rest
 static void p_update(const amg_hierarchy *h, int N, double2 *z, double2 *p, double2 *zold, double *scal,
                      int first, cudaStream_t s)
 {
-    if (h->sell.valid) k_p_update<true><<<kVecBlocks, kVecThreads, 0, s>>>(N, z, p, zold, scal, first);
+    if (h->fine.valid) k_p_update<true><<<kVecBlocks, kVecThreads, 0, s>>>(N, z, p, zold, scal, first);
     else k_p_update<false><<<kVecBlocks, kVecThreads, 0, s>>>(N, z, p, zold, scal, first);
     note_launch();
 }
@@ -1644,7 +1493,7 @@ static void p_update(const amg_hierarchy *h, int N, double2 *z, double2 *p, doub
 static void xr_update(const amg_hierarchy *h, int N, double2 *x, double2 *r, const double2 *p,
                       const double2 *q, const Fin &fin, cudaStream_t s, const D0Out &d0)
 {
-    if (h->sell.valid) k_xr_update<true><<<kVecBlocks, kVecThreads, 0, s>>>(N, x, r, p, q, fin, d0);
+    if (h->fine.valid) k_xr_update<true><<<kVecBlocks, kVecThreads, 0, s>>>(N, x, r, p, q, fin, d0);
     else k_xr_update<false><<<kVecBlocks, kVecThreads, 0, s>>>(N, x, r, p, q, fin, d0);
     note_launch();
 }
@@ -1662,7 +1511,7 @@ static D0Out d0_out(amg_hierarchy *h)
         d.invd32 = (const float2 *)L0.invdiag32.p;
         d.it32 = (float)L0.ch_inv_theta;
     } else if (h->nlev > 1) {
-        d.mode = h->sell.valid ? 1 : 2;
+        d.mode = h->fine.valid ? 1 : 2;
         d.d64 = (double2 *)L0.d.p;
         d.invd64 = (const double2 *)L0.invdiag.p;
         d.it = L0.ch_inv_theta;
@@ -1759,7 +1608,7 @@ static int autotune_lanes(amg_hierarchy *h, cudaStream_t s)
         Level &L = h->lev[l];
         const LV<S> lv = view<S>(h, l), cv = view<S>(h, l + 1);
         for (int op = 0; op < 3 && st == BD_OK; op++) {
-            if (op == 0 && l == 0 && h->sell.valid) continue;
+            if (op == 0 && l == 0 && h->fine.valid) continue;
             const BSR &M = op == 0 ? L.A : (op == 1 ? L.R : L.P);
             if (M.nb < kTuneMinBlocks) continue;
             const S *vals = op == 0 ? lv.Av : (op == 1 ? lv.Rv : lv.Pv);
@@ -1790,9 +1639,12 @@ int prepare_solve(amg_hierarchy *h, cudaStream_t s)
             BD_TRY(L.d32.alloc(n));
             BD_TRY(L.w32.alloc(n));
             BD_TRY(L.invdiag32.alloc(n));
-            BD_TRY(L.A32.alloc(4 * (size_t)L.A.nb));
+            const bool a32 = l > 0 || !h->fine.valid;  // the stencil has its own FP32 table
+            if (a32) BD_TRY(L.A32.alloc(4 * (size_t)L.A.nb));
             k_to_f32<<<grid_for(n, 256), 256, 0, s>>>((long long)n, L.invdiag.p, L.invdiag32.p); ::bd::note_launch();
-            k_to_f32<<<grid_for(4 * L.A.nb, 256), 256, 0, s>>>(4 * L.A.nb, L.A.v.p, L.A32.p); ::bd::note_launch();
+            if (a32) {
+                k_to_f32<<<grid_for(4 * L.A.nb, 256), 256, 0, s>>>(4 * L.A.nb, L.A.v.p, L.A32.p); ::bd::note_launch();
+            }
             if (l < h->nlev - 1) {
                 BD_TRY(L.P32.alloc(4 * (size_t)L.P.nb));
                 BD_TRY(L.R32.alloc(4 * (size_t)L.R.nb));
@@ -1815,26 +1667,15 @@ int prepare_solve(amg_hierarchy *h, cudaStream_t s)
             L.ch_inv_theta = 1.0 / theta;
             L.ch_c1 = rho1 * rho0;
             L.ch_c2 = 2.0 * rho1 / delta;
-            if (l == 0 && !p32 && h->sell.valid) {
-                // the FP64 finest level's scaled inverse diagonals (EpiPreX and kin)
-                BD_TRY(L.idc2.alloc(n));
-                BD_TRY(L.idt.alloc(n));
-                k_scale_vec<<<grid_for(n, 256), 256, 0, s>>>((long long)n, L.invdiag.p, L.ch_c2, L.idc2.p);
-                ::bd::note_launch();
-                k_scale_vec<<<grid_for(n, 256), 256, 0, s>>>((long long)n, L.invdiag.p, L.ch_inv_theta, L.idt.p);
-                ::bd::note_launch();
-                BD_LAUNCH_CHECK();
-            }
         }
     }
-    if (p32 && h->sell.valid) {
-        FineSell &F = h->sell;
-        size_t nk = 64 * (size_t)F.slots;
-        BD_TRY(F.kk32.alloc(nk));
-        BD_TRY(F.cm32.alloc((size_t)h->lev[0].N));
-        k_to_f32<<<grid_for(nk, 256), 256, 0, s>>>((long long)nk, F.kk.p, F.kk32.p); ::bd::note_launch();
-        k_to_f32<<<grid_for(h->lev[0].N, 256), 256, 0, s>>>(h->lev[0].N, F.cm.p, F.cm32.p); ::bd::note_launch();
-        BD_LAUNCH_CHECK();
+    if (h->fine.valid) {
+        FineStencil &F = h->fine;
+        const Level &L0 = h->lev[0];
+        const size_t len = 2 * (size_t)fine_row_len(F.sym) * 9 * F.NZ;
+        BD_TRY(F.tab.alloc(len));
+        if (p32) BD_TRY(F.tab32.alloc(len));
+        BD_TRY(fine_pack(F, F.sym, L0.ch_c2, L0.ch_inv_theta, F.tab.p, F.tab32.p, s));
     }
     size_t n0 = 2 * (size_t)h->lev[0].N;
     BD_TRY(h->x.alloc(n0));
@@ -1954,7 +1795,7 @@ static int pcg_solve_loop(amg_hierarchy *h, const double *f_dev, double *x_dev, 
             // when the V-cycle is FP64 too (one kernel family per profile)
             int sq = prof_begin(h, s, R_AP, !h->prec32);
             fine_reduce<0>(h, p, nullptr, q, make_fin(h, 4, 0), s);
-            prof_end(h, sq, h->prec32 ? 0.0 : fine_bytes<double>(h, L0, 2), fine_flops(h, L0, true), s,
+            prof_end(h, sq, h->prec32 ? 0.0 : fine_bytes<double>(h, L0, 2), fine_flops(h, L0), s,
                      fine_ops<double>(h, L0, FR_AP));
             int sx = prof_begin(h, s, R_XRUPDATE, false);
             xr_update(h, N, x, r, p, q, make_fin(h, 2, 0), s, d0);
@@ -2391,7 +2232,7 @@ extern "C" int amg_set_level_lanes(amg_hierarchy *h, int level, const int lanes[
     for (int op = 0; op < 3; op++) {
         const int T = lanes[op];
         if (T == 0) continue;
-        const bool applied = !last && !(op == 0 && level == 0 && h->sell.valid);
+        const bool applied = !last && !(op == 0 && level == 0 && h->fine.valid);
         const bool csr_ok = T > 0 && T <= 256 && (T & (T - 1)) == 0;
         const bool sliced_ok = T < 0 && sliced_k_ok(-T) && !(op == 0 && level == 0);
         if (!applied || !(csr_ok || sliced_ok)) return BD_EINVAL;

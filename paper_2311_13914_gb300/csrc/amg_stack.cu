@@ -24,6 +24,7 @@
 
 #include "amg_bsr.cuh"
 #include "amg_internal.cuh"
+#include "fine_stencil.cuh"
 
 namespace bd {
 namespace {
@@ -38,7 +39,7 @@ enum {
 };
 
 // node -> member, and each member's Chebyshev coefficients on one level:
-// coef[4k] = 1/theta, coef[4k+1] = c1, coef[4k+2] = c2, coef[4k+3] = 1 + c1
+// coef[4k] = 1/theta, coef[4k+1] = c1, coef[4k+2] = c2
 struct StCoef {
     const int *__restrict__ mem;
     const double *__restrict__ coef;
@@ -138,26 +139,6 @@ struct StStore {  // q = A p (FP64, PCG)
     __device__ __forceinline__ void operator()(int p, double y0, double y1) const { q[p] = make_double2(y0, y1); }
 };
 
-// The FP64 finest level's steps with the vectors its operator gathers (d0, u,
-// d, w) kept in (v + u, u) form and the inverse diagonal scaled per member
-// (idc2 = c2 D^{-1}, idt = D^{-1} / theta), as the single hierarchy's FP64
-// finest level does them: 2 FMA per stored node pair instead of 3 operations.
-// Pre-smoothing from zero with m = idc2 (f - A d0): u_s = (1 + c1) d0_s + (m_v
-// + m_u), u_u = (1 + c1) d0_u + m_u.
-struct StPreX {
-    const double2 *__restrict__ f;
-    const double2 *__restrict__ idc2;
-    const double2 *__restrict__ d0;  // (v + u, u)
-    double2 *__restrict__ u;         // (v + u, u)
-    StCoef c;
-    __device__ __forceinline__ void operator()(int p, double y0, double y1) const
-    {
-        const double c1p = c.at(p)[3];
-        const double2 fp = f[p], k = idc2[p], dp = d0[p];
-        const double m0 = k.x * (fp.x - y0), m1 = k.y * (fp.y - y1);
-        u[p] = make_double2(fma(c1p, dp.x, m0 + m1), fma(c1p, dp.y, m1));
-    }
-};
 struct StAddX {  // u += P e_c with u in (v + u, u) form
     double2 *__restrict__ u;
     __device__ __forceinline__ void operator()(int p, double y0, double y1) const
@@ -166,103 +147,6 @@ struct StAddX {  // u += P e_c with u in (v + u, u) form
         u[p] = make_double2(a.x + (y0 + y1), a.y + y1);
     }
 };
-// r = f - A u (plain), d = D^{-1} r / theta and w = u + d in (v + u, u) form
-struct StPost1X {
-    const double2 *__restrict__ f;
-    const double2 *__restrict__ idt;
-    const double2 *__restrict__ u;  // (v + u, u)
-    double2 *__restrict__ r;
-    double2 *__restrict__ d;
-    double2 *__restrict__ w;
-    __device__ __forceinline__ void operator()(int p, double y0, double y1) const
-    {
-        const double2 fp = f[p], k = idt[p], up = u[p];
-        const double r0 = fp.x - y0, r1 = fp.y - y1;
-        const double d1 = r1 * k.y, ds = r0 * k.x + d1;
-        r[p] = make_double2(r0, r1);
-        d[p] = make_double2(ds, d1);
-        w[p] = make_double2(up.x + ds, up.y + d1);
-    }
-};
-// u = w + (c1 d + c2 D^{-1} (r - A d)) in plain (v, u) form (the V-cycle's
-// output) from w and d in (v + u, u) form
-struct StPost2X {
-    const double2 *__restrict__ r;
-    const double2 *__restrict__ d;  // (v + u, u)
-    const double2 *__restrict__ idc2;
-    const double2 *__restrict__ w;  // (v + u, u)
-    double2 *__restrict__ u;
-    StCoef c;
-    __device__ __forceinline__ void operator()(int p, double y0, double y1) const
-    {
-        const double c1 = c.at(p)[1];
-        const double2 rp_ = r[p], dp = d[p], k = idc2[p], wp = w[p];
-        const double m0 = k.x * (rp_.x - y0), m1 = k.y * (rp_.y - y1);
-        const double uu = wp.y + fma(c1, dp.y, m1);
-        const double us = wp.x + fma(c1, dp.x, m0 + m1);
-        u[p] = make_double2(us - uu, uu);
-    }
-};
-
-// Finest level of the stack in sliced ELL with the shared Ki/Ke pattern of
-// the Bidomain operator (every member's own slices, its rows padded to whole
-// 32-row slices; padded rows, member -1, are skipped): one thread per row,
-// slot j of a slice holds entry j of its 32 rows; per node pair
-// a += Ki (v_q + u_q), b += Ke u_q, then y_v = c M_p v_p + a, y_u = a + b.
-// SU: the gathered vector is stored as (v + u, u), so a node pair costs two
-// FMAs and the row's own v is recovered once.
-template <class S, class E, bool SU = false>
-__global__ void __launch_bounds__(256) k_st_sell(int rows, const int *__restrict__ mem, const int *__restrict__ sptr,
-                                                 const int *__restrict__ col, const v2<S> *__restrict__ kk,
-                                                 const S *__restrict__ cm, StGather<S> g, E epi)
-{
-    for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < rows; p += gridDim.x * blockDim.x) {
-        if (mem[p] < 0) continue;
-        const int sl = p >> 5, lane = p & 31, j1 = sptr[sl + 1];
-        S a = 0, b = 0;
-#pragma unroll 4
-        for (int j = sptr[sl]; j < j1; j++) {
-            const size_t idx = (size_t)j * 32 + lane;
-            const v2<S> k = kk[idx];
-            const v2<S> x = g(col[idx]);
-            a = fma(k.x, SU ? x.x : x.x + x.y, a);
-            b = fma(k.y, x.y, b);
-        }
-        const v2<S> xp = g(p);
-        epi(p, fma(cm[p], SU ? xp.x - xp.y : xp.x, a), a + b);
-    }
-}
-
-// The same for a large FP64 level, as the single hierarchy's finest level runs
-// it: one block of 1024 threads per SM, each block an equal contiguous share of
-// the 32-row slices (the stack's rows are whole slices), rows unrolled deeper
-// with the registers one block per SM leaves.
-template <class S, class E, bool SU>
-__global__ void __launch_bounds__(1024, 1) k_st_sell_wide(int rows, const int *__restrict__ mem,
-                                                          const int *__restrict__ sptr, const int *__restrict__ col,
-                                                          const v2<S> *__restrict__ kk, const S *__restrict__ cm,
-                                                          StGather<S> g, E epi)
-{
-    const long long nsl = ((long long)rows + 31) >> 5;
-    const int lo = (int)(nsl * blockIdx.x / gridDim.x) * 32;
-    const int hi = min(rows, (int)(nsl * (blockIdx.x + 1) / gridDim.x) * 32);
-    for (int p = lo + threadIdx.x; p < hi; p += blockDim.x) {
-        if (mem[p] < 0) continue;
-        const int sl = p >> 5, lane = p & 31, j1 = sptr[sl + 1];
-        S a = 0, b = 0;
-#pragma unroll 8
-        for (int j = sptr[sl]; j < j1; j++) {
-            const size_t idx = (size_t)j * 32 + lane;
-            const v2<S> k = kk[idx];
-            const v2<S> x = g(col[idx]);
-            a = fma(k.x, SU ? x.x : x.x + x.y, a);
-            b = fma(k.y, x.y, b);
-        }
-        const v2<S> xp = g(p);
-        epi(p, fma(cm[p], SU ? xp.x - xp.y : xp.x, a), a + b);
-    }
-}
-
 // ------------------------------------------------------------------ assembly of the stack
 __global__ void k_st_shift(long long n, const int *__restrict__ src, int *__restrict__ dst, int add)
 {
@@ -274,7 +158,6 @@ __global__ void k_st_fill(long long n, int *__restrict__ dst, int v)
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
         dst[i] = v;
 }
-__global__ void k_st_set(int *dst, int v) { *dst = v; }
 
 // ------------------------------------------------------------------ coarsest levels
 struct StCoarseJob {
@@ -347,7 +230,7 @@ template <class S> struct StPcg {
     const v2<S> *u0, *invd0;
     StCoef c0;
     const int *mem;                // finest-level node -> member
-    int psu;                       // p stored as (v + u, u) (sliced-ELL finest level)
+    int psu;                       // p stored as (v + u, u) (stencil finest level)
     int dsu;                       // FP64 V-cycle: d0 stored as (v + u, u)
 };
 
@@ -564,7 +447,7 @@ __global__ void k_st_p(int N, StPcg<S> v, const double *__restrict__ scal)
 {
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < N; i += gridDim.x * blockDim.x) {
         const int m = v.mem[i];
-        if (m < 0) continue;  // padding of a member's last 32-row slice
+        if (m < 0) continue;  // padding after a member's last node
         const double *sc = scal + (size_t)m * T_NSLOTS;
         if (sc[T_ACTIVE] == 0.0) continue;
         double2 zi = v.z[i];
@@ -610,16 +493,18 @@ struct StLevel {
     DBuf<double> coef;         // 3 per member
     DBuf<double> f, u, r, d, w, invd;          // FP64 V-cycle (f unused on the finest level)
     DBuf<float> f32, u32, r32, d32, w32, invd32;
-    // finest level only, when every member has its sliced-ELL finest level:
-    // the members' slices end to end (columns shifted to the stack's nodes)
-    bool sell = false;
-    DBuf<int> ssptr, scol;
-    DBuf<double> skk, scm;     // FP64 (the PCG's A p always; the FP64 V-cycle)
-    DBuf<float> skk32, scm32;  // FP32 V-cycle
-    // FP64 V-cycle on the sliced finest level: its gathered vectors in
-    // (v + u, u) form, with the members' c2 D^{-1} and D^{-1} / theta
+    // finest level only, when every member's is a stencil: the members' packed
+    // tables and, per V-cycle precision, their grids in stack order (the first
+    // nsmooth smooth; the PCG applies all of them in FP64)
+    bool fine = false, sym = false;
+    int nsmooth = 0;
+    long long units = 0, units_smooth = 0;
+    DBuf<double> tab;
+    DBuf<float> tab32;
+    DBuf<FineGrid> grid, grid32;
+    // FP64 V-cycle on the stencil finest level: its gathered vectors in
+    // (v + u, u) form
     bool su = false;
-    DBuf<double> idc2, idt;
 };
 
 }  // namespace bd
@@ -707,7 +592,7 @@ struct StPart {
     long long col0;
 };
 // rows: the stacked operator's rows, the parts' rows at their row0 (ascending)
-// and empty rows in between (the finest level's padding to 32-row slices)
+// and empty rows in between (the finest level's padding to multiples of 32)
 int st_build(const std::vector<StPart> &parts, long long rows, int ncols, bool fp64, bool fp32, BSR &O,
              DBuf<float> &O32, cudaStream_t s)
 {
@@ -738,49 +623,50 @@ int st_build(const std::vector<StPart> &parts, long long rows, int ncols, bool f
     return BD_OK;
 }
 
-int st_sell_build(amg_stack *b, const std::vector<int> &order, const std::vector<long long> &off, cudaStream_t s)
+// The members' stencils as one launch: tables packed in one form (symmetric
+// only if every member's is) and each member's first node and work unit.
+int st_fine_build(amg_stack *b, const std::vector<int> &order, const std::vector<long long> &off, cudaStream_t s)
 {
     StLevel &S = b->lev[0];
-    long long slots = 0;
-    int nsl = 0;
+    S.sym = true;
+    size_t rows = 0;
     for (int k : order) {
-        slots += b->h[k]->sell.slots;
-        nsl += b->h[k]->sell.nslices;
+        S.sym = S.sym && b->h[k]->fine.sym;
+        rows += 9 * (size_t)b->h[k]->fine.NZ;
     }
-    if (slots * 32 > 2147483647LL) return BD_ERANGE;
-    BD_TRY(S.ssptr.alloc((size_t)nsl + 1));
-    BD_TRY(S.scol.alloc((size_t)slots * 32));
-    BD_TRY(S.skk.alloc((size_t)slots * 64));
-    BD_TRY(S.scm.alloc((size_t)std::max(S.N, 1)));
-    BD_CUDA(cudaMemsetAsync(S.scm.p, 0, S.scm.bytes(), s));
-    if (b->p32) {
-        BD_TRY(S.skk32.alloc((size_t)slots * 64));
-        BD_TRY(S.scm32.alloc((size_t)std::max(S.N, 1)));
-        BD_CUDA(cudaMemsetAsync(S.scm32.p, 0, S.scm32.bytes(), s));
-    }
-    long long so = 0;
+    const size_t len = 2 * (size_t)fine_row_len(S.sym);
+    BD_TRY(S.tab.alloc(rows * len));
+    if (b->p32) BD_TRY(S.tab32.alloc(rows * len));
+    std::vector<FineGrid> g64, g32;
+    size_t at = 0;
+    long long units = 0;
     for (int k : order) {
-        const FineSell &F = b->h[k]->sell;
-        const int N = b->h[k]->lev[0].N;
-        const long long sl0 = off[k] / 32;  // the member's first slice (offsets are 32-aligned)
-        k_st_shift<<<grid_for(F.nslices, 256), 256, 0, s>>>(F.nslices, F.sptr.p, S.ssptr.p + sl0, (int)so);
-        ::bd::note_launch();
-        k_st_shift<<<grid_for(F.slots * 32, 256), 256, 0, s>>>(F.slots * 32, F.col.p, S.scol.p + so * 32, (int)off[k]);
-        ::bd::note_launch();
-        BD_CUDA(cudaMemcpyAsync(S.skk.p + so * 64, F.kk.p, sizeof(double) * 64 * (size_t)F.slots,
-                                cudaMemcpyDeviceToDevice, s));
-        BD_CUDA(cudaMemcpyAsync(S.scm.p + off[k], F.cm.p, sizeof(double) * (size_t)N, cudaMemcpyDeviceToDevice, s));
-        if (b->p32) {
-            BD_CUDA(cudaMemcpyAsync(S.skk32.p + so * 64, F.kk32.p, sizeof(float) * 64 * (size_t)F.slots,
-                                    cudaMemcpyDeviceToDevice, s));
-            BD_CUDA(cudaMemcpyAsync(S.scm32.p + off[k], F.cm32.p, sizeof(float) * (size_t)N,
-                                    cudaMemcpyDeviceToDevice, s));
+        const FineStencil &F = b->h[k]->fine;
+        const Level &L0 = b->h[k]->lev[0];
+        double *t64 = S.tab.p + at * len;
+        float *t32 = b->p32 ? S.tab32.p + at * len : nullptr;
+        BD_TRY(fine_pack(F, S.sym, L0.ch_c2, L0.ch_inv_theta, t64, t32, s));
+        FineGrid g = fine_grid<double>(F, L0.ch_c1);
+        g.off = (int)off[k];
+        g.unit0 = (int)units;
+        g.tab = t64;
+        g64.push_back(g);
+        g.tab = t32;
+        g32.push_back(g);
+        units += (long long)g.ncb * g.NZ;
+        if (units > 2147483647LL) return BD_ERANGE;
+        at += 9 * (size_t)F.NZ;
+        if (b->nlev[k] > 1) {
+            S.nsmooth++;
+            S.units_smooth = units;
         }
-        so += F.slots;
     }
-    k_st_set<<<1, 1, 0, s>>>(S.ssptr.p + nsl, (int)slots);
-    ::bd::note_launch();
-    BD_LAUNCH_CHECK();
+    S.units = units;
+    BD_TRY(S.grid.alloc(g64.size()));
+    BD_TRY(S.grid32.alloc(g32.size()));
+    BD_CUDA(cudaMemcpyAsync(S.grid.p, g64.data(), sizeof(FineGrid) * g64.size(), cudaMemcpyHostToDevice, s));
+    BD_CUDA(cudaMemcpyAsync(S.grid32.p, g32.data(), sizeof(FineGrid) * g32.size(), cudaMemcpyHostToDevice, s));
+    BD_CUDA(cudaStreamSynchronize(s));  // the lists live on the host stack
     return BD_OK;
 }
 
@@ -801,12 +687,12 @@ int st_create(amg_stack *b, cudaStream_t s)
         L = std::max(L, b->nlev[k]);
     }
     b->L = L;
-    bool sell0 = true;
-    for (int k = 0; k < count; k++) sell0 = sell0 && b->h[k]->sell.valid;
-    b->lev[0].sell = sell0;
+    bool fine0 = true;
+    for (int k = 0; k < count; k++) fine0 = fine0 && b->h[k]->fine.valid;
+    b->lev[0].fine = fine0;
     // member order and node offsets per level: smoothing members, then the
-    // members whose coarsest level it is; on a sliced-ELL finest level every
-    // member starts on a 32-row slice
+    // members whose coarsest level it is; on a stencil finest level every
+    // member starts on a multiple of 32 nodes
     std::vector<std::vector<int>> order(L);
     std::vector<std::vector<long long>> off(L, std::vector<long long>(count, -1));
     for (int l = 0; l < L; l++) {
@@ -819,7 +705,7 @@ int st_create(amg_stack *b, cudaStream_t s)
                     order[l].push_back(k);
                     off[l][k] = o;
                     const long long nk = b->h[k]->lev[l].N;
-                    o += (l == 0 && sell0) ? (nk + 31) / 32 * 32 : nk;
+                    o += (l == 0 && fine0) ? (nk + 31) / 32 * 32 : nk;
                     if (pass == 0) ns = (int)o;
                 }
             }
@@ -835,7 +721,7 @@ int st_create(amg_stack *b, cudaStream_t s)
         for (int k : order[l]) {
             const Level &Lk = b->h[k]->lev[l];
             const bool smooth = b->nlev[k] - 1 > l;
-            if ((l == 0 && !sell0) || (l > 0 && smooth))
+            if ((l == 0 && !fine0) || (l > 0 && smooth))
                 pa.push_back({&Lk.A, p32 ? Lk.A32.p : nullptr, Lk.A.nbr, off[l][k], off[l][k]});
             if (smooth) pp.push_back({&Lk.P, p32 ? Lk.P32.p : nullptr, Lk.P.nbr, off[l][k], off[l + 1][k]});
         }
@@ -850,7 +736,7 @@ int st_create(amg_stack *b, cudaStream_t s)
             BD_TRY(st_build(pp, S.Ns, b->lev[l + 1].N, !p32, p32, S.P, S.P32, s));
             BD_TRY(st_build(pr, b->lev[l + 1].N, S.N, !p32, p32, S.R, S.R32, s));
         }
-        if (l == 0 && sell0) BD_TRY(st_sell_build(b, order[0], off[0], s));
+        if (l == 0 && fine0) BD_TRY(st_fine_build(b, order[0], off[0], s));
         // node -> member (-1 on padding), Chebyshev coefficients, inverse diagonals
         BD_TRY(S.mem.alloc((size_t)std::max(S.N, 1)));
         BD_CUDA(cudaMemsetAsync(S.mem.p, 0xff, S.mem.bytes(), s));
@@ -861,7 +747,6 @@ int st_create(amg_stack *b, cudaStream_t s)
             coef[4 * k] = Lk.ch_inv_theta;
             coef[4 * k + 1] = Lk.ch_c1;
             coef[4 * k + 2] = Lk.ch_c2;
-            coef[4 * k + 3] = 1.0 + Lk.ch_c1;
         }
         BD_TRY(S.coef.alloc(coef.size()));
         BD_CUDA(cudaMemcpyAsync(S.coef.p, coef.data(), sizeof(double) * coef.size(), cudaMemcpyHostToDevice, s));
@@ -882,25 +767,8 @@ int st_create(amg_stack *b, cudaStream_t s)
             for (int k : order[l])
                 BD_CUDA(cudaMemcpyAsync(S.invd.p + 2 * off[l][k], b->h[k]->lev[l].invdiag.p,
                                         sizeof(double) * 2 * b->h[k]->lev[l].N, cudaMemcpyDeviceToDevice, s));
-            // the (v + u, u) form on a sliced finest level whose members all carry
-            // their scaled inverse diagonals (every FP64 sliced finest level does)
-            // (only the members that smooth there, rows [0, Ns), use them)
-            bool su = l == 0 && sell0;
-            for (int k : order[l])
-                if (b->nlev[k] > 1) su = su && b->h[k]->lev[0].idc2.p && b->h[k]->lev[0].idt.p;
-            S.su = su;
-            if (su) {
-                BD_TRY(st_vec(S.idc2, n2, s));
-                BD_TRY(st_vec(S.idt, n2, s));
-                for (int k : order[l]) {
-                    if (b->nlev[k] <= 1) continue;
-                    const size_t bytes = sizeof(double) * 2 * b->h[k]->lev[0].N;
-                    BD_CUDA(cudaMemcpyAsync(S.idc2.p + 2 * off[0][k], b->h[k]->lev[0].idc2.p, bytes,
-                                            cudaMemcpyDeviceToDevice, s));
-                    BD_CUDA(cudaMemcpyAsync(S.idt.p + 2 * off[0][k], b->h[k]->lev[0].idt.p, bytes,
-                                            cudaMemcpyDeviceToDevice, s));
-                }
-            }
+            // FP64 on a stencil: its gathered vectors in (v + u, u) form
+            S.su = l == 0 && fine0;
             if (l > 0) BD_TRY(st_vec(S.f, n2, s));
             BD_TRY(st_vec(S.u, n2, s));
             BD_TRY(st_vec(S.r, n2, s));
@@ -997,59 +865,53 @@ template <> StView<float> st_view<float>(amg_stack *b, int l)
             (float2 *)S.d32.p, (float2 *)S.w32.p, (const float2 *)S.invd32.p};
 }
 
-template <class S> const v2<S> *st_kk(const StLevel &Lv);
-template <> const double2 *st_kk<double>(const StLevel &Lv) { return (const double2 *)Lv.skk.p; }
-template <> const float2 *st_kk<float>(const StLevel &Lv) { return (const float2 *)Lv.skk32.p; }
-template <class S> const S *st_cm(const StLevel &Lv);
-template <> const double *st_cm<double>(const StLevel &Lv) { return Lv.scm.p; }
-template <> const float *st_cm<float>(const StLevel &Lv) { return Lv.scm32.p; }
+template <class S> const FineGrid *st_grids(const StLevel &Lv);
+template <> const FineGrid *st_grids<double>(const StLevel &Lv) { return Lv.grid.p; }
+template <> const FineGrid *st_grids<float>(const StLevel &Lv) { return Lv.grid32.p; }
 
-// Operator of stack level l on rows [0, rows): the finest level's sliced ELL
-// when built, block CSR otherwise.
-template <class S, class E, bool SU = false>
-int st_apply(const StLevel &Lv, int l, int rows, const S *vals, const v2<S> *x, E e, cudaStream_t s)
+// The stencil finest level of every member (all) or of those that smooth;
+// make(SYM) gives the epilogue for the tables' form.
+template <class S, bool SU, class F>
+int st_fine(const StLevel &Lv, bool all, const v2<S> *x, F make, cudaStream_t s)
 {
-    if (l == 0 && Lv.sell) {
-        if (rows <= 0) return BD_OK;
-        // a large FP64 level: one 1024-thread block per SM on equal shares (measured
-        // against the grid-stride kernel: 64 slabs 2624 -> 2666 solves/s)
-        if (sizeof(S) == 8 && ((long long)rows + 31) / 32 >= (long long)kSM * 32) {
-            k_st_sell_wide<S, E, SU><<<kSM, 1024, 0, s>>>(rows, Lv.mem.p, Lv.ssptr.p, Lv.scol.p, st_kk<S>(Lv),
-                                                          st_cm<S>(Lv), StGather<S>{x}, e);
-        } else {
-            const int grid = (int)std::min<long long>(((long long)rows + 255) / 256, (long long)kSM * 8);
-            k_st_sell<S, E, SU><<<grid, 256, 0, s>>>(rows, Lv.mem.p, Lv.ssptr.p, Lv.scol.p, st_kk<S>(Lv),
-                                                     st_cm<S>(Lv), StGather<S>{x}, e);
-        }
-        ::bd::note_launch();
-        BD_LAUNCH_CHECK();
-        return BD_OK;
-    }
-    if constexpr (SU) return BD_ESTATE;  // the (v + u, u) form exists on the sliced level only
-    else return launch_bsr_rows<S>(rows, Lv.A.rp.p, Lv.A.ci.p, vals, Lv.lanes[0], StGather<S>{x}, e, s);
+    const int count = all ? (int)Lv.grid.n : Lv.nsmooth;
+    if (count <= 0) return BD_OK;
+    const long long units = all ? Lv.units : Lv.units_smooth;
+    if (Lv.sym)
+        k_fine_many<S, true, SU><<<fine_blocks<S, true>(units), kFineTPB, 0, s>>>(st_grids<S>(Lv), count, x,
+                                                                                  make(std::true_type{}));
+    else
+        k_fine_many<S, false, SU><<<fine_blocks<S, false>(units), kFineTPB, 0, s>>>(st_grids<S>(Lv), count, x,
+                                                                                    make(std::false_type{}));
+    ::bd::note_launch();
+    BD_LAUNCH_CHECK();
+    return BD_OK;
+}
+
+// Block-CSR operator of stack level l on rows [0, rows).
+template <class S, class E>
+int st_apply(const StLevel &Lv, int rows, const S *vals, const v2<S> *x, E e, cudaStream_t s)
+{
+    return launch_bsr_rows<S>(rows, Lv.A.rp.p, Lv.A.ci.p, vals, Lv.lanes[0], StGather<S>{x}, e, s);
 }
 
 template <class S>
 int st_vcycle(amg_stack *b, cudaStream_t s)
 {
+    constexpr bool SU = std::is_same<S, double>::value;
     const int L = b->L;
     for (int l = 0; l + 1 < L; l++) {
         StLevel &Lv = b->lev[l];
         if (Lv.Ns <= 0) continue;
         const StView<S> v = st_view<S>(b, l), cv = st_view<S>(b, l + 1);
         const StCoef c{Lv.mem.p, Lv.coef.p}, cc{b->lev[l + 1].mem.p, b->lev[l + 1].coef.p};
-        if constexpr (std::is_same<S, double>::value) {
-            if (l == 0 && Lv.su) {
-                BD_TRY((st_apply<S, StPreX, true>(Lv, l, Lv.Ns, v.Av, v.d,
-                                                  StPreX{v.f, (const double2 *)Lv.idc2.p, v.d, v.u, c}, s)));
-                BD_TRY((st_apply<S, StResid<S>, true>(Lv, l, Lv.Ns, v.Av, v.u, StResid<S>{v.f, v.r}, s)));
-                BD_TRY(launch_bsr<S>(Lv.R, v.Rv, Lv.lanes[1], StGather<S>{v.r},
-                                     StStoreD0<S>{cv.f, cv.d, cv.invd, cc}, s));
-                continue;
-            }
+        if (l == 0 && Lv.fine) {
+            BD_TRY((st_fine<S, SU>(Lv, false, v.d, [&](auto sym) { return FinePre<S, sym.value, SU>{v.f, v.u}; }, s)));
+            BD_TRY((st_fine<S, SU>(Lv, false, v.u, [&](auto sym) { return FineResid<S, sym.value>{v.f, v.r}; }, s)));
+        } else {
+            BD_TRY(st_apply<S>(Lv, Lv.Ns, v.Av, v.d, StPre<S>{v.f, v.invd, v.d, v.u, c}, s));
+            BD_TRY(st_apply<S>(Lv, Lv.Ns, v.Av, v.u, StResid<S>{v.f, v.r}, s));
         }
-        BD_TRY(st_apply<S>(Lv, l, Lv.Ns, v.Av, v.d, StPre<S>{v.f, v.invd, v.d, v.u, c}, s));
-        BD_TRY(st_apply<S>(Lv, l, Lv.Ns, v.Av, v.u, StResid<S>{v.f, v.r}, s));
         BD_TRY(launch_bsr<S>(Lv.R, v.Rv, Lv.lanes[1], StGather<S>{v.r}, StStoreD0<S>{cv.f, cv.d, cv.invd, cc}, s));
     }
     StLevelPtrs<S> lp{};
@@ -1068,21 +930,20 @@ int st_vcycle(amg_stack *b, cudaStream_t s)
         if (Lv.Ns <= 0) continue;
         const StView<S> v = st_view<S>(b, l), cv = st_view<S>(b, l + 1);
         const StCoef c{Lv.mem.p, Lv.coef.p};
-        if constexpr (std::is_same<S, double>::value) {
-            if (l == 0 && Lv.su) {
-                BD_TRY(launch_bsr<S>(Lv.P, v.Pv, Lv.lanes[2], StGather<S>{cv.u}, StAddX{v.u}, s));
-                BD_TRY((st_apply<S, StPost1X, true>(Lv, l, Lv.Ns, v.Av, v.u,
-                                                    StPost1X{v.f, (const double2 *)Lv.idt.p, v.u, v.r, v.d, v.w},
-                                                    s)));
-                BD_TRY((st_apply<S, StPost2X, true>(Lv, l, Lv.Ns, v.Av, v.d,
-                                                    StPost2X{v.r, v.d, (const double2 *)Lv.idc2.p, v.w, v.u, c},
-                                                    s)));
-                continue;
-            }
+        if (l == 0 && Lv.fine) {
+            if constexpr (SU) BD_TRY(launch_bsr<S>(Lv.P, v.Pv, Lv.lanes[2], StGather<S>{cv.u}, StAddX{v.u}, s));
+            else BD_TRY(launch_bsr<S>(Lv.P, v.Pv, Lv.lanes[2], StGather<S>{cv.u}, StAdd<S>{v.u}, s));
+            BD_TRY((st_fine<S, SU>(Lv, false, v.u, [&](auto sym) {
+                return FinePost1<S, sym.value, SU>{v.f, v.r, v.d, nullptr};
+            }, s)));
+            BD_TRY((st_fine<S, SU>(Lv, false, v.d, [&](auto sym) {
+                return FinePost2<S, sym.value, SU>{v.r, v.u, v.u};
+            }, s)));
+            continue;
         }
         BD_TRY(launch_bsr<S>(Lv.P, v.Pv, Lv.lanes[2], StGather<S>{cv.u}, StAdd<S>{v.u}, s));
-        BD_TRY(st_apply<S>(Lv, l, Lv.Ns, v.Av, v.u, StPost1<S>{v.f, v.invd, v.u, v.r, v.d, v.w, c}, s));
-        BD_TRY(st_apply<S>(Lv, l, Lv.Ns, v.Av, v.d, StPost2<S>{v.r, v.d, v.invd, v.w, v.u, c}, s));
+        BD_TRY(st_apply<S>(Lv, Lv.Ns, v.Av, v.u, StPost1<S>{v.f, v.invd, v.u, v.r, v.d, v.w, c}, s));
+        BD_TRY(st_apply<S>(Lv, Lv.Ns, v.Av, v.d, StPost2<S>{v.r, v.d, v.invd, v.w, v.u, c}, s));
     }
     return BD_OK;
 }
@@ -1107,7 +968,7 @@ StPcg<S> st_pcg(amg_stack *b)
     v.invd0 = v0.invd;
     v.c0 = StCoef{b->lev[0].mem.p, b->lev[0].coef.p};
     v.mem = b->lev[0].mem.p;
-    v.psu = b->lev[0].sell ? 1 : 0;
+    v.psu = b->lev[0].fine ? 1 : 0;
     v.dsu = b->lev[0].su ? 1 : 0;
     return v;
 }
@@ -1119,12 +980,14 @@ StRed st_red(amg_stack *b, cudaGraphConditionalHandle cond)
 }
 
 // q = A x on the finest level; su: x is stored in (v + u, u) form (the PCG's p
-// on a sliced level)
+// on a stencil level)
 int st_apply_a(amg_stack *b, const double2 *x, double2 *q, cudaStream_t s, bool su = false)
 {
     StLevel &S = b->lev[0];
-    if (S.sell && su) return st_apply<double, StStore, true>(S, 0, S.N, nullptr, x, StStore{q}, s);
-    if (S.sell) return st_apply<double>(S, 0, S.N, nullptr, x, StStore{q}, s);
+    if (S.fine) {
+        auto store = [&](auto) { return FineStore<double>{q}; };
+        return su ? st_fine<double, true>(S, true, x, store, s) : st_fine<double, false>(S, true, x, store, s);
+    }
     return launch_bsr_rows<double>(S.N, S.A.rp.p, S.A.ci.p, S.A.v.p, lanes_for(S.A, false), StGather<double>{x},
                                    StStore{q}, s);
 }

@@ -270,7 +270,7 @@ extern "C" int bd_dsim_create(const bd_system *sys, amg_hierarchy *h_elliptic, c
 {
     if (!sys || !h_elliptic || !out) return BD_EINVAL;
     *out = nullptr;
-    if (h_elliptic->lev[0].N != sys->N || h_elliptic->sell.valid) return BD_EINVAL;
+    if (h_elliptic->lev[0].N != sys->N || h_elliptic->fine.valid) return BD_EINVAL;
     cudaStream_t s = (cudaStream_t)stream;
     bd_dsim *S = new (std::nothrow) bd_dsim();
     if (!S) return BD_ENOMEM;
