@@ -22,14 +22,30 @@ struct SlicedOp {
     int rows = 0;               // block rows
     int nsl = 0;                // slices
     long long groups = 0;       // 32-entry groups
-    int warps = 0;              // warps of the launch (grid x 8)
+    int blocks = 0;             // blocks of the launch
     DBuf<int> order;            // rows padded to 32: row at each sorted position, -1 past the end
     DBuf<int> sptr;             // nsl + 1: first group of each slice
-    DBuf<int> wsl;              // warps + 1: first slice of each warp (balanced by groups)
+    DBuf<int> bsl;              // blocks + 1: first slice of each block (balanced by groups)
     DBuf<int> cnt;              // nsl: groups per slice (build scratch)
     DBuf<int> col;              // groups * 32 block columns
     DBuf<double> v;             // FP64: groups * 32 (a00, a01) pairs, then as many (a10, a11)
     DBuf<float> v32;            // FP32: groups * 32 float4 (a00, a01, a10, a11)
+    DBuf<double> alpha;         // pair form (values then are (ki, ke) pairs)
+    DBuf<float> alpha32;
+};
+
+// The finest level's P or R of an assembled slab with two numbers per block
+// (MatPair).  There A's blocks are [c M d + ki, ki; ki, ki + ke] (d: diagonal)
+// and the tentative prolongator has the same value in both fields, so a block of
+// the smoothed P = Pt - omega D^{-1} A Pt is kappa [ki + alpha, ki; ki, ki + ke]
+// with kappa = -omega D^{-1} of its row.  kappa is applied by P's epilogue and,
+// for R = P^T, to the vector R gathers.  Rows as in the block-CSR operator,
+// each row's own entries (P: its aggregate, R: its members) first.
+struct PairOp {
+    bool valid = false;
+    DBuf<int> ci;
+    DBuf<double> v, alpha;     // (ki, ke) per entry, alpha per entry (own ones only)
+    DBuf<float> v32, alpha32;
 };
 
 struct Level {
@@ -54,6 +70,11 @@ struct Level {
     // sliced form sl[op] with K lanes per row
     int lanes[3] = {0, 0, 0};
     SlicedOp sl[3];
+    // finest level of an assembled slab: R (0) and P (1) in pair form and
+    // kappa = -omega D^{-1} per node (2N, in the V-cycle's precision)
+    PairOp pair[2];
+    DBuf<double> kappa;
+    DBuf<float> kappa32;
 };
 
 // Finest level of an assembled slab as a layered stencil (fine_stencil.cuh):

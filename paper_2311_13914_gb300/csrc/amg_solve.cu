@@ -36,40 +36,76 @@ __device__ __forceinline__ BlkS<float> load_sliced(const float *__restrict__ v, 
     return {p.x, p.y, p.z, p.w};
 }
 
-// One warp per slice of 32/K rows with K lanes each; warp w takes slices
-// [wsl[w], wsl[w+1]), which split the groups evenly over the warps.  Lane k of
-// a row sums entries k, k+K, ... and the K partial sums meet in the lane-sum
-// tree k_bsr<K> uses (group_sum2), so both forms give the same bits.  Rows sorted by
-// length leave few padded positions, and every FP64 instruction of the loop
-// and the epilogue works on 32 lanes (the FP64 pipe, not HBM, bounds the
-// coarse levels in FP64).
-template <int K, class S, class G, class E, int MINB, int TPB = 256>
-__global__ void __launch_bounds__(TPB, MINB) k_bsell(const int *__restrict__ sptr, const int *__restrict__ wsl,
-                                                    const int *__restrict__ order, const int *__restrict__ col,
-                                                    const S *__restrict__ v, size_t plane, G gather, E epi)
+// One warp per slice of 32/K rows with K lanes each.  Block b owns slices
+// [bsl[b], bsl[b+1]), which split the groups evenly over the blocks, and its
+// warps take the next slice whenever they finish one: slices differ in length
+// (sorted rows: a window's first are its longest), and with a fixed share of
+// three or four slices per warp the slowest held its SM for a third of the
+// launch.  Lane k of a row sums entries k, k+K, ... and the K partial sums meet
+// in the lane-sum tree k_bsr<K> uses (group_sum2), so both forms give the same
+// bits.  Rows sorted by length leave few padded positions, and every FP64
+// instruction of the loop and the epilogue works on 32 lanes (the FP64 pipe,
+// not HBM, bounds the coarse levels in FP64).
+constexpr int kSlicedTPB = 512;
+template <class S> struct SlicedMinB { static constexpr int v = sizeof(S) == 8 ? 2 : 4; };
+template <int K, class M, class G, class E>
+__global__ void __launch_bounds__(kSlicedTPB, SlicedMinB<typename M::Sc>::v)
+    k_bsell(const int *__restrict__ sptr, const int *__restrict__ bsl, const int *__restrict__ order,
+            const int *__restrict__ col, M mat, G gather, E epi)
 {
-    const int w = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+    __shared__ int next;
+    if (threadIdx.x == 0) next = bsl[blockIdx.x];
+    const int s1 = bsl[blockIdx.x + 1];
+    __syncthreads();
     const int lane = threadIdx.x & 31;
-    const int s1 = wsl[w + 1];
-    for (int sl = wsl[w]; sl < s1; sl++) {
-        const int j1 = sptr[sl + 1];
-        S y0 = 0, y1 = 0;
+    for (;;) {
+        int sl = 0;
+        if (lane == 0) sl = atomicAdd(&next, 1);
+        sl = __shfl_sync(0xffffffffu, sl, 0);
+        if (sl >= s1) break;
+        const int j0 = sptr[sl], j1 = sptr[sl + 1];
+        const int r = order[sl * (32 / K) + lane / K];
+        typename M::Acc A;
+        typename M::Sc r0 = 0, r1 = 0;
+        if constexpr (M::OWN) {
+            for (int j = j0; j < j1; j++) {
+                const size_t idx = (size_t)j * 32 + lane;
+                const int q = col[idx];
+                if (q >= 0) break;
+                mat.own(A, idx, q, gather);
+            }
+        }
 #pragma unroll 4
-        for (int j = sptr[sl]; j < j1; j++) {
+        for (int j = j0; j < j1; j++) {
             const size_t idx = (size_t)j * 32 + lane;
-            const int q = col[idx];
-            const BlkS<S> a = load_sliced(v, idx, plane);
-            const v2<S> x = gather(q);
-            y0 = fma(a.a00, x.x, fma(a.a01, x.y, y0));
-            y1 = fma(a.a10, x.x, fma(a.a11, x.y, y1));
+            mat.step(A, idx, col[idx], gather);
         }
-        group_sum2<K>(y0, y1);
-        if ((lane & (K - 1)) == 0) {
-            const int r = order[sl * (32 / K) + lane / K];
-            if (r >= 0) epi(r, y0, y1);
-        }
+        mat.finish(A, r0, r1);
+        group_sum2<K>(r0, r1);
+        if ((lane & (K - 1)) == 0 && r >= 0) epi(r, r0, r1);
     }
 }
+
+// Full blocks in the sliced form: two planes of half blocks in FP64.
+template <class S> struct MatSliced {
+    using Sc = S;
+    static constexpr bool OWN = false;
+    using Acc = typename MatFull<S>::Acc;
+    const S *__restrict__ v;
+    size_t plane;
+    __device__ __forceinline__ void finish(const Acc &A, S &y0, S &y1) const
+    {
+        y0 = A.y0;
+        y1 = A.y1;
+    }
+    template <class G> __device__ __forceinline__ void step(Acc &A, size_t t, int q, const G &g) const
+    {
+        const BlkS<S> a = load_sliced(v, t, plane);
+        const v2<S> x = g(q);
+        A.y0 = fma(a.a00, x.x, fma(a.a01, x.y, A.y0));
+        A.y1 = fma(a.a10, x.x, fma(a.a11, x.y, A.y1));
+    }
+};
 
 // Sorted position of every row of a window: by block count, descending, ties
 // by row (a stable, deterministic order).  One thread block per window.
@@ -138,24 +174,47 @@ __global__ void k_slice_fill(int nsl, int K, const int *__restrict__ rp, const i
     }
 }
 
-// first slice of every warp: the lower bound of w * groups / warps in sptr
-__global__ void k_slice_warps(int nsl, long long groups, int warps, const int *__restrict__ sptr,
-                              int *__restrict__ wsl)
+// the same for an operator in pair form
+template <class S>
+__global__ void k_slice_fill_pair(int nsl, int K, const int *__restrict__ rp, const int *__restrict__ ci,
+                                  const v2<S> *__restrict__ pv, const S *__restrict__ alpha,
+                                  const int *__restrict__ order, const int *__restrict__ sptr, int *__restrict__ col,
+                                  v2<S> *__restrict__ v, S *__restrict__ al)
+{
+    const long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+    if (t >= (long long)nsl * 32) return;
+    const int sl = (int)(t >> 5), lane = (int)(t & 31);
+    const int r = order[sl * (32 / K) + lane / K], k = lane % K;
+    const int b = r >= 0 ? rp[r] : 0, len = r >= 0 ? rp[r + 1] - b : 0;
+    const int g0 = sptr[sl], g1 = sptr[sl + 1];
+    for (int g = g0; g < g1; g++) {
+        const int j = (g - g0) * K + k;
+        const size_t idx = (size_t)g * 32 + lane;
+        const bool in = j < len;
+        col[idx] = in ? ci[b + j] : 0;
+        v[idx] = in ? pv[b + j] : V2<S>::mk((S)0, (S)0);
+        al[idx] = in ? alpha[b + j] : (S)0;
+    }
+}
+
+// first slice of every block: the lower bound of b * groups / blocks in sptr
+__global__ void k_slice_blocks(int nsl, long long groups, int blocks, const int *__restrict__ sptr,
+                               int *__restrict__ bsl)
 {
     const int w = blockIdx.x * blockDim.x + threadIdx.x;
-    if (w > warps) return;
-    if (w == warps) {
-        wsl[w] = nsl;
+    if (w > blocks) return;
+    if (w == blocks) {
+        bsl[w] = nsl;
         return;
     }
-    const long long g = groups * w / warps;
+    const long long g = groups * w / blocks;
     int lo = 0, hi = nsl;
     while (lo < hi) {
         const int m = (lo + hi) >> 1;
         if (sptr[m] < g) lo = m + 1;
         else hi = m;
     }
-    wsl[w] = lo;
+    bsl[w] = lo;
 }
 
 // ------------------------------------------------------------------ vector kernels' shares
@@ -173,11 +232,6 @@ __device__ __forceinline__ int share_hi(int n)
 }
 
 // ------------------------------------------------------------------ fused epilogues
-template <class S> struct GatherVec {
-    const v2<S> *__restrict__ x;
-    __device__ __forceinline__ v2<S> operator()(int q) const { return x[q]; }
-};
-
 // Vectors the FP64 finest-level stencil gathers are kept in the (v + u, u)
 // form (SU): two operations per node pair instead of three.
 template <class S, bool SU> __device__ __forceinline__ v2<S> to_su(S v, S u)
@@ -222,11 +276,22 @@ template <class S> struct EpiResid {  // r = f - A u
     }
 };
 
-template <class S, bool SU = false> struct EpiAdd {  // u += P e_c
+template <class S> struct EpiAdd {  // u += P e_c
     v2<S> *__restrict__ u;
     __device__ __forceinline__ void operator()(int p, S y0, S y1) const {
         const v2<S> a = u[p];
-        u[p] = V2<S>::mk(a.x + (SU ? y0 + y1 : y0), a.y + y1);
+        u[p] = V2<S>::mk(a.x + y0, a.y + y1);
+    }
+};
+
+// the same for the finest P in pair form; u in (v + u, u) form in FP64
+template <class S, bool SU> struct EpiAddPair {
+    v2<S> *__restrict__ u;
+    const v2<S> *__restrict__ kappa;
+    __device__ __forceinline__ void operator()(int p, S y0, S y1) const {
+        const v2<S> a = u[p], k = kappa[p];
+        const S e1 = k.y * y1;
+        u[p] = V2<S>::mk(SU ? a.x + fma(k.x, y0, e1) : a.x + k.x * y0, a.y + e1);
     }
 };
 
@@ -250,7 +315,8 @@ template <class S> struct EpiPost1 {
 };
 
 // post-smoothing, second half: r1 = r0 - A d0, d1 = c1 d0 + c2 D^{-1} r1, u = w + d1
-template <class S> struct EpiPost2 {
+// (OSU: u in (v + u, u) form, which the finest prolongation in pair form gathers)
+template <class S, bool OSU = false> struct EpiPost2 {
     const v2<S> *__restrict__ r;
     const v2<S> *__restrict__ d;
     const v2<S> *__restrict__ invd;
@@ -260,7 +326,7 @@ template <class S> struct EpiPost2 {
     __device__ __forceinline__ void operator()(int p, S y0, S y1) const {
         const v2<S> rp_ = r[p], dp = d[p], id = invd[p], wp = w[p];
         const S r0 = rp_.x - y0, r1 = rp_.y - y1;
-        u[p] = V2<S>::mk(wp.x + (c1 * dp.x + c2 * id.x * r0), wp.y + (c1 * dp.y + c2 * id.y * r1));
+        u[p] = to_su<S, OSU>(wp.x + (c1 * dp.x + c2 * id.x * r0), wp.y + (c1 * dp.y + c2 * id.y * r1));
     }
 };
 
@@ -273,6 +339,10 @@ template <class S> struct LV {
 };
 
 template <class S> static LV<S> view(amg_hierarchy *h, int l);
+
+template <class S> static const v2<S> *kappa_of(const Level &L);
+template <> const double2 *kappa_of<double>(const Level &L) { return (const double2 *)L.kappa.p; }
+template <> const float2 *kappa_of<float>(const Level &L) { return (const float2 *)L.kappa32.p; }
 
 template <> LV<double> view<double>(amg_hierarchy *h, int l)
 {
@@ -308,34 +378,19 @@ template <> LV<float> view<float>(amg_hierarchy *h, int l)
 template <class S> static const S *sliced_vals(const SlicedOp &o);
 template <> const double *sliced_vals<double>(const SlicedOp &o) { return o.v.p; }
 template <> const float *sliced_vals<float>(const SlicedOp &o) { return o.v32.p; }
+template <class S> static const S *sliced_alpha(const SlicedOp &o);
+template <> const double *sliced_alpha<double>(const SlicedOp &o) { return o.alpha.p; }
+template <> const float *sliced_alpha<float>(const SlicedOp &o) { return o.alpha32.p; }
 
-template <class S, class G, class E>
-static int launch_sliced(const SlicedOp &o, int K, G g, E e, cudaStream_t s)
+template <class M, class G, class E>
+static int launch_sliced(const SlicedOp &o, int K, M mat, G g, E e, cudaStream_t s)
 {
-    if (o.K != K || !sliced_vals<S>(o)) return BD_ESTATE;
-    constexpr int MB = sizeof(S) == 8 ? 4 : 8;  // as the finest level's sliced ELL
-    const S *v = sliced_vals<S>(o);
-    const size_t plane = (size_t)o.groups * 32;
-    // FP64 operators whose warps fill one wave: one 1024-thread block per SM,
-    // the same warps and slices as 256-thread blocks (the finest R and P:
-    // 1.3-1.8 us shorter launches, measured)
-    if (sizeof(S) == 8 && o.warps == kSM * 32) {
-        switch (K) {
-        case 1: k_bsell<1, S, G, E, 1, 1024><<<kSM, 1024, 0, s>>>(o.sptr.p, o.wsl.p, o.order.p, o.col.p, v, plane, g, e); break;
-        case 2: k_bsell<2, S, G, E, 1, 1024><<<kSM, 1024, 0, s>>>(o.sptr.p, o.wsl.p, o.order.p, o.col.p, v, plane, g, e); break;
-        case 4: k_bsell<4, S, G, E, 1, 1024><<<kSM, 1024, 0, s>>>(o.sptr.p, o.wsl.p, o.order.p, o.col.p, v, plane, g, e); break;
-        default: k_bsell<8, S, G, E, 1, 1024><<<kSM, 1024, 0, s>>>(o.sptr.p, o.wsl.p, o.order.p, o.col.p, v, plane, g, e); break;
-        }
-        ::bd::note_launch();
-        BD_LAUNCH_CHECK();
-        return BD_OK;
-    }
-    const int grid = o.warps / 8;
+    if (o.K != K || !mat.v) return BD_ESTATE;
     switch (K) {
-    case 1: k_bsell<1, S, G, E, MB><<<grid, 256, 0, s>>>(o.sptr.p, o.wsl.p, o.order.p, o.col.p, v, plane, g, e); break;
-    case 2: k_bsell<2, S, G, E, MB><<<grid, 256, 0, s>>>(o.sptr.p, o.wsl.p, o.order.p, o.col.p, v, plane, g, e); break;
-    case 4: k_bsell<4, S, G, E, MB><<<grid, 256, 0, s>>>(o.sptr.p, o.wsl.p, o.order.p, o.col.p, v, plane, g, e); break;
-    default: k_bsell<8, S, G, E, MB><<<grid, 256, 0, s>>>(o.sptr.p, o.wsl.p, o.order.p, o.col.p, v, plane, g, e); break;
+    case 1: k_bsell<1><<<o.blocks, kSlicedTPB, 0, s>>>(o.sptr.p, o.bsl.p, o.order.p, o.col.p, mat, g, e); break;
+    case 2: k_bsell<2><<<o.blocks, kSlicedTPB, 0, s>>>(o.sptr.p, o.bsl.p, o.order.p, o.col.p, mat, g, e); break;
+    case 4: k_bsell<4><<<o.blocks, kSlicedTPB, 0, s>>>(o.sptr.p, o.bsl.p, o.order.p, o.col.p, mat, g, e); break;
+    default: k_bsell<8><<<o.blocks, kSlicedTPB, 0, s>>>(o.sptr.p, o.bsl.p, o.order.p, o.col.p, mat, g, e); break;
     }
     ::bd::note_launch();
     BD_LAUNCH_CHECK();
@@ -352,7 +407,7 @@ template <class T> static int ensure(DBuf<T> &b, size_t n)
     return b.p && b.n >= n ? BD_OK : b.alloc(n);
 }
 
-static int build_sliced(const BSR &M, int K, bool fp32, SlicedOp &o, cudaStream_t s)
+static int build_sliced(const BSR &M, const PairOp *pr, int K, bool fp32, SlicedOp &o, cudaStream_t s)
 {
     if (M.nbr <= 0 || M.nb <= 0 || !sliced_k_ok(K)) return BD_EINVAL;
     const int rows = M.nbr, H = 32 / K;
@@ -377,24 +432,38 @@ static int build_sliced(const BSR &M, int K, bool fp32, SlicedOp &o, cudaStream_
     BD_TRY(ensure(o.col, ent));
     const long long fill_threads = (long long)o.nsl * 32;
     const int fill_grid = (int)((fill_threads + 255) / 256);
-    if (fp32) {
-        o.v.release();
+    if (fp32) o.v.release();
+    else o.v32.release();
+    if (pr) {
+        if (fp32) {
+            BD_TRY(ensure(o.v32, 2 * ent));
+            BD_TRY(ensure(o.alpha32, ent));
+            k_slice_fill_pair<float><<<fill_grid, 256, 0, s>>>(o.nsl, K, M.rp.p, pr->ci.p, (const float2 *)pr->v32.p,
+                                                               pr->alpha32.p, o.order.p, o.sptr.p, o.col.p,
+                                                               (float2 *)o.v32.p, o.alpha32.p);
+        } else {
+            BD_TRY(ensure(o.v, 2 * ent));
+            BD_TRY(ensure(o.alpha, ent));
+            k_slice_fill_pair<double><<<fill_grid, 256, 0, s>>>(o.nsl, K, M.rp.p, pr->ci.p, (const double2 *)pr->v.p,
+                                                                pr->alpha.p, o.order.p, o.sptr.p, o.col.p,
+                                                                (double2 *)o.v.p, o.alpha.p);
+        }
+    } else if (fp32) {
         BD_TRY(ensure(o.v32, 4 * ent));
         k_slice_fill<float><<<fill_grid, 256, 0, s>>>(o.nsl, K, M.rp.p, M.ci.p, M.v.p, o.order.p, o.sptr.p,
                                                      o.col.p, o.v32.p, ent);
     } else {
-        o.v32.release();
         BD_TRY(ensure(o.v, 4 * ent));
         k_slice_fill<double><<<fill_grid, 256, 0, s>>>(o.nsl, K, M.rp.p, M.ci.p, M.v.p, o.order.p, o.sptr.p,
                                                       o.col.p, o.v.p, ent);
     }
     ::bd::note_launch();
     BD_LAUNCH_CHECK();
-    const int MB = fp32 ? 8 : 4;
-    const long long cap = (long long)kSM * MB * 8;  // one resident wave of 256-thread blocks
-    o.warps = (int)std::min<long long>(cap, ((long long)o.nsl + 7) / 8 * 8);
-    BD_TRY(ensure(o.wsl, (size_t)o.warps + 1));
-    k_slice_warps<<<(o.warps + 256) / 256, 256, 0, s>>>(o.nsl, o.groups, o.warps, o.sptr.p, o.wsl.p);
+    // one resident wave, a slice per warp at least
+    const long long cap = (long long)kSM * (fp32 ? SlicedMinB<float>::v : SlicedMinB<double>::v);
+    o.blocks = (int)std::min<long long>(cap, ((long long)o.nsl + kSlicedTPB / 32 - 1) / (kSlicedTPB / 32));
+    BD_TRY(ensure(o.bsl, (size_t)o.blocks + 1));
+    k_slice_blocks<<<o.blocks / 256 + 1, 256, 0, s>>>(o.nsl, o.groups, o.blocks, o.sptr.p, o.bsl.p);
     ::bd::note_launch();
     BD_LAUNCH_CHECK();
     o.K = K;
@@ -408,8 +477,21 @@ static void drop_sliced(SlicedOp &o)
     o.col.release();
     o.v.release();
     o.v32.release();
+    o.alpha.release();
+    o.alpha32.release();
     o.sptr.release();
-    o.wsl.release();
+    o.bsl.release();
+}
+
+static const BSR &op_of(const Level &L, int op) { return op == 0 ? L.A : (op == 1 ? L.R : L.P); }
+static const PairOp *pair_of(const Level &L, int op)
+{
+    return op > 0 && L.pair[op - 1].valid ? &L.pair[op - 1] : nullptr;
+}
+// sliced form of operator op with K lanes per row
+static int build_op(Level &L, int op, int K, bool fp32, cudaStream_t s)
+{
+    return build_sliced(op_of(L, op), pair_of(L, op), K, fp32, L.sl[op], s);
 }
 
 // Operator op (0: A, 1: R, 2: P) of level L in the form its lanes entry names.
@@ -417,25 +499,142 @@ template <class S, class G, class E>
 static int apply_op(const Level &L, int op, const S *csr_vals, G g, E e, cudaStream_t s)
 {
     const int T = L.lanes[op];
-    if (T < 0) return launch_sliced<S>(L.sl[op], -T, g, e, s);
-    return launch_bsr<S>(op == 0 ? L.A : (op == 1 ? L.R : L.P), csr_vals, T, g, e, s);
+    const SlicedOp &o = L.sl[op];
+    if (T < 0) return launch_sliced(o, -T, MatSliced<S>{sliced_vals<S>(o), (size_t)o.groups * 32}, g, e, s);
+    return launch_bsr<S>(op_of(L, op), csr_vals, T, g, e, s);
+}
+
+// The finest R or P in pair form; the caller applies kappa.
+template <class S, class G, class E>
+static int apply_pair(const Level &L, int op, G g, E e, cudaStream_t s)
+{
+    const int T = L.lanes[op];
+    const SlicedOp &o = L.sl[op];
+    if (T < 0) return launch_sliced(o, -T, MatPair<S>{(const v2<S> *)sliced_vals<S>(o), sliced_alpha<S>(o)}, g, e, s);
+    const BSR &M = op_of(L, op);
+    return launch_bsr_rows(M.nbr, M.rp.p, pair_of(L, op)->ci.p, mat_pair<S>(*pair_of(L, op)), T, g, e, s);
+}
+
+// Pair form of P (rows: fine nodes, own entry: the node's aggregate) or of its
+// transpose R (rows: aggregates, own entries: the members).  One warp per row:
+// own entries keep their order at the front, the others theirs behind.
+__global__ void k_pair_fill(int rows, int is_r, const int *__restrict__ rp, const int *__restrict__ ci,
+                            const double *__restrict__ bv, const int *__restrict__ agg,
+                            const double *__restrict__ kappa, int *__restrict__ oci, double2 *__restrict__ ov,
+                            double *__restrict__ oal, float2 *__restrict__ ov32, float *__restrict__ oal32)
+{
+    const int lane = threadIdx.x & 31, warps = (gridDim.x * blockDim.x) >> 5;
+    for (int row = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; row < rows; row += warps) {
+        const int b = rp[row], e = rp[row + 1];
+        int nown = 0;
+        for (int t0 = b; t0 < e; t0 += 32) {
+            const int t = t0 + lane;
+            const bool own = t < e && (is_r ? agg[ci[t]] == row : ci[t] == agg[row]);
+            nown += __popc(__ballot_sync(0xffffffffu, own));
+        }
+        int po = b, pn = b + nown;  // next own and next other position
+        for (int t0 = b; t0 < e; t0 += 32) {
+            const int t = t0 + lane;
+            const bool in = t < e;
+            const int q = in ? ci[t] : 0;
+            const bool own = in && (is_r ? agg[q] == row : q == agg[row]);
+            const unsigned mo = __ballot_sync(0xffffffffu, own), mi = __ballot_sync(0xffffffffu, in);
+            const unsigned below = (1u << lane) - 1u;
+            if (in) {
+                const int pos = own ? po + __popc(mo & below) : pn + __popc(mi & ~mo & below);
+                const int node = is_r ? q : row;
+                const double kv = kappa[2 * node], ku = kappa[2 * node + 1];
+                const double *a = bv + 4 * (size_t)t;
+                // P's block [a00 a01; a10 a11]; R holds its transpose
+                const double a01 = is_r ? a[2] : a[1];
+                const double ki = a01 / kv, ke = a[3] / ku - ki, al = own ? (a[0] - a01) / kv : 0.0;
+                oci[pos] = own ? (q | ~kColMask) : q;
+                if (ov) {
+                    ov[pos] = make_double2(ki, ke);
+                    oal[pos] = al;
+                } else {
+                    ov32[pos] = make_float2((float)ki, (float)ke);
+                    oal32[pos] = (float)al;
+                }
+            }
+            po += __popc(mo);
+            pn += __popc(mi & ~mo);
+        }
+    }
+}
+
+__global__ void k_kappa(long long n, const double *__restrict__ invd, double omega, double *__restrict__ k64,
+                        float *__restrict__ k32)
+{
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
+         i += (long long)gridDim.x * blockDim.x) {
+        const double k = -omega * invd[i];
+        k64[i] = k;
+        if (k32) k32[i] = (float)k;
+    }
+}
+
+static int build_pairs(Level &L, bool fp32, cudaStream_t s)
+{
+    const long long n = 2LL * L.N;
+    BD_TRY(L.kappa.alloc((size_t)n));
+    if (fp32) BD_TRY(L.kappa32.alloc((size_t)n));
+    k_kappa<<<grid_for(n, 256), 256, 0, s>>>(n, L.invdiag.p, fine_omega(L), L.kappa.p, L.kappa32.p);
+    ::bd::note_launch();
+    for (int op = 1; op <= 2; op++) {
+        const BSR &M = op_of(L, op);
+        PairOp &o = L.pair[op - 1];
+        BD_TRY(o.ci.alloc((size_t)M.nb));
+        if (fp32) {
+            BD_TRY(o.v32.alloc(2 * (size_t)M.nb));
+            BD_TRY(o.alpha32.alloc((size_t)M.nb));
+        } else {
+            BD_TRY(o.v.alloc(2 * (size_t)M.nb));
+            BD_TRY(o.alpha.alloc((size_t)M.nb));
+        }
+        k_pair_fill<<<grid_for(32LL * M.nbr, 256), 256, 0, s>>>(M.nbr, op == 1, M.rp.p, M.ci.p, M.v.p, L.agg.p,
+                                                                L.kappa.p, o.ci.p, (double2 *)o.v.p, o.alpha.p,
+                                                                (float2 *)o.v32.p, o.alpha32.p);
+        ::bd::note_launch();
+        o.valid = true;
+    }
+    BD_LAUNCH_CHECK();
+    return BD_OK;
 }
 
 // The sliced form (FP64 only: in FP32 block-CSR with more lanes was as fast
-// or faster on every level) where it beat block-CSR inside the V-cycle: many
-// short, ragged rows (the prolongators of levels of 65536 rows and more:
-// sorted rows leave few idle lanes, one lane per row needs no reduction), many
-// long rows (restrictions, 8 lanes per row) and, on levels of 65536 rows and
-// more, rows in between (4 lanes; the autotuner's choices on the 256x256x64
-// slab's second level, while block-CSR with 4 lanes won on the 31542 rows of
-// the 128x128x32 slab's).  Elsewhere the block-CSR rule.
+// or faster on every level) where it beat block-CSR inside the V-cycle (us per
+// V-cycle, forms.time_forms): many short, ragged rows (the prolongators of levels
+// of 65536 rows and more: sorted rows leave few idle lanes, one lane per row needs
+// no reduction), rows of 64 to 400 blocks on 24576 rows and more (8 lanes; the
+// 128x128x32 slab's second level, 32001 rows: 145 -> 137, on the 13197 rows of
+// 96x96x24 block-CSR wins, 78 against 93) and, on levels of 65536 rows and more,
+// rows in between and long ones (4 lanes; 256x256x64, 249682 rows: 840 -> 743).
+// Restrictions from 96 blocks a row from 8192 rows on.  Longer rows still (the
+// nearly dense levels of large slabs): a thread block per row in both
+// precisions (11501 rows of 2830 blocks: FP64 sliced 8 1980, 128 threads 1061;
+// FP32 32 lanes 528, 256 threads 403).  Elsewhere the block-CSR rule.
+//
+// The finest R and P in pair form have their own crossovers.  R: few lanes
+// where rows fill the GPU (T rows >= 200 K), else up to 16 (31542 rows: 8 lanes
+// 35.8, sliced 8 38.9; 13197 rows: 16 lanes 23.2, 8 24.8; 249682 rows: 4 lanes
+// 199, 8 211).  P: one lane per row on a million rows and more (256x256x64: FP64
+// sliced 254, one lane 240; FP32 two lanes 127, one 107); the rule above below.
 constexpr int kSlicedMinRows = 8192;
-static int lanes_rule(const BSR &A, bool fp32, bool sliced_ok)
+constexpr double kLongRow = 1000.0;
+static int lanes_rule(const BSR &A, bool fp32, bool sliced_ok, const PairOp *pr = nullptr)
 {
     const double avg = A.nbr > 0 ? (double)A.nb / A.nbr : 1.0;
+    if (avg >= kLongRow) return fp32 ? 256 : 128;
+    if (pr && !fp32 && avg >= 48.0 && A.nbr >= 4096) {
+        int T = 4;
+        while (T < 16 && (long long)A.nbr * T < 200000) T <<= 1;
+        return T;
+    }
+    if (pr && avg < 48.0 && A.nbr >= 1 << 20) return 1;
     if (sliced_ok && !fp32 && A.nbr >= kSlicedMinRows) {
         if (A.nbr >= 65536 && avg <= 24.0) return -1;
-        if (avg >= 96.0) return -8;
+        if (avg < 400.0 && (A.nbr == A.nbc ? avg >= 64.0 && A.nbr >= 24576 && A.nbr < 65536 : avg >= 96.0)) return -8;
         if (A.nbr >= 65536) return -4;  // middle-length rows of a big level
     }
     return lanes_for(A, fp32);
@@ -534,8 +733,8 @@ int build_fine_stencil(amg_hierarchy *h, const bd_system *sys, cudaStream_t s)
 // Packed row from a raw one; a pair's coefficient is taken from its member
 // that exists on this row type.
 template <bool SYM>
-__global__ void k_fine_pack(int rows, const double *__restrict__ raw, double c2, double it, double *__restrict__ tab,
-                            float *__restrict__ tab32)
+__global__ void k_fine_pack(int rows, const double *__restrict__ raw, double c2, double it, double omega,
+                            double *__restrict__ tab, float *__restrict__ tab32)
 {
     using Row = FineRow<SYM>;
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
@@ -564,13 +763,16 @@ __global__ void k_fine_pack(int rows, const double *__restrict__ raw, double c2,
     }
     put(Row::IDC2, c2 * o[55], c2 * o[56]);
     put(Row::IDT, o[55] * it, o[56] * it);
+    put(Row::KAPPA, -omega * o[55], -omega * o[56]);
+    put(Row::KAPPA + 1, 0.0, 0.0);
 }
 
-int fine_pack(const FineStencil &F, bool sym, double c2, double inv_theta, double *tab, float *tab32, cudaStream_t s)
+int fine_pack(const FineStencil &F, bool sym, double c2, double inv_theta, double omega, double *tab, float *tab32,
+              cudaStream_t s)
 {
     const int rows = 9 * F.NZ, grid = (rows + 63) / 64;
-    if (sym) k_fine_pack<true><<<grid, 64, 0, s>>>(rows, F.raw.p, c2, inv_theta, tab, tab32);
-    else k_fine_pack<false><<<grid, 64, 0, s>>>(rows, F.raw.p, c2, inv_theta, tab, tab32);
+    if (sym) k_fine_pack<true><<<grid, 64, 0, s>>>(rows, F.raw.p, c2, inv_theta, omega, tab, tab32);
+    else k_fine_pack<false><<<grid, 64, 0, s>>>(rows, F.raw.p, c2, inv_theta, omega, tab, tab32);
     ::bd::note_launch();
     BD_LAUNCH_CHECK();
     return BD_OK;
@@ -826,6 +1028,9 @@ static int vcycle_impl(amg_hierarchy *h, const v2<S> *f0, v2<S> *u0, cudaStream_
     constexpr bool SU = std::is_same<S, double>::value;
     const int nl = h->nlev;
     const bool deg2 = h->opts.cheb_degree == 2;
+    // level whose smoothed correction the finest P in pair form gathers: kept in
+    // (v + u, u) form in FP64 (an addition per coarse node instead of per entry)
+    auto OSU = [&](int l) { return SU && l == 1 && h->fine.valid && deg2 && nl > 2; };
     auto down = [&](int l) -> int {
         Level &L = h->lev[l];
         const LV<S> lv = view<S>(h, l);
@@ -850,15 +1055,16 @@ static int vcycle_impl(amg_hierarchy *h, const v2<S> *f0, v2<S> *u0, cudaStream_
         }
         int sr = prof_begin(h, s, 16 * l + R_RESID, l == 0);
         if (fine)
-            BD_TRY((fine_apply<S, SU>(h, u, [&](auto sym) { return FineResid<S, sym.value>{f, lv.r}; }, s)));
+            BD_TRY((fine_apply<S, SU>(h, u, [&](auto sym) { return FineResid<S, sym.value, SU>{f, lv.r}; }, s)));
         else
             BD_TRY(apply_op<S>(L, 0, lv.Av, GatherVec<S>{u}, EpiResid<S>{f, lv.r}, s));
         prof_end(h, sr, l == 0 ? fine_bytes<S>(h, L, 3) : 0.0, fine_flops(h, L), s, fine_ops<S>(h, L, FR_RESID));
         const Level &C = h->lev[l + 1];
         const LV<S> cv = view<S>(h, l + 1);
         int sx = prof_begin(h, s, 16 * l + R_RESTRICT, false);
-        BD_TRY(apply_op<S>(L, 1, lv.Rv, GatherVec<S>{lv.r},
-                             EpiStoreD0<S>{cv.f, cv.d, cv.invd, (S)C.ch_inv_theta}, s));
+        const EpiStoreD0<S> rest{cv.f, cv.d, cv.invd, (S)C.ch_inv_theta};
+        if (fine) BD_TRY((apply_pair<S>(L, 1, GatherVec<S, SU>{lv.r}, rest, s)));
+        else BD_TRY(apply_op<S>(L, 1, lv.Rv, GatherVec<S>{lv.r}, rest, s));
         prof_end(h, sx, 0.0, 0.0, s);
         return BD_OK;
     };
@@ -870,8 +1076,11 @@ static int vcycle_impl(amg_hierarchy *h, const v2<S> *f0, v2<S> *u0, cudaStream_
         v2<S> *u = l == 0 ? u0 : lv.u;
         const LV<S> cv = view<S>(h, l + 1);
         int sp = prof_begin(h, s, 16 * l + R_PROLONG, false);
-        if (fine) BD_TRY(apply_op<S>(L, 2, lv.Pv, GatherVec<S>{cv.u}, EpiAdd<S, SU>{u}, s));
-        else BD_TRY(apply_op<S>(L, 2, lv.Pv, GatherVec<S>{cv.u}, EpiAdd<S>{u}, s));
+        if (fine) {
+            const EpiAddPair<S, SU> add{u, kappa_of<S>(L)};
+            if (OSU(1)) BD_TRY((apply_pair<S>(L, 2, GatherVec<S, SU>{cv.u}, add, s)));
+            else BD_TRY((apply_pair<S>(L, 2, GatherVec<S>{cv.u}, add, s)));
+        } else BD_TRY(apply_op<S>(L, 2, lv.Pv, GatherVec<S>{cv.u}, EpiAdd<S>{u}, s));
         prof_end(h, sp, 0.0, 0.0, s);
         int s1 = prof_begin(h, s, 16 * l + R_POST1, l == 0);
         if (fine)
@@ -898,6 +1107,9 @@ static int vcycle_impl(amg_hierarchy *h, const v2<S> *f0, v2<S> *u0, cudaStream_
                 BD_TRY((fine_apply<S, SU>(h, lv.d, [&](auto sym) {
                     return FinePost2<S, sym.value, SU>{lv.r, u, u};
                 }, s)));
+            } else if (OSU(l)) {
+                BD_TRY(apply_op<S>(L, 0, lv.Av, GatherVec<S>{lv.d},
+                                   EpiPost2<S, true>{lv.r, lv.d, lv.invd, lv.w, u, (S)L.ch_c1, (S)L.ch_c2}, s));
             } else {
                 BD_TRY(apply_op<S>(L, 0, lv.Av, GatherVec<S>{lv.d},
                                    EpiPost2<S>{lv.r, lv.d, lv.invd, lv.w, u, (S)L.ch_c1, (S)L.ch_c2}, s));
@@ -1556,13 +1768,17 @@ static int tune_operator(Level &L, int op, bool sliced_ok, const v2<S> *x, const
     if (sliced_ok && !fp32 && M.nbr >= kSlicedMinRows)
         for (int K = 1; K <= 8; K <<= 1) cand[nc++] = -K;
     const int rule = L.lanes[op];
+    auto run = [&]() {
+        return pair_of(L, op) ? apply_pair<S>(L, op, GatherVec<S, sizeof(S) == 8>{x}, epi, s)
+                              : apply_op<S>(L, op, vals, GatherVec<S>{x}, epi, s);
+    };
     for (int c = 0; c < nc; c++) {
-        if (cand[c] < 0) BD_TRY(build_sliced(M, -cand[c], fp32, L.sl[op], s));
+        if (cand[c] < 0) BD_TRY(build_op(L, op, -cand[c], fp32, s));
         L.lanes[op] = cand[c];
-        BD_TRY(apply_op<S>(L, op, vals, GatherVec<S>{x}, epi, s));
+        BD_TRY(run());
         for (int k = 0; k < kLaneReps; k++) {
             BD_CUDA(cudaEventRecord(ev[c][k][0], s));
-            BD_TRY(apply_op<S>(L, op, vals, GatherVec<S>{x}, epi, s));
+            BD_TRY(run());
             BD_CUDA(cudaEventRecord(ev[c][k][1], s));
         }
         if (cand[c] < 0 || c + 1 == ncsr) BD_CUDA(cudaStreamSynchronize(s));
@@ -1586,7 +1802,7 @@ static int tune_operator(Level &L, int op, bool sliced_ok, const v2<S> *x, const
     const int pick = (t_rule >= 0.0f && t_rule <= 1.03f * best) ? rule : bestT;
     L.lanes[op] = pick;
     if (pick > 0) drop_sliced(L.sl[op]);
-    else if (L.sl[op].K != -pick) BD_TRY(build_sliced(M, -pick, fp32, L.sl[op], s));
+    else if (L.sl[op].K != -pick) BD_TRY(build_op(L, op, -pick, fp32, s));
     return BD_OK;
 }
 
@@ -1645,7 +1861,7 @@ int prepare_solve(amg_hierarchy *h, cudaStream_t s)
             if (a32) {
                 k_to_f32<<<grid_for(4 * L.A.nb, 256), 256, 0, s>>>(4 * L.A.nb, L.A.v.p, L.A32.p); ::bd::note_launch();
             }
-            if (l < h->nlev - 1) {
+            if (l < h->nlev - 1 && a32) {  // the finest level has them in pair form
                 BD_TRY(L.P32.alloc(4 * (size_t)L.P.nb));
                 BD_TRY(L.R32.alloc(4 * (size_t)L.R.nb));
                 k_to_f32<<<grid_for(4 * L.P.nb, 256), 256, 0, s>>>(4 * L.P.nb, L.P.v.p, L.P32.p); ::bd::note_launch();
@@ -1675,8 +1891,9 @@ int prepare_solve(amg_hierarchy *h, cudaStream_t s)
         const size_t len = 2 * (size_t)fine_row_len(F.sym) * 9 * F.NZ;
         BD_TRY(F.tab.alloc(len));
         if (p32) BD_TRY(F.tab32.alloc(len));
-        BD_TRY(fine_pack(F, F.sym, L0.ch_c2, L0.ch_inv_theta, F.tab.p, F.tab32.p, s));
+        BD_TRY(fine_pack(F, F.sym, L0.ch_c2, L0.ch_inv_theta, fine_omega(L0), F.tab.p, F.tab32.p, s));
     }
+    if (h->fine.valid && h->nlev > 1) BD_TRY(build_pairs(h->lev[0], p32, s));
     size_t n0 = 2 * (size_t)h->lev[0].N;
     BD_TRY(h->x.alloc(n0));
     BD_TRY(h->r.alloc(n0));
@@ -1703,11 +1920,11 @@ int prepare_solve(amg_hierarchy *h, cudaStream_t s)
         Level &L = h->lev[l];
         const bool last = l == h->nlev - 1;
         L.lanes[0] = lanes_rule(L.A, p32, l > 0 && !last);
-        L.lanes[1] = last ? 0 : lanes_rule(L.R, p32, true);
-        L.lanes[2] = last ? 0 : lanes_rule(L.P, p32, true);
+        L.lanes[1] = last ? 0 : lanes_rule(L.R, p32, true, pair_of(L, 1));
+        L.lanes[2] = last ? 0 : lanes_rule(L.P, p32, true, pair_of(L, 2));
         for (int op = 0; op < 3; op++) {
             if (L.lanes[op] < 0)
-                BD_TRY(build_sliced(op == 0 ? L.A : (op == 1 ? L.R : L.P), -L.lanes[op], p32, L.sl[op], s));
+                BD_TRY(build_op(L, op, -L.lanes[op], p32, s));
             else drop_sliced(L.sl[op]);
         }
     }
@@ -2252,7 +2469,7 @@ extern "C" int amg_set_level_lanes(amg_hierarchy *h, int level, const int lanes[
         if (T == 0) continue;
         const BSR &M = op == 0 ? L.A : (op == 1 ? L.R : L.P);
         if (T < 0) {
-            const int rc = build_sliced(M, -T, h->prec32, L.sl[op], s);
+            const int rc = build_op(L, op, -T, h->prec32, s);
             if (rc != BD_OK) {
                 // a half-built sliced form is unusable: fall back to the
                 // block-CSR form the rule gives, which needs no extra buffers

@@ -46,11 +46,6 @@ struct StCoef {
     __device__ __forceinline__ const double *at(int p) const { return coef + 4 * mem[p]; }
 };
 
-template <class S> struct StGather {
-    const v2<S> *__restrict__ x;
-    __device__ __forceinline__ v2<S> operator()(int q) const { return x[q]; }
-};
-
 // Epilogues of the stacked V-cycle: the single-hierarchy Chebyshev steps
 // (Saad, Alg. 12.1 on D^{-1}A, degree 2) with the coefficients of the row's
 // member.
@@ -139,14 +134,19 @@ struct StStore {  // q = A p (FP64, PCG)
     __device__ __forceinline__ void operator()(int p, double y0, double y1) const { q[p] = make_double2(y0, y1); }
 };
 
-struct StAddX {  // u += P e_c with u in (v + u, u) form
-    double2 *__restrict__ u;
-    __device__ __forceinline__ void operator()(int p, double y0, double y1) const
+// u += P e_c on a stencil finest level, P in pair form (PairOp): kappa scales
+// the row; u in (v + u, u) form in FP64
+template <class S, bool SU> struct StAddPair {
+    v2<S> *__restrict__ u;
+    const v2<S> *__restrict__ kappa;
+    __device__ __forceinline__ void operator()(int p, S y0, S y1) const
     {
-        const double2 a = u[p];
-        u[p] = make_double2(a.x + (y0 + y1), a.y + y1);
+        const v2<S> a = u[p], k = kappa[p];
+        const S e1 = k.y * y1;
+        u[p] = V2<S>::mk(SU ? a.x + fma(k.x, y0, e1) : a.x + k.x * y0, a.y + e1);
     }
 };
+
 // ------------------------------------------------------------------ assembly of the stack
 __global__ void k_st_shift(long long n, const int *__restrict__ src, int *__restrict__ dst, int add)
 {
@@ -157,6 +157,12 @@ __global__ void k_st_fill(long long n, int *__restrict__ dst, int v)
 {
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
         dst[i] = v;
+}
+
+__global__ void k_st_f32(long long n, const double *__restrict__ src, float *__restrict__ dst)
+{
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
+        dst[i] = (float)src[i];
 }
 
 // ------------------------------------------------------------------ coarsest levels
@@ -488,6 +494,10 @@ struct StLevel {
     int rowsA = 0;             // rows of the stacked A (N on the finest level, Ns below)
     BSR A, R, P;               // FP64 values (A of the finest level always: the PCG's A p)
     DBuf<float> A32, R32, P32; // FP32 V-cycle values
+    // a stencil finest level: R and P in pair form (their A32, P32 stay empty)
+    PairOp pair[2];
+    DBuf<double> kappa;
+    DBuf<float> kappa32;
     int lanes[3] = {0, 0, 0};
     DBuf<int> mem;             // member of each node
     DBuf<double> coef;         // 3 per member
@@ -562,21 +572,38 @@ namespace bd {
 namespace {
 
 // One member's block rows [0, nbr) of M appended to the stacked operator at
-// row `row0` / block `blk0`, its columns shifted by `col0`.
-int st_append(const BSR &M, int nbr, const float *v32, BSR &O, DBuf<float> *O32, int row0, long long blk0, int col0,
-              bool fp64, cudaStream_t s)
+// row `row0` / block `blk0`, its columns shifted by `col0`: full blocks (FP64
+// and/or FP32 values), or M's pair form into OP.
+int st_append(const BSR &M, int nbr, const float *v32, const PairOp *pr, BSR &O, DBuf<float> *O32, PairOp *OP, int row0,
+              long long blk0, int col0, bool fp64, cudaStream_t s)
 {
     if (nbr <= 0) return BD_OK;
     int nb = 0;
     BD_CUDA(cudaMemcpyAsync(&nb, M.rp.p + nbr, sizeof(int), cudaMemcpyDeviceToHost, s));
     BD_CUDA(cudaStreamSynchronize(s));
     k_st_shift<<<grid_for(nbr, 256), 256, 0, s>>>(nbr, M.rp.p, O.rp.p + row0, (int)blk0); ::bd::note_launch();
+    auto copy = [&](auto *dst, const auto *src, int per) {
+        return cudaMemcpyAsync(dst + per * blk0, src, sizeof(*dst) * per * (size_t)nb, cudaMemcpyDeviceToDevice, s);
+    };
     if (nb > 0) {
-        k_st_shift<<<grid_for(nb, 256), 256, 0, s>>>(nb, M.ci.p, O.ci.p + blk0, col0); ::bd::note_launch();
-        if (fp64) BD_CUDA(cudaMemcpyAsync(O.v.p + 4 * blk0, M.v.p, sizeof(double) * 4 * (size_t)nb,
-                                          cudaMemcpyDeviceToDevice, s));
-        if (O32) BD_CUDA(cudaMemcpyAsync(O32->p + 4 * blk0, v32, sizeof(float) * 4 * (size_t)nb,
-                                         cudaMemcpyDeviceToDevice, s));
+        // (an own entry's column keeps its sign bit: q + col0 < 2^31)
+        k_st_shift<<<grid_for(nb, 256), 256, 0, s>>>(nb, pr ? pr->ci.p : M.ci.p, (pr ? OP->ci.p : O.ci.p) + blk0, col0);
+        ::bd::note_launch();
+        if (pr && O32) {
+            BD_CUDA(copy(OP->v32.p, pr->v32.p, 2));
+            BD_CUDA(copy(OP->alpha32.p, pr->alpha32.p, 1));
+        } else if (pr) {
+            BD_CUDA(copy(OP->v.p, pr->v.p, 2));
+            BD_CUDA(copy(OP->alpha.p, pr->alpha.p, 1));
+        } else {
+            if (fp64) BD_CUDA(copy(O.v.p, M.v.p, 4));
+            if (O32 && v32) {
+                BD_CUDA(copy(O32->p, v32, 4));
+            } else if (O32) {  // a stencil finest level keeps no FP32 blocks (stacked with a block-CSR one)
+                k_st_f32<<<grid_for(4LL * nb, 256), 256, 0, s>>>(4LL * nb, M.v.p, O32->p + 4 * blk0);
+                ::bd::note_launch();
+            }
+        }
     }
     BD_LAUNCH_CHECK();
     return BD_OK;
@@ -587,6 +614,7 @@ int st_append(const BSR &M, int nbr, const float *v32, BSR &O, DBuf<float> *O32,
 struct StPart {
     const BSR *M;
     const float *v32;
+    const PairOp *pr;  // pair form to stack instead of the blocks (all parts, or none)
     int nbr;
     long long row0;
     long long col0;
@@ -594,7 +622,7 @@ struct StPart {
 // rows: the stacked operator's rows, the parts' rows at their row0 (ascending)
 // and empty rows in between (the finest level's padding to multiples of 32)
 int st_build(const std::vector<StPart> &parts, long long rows, int ncols, bool fp64, bool fp32, BSR &O,
-             DBuf<float> &O32, cudaStream_t s)
+             DBuf<float> &O32, PairOp *OP, cudaStream_t s)
 {
     long long blocks = 0;
     for (const StPart &pt : parts) blocks += pt.nbr > 0 ? pt.M->nb : 0;  // full operators: nbr == M->nbr
@@ -602,10 +630,24 @@ int st_build(const std::vector<StPart> &parts, long long rows, int ncols, bool f
     O.nbr = (int)rows;
     O.nbc = ncols;
     O.nb = blocks;
+    const size_t nb = (size_t)std::max<long long>(blocks, 1);
+    const bool pairs = OP && !parts.empty() && parts[0].pr;
     BD_TRY(O.rp.alloc((size_t)rows + 1));
-    BD_TRY(O.ci.alloc((size_t)std::max<long long>(blocks, 1)));
-    if (fp64) BD_TRY(O.v.alloc(4 * (size_t)std::max<long long>(blocks, 1)));
-    if (fp32) BD_TRY(O32.alloc(4 * (size_t)std::max<long long>(blocks, 1)));
+    if (pairs) {
+        BD_TRY(OP->ci.alloc(nb));
+        if (fp32) {
+            BD_TRY(OP->v32.alloc(2 * nb));
+            BD_TRY(OP->alpha32.alloc(nb));
+        } else {
+            BD_TRY(OP->v.alloc(2 * nb));
+            BD_TRY(OP->alpha.alloc(nb));
+        }
+        OP->valid = true;
+    } else {
+        BD_TRY(O.ci.alloc(nb));
+        if (fp64) BD_TRY(O.v.alloc(4 * nb));
+        if (fp32) BD_TRY(O32.alloc(4 * nb));
+    }
     long long blk = 0, next = 0;
     for (const StPart &pt : parts) {
         if (pt.nbr <= 0) continue;
@@ -613,7 +655,8 @@ int st_build(const std::vector<StPart> &parts, long long rows, int ncols, bool f
             k_st_fill<<<grid_for(pt.row0 - next, 256), 256, 0, s>>>(pt.row0 - next, O.rp.p + next, (int)blk);
             ::bd::note_launch();
         }
-        BD_TRY(st_append(*pt.M, pt.nbr, pt.v32, O, fp32 ? &O32 : nullptr, (int)pt.row0, blk, (int)pt.col0, fp64, s));
+        BD_TRY(st_append(*pt.M, pt.nbr, pt.v32, pairs ? pt.pr : nullptr, O, fp32 ? &O32 : nullptr, OP, (int)pt.row0, blk,
+                         (int)pt.col0, fp64, s));
         blk += pt.M->nb;
         next = pt.row0 + pt.nbr;
     }
@@ -645,7 +688,7 @@ int st_fine_build(amg_stack *b, const std::vector<int> &order, const std::vector
         const Level &L0 = b->h[k]->lev[0];
         double *t64 = S.tab.p + at * len;
         float *t32 = b->p32 ? S.tab32.p + at * len : nullptr;
-        BD_TRY(fine_pack(F, S.sym, L0.ch_c2, L0.ch_inv_theta, t64, t32, s));
+        BD_TRY(fine_pack(F, S.sym, L0.ch_c2, L0.ch_inv_theta, fine_omega(L0), t64, t32, s));
         FineGrid g = fine_grid<double>(F, L0.ch_c1);
         g.off = (int)off[k];
         g.unit0 = (int)units;
@@ -722,19 +765,23 @@ int st_create(amg_stack *b, cudaStream_t s)
             const Level &Lk = b->h[k]->lev[l];
             const bool smooth = b->nlev[k] - 1 > l;
             if ((l == 0 && !fine0) || (l > 0 && smooth))
-                pa.push_back({&Lk.A, p32 ? Lk.A32.p : nullptr, Lk.A.nbr, off[l][k], off[l][k]});
-            if (smooth) pp.push_back({&Lk.P, p32 ? Lk.P32.p : nullptr, Lk.P.nbr, off[l][k], off[l + 1][k]});
+                pa.push_back({&Lk.A, p32 ? Lk.A32.p : nullptr, nullptr, Lk.A.nbr, off[l][k], off[l][k]});
+            const bool pairs = l == 0 && fine0;
+            if (smooth)
+                pp.push_back({&Lk.P, p32 ? Lk.P32.p : nullptr, pairs ? &Lk.pair[1] : nullptr, Lk.P.nbr, off[l][k],
+                              off[l + 1][k]});
         }
         if (l + 1 < L)
             for (int k : order[l + 1]) {
                 const Level &Lk = b->h[k]->lev[l];
-                pr.push_back({&Lk.R, p32 ? Lk.R32.p : nullptr, Lk.R.nbr, off[l + 1][k], off[l][k]});
+                pr.push_back({&Lk.R, p32 ? Lk.R32.p : nullptr, l == 0 && fine0 ? &Lk.pair[0] : nullptr, Lk.R.nbr,
+                              off[l + 1][k], off[l][k]});
             }
-        BD_TRY(st_build(pa, l == 0 ? S.N : S.Ns, S.N, l == 0 || !p32, p32, S.A, S.A32, s));
+        BD_TRY(st_build(pa, l == 0 ? S.N : S.Ns, S.N, l == 0 || !p32, p32, S.A, S.A32, nullptr, s));
         S.rowsA = S.A.nbr;
         if (!pp.empty()) {
-            BD_TRY(st_build(pp, S.Ns, b->lev[l + 1].N, !p32, p32, S.P, S.P32, s));
-            BD_TRY(st_build(pr, b->lev[l + 1].N, S.N, !p32, p32, S.R, S.R32, s));
+            BD_TRY(st_build(pp, S.Ns, b->lev[l + 1].N, !p32, p32, S.P, S.P32, &S.pair[1], s));
+            BD_TRY(st_build(pr, b->lev[l + 1].N, S.N, !p32, p32, S.R, S.R32, &S.pair[0], s));
         }
         if (l == 0 && fine0) BD_TRY(st_fine_build(b, order[0], off[0], s));
         // node -> member (-1 on padding), Chebyshev coefficients, inverse diagonals
@@ -752,6 +799,20 @@ int st_create(amg_stack *b, cudaStream_t s)
         BD_CUDA(cudaMemcpyAsync(S.coef.p, coef.data(), sizeof(double) * coef.size(), cudaMemcpyHostToDevice, s));
         BD_CUDA(cudaStreamSynchronize(s));  // coef lives on the host stack
         const long long n2 = 2LL * S.N;
+        if (l == 0 && fine0) {
+            if (p32) BD_TRY(st_vec(S.kappa32, n2, s));
+            else BD_TRY(st_vec(S.kappa, n2, s));
+            for (int k : order[l]) {
+                const Level &Lk = b->h[k]->lev[0];
+                if (b->nlev[k] <= 1) continue;
+                if (p32)
+                    BD_CUDA(cudaMemcpyAsync(S.kappa32.p + 2 * off[l][k], Lk.kappa32.p, sizeof(float) * 2 * Lk.N,
+                                            cudaMemcpyDeviceToDevice, s));
+                else
+                    BD_CUDA(cudaMemcpyAsync(S.kappa.p + 2 * off[l][k], Lk.kappa.p, sizeof(double) * 2 * Lk.N,
+                                            cudaMemcpyDeviceToDevice, s));
+            }
+        }
         if (p32) {
             BD_TRY(st_vec(S.invd32, n2, s));
             for (int k : order[l])
@@ -865,6 +926,9 @@ template <> StView<float> st_view<float>(amg_stack *b, int l)
             (float2 *)S.d32.p, (float2 *)S.w32.p, (const float2 *)S.invd32.p};
 }
 
+template <class S> const v2<S> *st_kappa(const StLevel &Lv);
+template <> const double2 *st_kappa<double>(const StLevel &Lv) { return (const double2 *)Lv.kappa.p; }
+template <> const float2 *st_kappa<float>(const StLevel &Lv) { return (const float2 *)Lv.kappa32.p; }
 template <class S> const FineGrid *st_grids(const StLevel &Lv);
 template <> const FineGrid *st_grids<double>(const StLevel &Lv) { return Lv.grid.p; }
 template <> const FineGrid *st_grids<float>(const StLevel &Lv) { return Lv.grid32.p; }
@@ -892,7 +956,7 @@ int st_fine(const StLevel &Lv, bool all, const v2<S> *x, F make, cudaStream_t s)
 template <class S, class E>
 int st_apply(const StLevel &Lv, int rows, const S *vals, const v2<S> *x, E e, cudaStream_t s)
 {
-    return launch_bsr_rows<S>(rows, Lv.A.rp.p, Lv.A.ci.p, vals, Lv.lanes[0], StGather<S>{x}, e, s);
+    return launch_bsr_rows(rows, Lv.A.rp.p, Lv.A.ci.p, MatFull<S>{vals}, Lv.lanes[0], GatherVec<S>{x}, e, s);
 }
 
 template <class S>
@@ -907,12 +971,17 @@ int st_vcycle(amg_stack *b, cudaStream_t s)
         const StCoef c{Lv.mem.p, Lv.coef.p}, cc{b->lev[l + 1].mem.p, b->lev[l + 1].coef.p};
         if (l == 0 && Lv.fine) {
             BD_TRY((st_fine<S, SU>(Lv, false, v.d, [&](auto sym) { return FinePre<S, sym.value, SU>{v.f, v.u}; }, s)));
-            BD_TRY((st_fine<S, SU>(Lv, false, v.u, [&](auto sym) { return FineResid<S, sym.value>{v.f, v.r}; }, s)));
+            BD_TRY((st_fine<S, SU>(Lv, false, v.u, [&](auto sym) { return FineResid<S, sym.value, SU>{v.f, v.r}; }, s)));
         } else {
             BD_TRY(st_apply<S>(Lv, Lv.Ns, v.Av, v.d, StPre<S>{v.f, v.invd, v.d, v.u, c}, s));
             BD_TRY(st_apply<S>(Lv, Lv.Ns, v.Av, v.u, StResid<S>{v.f, v.r}, s));
         }
-        BD_TRY(launch_bsr<S>(Lv.R, v.Rv, Lv.lanes[1], StGather<S>{v.r}, StStoreD0<S>{cv.f, cv.d, cv.invd, cc}, s));
+        const StStoreD0<S> rest{cv.f, cv.d, cv.invd, cc};
+        if (Lv.pair[0].valid)
+            BD_TRY((launch_bsr_rows(Lv.R.nbr, Lv.R.rp.p, Lv.pair[0].ci.p, mat_pair<S>(Lv.pair[0]), Lv.lanes[1],
+                                    GatherVec<S, SU>{v.r}, rest, s)));
+        else
+            BD_TRY(launch_bsr<S>(Lv.R, v.Rv, Lv.lanes[1], GatherVec<S>{v.r}, rest, s));
     }
     StLevelPtrs<S> lp{};
     for (int l = 0; l < L; l++) {
@@ -931,8 +1000,8 @@ int st_vcycle(amg_stack *b, cudaStream_t s)
         const StView<S> v = st_view<S>(b, l), cv = st_view<S>(b, l + 1);
         const StCoef c{Lv.mem.p, Lv.coef.p};
         if (l == 0 && Lv.fine) {
-            if constexpr (SU) BD_TRY(launch_bsr<S>(Lv.P, v.Pv, Lv.lanes[2], StGather<S>{cv.u}, StAddX{v.u}, s));
-            else BD_TRY(launch_bsr<S>(Lv.P, v.Pv, Lv.lanes[2], StGather<S>{cv.u}, StAdd<S>{v.u}, s));
+            BD_TRY((launch_bsr_rows(Lv.P.nbr, Lv.P.rp.p, Lv.pair[1].ci.p, mat_pair<S>(Lv.pair[1]), Lv.lanes[2],
+                                    GatherVec<S>{cv.u}, StAddPair<S, SU>{v.u, st_kappa<S>(Lv)}, s)));
             BD_TRY((st_fine<S, SU>(Lv, false, v.u, [&](auto sym) {
                 return FinePost1<S, sym.value, SU>{v.f, v.r, v.d, nullptr};
             }, s)));
@@ -941,7 +1010,7 @@ int st_vcycle(amg_stack *b, cudaStream_t s)
             }, s)));
             continue;
         }
-        BD_TRY(launch_bsr<S>(Lv.P, v.Pv, Lv.lanes[2], StGather<S>{cv.u}, StAdd<S>{v.u}, s));
+        BD_TRY(launch_bsr<S>(Lv.P, v.Pv, Lv.lanes[2], GatherVec<S>{cv.u}, StAdd<S>{v.u}, s));
         BD_TRY(st_apply<S>(Lv, Lv.Ns, v.Av, v.u, StPost1<S>{v.f, v.invd, v.u, v.r, v.d, v.w, c}, s));
         BD_TRY(st_apply<S>(Lv, Lv.Ns, v.Av, v.d, StPost2<S>{v.r, v.d, v.invd, v.w, v.u, c}, s));
     }
@@ -988,8 +1057,8 @@ int st_apply_a(amg_stack *b, const double2 *x, double2 *q, cudaStream_t s, bool 
         auto store = [&](auto) { return FineStore<double>{q}; };
         return su ? st_fine<double, true>(S, true, x, store, s) : st_fine<double, false>(S, true, x, store, s);
     }
-    return launch_bsr_rows<double>(S.N, S.A.rp.p, S.A.ci.p, S.A.v.p, lanes_for(S.A, false), StGather<double>{x},
-                                   StStore{q}, s);
+    return launch_bsr_rows(S.N, S.A.rp.p, S.A.ci.p, MatFull<double>{S.A.v.p}, lanes_for(S.A, false),
+                           GatherVec<double>{x}, StStore{q}, s);
 }
 
 template <class S>

@@ -32,7 +32,7 @@ namespace bd {
 // the same for dz = +1 and a pad; in the general form for dz = -1 too (in the
 // symmetric form a plane's dz = +1 coefficients are those of the plane above
 // for dz = -1, and each group is loaded once for both); c2 D^{-1}; D^{-1} /
-// theta.  In-plane positions: symmetric form 0 centre, 1 x pair, 2 y pair, 3
+// theta; kappa = -omega D^{-1} (PairOp); a pad.  In-plane positions: symmetric form 0 centre, 1 x pair, 2 y pair, 3
 // the (-1,-1), (1,1) pair, 4 the (1,-1), (-1,1) pair; general form 3 (dy + 1) +
 // dx + 1.
 template <bool SYM> struct FineRow {
@@ -43,7 +43,8 @@ template <bool SYM> struct FineRow {
     static constexpr int DN = 2 * G;          // general form only
     static constexpr int IDC2 = (SYM ? 2 : 3) * G;
     static constexpr int IDT = IDC2 + 1;
-    static constexpr int LEN = IDC2 + 2;
+    static constexpr int KAPPA = IDC2 + 2;
+    static constexpr int LEN = IDC2 + 4;
 };
 
 // One slab of a launch: extents in nodes, first node and first work unit.  A
@@ -238,6 +239,7 @@ template <class S, bool SYM> struct FineConst {
     using Row = FineRow<SYM>;
     static __device__ __forceinline__ v2<S> idc2(const v2<S> *t) { return t[Row::IDC2]; }
     static __device__ __forceinline__ v2<S> idt(const v2<S> *t) { return t[Row::IDT]; }
+    static __device__ __forceinline__ v2<S> kappa(const v2<S> *t) { return t[Row::KAPPA]; }
 };
 
 // pre-smoothing from zero: u = d0 + (c1 d0 + c2 D^{-1} (f - A d0)), d0 gathered
@@ -254,13 +256,17 @@ template <class S, bool SYM, bool SU> struct FinePre {
     }
 };
 
-template <class S, bool SYM> struct FineResid {  // r = f - A u
+// what the restriction gathers: kappa (f - A u), kappa R's row scaling (PairOp);
+// in (v + u, u) form in FP64, plain in FP32 (whose additions are free)
+template <class S, bool SYM, bool SU> struct FineResid {
     const v2<S> *__restrict__ f;
     v2<S> *__restrict__ r;
     __device__ __forceinline__ v2<S> load(int p, bool ok) const { return fine_ld<S>(f, p, ok); }
-    __device__ __forceinline__ void operator()(int p, const v2<S> *, v2<S> fp, v2<S>, S, S y0, S y1)
+    __device__ __forceinline__ void operator()(int p, const v2<S> *t, v2<S> fp, v2<S>, S, S y0, S y1)
     {
-        r[p] = V2<S>::mk(fp.x - y0, fp.y - y1);
+        const v2<S> k = FineConst<S, SYM>::kappa(t);
+        const S t1 = k.y * (fp.y - y1), r0 = fp.x - y0;
+        r[p] = V2<S>::mk(SU ? fma(k.x, r0, t1) : k.x * r0, t1);
     }
 };
 
@@ -377,7 +383,10 @@ template <class S> static FineGrid fine_grid(const FineStencil &F, double c1)
 
 // Table of one slab from its raw rows and the level's Chebyshev constants, in
 // the symmetric or the general form.
-int fine_pack(const FineStencil &F, bool sym, double c2, double inv_theta, double *tab, float *tab32, cudaStream_t s);
+int fine_pack(const FineStencil &F, bool sym, double c2, double inv_theta, double omega, double *tab, float *tab32,
+              cudaStream_t s);
+// the prolongator smoother's omega on a level (0 on a hierarchy's only level)
+inline double fine_omega(const Level &L) { return L.lam > 0.0 ? 4.0 / (3.0 * L.lam) : 0.0; }
 constexpr int fine_row_len(bool sym) { return sym ? FineRow<true>::LEN : FineRow<false>::LEN; }
 
 }  // namespace bd

@@ -76,3 +76,22 @@ def test_stack_of_both_forms(B, precision):
     for (xr, ir), x, i in zip(ref, xs, B.amg_stack_solve(B.amg_stack_create(hs), fs, xs)):
         assert i["status"] == 0 and abs(i["iters"] - ir["iters"]) <= 1
         assert float((x - xr).norm()) <= 1e-7 * float(xr.norm())
+
+
+@pytest.mark.parametrize("precision", [0, 1])
+def test_stack_of_stencil_and_csr_members(B, precision):
+    """A member given as a caller's CSR has no stencil: the whole stack then runs
+    on blocks, the slab's included."""
+    import torch
+
+    m = W.mesh(14, 8, 9)
+    sysh = B.bd_assemble(m, W.DEFAULT_PARAMS, _fib(m, False))
+    rp, ci, v, _ = B.bd_system_export(sysh)
+    n = rp.size - 1
+    o = B.amg_options_default(coarse_eq_limit=30, precision=precision)
+    hs = [B.amg_setup(sysh, o), B.amg_setup_from_csr(n, rp, ci, v, o)]
+    fs = [torch.tensor(W.rhs(n, k), device="cuda") for k in range(2)]
+    ref = [B.amg_solve(h, f, torch.zeros_like(f))[0] for h, f in zip(hs, fs)]
+    xs = [torch.zeros_like(f) for f in fs]
+    for x, xr, i in zip(xs, ref, B.amg_stack_solve(B.amg_stack_create(hs), fs, xs)):
+        assert i["status"] == 0 and float((x - xr).norm()) <= 1e-7 * float(xr.norm())
