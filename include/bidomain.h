@@ -148,7 +148,7 @@ int bd_dot_exact(const double *x, const double *y, long long n, int on_device, d
  * leaving none for the library to take), and latency-critical loops in which
  * an allocation would synchronise the device and stall the pipeline.
  * x, y: n doubles in device memory; out: one double in device memory, written
- * in stream order (the call does not synchronise).  Scratch: one 552-byte
+ * in stream order (the call does not synchronise).  Scratch: one 560-byte
  * accumulator in a static device array that every GPU loading the library
  * holds until exit; each call clears it on `stream` before use.  All calls
  * share that array, so calls whose work overlaps on the GPU (different

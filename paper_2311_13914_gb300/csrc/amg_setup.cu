@@ -1613,7 +1613,7 @@ static int build_coarsest(amg_hierarchy *h, int l, cudaStream_t s)
 static int setup_from_level0(amg_hierarchy *h, cudaStream_t s)
 {
     Level &L0 = h->lev[0];
-    BD_TRY(h->exact_acc.alloc(kExactLimbs + 1));
+    BD_TRY(h->exact_acc.alloc(kExactScratch));
     BD_TRY(L0.B.alloc(2 * (size_t)L0.N));
     k_fill<<<nblk(2LL * L0.N), 256, 0, s>>>(2 * L0.N, 1.0, L0.B.p); ::bd::note_launch();
     BD_LAUNCH_CHECK();

@@ -126,8 +126,10 @@ int sort_segments(int *keys, int *payload, const int *seg, int nseg, int max_len
 // Correctly rounded dot product sum_i x[i]*y[i] (each product rounded, then an
 // exact long accumulator and one rounding to nearest-even), written to *out on
 // the device.  Order-independent, hence bit-reproducible.  `acc` must hold
-// kExactLimbs+1 long longs of scratch.
+// kExactScratch long longs: the limbs, the flags of infinities and NaNs, and the
+// blocks' arrival counter.
 constexpr int kExactLimbs = 68;
+constexpr int kExactScratch = kExactLimbs + 2;
 int exact_dot(const double *x, const double *y, int n, double *out, long long *acc,
               cudaStream_t s);
 

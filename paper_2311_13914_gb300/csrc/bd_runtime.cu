@@ -1,6 +1,7 @@
 // bd_runtime.cu -- status codes, option defaults, device utilities (prefix
 // scan, segmented sort, correctly rounded dot product), copies and format
 // conversion used by the other translation units.
+#include <algorithm>
 #include <atomic>
 #include <climits>
 #include <cstring>
@@ -270,131 +271,195 @@ __device__ __forceinline__ void exact_acc_digits(long long *acc, int li, unsigne
     if (d2) atomicAdd(a + li + 2, d2);
 }
 
-// Whole warps step through the elements.  When every nonzero finite product
-// of a warp's step falls on the same limb index (the usual case: products of
-// similar magnitude), the warp sums its digits exactly (32 signed 33-bit
-// digits fit 64 bits) and one lane adds them; otherwise every lane adds its
-// own.  Integer sums are associative, so the total is the same either way.
-__global__ void k_exact_dot_partial(const double *__restrict__ x, const double *__restrict__ y,
-                                    int n, long long *gacc)
+// A thread's window: a 256-bit two's complement integer in units of
+// 2^(b0 - 1074), b0 a multiple of 32.
+struct ExactWindow {
+    unsigned long long w[4] = {0, 0, 0, 0};
+    __device__ __forceinline__ void add(unsigned long long v0, unsigned long long v1, unsigned long long v2,
+                                        unsigned long long v3)
+    {
+        asm("add.cc.u64 %0, %0, %4;\n\t"
+            "addc.cc.u64 %1, %1, %5;\n\t"
+            "addc.cc.u64 %2, %2, %6;\n\t"
+            "addc.u64 %3, %3, %7;"
+            : "+l"(w[0]), "+l"(w[1]), "+l"(w[2]), "+l"(w[3])
+            : "l"(v0), "l"(v1), "l"(v2), "l"(v3));
+    }
+};
+// Highest position of a product's last bit in the window: 53 bits above it and
+// 2^31 of them stay below 2^255.
+constexpr int kWindowTop = 169;
+
+// The exact total of gacc's limbs rounded to the nearest double (ties to even).
+// Called by one whole warp with the limbs in shared memory.
+__device__ double exact_round(long long *l, int flags)
+{
+    const int lane = threadIdx.x & 31;
+    int lo = kExactLimbs, hi = -1;
+    for (int i0 = 0; i0 < kExactLimbs; i0 += 32) {
+        const int i = i0 + lane;
+        const unsigned m = __ballot_sync(0xffffffffu, i < kExactLimbs && l[i] != 0);
+        if (m) {
+            if (lo == kExactLimbs) lo = i0 + __ffs(m) - 1;
+            hi = i0 + 31 - __clz(m);
+        }
+    }
+    if (lane != 0) return 0.0;
+    if (flags) {
+        if ((flags & 1) || ((flags & 2) && (flags & 4))) return __longlong_as_double(0x7ff8000000000000LL);
+        return __longlong_as_double((flags & 2) ? 0x7ff0000000000000LL : (long long)0xfff0000000000000ULL);
+    }
+    if (hi < 0) return 0.0;
+    // carries into 32-bit digits; the limb above the highest nonzero one takes the
+    // last carry and the sign
+    const int end = hi < kExactLimbs - 1 ? hi + 1 : hi;
+    bool negative = false;
+    for (int pass = 0; pass < 2; pass++) {
+        for (int i = lo; i < end; i++) {
+            const long long d = l[i] & 0xffffffffLL;
+            l[i + 1] += (l[i] - d) >> 32;  // exact: l[i] - d is a multiple of 2^32
+            l[i] = d;
+        }
+        if (pass || l[end] >= 0) break;
+        negative = true;
+        for (int i = lo; i <= end; i++) l[i] = -l[i];
+    }
+    int top = end;
+    while (top > lo && l[top] == 0) top--;
+    double r;
+    if (l[top] == 0) return 0.0;
+    if (l[top] >= (1LL << 32)) {
+        r = __longlong_as_double(0x7ff0000000000000LL);
+    } else {
+        auto limb = [&](int i) -> unsigned long long { return i >= lo ? (unsigned long long)l[i] : 0ULL; };
+        const int H = 32 * top + 31 - __clz((unsigned)l[top]);  // the highest bit
+        const unsigned long long u = (limb(top) << 32) | limb(top - 1), v = (limb(top - 2) << 32) | limb(top - 3);
+        if (H < 53) {
+            r = scalbn((double)(top == 0 ? u >> 32 : u), -1074);
+        } else {
+            // 128 bits from limb top down; bit H sits at position P
+            const int P = 96 + (H & 31), sh = P - 52;  // 44 .. 75
+            unsigned long long mant = sh < 64 ? (u << (64 - sh)) | (v >> sh) : u >> (sh - 64);
+            const int rb = sh - 1;
+            const bool round = rb < 64 ? (v >> rb) & 1 : (u >> (rb - 64)) & 1;
+            bool sticky = rb < 64 ? (v & ((1ULL << rb) - 1)) != 0 : v != 0 || (u & ((1ULL << (rb - 64)) - 1)) != 0;
+            for (int i = top - 4; i >= lo && !sticky; i--) sticky = l[i] != 0;
+            int e = H;
+            if (round && (sticky || (mant & 1)) && ++mant == (1ULL << 53)) {
+                mant >>= 1;
+                e++;
+            }
+            r = scalbn((double)mant, e - 52 - 1074);
+        }
+    }
+    return negative ? -r : r;
+}
+
+// Every thread sums its products in a register window placed by its block's
+// first products (the largest of them 128 to 159 bits above the window's
+// base), about 45 integer instructions a product; the few that do not fit go
+// to the block's limbs one by one.  The warps fold their windows by shuffles,
+// the blocks add their limbs to the global accumulator, and the last block to
+// arrive rounds it.  One launch and a clear, where a digit-wise sum per warp
+// step, shared by three launches with a one-thread rounding, took 57 us for 1.1 M
+// products (now 16, the call included; reading them takes 2.6 us of HBM).
+constexpr int kDotThreads = 512, kDotUnroll = 4;
+__global__ void __launch_bounds__(kDotThreads) k_exact_dot(const double *__restrict__ x, const double *__restrict__ y,
+                                                           int n, long long *gacc, double *__restrict__ out)
 {
     __shared__ long long acc[kExactLimbs];
-    __shared__ int flags;
+    __shared__ int flags, emax;
+    __shared__ bool last;
     for (int i = threadIdx.x; i < kExactLimbs; i += blockDim.x) acc[i] = 0;
-    if (threadIdx.x == 0) flags = 0;
+    if (threadIdx.x == 0) {
+        flags = 0;
+        emax = 0;
+    }
     __syncthreads();
-    const int lane = threadIdx.x & 31;
     const long long stride = (long long)gridDim.x * blockDim.x;
-    for (long long base = (long long)blockIdx.x * blockDim.x + (threadIdx.x & ~31); base < n; base += stride) {
-        const long long i = base + lane;
-        const double p = i < n ? __dmul_rn(x[i], y[i]) : 0.0;
-        int li, nf;
-        unsigned long long d0, d1, d2;
-        const bool fin = exact_digits(p, li, d0, d1, d2, nf);
-        const bool nz = fin && (d0 | d1 | d2);
-        const unsigned nzm = __ballot_sync(0xffffffffu, nz);
-        const bool allfin = __all_sync(0xffffffffu, fin);
-        if (nzm == 0 && allfin) continue;
-        const int li0 = __shfl_sync(0xffffffffu, li, __ffs(nzm ? nzm : 1u) - 1);
-        if (allfin && __all_sync(0xffffffffu, !nz || li == li0)) {
+    const long long i0 = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+    double p[kDotUnroll];
+    auto fetch = [&](long long i) {
 #pragma unroll
-            for (int o = 16; o > 0; o >>= 1) {
-                d0 += __shfl_xor_sync(0xffffffffu, d0, o);
-                d1 += __shfl_xor_sync(0xffffffffu, d1, o);
-                d2 += __shfl_xor_sync(0xffffffffu, d2, o);
-            }
-            if (lane == 0) exact_acc_digits(acc, li0, d0, d1, d2);
-        } else {
-            if (!fin) atomicOr(&flags, nf);
-            else if (nz) exact_acc_digits(acc, li, d0, d1, d2);
+        for (int k = 0; k < kDotUnroll; k++) {
+            const long long j = i + k * stride;
+            p[k] = j < n ? __dmul_rn(x[j], y[j]) : 0.0;
         }
+    };
+    fetch(i0);
+    unsigned em = 0;
+#pragma unroll
+    for (int k = 0; k < kDotUnroll; k++) {
+        const unsigned e = ((unsigned)__double2hiint(p[k]) >> 20) & 0x7ff;
+        if (e != 0x7ff) em = max(em, e);
+    }
+    em = __reduce_max_sync(0xffffffffu, em);
+    if ((threadIdx.x & 31) == 0) atomicMax(&emax, (int)em);
+    __syncthreads();
+    const int b0 = max(0, emax - 1 - 128) & ~31;
+    ExactWindow W;
+    for (long long i = i0; i < n; i += kDotUnroll * stride) {
+        if (i != i0) fetch(i);
+#pragma unroll
+        for (int k = 0; k < kDotUnroll; k++) {
+            const unsigned long long bits = (unsigned long long)__double_as_longlong(p[k]);
+            if ((bits << 1) == 0) continue;
+            const int E = (int)((bits >> 52) & 0x7ff);
+            const unsigned long long m = (bits & 0xFFFFFFFFFFFFFULL) | (E ? 1ULL << 52 : 0);
+            const int s = max(E, 1) - 1 - b0;
+            if (E < 0x7ff && s >= 0 && s <= kWindowTop) {
+                const int r = s & 63, w = s >> 6;
+                const unsigned long long neg = (unsigned long long)((long long)bits >> 63);
+                // (m << s) negated where the sign is set: xor and add one
+                const unsigned long long a = m << r, c = r ? m >> (64 - r) : 0;
+                unsigned long long v0 = w == 0 ? a : 0, v1 = w == 1 ? a : (w == 0 ? c : 0);
+                unsigned long long v2 = w == 2 ? a : (w == 1 ? c : 0), v3 = w == 2 ? c : 0;
+                W.add(v0 ^ neg, v1 ^ neg, v2 ^ neg, v3 ^ neg);
+                W.add(neg & 1, 0, 0, 0);
+            } else {
+                int li, nf;
+                unsigned long long d0, d1, d2;
+                if (!exact_digits(p[k], li, d0, d1, d2, nf)) atomicOr(&flags, nf);
+                else exact_acc_digits(acc, li, d0, d1, d2);
+            }
+        }
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        unsigned long long v[4];
+#pragma unroll
+        for (int k = 0; k < 4; k++) v[k] = __shfl_xor_sync(0xffffffffu, W.w[k], o);
+        W.add(v[0], v[1], v[2], v[3]);
+    }
+    const int lane = threadIdx.x & 31;
+    if (lane < 8) {  // every lane holds the warp's total: lane d adds digit d, the top one signed
+        const int q = lane >> 1;
+        const unsigned long long w = q == 0 ? W.w[0] : (q == 1 ? W.w[1] : (q == 2 ? W.w[2] : W.w[3]));
+        const long long d = lane == 7 ? (long long)w >> 32 : (long long)((lane & 1) ? w >> 32 : w & 0xffffffffULL);
+        if (d) atomicAdd((unsigned long long *)&acc[(b0 >> 5) + lane], (unsigned long long)d);
     }
     __syncthreads();
     for (int i = threadIdx.x; i < kExactLimbs; i += blockDim.x)
         if (acc[i]) atomicAdd((unsigned long long *)&gacc[i], (unsigned long long)acc[i]);
     if (threadIdx.x == 0 && flags) atomicOr((int *)&gacc[kExactLimbs], flags);
-}
-
-// Round the exact total to the nearest double (ties to even).
-__global__ void k_exact_round(long long *gacc, double *out)
-{
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
-    int flags = (int)gacc[kExactLimbs];
-    if (flags) {
-        double r;
-        if ((flags & 1) || ((flags & 2) && (flags & 4))) r = __longlong_as_double(0x7ff8000000000000LL);
-        else if (flags & 2) r = __longlong_as_double(0x7ff0000000000000LL);
-        else r = __longlong_as_double((long long)0xfff0000000000000ULL);
-        *out = r;
-        return;
-    }
-    long long l[kExactLimbs];
-    for (int i = 0; i < kExactLimbs; i++) l[i] = gacc[i];
-    // carry propagation into 32-bit digits, the top limb keeps the sign
-    for (int i = 0; i < kExactLimbs - 1; i++) {
-        long long lo = l[i] & 0xffffffffLL;
-        long long c = (l[i] - lo) >> 32;  // exact: l[i]-lo is a multiple of 2^32
-        l[i] = lo;
-        l[i + 1] += c;
-    }
-    bool negative = l[kExactLimbs - 1] < 0;
-    if (negative) {
-        for (int i = 0; i < kExactLimbs; i++) l[i] = -l[i];
-        for (int i = 0; i < kExactLimbs - 1; i++) {
-            long long lo = l[i] & 0xffffffffLL;
-            long long c = (l[i] - lo) >> 32;
-            l[i] = lo;
-            l[i + 1] += c;
-        }
-    }
-    int top = -1;
-    for (int i = kExactLimbs - 1; i >= 0; i--)
-        if (l[i] != 0) {
-            top = i;
-            break;
-        }
-    double r;
-    if (top < 0) {
-        r = 0.0;
-    } else if (l[top] >= (1LL << 32)) {
-        r = __longlong_as_double(0x7ff0000000000000LL);
-    } else {
-        int H = 32 * top + 31 - __clz((unsigned)l[top]);
-        auto bit = [&](int pos) -> unsigned long long {
-            return (unsigned long long)((l[pos >> 5] >> (pos & 31)) & 1);
-        };
-        unsigned long long mant = 0;
-        if (H < 53) {
-            for (int p = H; p >= 0; p--) mant = (mant << 1) | bit(p);
-            r = scalbn((double)mant, -1074);
-        } else {
-            for (int p = H; p >= H - 52; p--) mant = (mant << 1) | bit(p);
-            unsigned long long rb = bit(H - 53);
-            unsigned long long sticky = 0;
-            for (int p = H - 54; p >= 0 && !sticky; p--) sticky |= bit(p);
-            if (rb && (sticky || (mant & 1))) {
-                mant += 1;
-                if (mant == (1ULL << 53)) {
-                    mant >>= 1;
-                    H += 1;
-                }
-            }
-            r = scalbn((double)mant, H - 52 - 1074);
-        }
-        if (negative) r = -r;
-    }
-    *out = r;
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) last = atomicAdd((unsigned int *)&gacc[kExactLimbs + 1], 1u) == gridDim.x - 1;
+    __syncthreads();
+    if (!last || threadIdx.x >= 32) return;
+    __threadfence();
+    for (int i = threadIdx.x; i < kExactLimbs; i += 32) acc[i] = __ldcg(gacc + i);
+    __syncwarp();
+    const double r = exact_round(acc, (int)__ldcg(gacc + kExactLimbs));
+    if (threadIdx.x == 0) *out = r;
 }
 
 int exact_dot(const double *x, const double *y, int n, double *out, long long *acc, cudaStream_t s)
 {
-    BD_CUDA(cudaMemsetAsync(acc, 0, sizeof(long long) * (kExactLimbs + 1), s));
-    if (n > 0) {
-        int grid = grid_for(n, 256, 2);
-        k_exact_dot_partial<<<grid, 256, 0, s>>>(x, y, n, acc); ::bd::note_launch();
-        BD_LAUNCH_CHECK();
-    }
-    k_exact_round<<<1, 1, 0, s>>>(acc, out); ::bd::note_launch();
+    BD_CUDA(cudaMemsetAsync(acc, 0, sizeof(long long) * kExactScratch, s));
+    const long long per = (long long)kDotThreads * kDotUnroll;
+    const int grid = (int)std::max<long long>(1, std::min<long long>(2 * kSM, (n + per - 1) / per));
+    k_exact_dot<<<grid, kDotThreads, 0, s>>>(x, y, n, acc, out); ::bd::note_launch();
     BD_LAUNCH_CHECK();
     return BD_OK;
 }
@@ -513,10 +578,10 @@ int bsr_to_scalar_csr_host(const BSR &a, int *rp, int *ci, double *v, cudaStream
 
 // ------------------------------------------------------------------ allocation-free dot
 // Scratch of bd_dot_exact_noalloc: one long accumulator (kExactLimbs limbs and
-// a flags word, 552 bytes) in device memory that every GPU loading the library
+// two words, 560 bytes) in device memory that every GPU loading the library
 // holds until the process exits.  Host code must not use the array's name as a
 // device address: the address is looked up once per device below.
-static __device__ __align__(256) long long g_noalloc_dot_acc[kExactLimbs + 1];
+static __device__ __align__(256) long long g_noalloc_dot_acc[kExactScratch];
 
 constexpr int kNoallocMaxDevices = 64;
 static std::mutex g_noalloc_mu;
@@ -577,7 +642,7 @@ extern "C" int bd_dot_exact(const double *x, const double *y, long long n, int o
     cudaStream_t s = (cudaStream_t)stream;
     bd::DBuf<long long> acc;
     bd::DBuf<double> res, dx, dy;
-    BD_TRY(acc.alloc(bd::kExactLimbs + 1));
+    BD_TRY(acc.alloc(bd::kExactScratch));
     BD_TRY(res.alloc(1));
     const double *px = x, *py = y;
     if (!on_device && n > 0) {
