@@ -27,6 +27,7 @@ UNITS = {
     "amg_setup.cu": ["-fmad=false"],
     "amg_solve.cu": [],
     "amg_stack.cu": [],
+    "amg_scalar.cu": [],
     "bd_step.cu": [],
     "bd_serve.cu": [],
     "bd_decoupled.cu": [],

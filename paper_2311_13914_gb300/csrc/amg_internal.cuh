@@ -1,6 +1,8 @@
 // amg_internal.cuh -- hierarchy layout shared by the setup and solve units.
 #pragma once
 
+#include <memory>
+
 #include "bd_common.cuh"
 
 namespace bd {
@@ -94,11 +96,16 @@ struct FineStencil {
 
 }  // namespace bd
 
+namespace bd {
+struct ScalarEll;  // an elliptic hierarchy's solve on its one field (amg_scalar.cu)
+}
+
 struct amg_hierarchy {
     amg_options opts{};
     int nlev = 0;
     bool prec32 = false;        // V-cycle in FP32 inside an FP64 flexible CG
     bd::FineStencil fine;
+    std::shared_ptr<bd::ScalarEll> scalar;
     bd::Level lev[bd::kMaxLevels];
     // coarsest level: dense inverse of A_c + s z z^T / z^T z, null vector z
     int nc = 0;
@@ -153,6 +160,8 @@ int prepare_solve(amg_hierarchy *h, cudaStream_t s);
 int pcg_solve_begin(amg_hierarchy *h, const double *f_dev, double *x_dev, int warm,
                     const solve_options *o, cudaStream_t s, solve_info *info, bool *pending);
 int pcg_solve_end(amg_hierarchy *h, cudaStream_t s, solve_info *info);
+// raw rows and symmetry of sys's operators (invd: interleaved inverse diagonals, or null)
+int fine_raw_build(FineStencil &F, const bd_system *sys, const double *invd, cudaStream_t s);
 int build_fine_stencil(amg_hierarchy *h, const bd_system *sys, cudaStream_t s);
 // Timed step of the solve phase (host-driven loop only).  `fine`: a
 // finest-operator application, timed at profiling level 1 and summed into

@@ -15,6 +15,7 @@
 #include <cmath>
 
 #include "amg_internal.cuh"
+#include "scalar.cuh"
 
 namespace bd {
 
@@ -1735,7 +1736,7 @@ extern "C" int bd_elliptic_setup(const bd_system *sys, const amg_options *opts, 
         delete h;
         return BD_ECUDA;
     }
-    if ((st = setup_from_level0(h, s)) || (st = prepare_solve(h, s))) {
+    if ((st = setup_from_level0(h, s)) || (st = prepare_solve(h, s)) || (st = scalar_build(h, sys, s))) {
         delete h;
         return st;
     }

@@ -19,6 +19,8 @@
 #include "amg_bsr.cuh"
 #include "amg_internal.cuh"
 #include "fine_stencil.cuh"
+#include "pcg_reduce.cuh"
+#include "scalar.cuh"
 
 namespace bd {
 
@@ -215,20 +217,6 @@ __global__ void k_slice_blocks(int nsl, long long groups, int blocks, const int 
         else hi = m;
     }
     bsl[w] = lo;
-}
-
-// ------------------------------------------------------------------ vector kernels' shares
-// Block b's share [share_lo(n), share_hi(n)) of n rows or nodes: the grid
-// splits the 32-row slices in equal contiguous parts, so with one resident
-// wave of blocks every SM gets the same work (a grid-stride loop leaves the
-// SMs whose blocks drew one row fewer per thread idle for part of the launch).
-__device__ __forceinline__ int share_lo(int n)
-{
-    return (int)((((long long)n + 31) >> 5) * blockIdx.x / gridDim.x) * 32;
-}
-__device__ __forceinline__ int share_hi(int n)
-{
-    return min(n, (int)((((long long)n + 31) >> 5) * (blockIdx.x + 1) / gridDim.x) * 32);
 }
 
 // ------------------------------------------------------------------ fused epilogues
@@ -610,10 +598,8 @@ static int build_pairs(Level &L, bool fp32, cudaStream_t s)
 // 128x128x32 slab's second level, 32001 rows: 145 -> 137, on the 13197 rows of
 // 96x96x24 block-CSR wins, 78 against 93) and, on levels of 65536 rows and more,
 // rows in between and long ones (4 lanes; 256x256x64, 249682 rows: 840 -> 743).
-// Restrictions from 96 blocks a row from 8192 rows on.  Longer rows still (the
-// nearly dense levels of large slabs): a thread block per row in both
-// precisions (11501 rows of 2830 blocks: FP64 sliced 8 1980, 128 threads 1061;
-// FP32 32 lanes 528, 256 threads 403).  Elsewhere the block-CSR rule.
+// Restrictions from 96 blocks a row from 8192 rows on.  Longer rows still and
+// everything else: the block-CSR rule.
 //
 // The finest R and P in pair form have their own crossovers.  R: few lanes
 // where rows fill the GPU (T rows >= 200 K), else up to 16 (31542 rows: 8 lanes
@@ -621,11 +607,10 @@ static int build_pairs(Level &L, bool fp32, cudaStream_t s)
 // 199, 8 211).  P: one lane per row on a million rows and more (256x256x64: FP64
 // sliced 254, one lane 240; FP32 two lanes 127, one 107); the rule above below.
 constexpr int kSlicedMinRows = 8192;
-constexpr double kLongRow = 1000.0;
 static int lanes_rule(const BSR &A, bool fp32, bool sliced_ok, const PairOp *pr = nullptr)
 {
     const double avg = A.nbr > 0 ? (double)A.nb / A.nbr : 1.0;
-    if (avg >= kLongRow) return fp32 ? 256 : 128;
+    if (avg >= kLongRow) return lanes_for(A, fp32);
     if (pr && !fp32 && avg >= 48.0 && A.nbr >= 4096) {
         int T = 4;
         while (T < 16 && (long long)A.nbr * T < 200000) T <<= 1;
@@ -669,8 +654,10 @@ __global__ void k_fine_raw(int NX, int NY, int NZ, const int *__restrict__ rp, c
                 b++;
             }
     o[54] = c * M[p];
-    o[55] = invd[2 * p];
-    o[56] = invd[2 * p + 1];
+    if (invd) {
+        o[55] = invd[2 * p];
+        o[56] = invd[2 * p + 1];
+    }
 }
 
 // bad[0]: a node whose row is not its type's (the assembled system was
@@ -703,9 +690,8 @@ __global__ void k_fine_check(int NX, int NY, int NZ, const int *__restrict__ rp,
     }
 }
 
-int build_fine_stencil(amg_hierarchy *h, const bd_system *sys, cudaStream_t s)
+int fine_raw_build(FineStencil &F, const bd_system *sys, const double *invd, cudaStream_t s)
 {
-    FineStencil &F = h->fine;
     F.NX = sys->mesh.nx + 1;
     F.NY = sys->mesh.ny + 1;
     F.NZ = sys->mesh.nz + 1;
@@ -715,7 +701,7 @@ int build_fine_stencil(amg_hierarchy *h, const bd_system *sys, cudaStream_t s)
     BD_CUDA(cudaMemsetAsync(bad.p, 0, 2 * sizeof(int), s));
     const bd_params &P = sys->params;
     k_fine_raw<<<(9 * F.NZ + 63) / 64, 64, 0, s>>>(F.NX, F.NY, F.NZ, sys->A.rp.p, sys->Ki.p, sys->Ke.p, sys->M.p,
-                                                   (P.chi * P.cm) / P.dt, h->lev[0].invdiag.p, F.raw.p);
+                                                   (P.chi * P.cm) / P.dt, invd, F.raw.p);
     ::bd::note_launch();
     k_fine_check<<<grid_for(sys->N, 256), 256, 0, s>>>(F.NX, F.NY, F.NZ, sys->A.rp.p, sys->A.ci.p, sys->Ki.p,
                                                        sys->Ke.p, F.raw.p, bad.p);
@@ -726,7 +712,13 @@ int build_fine_stencil(amg_hierarchy *h, const bd_system *sys, cudaStream_t s)
     BD_CUDA(cudaStreamSynchronize(s));
     if (hbad[0]) return BD_EINVAL;
     F.sym = !hbad[1];
-    F.valid = true;
+    return BD_OK;
+}
+
+int build_fine_stencil(amg_hierarchy *h, const bd_system *sys, cudaStream_t s)
+{
+    BD_TRY(fine_raw_build(h->fine, sys, h->lev[0].invdiag.p, s));
+    h->fine.valid = true;
     return BD_OK;
 }
 
@@ -749,14 +741,7 @@ __global__ void k_fine_pack(int rows, const double *__restrict__ raw, double c2,
     for (int z = 0; z < (SYM ? 2 : 3); z++) {
         const int b = 9 * (z == 0 ? 1 : (z == 1 ? 2 : 0));  // dz = 0, +1, -1
         for (int k = 0; k < Row::NP; k++) {
-            int q = k;
-            if (SYM) {
-                if (k == 0) q = 4;
-                else if (k == 1) q = ti == 2 ? 3 : 5;
-                else if (k == 2) q = tj == 2 ? 1 : 7;
-                else if (k == 3) q = (ti == 2 || tj == 2) ? 0 : 8;
-                else q = (ti == 2 || tj == 0) ? 6 : 2;
-            }
+            const int q = SYM ? fine_pair_pos(k, ti, tj) : k;
             put(z * Row::G + k, o[2 * (b + q)], o[2 * (b + q) + 1]);
         }
         put(z * Row::G + Row::NP, z == 0 ? o[54] : 0.0, 0.0);
@@ -963,6 +948,25 @@ __global__ void __launch_bounds__(256) k_coarse_solve_wide(int n, const double *
 }
 
 template <class S>
+static int launch_coarse(int n, const double *cinv, const double *z, double zz, const S *r, S *x, cudaStream_t s)
+{
+    const size_t smem = sizeof(double) * (size_t)n;
+    if (n <= 256) k_coarse_solve<S><<<1, 1024, smem, s>>>(n, cinv, z, zz, r, x);
+    else k_coarse_solve_wide<S><<<(n + 7) / 8, 256, smem, s>>>(n, cinv, z, zz, r, x);
+    ::bd::note_launch();
+    BD_LAUNCH_CHECK();
+    return BD_OK;
+}
+int coarse_solve(int n, const double *cinv, const double *z, double zz, const double *r, double *x, cudaStream_t s)
+{
+    return launch_coarse(n, cinv, z, zz, r, x, s);
+}
+int coarse_solve(int n, const double *cinv, const double *z, double zz, const float *r, float *x, cudaStream_t s)
+{
+    return launch_coarse(n, cinv, z, zz, r, x, s);
+}
+
+template <class S>
 __global__ void k_copy2(int N, const v2<S> *__restrict__ a, v2<S> *__restrict__ b)
 {
     for (int i = share_lo(N) + threadIdx.x, e = share_hi(N); i < e; i += blockDim.x) b[i] = a[i];
@@ -1134,15 +1138,8 @@ static int vcycle_impl(amg_hierarchy *h, const v2<S> *f0, v2<S> *u0, cudaStream_
         const LV<S> cv = view<S>(h, nl - 1);
         const S *f = (const S *)(nl == 1 ? f0 : cv.f);
         S *u = (S *)(nl == 1 ? u0 : cv.u);
-        size_t smem = sizeof(double) * (size_t)h->nc;
         int sc = prof_begin(h, s, R_COARSE, false);
-        if (h->nc <= 256) {
-            k_coarse_solve<S><<<1, 1024, smem, s>>>(h->nc, h->cinv.p, h->zc.p, h->zz, f, u); ::bd::note_launch();
-        } else {
-            k_coarse_solve_wide<S><<<(h->nc + 7) / 8, 256, smem, s>>>(h->nc, h->cinv.p, h->zc.p, h->zz, f, u);
-            ::bd::note_launch();
-        }
-        BD_LAUNCH_CHECK();
+        BD_TRY(coarse_solve(h->nc, h->cinv.p, h->zc.p, h->zz, f, u, s));
         prof_end(h, sc, 0.0, 0.0, s);
     }
     for (int l = nl - 2; l >= 0; l--) BD_TRY(up(l));
@@ -1198,166 +1195,6 @@ static int vcycle_run(amg_hierarchy *h, const double *r_dev, double *z_dev, cuda
 int vcycle_device(amg_hierarchy *h, const double *r_dev, double *z_dev, cudaStream_t s)
 {
     return vcycle_run(h, r_dev, z_dev, s, false, nullptr, nullptr);
-}
-
-// ------------------------------------------------------------------ PCG reductions
-// scal[] slots of the device scalars
-enum {
-    S_SUMFU = 0, S_FF, S_NF2, S_RR, S_RZ, S_PQ, S_ALPHA, S_BETA, S_MEANZ,
-    S_BREAK, S_MEANF, S_TRR, S_MEANX,
-    // device-side loop control of the graph form
-    S_RTOL, S_MAXIT, S_WARM, S_IT, S_STATUS,
-    S_NSLOTS
-};
-constexpr int kPart = 4;  // partial sums per block
-// Grid of the PCG vector kernels: one resident wave of fewer, larger blocks
-// than kRedBlocks, so the last block's reduction of the partials is shorter.
-constexpr int kVecBlocks = 608, kVecThreads = 512;
-constexpr int kMaxBlockThreads = 512;  // largest block of a reduction kernel
-
-// What the last block of a reduction kernel does with the totals.
-// first < 0: "first iteration" is read from the device iteration counter
-// (graph form).  Stages 6 and 7 are the graph form's loop control: 6 opens
-// the loop after the initial residual, 7 closes an iteration; both set the
-// WHILE node's condition.
-struct Fin {
-    double *scal;
-    double *partial;
-    unsigned int *counter;
-    int stage, N, first, flex;
-    cudaGraphConditionalHandle cond;
-};
-
-__device__ void finish_stage(const Fin &f, double a, double b, double c, double d)
-{
-    double *scal = f.scal;
-    const int N = f.N;
-    const int first = f.first < 0 ? (scal[S_IT] == 0.0) : f.first;
-    switch (f.stage) {
-    case 0:  // f statistics: sum f_u, ||f||^2
-        scal[S_SUMFU] = a;
-        scal[S_FF] = b;
-        scal[S_MEANF] = a / N;
-        break;
-    case 1:  // ||fp||^2
-        scal[S_NF2] = a;
-        break;
-    case 2:  // ||r||^2
-        scal[S_RR] = a;
-        break;
-    case 3: {  // z statistics: sum z_u, sum r_u, r.z, r.z_old
-        double mz = a / N;
-        double rz = c - mz * b;  // r . (z projected)
-        scal[S_MEANZ] = mz;
-        // standard CG: beta = rz_new / rz_old; flexible (Polak-Ribiere):
-        // beta = (r.z_new - r.z_old) / rz_old with z_old the previous projected z
-        double num = f.flex ? rz - d : rz;
-        scal[S_BETA] = first ? 0.0 : num / scal[S_RZ];
-        scal[S_RZ] = rz;
-        break;
-    }
-    case 4:  // p.q
-        scal[S_PQ] = a;
-        if (!(a > 0.0) || !isfinite(a) || !isfinite(scal[S_RZ])) scal[S_BREAK] = 1.0;
-        scal[S_ALPHA] = scal[S_RZ] / a;
-        break;
-    case 5:  // true residual and mean of x_u
-        scal[S_TRR] = a;
-        scal[S_MEANX] = b / N;
-        break;
-    case 6: {  // initial ||r||^2; open the loop unless already converged
-        scal[S_RR] = a;
-        const double nf = sqrt(scal[S_NF2]);
-        const bool go = nf > 0.0 && !(sqrt(a) <= scal[S_RTOL] * nf) && scal[S_MAXIT] > 0.0;
-        scal[S_IT] = 0.0;
-        scal[S_STATUS] = go ? (double)BD_ENOTCONV : (double)BD_OK;
-        cudaGraphSetConditional(f.cond, go ? 1u : 0u);
-        break;
-    }
-    case 7: {  // ||r||^2 after the update; close or continue the loop
-        scal[S_RR] = a;
-        const double it = scal[S_IT] + 1.0;
-        scal[S_IT] = it;
-        const double nf = sqrt(scal[S_NF2]), rr = sqrt(a);
-        bool go = true;
-        if (scal[S_BREAK] != 0.0 || !isfinite(rr)) {
-            scal[S_STATUS] = (double)BD_EBREAKDOWN;
-            go = false;
-        } else if (rr <= scal[S_RTOL] * nf) {
-            scal[S_STATUS] = (double)BD_OK;
-            go = false;
-        } else if (it >= scal[S_MAXIT]) {
-            go = false;  // status stays BD_ENOTCONV
-        }
-        cudaGraphSetConditional(f.cond, go ? 1u : 0u);
-        break;
-    }
-    }
-}
-
-// Block sums of the first NV of a thread's values, in a fixed order: every
-// thread stores its values, then warp k adds column k (the entries of lanes
-// l, l + 32, ... in index order) and folds its 32 lane sums by shuffles into
-// tot[k].  That is 12 FP64 warp additions per value and block for 256 threads
-// (36 for 1024), where a shuffle tree in every warp costs 45 for 256.
-template <int NV, int BT>
-__device__ __forceinline__ void block_sum(const double (&v)[4], double (*buf)[BT], double *tot)
-{
-#pragma unroll
-    for (int k = 0; k < NV; k++) buf[k][threadIdx.x] = v[k];
-    __syncthreads();
-    const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
-    if (w < NV) {
-        double t = buf[w][l];
-        for (int i = l + 32; i < (int)blockDim.x; i += 32) t += buf[w][i];
-        for (int o = 16; o; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-        if (l == 0) tot[w] = t;
-    }
-    __syncthreads();
-}
-
-// Block sums -> partial[blockIdx]; the last block to arrive reduces all
-// partials in a fixed order (independent of which block is last, so the
-// result is reproducible) and applies the stage.  No waiting: blocks that are
-// not last simply exit.  NV of (a, b, c, d) are live; the stage sees zeros for
-// the rest.  Needs blockDim.x <= BT and a multiple of 32 (the shared buffer
-// holds BT values per sum: kernels of 256 threads keep the rest of shared
-// memory for L1).
-template <int NV, int BT = kMaxBlockThreads>
-__device__ void block_finish(double a, double b, double c, double d, const Fin &f)
-{
-    __shared__ double buf[NV][BT];
-    __shared__ double tot[4];
-    __shared__ bool last;
-    double v[4] = {a, b, c, d};
-    block_sum<NV, BT>(v, buf, tot);
-    if (threadIdx.x == 0) {
-        double *o = f.partial + kPart * blockIdx.x;
-#pragma unroll
-        for (int k = 0; k < NV; k++) o[k] = tot[k];
-        __threadfence();
-        const unsigned int ticket = atomicAdd(f.counter, 1u);
-        last = ticket == gridDim.x - 1;
-    }
-    __syncthreads();
-    if (!last) return;
-    __threadfence();
-#pragma unroll
-    for (int k = 0; k < 4; k++) v[k] = 0.0;
-    // L2 loads (the partials were published by the other blocks' fences and
-    // tickets), not volatile ones, so that the unrolled loads of several
-    // partials are in flight together: the last block's serial tail
-#pragma unroll 4
-    for (int i = threadIdx.x; i < (int)gridDim.x; i += blockDim.x) {
-        const double *q = f.partial + kPart * i;
-#pragma unroll
-        for (int k = 0; k < NV; k++) v[k] += __ldcg(q + k);
-    }
-    block_sum<NV, BT>(v, buf, tot);
-    if (threadIdx.x == 0) {
-        finish_stage(f, tot[0], NV > 1 ? tot[1] : 0.0, NV > 2 ? tot[2] : 0.0, NV > 3 ? tot[3] : 0.0);
-        *f.counter = 0u;
-    }
 }
 
 __global__ void k_f_stats(int N, const double2 *__restrict__ f, Fin fin)
@@ -2063,7 +1900,7 @@ static int pcg_solve_loop(amg_hierarchy *h, const double *f_dev, double *x_dev, 
 // and sets the node's condition, so a solve costs one graph launch and one
 // host synchronisation.  The loop is bounded by max_it.  The graph works on the
 // hierarchy's own buffers (right-hand side in `fin`, iterate in `x`).
-static void end_capture_quietly(cudaStream_t s)
+void drop_capture(cudaStream_t s)
 {
     cudaStreamCaptureStatus cs;
     if (cudaStreamIsCapturing(s, &cs) == cudaSuccess && cs != cudaStreamCaptureStatusNone) {
@@ -2072,6 +1909,43 @@ static void end_capture_quietly(cudaStream_t s)
         if (g) cudaGraphDestroy(g);
     }
     cudaGetLastError();
+}
+
+int while_handle(cudaStream_t s, WhileNode *w)
+{
+    cudaStreamCaptureStatus cs;
+    cudaGraph_t g = nullptr;
+    const cudaGraphNode_t *deps = nullptr;
+    size_t nd = 0;
+    BD_CUDA(cudaStreamGetCaptureInfo(s, &cs, nullptr, &g, &deps, nullptr, &nd));
+    BD_CUDA(cudaGraphConditionalHandleCreate(&w->cond, g, 0, 0));
+    return BD_OK;
+}
+
+int while_begin(cudaStream_t s, cudaStream_t s2, WhileNode *w)
+{
+    cudaStreamCaptureStatus cs;
+    cudaGraph_t g = nullptr;
+    const cudaGraphNode_t *deps = nullptr;
+    size_t nd = 0;
+    BD_CUDA(cudaStreamGetCaptureInfo(s, &cs, nullptr, &g, &deps, nullptr, &nd));
+    cudaGraphNodeParams np = {};
+    np.type = cudaGraphNodeTypeConditional;
+    np.conditional.handle = w->cond;
+    np.conditional.type = cudaGraphCondTypeWhile;
+    np.conditional.size = 1;
+    BD_CUDA(cudaGraphAddNode(&w->node, g, deps, nullptr, nd, &np));
+    BD_CUDA(cudaStreamBeginCaptureToGraph(s2, np.conditional.phGraph_out[0], nullptr, nullptr, 0,
+                                          cudaStreamCaptureModeThreadLocal));
+    return BD_OK;
+}
+
+int while_end(cudaStream_t s, cudaStream_t s2, WhileNode *w)
+{
+    cudaGraph_t body = nullptr;
+    BD_CUDA(cudaStreamEndCapture(s2, &body));
+    BD_CUDA(cudaStreamUpdateCaptureDependencies(s, &w->node, nullptr, 1, cudaStreamSetCaptureDependencies));
+    return BD_OK;
 }
 
 // Capture one whole solve of h into the graph being captured on stream s:
@@ -2095,27 +1969,13 @@ static int capture_solve(amg_hierarchy *h, cudaStream_t s, cudaStream_t s2)
     k_project_f<<<kVecBlocks, kVecThreads, 0, s>>>(N, fin, fp, make_fin(h, 1, 0)); ::bd::note_launch();
     k_zero_if<<<kVecBlocks, kVecThreads, 0, s>>>(N, x, scal, 0); ::bd::note_launch();
     BD_LAUNCH_CHECK();
-    cudaStreamCaptureStatus cs;
-    cudaGraph_t g = nullptr;
-    const cudaGraphNode_t *deps = nullptr;
-    size_t nd = 0;
-    BD_CUDA(cudaStreamGetCaptureInfo(s, &cs, nullptr, &g, &deps, nullptr, &nd));
-    cudaGraphConditionalHandle cond;
-    BD_CUDA(cudaGraphConditionalHandleCreate(&cond, g, 0, 0));
+    WhileNode w;
+    BD_TRY(while_handle(s, &w));
     const D0Out d0 = d0_out(h);
-    fine_reduce<1>(h, x, fp, r, make_fin(h, 6, 0, cond), s, d0);
+    fine_reduce<1>(h, x, fp, r, make_fin(h, 6, 0, w.cond), s, d0);
     BD_LAUNCH_CHECK();
-    BD_CUDA(cudaStreamGetCaptureInfo(s, &cs, nullptr, &g, &deps, nullptr, &nd));
-    cudaGraphNodeParams np = {};
-    np.type = cudaGraphNodeTypeConditional;
-    np.conditional.handle = cond;
-    np.conditional.type = cudaGraphCondTypeWhile;
-    np.conditional.size = 1;
-    cudaGraphNode_t wnode;
-    BD_CUDA(cudaGraphAddNode(&wnode, g, deps, nullptr, nd, &np));
-    cudaGraph_t body = np.conditional.phGraph_out[0];
+    BD_TRY(while_begin(s, s2, &w));
     const long long c1 = launch_count();
-    BD_CUDA(cudaStreamBeginCaptureToGraph(s2, body, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal));
     const ZOut zo{z, r, zold, make_fin(h, 3, -1)};
     bool zd = false;
     BD_TRY(vcycle_run(h, (const double *)r, (double *)z, s2, true, &zo, &zd));
@@ -2124,12 +1984,10 @@ static int capture_solve(amg_hierarchy *h, cudaStream_t s, cudaStream_t s2)
     }
     p_update(h, N, z, p, zold, scal, -1, s2);
     fine_reduce<0>(h, p, nullptr, q, make_fin(h, 4, 0), s2);
-    xr_update(h, N, x, r, p, q, make_fin(h, 7, 0, cond), s2, d0);
+    xr_update(h, N, x, r, p, q, make_fin(h, 7, 0, w.cond), s2, d0);
     BD_LAUNCH_CHECK();
-    cudaGraph_t body_out = nullptr;
-    BD_CUDA(cudaStreamEndCapture(s2, &body_out));
     const long long c2 = launch_count();
-    BD_CUDA(cudaStreamUpdateCaptureDependencies(s, &wnode, nullptr, 1, cudaStreamSetCaptureDependencies));
+    BD_TRY(while_end(s, s2, &w));
     k_zero_if<<<kVecBlocks, kVecThreads, 0, s>>>(N, x, scal, 1); ::bd::note_launch();
     fine_reduce<1>(h, x, fp, nullptr, make_fin(h, 5, 0), s);
     k_project_x<<<kVecBlocks, kVecThreads, 0, s>>>(N, x, scal); ::bd::note_launch();
@@ -2157,8 +2015,8 @@ static int build_graph(amg_hierarchy *h)
     if (!h->cap_stream2) BD_CUDA(cudaStreamCreateWithFlags(&h->cap_stream2, cudaStreamNonBlocking));
     int st = capture_graph(h);
     if (st != BD_OK) {
-        end_capture_quietly(h->cap_stream2);
-        end_capture_quietly(h->cap_stream);
+        drop_capture(h->cap_stream2);
+        drop_capture(h->cap_stream);
         if (h->graph_exec) cudaGraphExecDestroy(h->graph_exec);
         if (h->graph) cudaGraphDestroy(h->graph);
         h->graph_exec = nullptr;
@@ -2210,13 +2068,18 @@ static int pcg_solve_graph(amg_hierarchy *h, const double *f_dev, double *x_dev,
     return pcg_graph_finish(h, s, info);
 }
 
-static bool graph_form(amg_hierarchy *h, const solve_options *o)
+bool solve_graph_off()
 {
-    static const bool graph_off = [] {
+    static const bool off = [] {
         const char *e = getenv("BD_SOLVE_GRAPH");
         return e && e[0] == '0';
     }();
-    if (h->prof || o->strict || h->graph_failed || graph_off) return false;
+    return off;
+}
+
+static bool graph_form(amg_hierarchy *h, const solve_options *o)
+{
+    if (h->prof || o->strict || h->graph_failed || solve_graph_off()) return false;
     if (!h->graph_exec && build_graph(h) != BD_OK) h->graph_failed = true;
     return h->graph_exec != nullptr;
 }
@@ -2251,9 +2114,14 @@ int pcg_solve_device(amg_hierarchy *h, const double *f_dev, double *x_dev, int w
 // residuals; counts its kernel executions.
 static int report_from_scal(amg_hierarchy *h, const double *sc, float ms, solve_info *info)
 {
+    note_launches(h->graph_pre + h->graph_post + (long long)sc[S_IT] * h->graph_body);
+    return info_from_scal(sc, ms, info);
+}
+
+int info_from_scal(const double *sc, float ms, solve_info *info)
+{
     const double nf = sqrt(sc[S_NF2]);
     const int status = (int)sc[S_STATUS];
-    note_launches(h->graph_pre + h->graph_post + (long long)sc[S_IT] * h->graph_body);
     if (info) {
         info->status = status;
         info->iters = (int)sc[S_IT];
@@ -2402,9 +2270,9 @@ extern "C" int amg_batch_solve(amg_batch *b, const double *const *f, double *con
         g.x.assign(x, x + count);
         const int st = batch_capture(g);
         if (st != BD_OK) {
-            end_capture_quietly(g.body);
-            for (cudaStream_t q : g.st) end_capture_quietly(q);
-            end_capture_quietly(g.origin);
+            drop_capture(g.body);
+            for (cudaStream_t q : g.st) drop_capture(q);
+            drop_capture(g.origin);
             g.drop_graph();
             return st;
         }

@@ -6,73 +6,134 @@
 // unpreconditioned (the paper's GPU runs leave it unpreconditioned).
 //
 // The elliptic hierarchy is the block hierarchy of [I, 0; 0, Ai + Ae]
-// (bd_elliptic_setup); its iterate is kept as (0, u_e) pairs, whose zero
-// v-field the solve preserves.  The parabolic CG runs on the host loop with
-// its inner products summed in a fixed order (per-block partials added on
-// the host in block order), so it is reproducible run to run.
+// (bd_elliptic_setup), solved on its one field (amg_scalar.cu).  Ai and c M + Ai
+// are scalar layered stencils (fine_scalar.cuh).  The parabolic CG runs as one
+// CUDA graph: three kernels per iteration under a WHILE node whose condition the
+// last reduction sets; the host synchronises once per solve, where a host-driven
+// loop read 1216 partial sums back twice per iteration (128x128x32, 24
+// iterations: 3.9 -> 1.25 ms).  Reductions sum in a fixed order, so it is
+// reproducible run to run.
 #include <cmath>
 #include <new>
 
 #include "amg_internal.cuh"
+#include "fine_scalar.cuh"
+#include "pcg_reduce.cuh"
+#include "scalar.cuh"
 
+namespace bd {
 namespace {
 
-constexpr int kParBlocks = 1216;  // fixed grid of the parabolic reductions
-constexpr int kParVals = 3;       // partial sums per block
+// elliptic right-hand side -Ai v
+struct DEllRhs {
+    double *__restrict__ f;
+    __device__ __forceinline__ int load(int, bool) const { return 0; }
+    __device__ __forceinline__ void operator()(int p, const double *, int, double, double, double y) { f[p] = -y; }
+};
 
-// sums of up to kParVals values over the block, in a fixed order, by thread 0
-__device__ void block_partials(double a, double b, double c, double *partial)
-{
-    __shared__ double buf[kParVals][256];
-    buf[0][threadIdx.x] = a;
-    buf[1][threadIdx.x] = b;
-    buf[2][threadIdx.x] = c;
-    __syncthreads();
-    const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
-    if (w < kParVals) {
-        double t = buf[w][l];
-        for (int i = l + 32; i < (int)blockDim.x; i += 32) t += buf[w][i];
-        for (int o = 16; o; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-        if (l == 0) partial[kParVals * blockIdx.x + w] = t;
+// gating update (Eq. 4) and parabolic right-hand side (Eq. 7); y = Ai u_e
+struct DParRhs {
+    const double *__restrict__ M, *__restrict__ stim, *__restrict__ v;
+    double *__restrict__ w, *__restrict__ b;
+    double chi, cm, dt;
+    bd_rm_params rm;
+    int stim_on;
+    struct Pre {
+        double M, stim, v, w;
+    };
+    __device__ __forceinline__ Pre load(int p, bool ok) const
+    {
+        return ok ? Pre{M[p], stim_on ? stim[p] : 0.0, v[p], w[p]} : Pre{0.0, 0.0, 0.0, 0.0};
     }
-}
-
-// Ai x on the node pattern, row p
-__device__ __forceinline__ double ki_row(int p, const int *__restrict__ rp, const int *__restrict__ ci,
-                                         const double *__restrict__ Ki, const double *__restrict__ x,
-                                         int stride, int off)
-{
-    double a = 0.0;
-    for (int t = rp[p]; t < rp[p + 1]; t++) a = fma(Ki[t], x[(size_t)stride * ci[t] + off], a);
-    return a;
-}
-
-// elliptic right-hand side (0, -Ai v)
-__global__ void k_ell_rhs(int N, const int *__restrict__ rp, const int *__restrict__ ci,
-                          const double *__restrict__ Ki, const double *__restrict__ v, double2 *__restrict__ fe)
-{
-    for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < N; p += gridDim.x * blockDim.x)
-        fe[p] = make_double2(0.0, -ki_row(p, rp, ci, Ki, v, 1, 0));
-}
-
-// gating update (Eq. 4) and parabolic right-hand side (Eq. 7); u_e from the
-// elliptic iterate (0, u_e)
-__global__ void k_par_rhs(int N, const int *__restrict__ rp, const int *__restrict__ ci,
-                          const double *__restrict__ Ki, const double *__restrict__ M,
-                          const double *__restrict__ stim, int stim_on, double chi, double cm, double dt,
-                          bd_rm_params rm, const double *__restrict__ v, double *__restrict__ w,
-                          const double *__restrict__ xe, double *__restrict__ b)
-{
-    const double c = (chi * cm) / dt;
-    for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < N; p += gridDim.x * blockDim.x) {
-        const double a = ki_row(p, rp, ci, Ki, xe, 2, 1);
-        const double vk = v[p];
-        const double wn = (w[p] + dt * rm.eta2 * vk / rm.vp) / (1.0 + dt * rm.eta2 * rm.eta3);
-        const double iion = rm.G * vk * (1.0 - vk / rm.vth) * (1.0 - vk / rm.vp) + rm.eta1 * vk * wn;
-        const double iapp = stim_on ? stim[p] : 0.0;
-        b[p] = c * M[p] * vk - a + M[p] * (iapp - chi * iion);
+    __device__ __forceinline__ void operator()(int p, const double *, const Pre &q, double, double, double y)
+    {
+        const double c = (chi * cm) / dt;
+        const double wn = (q.w + dt * rm.eta2 * q.v / rm.vp) / (1.0 + dt * rm.eta2 * rm.eta3);
+        const double iion = rm.G * q.v * (1.0 - q.v / rm.vth) * (1.0 - q.v / rm.vp) + rm.eta1 * q.v * wn;
+        b[p] = c * q.M * q.v - y + q.M * (q.stim - chi * iion);
         w[p] = wn;
     }
+};
+
+// r = b - A v; partials r.r, r.D^{-1}r, b.b
+struct DResid {
+    const double *__restrict__ b, *__restrict__ dinv;
+    double *__restrict__ r;
+    double rr, rz, bb;
+    struct Pre {
+        double b, d;
+    };
+    __device__ __forceinline__ Pre load(int p, bool ok) const { return ok ? Pre{b[p], dinv[p]} : Pre{0.0, 0.0}; }
+    __device__ __forceinline__ void operator()(int p, const double *, const Pre &q, double, double, double y)
+    {
+        const double rv = q.b - y;
+        r[p] = rv;
+        rr += rv * rv;
+        rz += rv * (q.d * rv);
+        bb += q.b * q.b;
+    }
+};
+template <bool SYM>
+__global__ void __launch_bounds__(kFineTPB, ScMinB<double>::v)
+    k_par_resid(ScGrid g, const double *__restrict__ v, DResid e, Fin fin)
+{
+    sc_block<double, SYM>(g, v, e);
+    block_finish<3, kFineTPB>(e.rr, e.rz, e.bb, 0.0, fin);
+}
+
+// q = A p; partial p.q
+struct DApply {
+    double *__restrict__ q;
+    double pq;
+    __device__ __forceinline__ int load(int, bool) const { return 0; }
+    __device__ __forceinline__ void operator()(int p, const double *, int, double c, double, double y)
+    {
+        q[p] = y;
+        pq = fma(c, y, pq);
+    }
+};
+template <bool SYM>
+__global__ void __launch_bounds__(kFineTPB, ScMinB<double>::v)
+    k_par_apply(ScGrid g, const double *__restrict__ p, DApply e, Fin fin)
+{
+    sc_block<double, SYM>(g, p, e);
+    block_finish<1, kFineTPB>(e.pq, 0.0, 0.0, 0.0, fin);
+}
+
+// p = D^{-1} r, + beta p after the first iteration
+__global__ void k_par_direction(int N, const double *__restrict__ dinv, const double *__restrict__ r,
+                                double *__restrict__ p, const double *__restrict__ scal)
+{
+    const double beta = scal[S_BETA];
+    const bool first = scal[S_IT] == 0.0;
+    for (int i = share_lo(N) + threadIdx.x, e = share_hi(N); i < e; i += blockDim.x) {
+        const double z = dinv[i] * r[i];
+        p[i] = first ? z : fma(beta, p[i], z);
+    }
+}
+
+// v += alpha p, r -= alpha q; partials r.r, r.D^{-1}r
+__global__ void k_par_update(int N, const double *__restrict__ p, const double *__restrict__ q,
+                             const double *__restrict__ dinv, double *__restrict__ v, double *__restrict__ r, Fin fin)
+{
+    const double alpha = fin.scal[S_ALPHA];
+    double rr = 0.0, rz = 0.0;
+    if (fin.scal[S_BREAK] == 0.0)
+        for (int i = share_lo(N) + threadIdx.x, e = share_hi(N); i < e; i += blockDim.x) {
+            v[i] = fma(alpha, p[i], v[i]);
+            const double rv = fma(-alpha, q[i], r[i]);
+            r[i] = rv;
+            rr += rv * rv;
+            rz += rv * (dinv[i] * rv);
+        }
+    block_finish<2>(rr, rz, 0.0, 0.0, fin);
+}
+
+// v = 0 for a zero right-hand side
+__global__ void k_par_zero(int N, double *__restrict__ v, const double *__restrict__ scal)
+{
+    if (scal[S_NF2] != 0.0) return;
+    for (int i = share_lo(N) + threadIdx.x, e = share_hi(N); i < e; i += blockDim.x) v[i] = 0.0;
 }
 
 // inverse diagonal of c M + Ai (ones when unpreconditioned)
@@ -88,70 +149,11 @@ __global__ void k_par_dinv(int N, const int *__restrict__ rp, const int *__restr
     }
 }
 
-// r = b - (c M + Ai) v, z = D^{-1} r; partials r.r, r.z, b.b
-__global__ void __launch_bounds__(256) k_par_resid(int N, const int *__restrict__ rp, const int *__restrict__ ci,
-                                                   const double *__restrict__ Ki, const double *__restrict__ M, double c,
-                                                   const double *__restrict__ v, const double *__restrict__ b,
-                                                   const double *__restrict__ dinv, double *__restrict__ r,
-                                                   double *__restrict__ z, double *__restrict__ partial)
-{
-    double rr = 0.0, rz = 0.0, bb = 0.0;
-    for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < N; p += gridDim.x * blockDim.x) {
-        const double y = fma(c * M[p], v[p], ki_row(p, rp, ci, Ki, v, 1, 0));
-        const double bp = b[p], rv = bp - y, zv = dinv[p] * rv;
-        r[p] = rv;
-        z[p] = zv;
-        rr += rv * rv;
-        rz += rv * zv;
-        bb += bp * bp;
-    }
-    block_partials(rr, rz, bb, partial);
-}
-
-// q = (c M + Ai) p; partial p.q
-__global__ void __launch_bounds__(256) k_par_apply(int N, const int *__restrict__ rp, const int *__restrict__ ci,
-                                                   const double *__restrict__ Ki, const double *__restrict__ M, double c,
-                                                   const double *__restrict__ pv, double *__restrict__ q,
-                                                   double *__restrict__ partial)
-{
-    double pq = 0.0;
-    for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < N; p += gridDim.x * blockDim.x) {
-        const double y = fma(c * M[p], pv[p], ki_row(p, rp, ci, Ki, pv, 1, 0));
-        q[p] = y;
-        pq += pv[p] * y;
-    }
-    block_partials(pq, 0.0, 0.0, partial);
-}
-
-// v += alpha p, r -= alpha q, z = D^{-1} r; partials r.r, r.z
-__global__ void __launch_bounds__(256) k_par_update(int N, double alpha, const double *__restrict__ pv,
-                                                    const double *__restrict__ q, const double *__restrict__ dinv,
-                                                    double *__restrict__ v, double *__restrict__ r,
-                                                    double *__restrict__ z, double *__restrict__ partial)
-{
-    double rr = 0.0, rz = 0.0;
-    for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < N; p += gridDim.x * blockDim.x) {
-        v[p] = fma(alpha, pv[p], v[p]);
-        const double rv = fma(-alpha, q[p], r[p]), zv = dinv[p] * rv;
-        r[p] = rv;
-        z[p] = zv;
-        rr += rv * rv;
-        rz += rv * zv;
-    }
-    block_partials(rr, rz, 0.0, partial);
-}
-
-__global__ void k_par_direction(int N, double beta, const double *__restrict__ z, double *__restrict__ pv, int first)
-{
-    for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < N; p += gridDim.x * blockDim.x)
-        pv[p] = first ? z[p] : fma(beta, pv[p], z[p]);
-}
-
+// (0, u) pairs of the block solve
 __global__ void k_split(int N, const double2 *__restrict__ xe, double *__restrict__ ue)
 {
     for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < N; p += gridDim.x * blockDim.x) ue[p] = xe[p].y;
 }
-
 __global__ void k_join(int N, const double *__restrict__ ue, double2 *__restrict__ xe)
 {
     for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < N; p += gridDim.x * blockDim.x)
@@ -159,6 +161,7 @@ __global__ void k_join(int N, const double *__restrict__ ue, double2 *__restrict
 }
 
 }  // namespace
+}  // namespace bd
 
 struct bd_dsim {
     const bd_system *sys = nullptr;
@@ -167,14 +170,26 @@ struct bd_dsim {
     int N = 0, jacobi = 1;
     long long step = 0;
     double stim_ms = 0.0;
-    bd::DBuf<double> v, w, stim;   // N each
-    bd::DBuf<double> xe, fe;       // elliptic iterate (0, u_e) and right-hand side, 2N
-    bd::DBuf<double> b, r, z, p, q, dinv, partial;
-    double *host_part = nullptr;   // pinned kParBlocks x kParVals
+    bd::FineStencil raw;
+    bd::ScOp ki, par;              // Ai; c M + Ai
+    bd::DBuf<double> v, w, stim, ue;  // N each
+    bd::DBuf<double> f;            // elliptic right-hand side
+    bd::DBuf<double> xe, fe;       // block solve only: (0, u_e) pairs
+    bd::DBuf<double> b, r, p, q, dinv, partial, scal;
+    bd::DBuf<unsigned int> counter;
+    double *host = nullptr;        // pinned: initial scalars, then results
     cudaEvent_t ev[2] = {nullptr, nullptr};
+    cudaGraph_t graph = nullptr;
+    cudaGraphExec_t exec = nullptr;
+    cudaStream_t cap = nullptr, cap2 = nullptr;
+    bool graph_failed = false;
     ~bd_dsim()
     {
-        if (host_part) cudaFreeHost(host_part);
+        if (exec) cudaGraphExecDestroy(exec);
+        if (graph) cudaGraphDestroy(graph);
+        if (cap) cudaStreamDestroy(cap);
+        if (cap2) cudaStreamDestroy(cap2);
+        if (host) cudaFreeHost(host);
         if (ev[0]) cudaEventDestroy(ev[0]);
         if (ev[1]) cudaEventDestroy(ev[1]);
     }
@@ -184,82 +199,122 @@ using namespace bd;
 
 namespace {
 
-// block partials -> host, summed in block order
-int read_sums(bd_dsim *S, cudaStream_t s, int nv, double *out)
+constexpr int kParBody = 3;  // kernels of an iteration
+
+Fin par_fin(bd_dsim *S, int stage, cudaGraphConditionalHandle cond = 0)
 {
-    BD_CUDA(cudaMemcpyAsync(S->host_part, S->partial.p, sizeof(double) * kParVals * kParBlocks,
-                            cudaMemcpyDeviceToHost, s));
-    BD_CUDA(cudaStreamSynchronize(s));
-    for (int k = 0; k < nv; k++) {
-        double t = 0.0;
-        for (int i = 0; i < kParBlocks; i++) t += S->host_part[kParVals * i + k];
-        out[k] = t;
-    }
+    return Fin{S->scal.p, S->partial.p, S->counter.p, stage, S->N, -1, 0, cond};
+}
+
+int par_resid(bd_dsim *S, const Fin &fin, cudaStream_t s)
+{
+    const DResid e{S->b.p, S->dinv.p, S->r.p, 0.0, 0.0, 0.0};
+    const int grid = S->par.blocks<double>();
+    if (S->par.sym) k_par_resid<true><<<grid, kFineTPB, 0, s>>>(S->par.grid<double>(), S->v.p, e, fin);
+    else k_par_resid<false><<<grid, kFineTPB, 0, s>>>(S->par.grid<double>(), S->v.p, e, fin);
+    note_launch();
+    BD_LAUNCH_CHECK();
     return BD_OK;
 }
 
-// (c M + Ai) v = b by (Jacobi-)CG from the current v; iterations and the
-// recurrence / true residuals into info
+int par_body(bd_dsim *S, cudaGraphConditionalHandle cond, cudaStream_t s)
+{
+    const int N = S->N, grid = S->par.blocks<double>();
+    k_par_direction<<<kVecBlocks, kVecThreads, 0, s>>>(N, S->dinv.p, S->r.p, S->p.p, S->scal.p); note_launch();
+    const DApply e{S->q.p, 0.0};
+    if (S->par.sym) k_par_apply<true><<<grid, kFineTPB, 0, s>>>(S->par.grid<double>(), S->p.p, e, par_fin(S, 10));
+    else k_par_apply<false><<<grid, kFineTPB, 0, s>>>(S->par.grid<double>(), S->p.p, e, par_fin(S, 10));
+    note_launch();
+    k_par_update<<<kVecBlocks, kVecThreads, 0, s>>>(N, S->p.p, S->q.p, S->dinv.p, S->v.p, S->r.p, par_fin(S, 8, cond));
+    note_launch();
+    BD_LAUNCH_CHECK();
+    return BD_OK;
+}
+
+int par_post(bd_dsim *S, cudaStream_t s)
+{
+    k_par_zero<<<kVecBlocks, kVecThreads, 0, s>>>(S->N, S->v.p, S->scal.p); note_launch();
+    return par_resid(S, par_fin(S, 11), s);
+}
+
+int par_capture(bd_dsim *S)
+{
+    if (!S->cap) BD_CUDA(cudaStreamCreateWithFlags(&S->cap, cudaStreamNonBlocking));
+    if (!S->cap2) BD_CUDA(cudaStreamCreateWithFlags(&S->cap2, cudaStreamNonBlocking));
+    const long long c0 = launch_count();
+    BD_CUDA(cudaStreamBeginCapture(S->cap, cudaStreamCaptureModeThreadLocal));
+    WhileNode w;
+    BD_TRY(while_handle(S->cap, &w));
+    BD_TRY(par_resid(S, par_fin(S, 9, w.cond), S->cap));
+    BD_TRY(while_begin(S->cap, S->cap2, &w));
+    BD_TRY(par_body(S, w.cond, S->cap2));
+    BD_TRY(while_end(S->cap, S->cap2, &w));
+    BD_TRY(par_post(S, S->cap));
+    BD_CUDA(cudaStreamEndCapture(S->cap, &S->graph));
+    BD_CUDA(cudaGraphInstantiate(&S->exec, S->graph, 0));
+    note_launches(-(launch_count() - c0));
+    return BD_OK;
+}
+
+// (c M + Ai) v = b by (Jacobi-)CG from the current v; iterations, the recurrence
+// and true residuals and the device time into info
 int parabolic_cg(bd_dsim *S, const solve_options *o, cudaStream_t s, solve_info *info)
 {
-    const bd_system *sys = S->sys;
-    const bd_params &P = sys->params;
-    const int N = S->N;
-    const double c = (P.chi * P.cm) / P.dt;
-    const int *rp = sys->A.rp.p, *ci = sys->A.ci.p;
-    const int G = kParBlocks;
-    double sums[3];
-    k_par_resid<<<G, 256, 0, s>>>(N, rp, ci, sys->Ki.p, sys->M.p, c, S->v.p, S->b.p, S->dinv.p, S->r.p, S->z.p,
-                                  S->partial.p); note_launch();
-    BD_LAUNCH_CHECK();
-    BD_TRY(read_sums(S, s, 3, sums));
-    const double nb = std::sqrt(sums[2]);
-    double rr = std::sqrt(sums[0]), rz = sums[1];
-    int it = 0, status = BD_OK;
-    if (nb == 0.0) {
-        BD_CUDA(cudaMemsetAsync(S->v.p, 0, S->v.bytes(), s));
-        rr = 0.0;
-    } else if (!(rr <= o->rtol * nb)) {
-        status = BD_ENOTCONV;
-        k_par_direction<<<grid_for(N, 256), 256, 0, s>>>(N, 0.0, S->z.p, S->p.p, 1); note_launch();
-        while (it < o->max_it) {
-            k_par_apply<<<G, 256, 0, s>>>(N, rp, ci, sys->Ki.p, sys->M.p, c, S->p.p, S->q.p, S->partial.p);
-            note_launch();
-            BD_LAUNCH_CHECK();
-            BD_TRY(read_sums(S, s, 1, sums));
-            const double pq = sums[0];
-            if (!(pq > 0.0) || !std::isfinite(pq)) {
-                status = BD_EBREAKDOWN;
-                break;
-            }
-            const double alpha = rz / pq;
-            k_par_update<<<G, 256, 0, s>>>(N, alpha, S->p.p, S->q.p, S->dinv.p, S->v.p, S->r.p, S->z.p,
-                                           S->partial.p); note_launch();
-            BD_LAUNCH_CHECK();
-            BD_TRY(read_sums(S, s, 2, sums));
-            it++;
-            rr = std::sqrt(sums[0]);
-            if (rr <= o->rtol * nb) {
-                status = BD_OK;
-                break;
-            }
-            const double beta = sums[1] / rz;
-            rz = sums[1];
-            k_par_direction<<<grid_for(N, 256), 256, 0, s>>>(N, beta, S->z.p, S->p.p, 0); note_launch();
+    double *in = S->host, *out = S->host + S_NSLOTS;
+    for (int i = 0; i < S_NSLOTS; i++) in[i] = 0.0;
+    in[S_RTOL] = o->rtol;
+    in[S_MAXIT] = (double)o->max_it;
+    BD_CUDA(cudaEventRecord(S->ev[0], s));
+    BD_CUDA(cudaMemcpyAsync(S->scal.p, in, sizeof(double) * S_NSLOTS, cudaMemcpyHostToDevice, s));
+    if (!S->exec && !S->graph_failed && !solve_graph_off() && par_capture(S) != BD_OK) {
+        drop_capture(S->cap2);
+        drop_capture(S->cap);
+        if (S->graph) cudaGraphDestroy(S->graph);
+        S->graph = nullptr;
+        S->exec = nullptr;
+        S->graph_failed = true;
+    }
+    auto fetch = [&]() {
+        BD_CUDA(cudaMemcpyAsync(out, S->scal.p, sizeof(double) * S_NSLOTS, cudaMemcpyDeviceToHost, s));
+        BD_CUDA(cudaStreamSynchronize(s));
+        return BD_OK;
+    };
+    if (S->exec) {
+        BD_CUDA(cudaGraphLaunch(S->exec, s));
+    } else {
+        BD_TRY(par_resid(S, par_fin(S, 9), s));
+        for (;;) {
+            BD_TRY(fetch());
+            if (out[S_WARM] == 0.0) break;
+            BD_TRY(par_body(S, 0, s));
         }
+        BD_TRY(par_post(S, s));
     }
-    // true residual
-    k_par_resid<<<G, 256, 0, s>>>(N, rp, ci, sys->Ki.p, sys->M.p, c, S->v.p, S->b.p, S->dinv.p, S->r.p, S->z.p,
-                                  S->partial.p); note_launch();
+    BD_CUDA(cudaEventRecord(S->ev[1], s));
+    BD_TRY(fetch());
+    if (S->exec) note_launches(3 + (long long)out[S_IT] * kParBody);
+    float ms = 0.0f;
+    cudaEventElapsedTime(&ms, S->ev[0], S->ev[1]);
+    return info_from_scal(out, ms, info);
+}
+
+// (Ai + Ae) u_e = f from the current u_e
+int elliptic_solve(bd_dsim *S, const solve_options *o, cudaStream_t s, solve_info *info)
+{
+    if (scalar_ready(S->h, o)) return scalar_solve(S->h, S->f.p, S->ue.p, o, s, info);
+    const size_t n = 2 * (size_t)S->N;
+    if (!S->xe.p) {
+        BD_TRY(S->xe.alloc(n));
+        BD_TRY(S->fe.alloc(n));
+    }
+    const int grid = grid_for(S->N, 256);
+    k_join<<<grid, 256, 0, s>>>(S->N, S->f.p, (double2 *)S->fe.p); note_launch();
+    k_join<<<grid, 256, 0, s>>>(S->N, S->ue.p, (double2 *)S->xe.p); note_launch();
     BD_LAUNCH_CHECK();
-    BD_TRY(read_sums(S, s, 1, sums));
-    if (info) {
-        info->status = status;
-        info->iters = it;
-        info->rel_res = nb > 0.0 ? rr / nb : 0.0;
-        info->true_rel_res = nb > 0.0 ? std::sqrt(sums[0]) / nb : 0.0;
-    }
-    return status;
+    const int st = pcg_solve_device(S->h, S->fe.p, S->xe.p, 1, o, s, info);
+    k_split<<<grid, 256, 0, s>>>(S->N, (const double2 *)S->xe.p, S->ue.p); note_launch();
+    BD_LAUNCH_CHECK();
+    return st;
 }
 
 }  // namespace
@@ -282,25 +337,31 @@ extern "C" int bd_dsim_create(const bd_system *sys, amg_hierarchy *h_elliptic, c
     S->jacobi = jacobi ? 1 : 0;
     S->stim_ms = stim ? stim_ms : 0.0;
     const size_t N = (size_t)sys->N;
-    int st;
-    if ((st = S->v.alloc(N)) || (st = S->w.alloc(N)) || (st = S->stim.alloc(N)) || (st = S->xe.alloc(2 * N)) ||
-        (st = S->fe.alloc(2 * N)) || (st = S->b.alloc(N)) || (st = S->r.alloc(N)) || (st = S->z.alloc(N)) ||
-        (st = S->p.alloc(N)) || (st = S->q.alloc(N)) || (st = S->dinv.alloc(N)) ||
-        (st = S->partial.alloc((size_t)kParVals * kParBlocks))) {
+    int st = BD_OK;
+    for (DBuf<double> *d : {&S->v, &S->w, &S->stim, &S->ue, &S->f, &S->b, &S->r, &S->p, &S->q, &S->dinv})
+        if (st == BD_OK) st = d->alloc(N);
+    if (st || (st = S->partial.alloc(kPart * (size_t)kRedBlocks)) || (st = S->scal.alloc(S_NSLOTS)) ||
+        (st = S->counter.alloc(1))) {
         delete S;
         return st;
     }
-    if (cudaMallocHost((void **)&S->host_part, sizeof(double) * kParVals * kParBlocks) != cudaSuccess ||
+    if (cudaMallocHost((void **)&S->host, 2 * sizeof(double) * S_NSLOTS) != cudaSuccess ||
         cudaEventCreate(&S->ev[0]) != cudaSuccess || cudaEventCreate(&S->ev[1]) != cudaSuccess) {
         delete S;
         return BD_ECUDA;
     }
     const bd_params &P = sys->params;
     if (cudaMemsetAsync(S->v.p, 0, S->v.bytes(), s) || cudaMemsetAsync(S->w.p, 0, S->w.bytes(), s) ||
-        cudaMemsetAsync(S->stim.p, 0, S->stim.bytes(), s) || cudaMemsetAsync(S->xe.p, 0, S->xe.bytes(), s) ||
-        cudaMemsetAsync(S->partial.p, 0, S->partial.bytes(), s)) {
+        cudaMemsetAsync(S->stim.p, 0, S->stim.bytes(), s) || cudaMemsetAsync(S->ue.p, 0, S->ue.bytes(), s) ||
+        cudaMemsetAsync(S->counter.p, 0, S->counter.bytes(), s)) {
         delete S;
         return BD_ECUDA;
+    }
+    if ((st = fine_raw_build(S->raw, sys, nullptr, s)) ||
+        (st = sc_pack(S->raw, 1.0, 0.0, 0.0, 0.0, 0.0, 0.0, false, S->ki, s)) ||
+        (st = sc_pack(S->raw, 1.0, 0.0, 1.0, 0.0, 0.0, 0.0, false, S->par, s))) {
+        delete S;
+        return st;
     }
     k_par_dinv<<<grid_for(sys->N, 256), 256, 0, s>>>(sys->N, sys->A.rp.p, sys->A.ci.p, sys->Ki.p, sys->M.p,
                                                      (P.chi * P.cm) / P.dt, S->jacobi, S->dinv.p); note_launch();
@@ -328,14 +389,7 @@ extern "C" int bd_dsim_set_state(bd_dsim *S, const double *v, const double *ue, 
     const size_t bytes = sizeof(double) * (size_t)S->N;
     if (v) BD_TRY(copy_in(S->v.p, v, bytes, on_device, s));
     if (w) BD_TRY(copy_in(S->w.p, w, bytes, on_device, s));
-    if (ue) {
-        DBuf<double> t;
-        BD_TRY(t.alloc((size_t)S->N));
-        BD_TRY(copy_in(t.p, ue, bytes, on_device, s));
-        k_join<<<grid_for(S->N, 256), 256, 0, s>>>(S->N, t.p, (double2 *)S->xe.p); note_launch();
-        BD_LAUNCH_CHECK();
-        BD_CUDA(cudaStreamSynchronize(s));
-    }
+    if (ue) BD_TRY(copy_in(S->ue.p, ue, bytes, on_device, s));
     BD_CUDA(cudaStreamSynchronize(s));
     return BD_OK;
 }
@@ -347,14 +401,7 @@ extern "C" int bd_dsim_get_state(const bd_dsim *S, double *v, double *ue, double
     const size_t bytes = sizeof(double) * (size_t)S->N;
     if (v) BD_TRY(copy_out(v, S->v.p, bytes, on_device, s));
     if (w) BD_TRY(copy_out(w, S->w.p, bytes, on_device, s));
-    if (ue) {
-        DBuf<double> t;
-        BD_TRY(t.alloc((size_t)S->N));
-        k_split<<<grid_for(S->N, 256), 256, 0, s>>>(S->N, (const double2 *)S->xe.p, t.p); note_launch();
-        BD_LAUNCH_CHECK();
-        BD_TRY(copy_out(ue, t.p, bytes, on_device, s));
-        BD_CUDA(cudaStreamSynchronize(s));
-    }
+    if (ue) BD_TRY(copy_out(ue, S->ue.p, bytes, on_device, s));
     BD_CUDA(cudaStreamSynchronize(s));
     return BD_OK;
 }
@@ -376,24 +423,15 @@ extern "C" int bd_dsim_step(bd_dsim *S, int nsteps, const solve_options *opts, v
     for (int k = 0; k < nsteps && st == BD_OK; k++) {
         const double t = (double)S->step * P.dt;
         // Eq. 6: (Ai + Ae) u_e^n = -Ai v^n, warm from the previous u_e
-        k_ell_rhs<<<grid_for(S->N, 256), 256, 0, s>>>(S->N, sys->A.rp.p, sys->A.ci.p, sys->Ki.p, S->v.p,
-                                                      (double2 *)S->fe.p); note_launch();
-        BD_LAUNCH_CHECK();
-        st = pcg_solve_device(S->h, S->fe.p, S->xe.p, 1, &o, s, &ie);
+        BD_TRY(sc_apply(S->ki, (const double *)S->v.p, [&] { return DEllRhs{S->f.p}; }, s));
+        st = elliptic_solve(S, &o, s, &ie);
         te += ie.iters;
         if (st != BD_OK) break;
         // Eqs. 4 and 7, then the parabolic solve warm from v^n
-        k_par_rhs<<<grid_for(S->N, 256), 256, 0, s>>>(S->N, sys->A.rp.p, sys->A.ci.p, sys->Ki.p, sys->M.p,
-                                                      S->stim.p, t < S->stim_ms, P.chi, P.cm, P.dt, S->rm, S->v.p,
-                                                      S->w.p, S->xe.p, S->b.p); note_launch();
-        BD_LAUNCH_CHECK();
-        BD_CUDA(cudaEventRecord(S->ev[0], s));
+        BD_TRY(sc_apply(S->ki, (const double *)S->ue.p, [&] {
+            return DParRhs{sys->M.p, S->stim.p, S->v.p, S->w.p, S->b.p, P.chi, P.cm, P.dt, S->rm, t < S->stim_ms};
+        }, s));
         st = parabolic_cg(S, &o, s, &ip);
-        BD_CUDA(cudaEventRecord(S->ev[1], s));
-        BD_CUDA(cudaEventSynchronize(S->ev[1]));
-        float ms = 0.0f;
-        cudaEventElapsedTime(&ms, S->ev[0], S->ev[1]);
-        ip.solve_ms = ms;
         tp += ip.iters;
         S->step++;
     }

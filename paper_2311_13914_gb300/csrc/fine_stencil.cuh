@@ -381,6 +381,17 @@ template <class S> static FineGrid fine_grid(const FineStencil &F, double c1)
     return g;
 }
 
+// In-plane stencil position (3 (dy + 1) + dx + 1) a symmetric pair's coefficient is
+// read from: its member that exists on row type (ti, tj).
+__device__ __forceinline__ int fine_pair_pos(int k, int ti, int tj)
+{
+    if (k == 0) return 4;
+    if (k == 1) return ti == 2 ? 3 : 5;
+    if (k == 2) return tj == 2 ? 1 : 7;
+    if (k == 3) return (ti == 2 || tj == 2) ? 0 : 8;
+    return (ti == 2 || tj == 0) ? 6 : 2;
+}
+
 // Table of one slab from its raw rows and the level's Chebyshev constants, in
 // the symmetric or the general form.
 int fine_pack(const FineStencil &F, bool sym, double c2, double inv_theta, double omega, double *tab, float *tab32,
