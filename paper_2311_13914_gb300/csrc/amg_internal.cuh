@@ -107,10 +107,10 @@ struct amg_hierarchy {
     bd::FineStencil fine;
     std::shared_ptr<bd::ScalarEll> scalar;
     bd::Level lev[bd::kMaxLevels];
-    // coarsest level: dense inverse of A_c + s z z^T / z^T z, null vector z
+    // coarsest level: dense inverse of A_c + s z z^T / z^T z (null vector z) times
+    // the projection orthogonal to z
     int nc = 0;
     bd::DBuf<double> cinv, zc;
-    double zz = 0.0;
     // PCG workspace on the finest level
     bd::DBuf<double> x, r, z, p, q, fp, zold, fin;
     // whole-solve CUDA graph: pre-loop, a device-controlled WHILE node over one

@@ -377,7 +377,7 @@ struct ScalarEll {
     ScOp op;
     FineStencil F;
     ScLevel lev[kMaxLevels];
-    DBuf<double> cinv, zc;
+    DBuf<double> cinv;
     DBuf<double> fin, fp, x, r, z, p, q, zold, partial, scal;
     DBuf<unsigned int> counter;
     cudaGraph_t graph = nullptr;
@@ -431,9 +431,7 @@ int scalar_build(amg_hierarchy *h, const bd_system *sys, cudaStream_t s)
     }
     const int n = h->nc / 2;
     BD_TRY(E.cinv.alloc((size_t)n * n));
-    BD_TRY(E.zc.alloc((size_t)n));
     k_uu_dense<<<grid_for((long long)n * n, 256), 256, 0, s>>>(n, h->cinv.p, E.cinv.p); ::bd::note_launch();
-    k_u_field<<<grid_for(n, 256), 256, 0, s>>>(n, h->zc.p, E.zc.p, nullptr); ::bd::note_launch();
     BD_LAUNCH_CHECK();
     const size_t N = (size_t)L0.N;
     for (DBuf<double> *v : {&E.fin, &E.fp, &E.x, &E.r, &E.z, &E.p, &E.q}) BD_TRY(v->alloc(N));
@@ -486,7 +484,7 @@ int vcycle1(amg_hierarchy *h, const S *f0, const Fin &zf, cudaStream_t s)
                       E1Restrict<S>{P(D.f), P(D.d), P(D.invd), (S)h->lev[l + 1].ch_inv_theta}, s));
     }
     ScLevel &K = E.lev[nl - 1];
-    BD_TRY(coarse_solve(h->nc / 2, E.cinv.p, E.zc.p, h->zz, nl == 1 ? f0 : (const S *)P(K.f), P(K.u), s));
+    BD_TRY(coarse_solve(h->nc / 2, E.cinv.p, nl == 1 ? f0 : (const S *)P(K.f), P(K.u), s));
     for (int l = nl - 2; l >= 0; l--) {
         Level &L = h->lev[l];
         ScLevel &C = E.lev[l], &D = E.lev[l + 1];

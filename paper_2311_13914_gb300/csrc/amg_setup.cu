@@ -1304,6 +1304,24 @@ __global__ void k_gj_update(int n, int K, int bb, double *__restrict__ A, const 
     }
 }
 
+// C = Cinv (I - z z^T / z.z): the solve's projection of the residual orthogonal
+// to the null vector z, folded into the inverse once.  One block per row.
+__global__ void __launch_bounds__(128) k_coarse_project(int n, double *__restrict__ C, const double *__restrict__ z,
+                                                        const double *__restrict__ zz)
+{
+    __shared__ double part[4];
+    double *row = C + (size_t)blockIdx.x * n;
+    double s = 0.0;
+    for (int j = threadIdx.x; j < n; j += blockDim.x) s = s + row[j] * z[j];
+    for (int o = 16; o; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = s;
+    __syncthreads();
+    s = ((part[0] + part[1]) + part[2]) + part[3];
+    if (!(*zz > 0.0)) return;
+    const double a = s / *zz;
+    for (int j = threadIdx.x; j < n; j += blockDim.x) row[j] = row[j] - a * z[j];
+}
+
 __global__ void k_null_vector(int N, const double *__restrict__ B, double *z)
 {
     int p = blockIdx.x * blockDim.x + threadIdx.x;
@@ -1604,9 +1622,10 @@ static int build_coarsest(amg_hierarchy *h, int l, cudaStream_t s)
         BD_CUDA(cudaMemcpyAsync(zz.p, st.p + 1, sizeof(double), cudaMemcpyDeviceToDevice, s));
         BD_CUDA(cudaStreamSynchronize(s));  // the scratch buffers are freed on return
     }
+    k_coarse_project<<<n, 128, 0, s>>>(n, h->cinv.p, h->zc.p, zz.p); ::bd::note_launch();
+    BD_LAUNCH_CHECK();
     int hbad = 0;
     BD_CUDA(cudaMemcpyAsync(&hbad, bad.p, sizeof(int), cudaMemcpyDeviceToHost, s));
-    BD_CUDA(cudaMemcpyAsync(&h->zz, zz.p, sizeof(double), cudaMemcpyDeviceToHost, s));
     BD_CUDA(cudaStreamSynchronize(s));
     return hbad ? BD_EINVAL : BD_OK;
 }

@@ -877,94 +877,67 @@ static double fine_ops(const amg_hierarchy *h, const Level &L, int role)
 }
 
 // ------------------------------------------------------------------ coarsest level
-// x = Cinv (r - (z.r / z.z) z) in FP64 whatever the storage precision; one
-// block, one warp per output row.
-template <class S>
-__global__ void k_coarse_solve(int n, const double *__restrict__ cinv, const double *__restrict__ z,
-                               double zz, const S *__restrict__ r, S *__restrict__ x)
+// x = C r in FP64 whatever the storage precision, C the inverse of the
+// rank-one-fixed coarsest operator with the projection orthogonal to its null
+// vector folded in (k_coarse_project): one dense mat-vec, a warp per row, the rows
+// spread evenly over the SMs.  Larger FP32 right-hand sides are widened once per
+// block in shared memory (a conversion costs the FP64 pipe what a multiply-add
+// does).  The separate projection made every block reduce z.r first: 62
+// unknowns 12.1 us in one block, 1942 unknowns 21.5 us; event-timed inside the
+// solve 14.8 -> 6.3 and 22.1 -> 16.1 (FP32 24.3 -> 18.1), bound by the latency of
+// streaming 30 MB with 13 warps per SM (two blocks' worth of loads in flight need
+// the 64 registers the launch bound leaves).
+template <class S, bool STAGE>
+__global__ void __launch_bounds__(1024, 1) k_coarse_solve(int n, const double *__restrict__ C, const S *__restrict__ r,
+                                                       S *__restrict__ x)
 {
-    extern __shared__ double rs[];
-    __shared__ double red[32];
-    double part = 0.0;
-    for (int i = threadIdx.x; i < n; i += blockDim.x) part += z[i] * (double)r[i];
-    for (int o = 16; o; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = part;
-    __syncthreads();
-    if (threadIdx.x < 32) {
-        double v = threadIdx.x < (blockDim.x >> 5) ? red[threadIdx.x] : 0.0;
-        for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-        if (threadIdx.x == 0) red[0] = v;
+    extern __shared__ double2 rs[];
+    if constexpr (STAGE) {
+        for (int j = threadIdx.x; j < n / 2; j += blockDim.x) {
+            const v2<S> v = ((const v2<S> *)r)[j];
+            rs[j] = make_double2((double)v.x, (double)v.y);
+        }
+        __syncthreads();
     }
-    __syncthreads();
-    double a = zz > 0.0 ? red[0] / zz : 0.0;
-    for (int i = threadIdx.x; i < n; i += blockDim.x) rs[i] = (double)r[i] - a * z[i];
-    __syncthreads();
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    for (int i = warp; i < n; i += nw) {
-        const double *row = cinv + (size_t)i * n;
-        double sacc = 0.0;
-        for (int j = lane; j < n; j += 32) sacc += row[j] * rs[j];
-        for (int o = 16; o; o >>= 1) sacc += __shfl_xor_sync(0xffffffffu, sacc, o);
-        if (lane == 0) x[i] = (S)sacc;
+    const int lane = threadIdx.x & 31, i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    if (i >= n) return;
+    const double *row = C + (size_t)i * n;
+    double s0 = 0.0, s1 = 0.0;
+    if (n & 1) {
+        for (int j = lane; j < n; j += 32) s0 = fma(row[j], (double)r[j], s0);
+    } else {  // even rows start on 16 bytes
+#pragma unroll 8
+        for (int j = lane; j < n / 2; j += 32) {
+            const double2 c = ((const double2 *)row)[j];
+            double2 v;
+            if constexpr (STAGE) {
+                v = rs[j];
+            } else {
+                const v2<S> t = ((const v2<S> *)r)[j];
+                v = make_double2((double)t.x, (double)t.y);
+            }
+            s0 = fma(c.x, v.x, s0);
+            s1 = fma(c.y, v.y, s1);
+        }
     }
+    s0 += s1;
+    for (int o = 16; o; o >>= 1) s0 += __shfl_xor_sync(0xffffffffu, s0, o);
+    if (lane == 0) x[i] = (S)s0;
 }
 
-// The same for larger coarsest levels, over the whole GPU: every block forms
-// z.r and the projected right-hand side r - (z.r/z.z) z in shared memory
-// itself (same order in each block, so all agree), then one warp per row: one
-// FP64 FMA per matrix entry.
-template <class S>
-__global__ void __launch_bounds__(256) k_coarse_solve_wide(int n, const double *__restrict__ cinv,
-                                                           const double *__restrict__ z, double zz,
-                                                           const S *__restrict__ r, S *__restrict__ x)
+template <class S> static int launch_coarse(int n, const double *C, const S *r, S *x, cudaStream_t s)
 {
-    extern __shared__ double rs[];
-    __shared__ double red[8];
-    __shared__ double alpha;
-    double part = 0.0;
-    for (int i = threadIdx.x; i < n; i += blockDim.x) part += z[i] * (double)r[i];
-    for (int o = 16; o; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = part;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double v = 0.0;
-        for (int w = 0; w < (int)(blockDim.x >> 5); w++) v += red[w];
-        alpha = zz > 0.0 ? v / zz : 0.0;
-    }
-    __syncthreads();
-    const double a = alpha;
-    for (int i = threadIdx.x; i < n; i += blockDim.x) rs[i] = (double)r[i] - a * z[i];
-    __syncthreads();
-    const int lane = threadIdx.x & 31;
-    const int warp = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    const int nw = gridDim.x * (blockDim.x >> 5);
-    for (int i = warp; i < n; i += nw) {
-        const double *row = cinv + (size_t)i * n;
-        double sacc = 0.0;
-        for (int j = lane; j < n; j += 32) sacc = fma(row[j], rs[j], sacc);
-        for (int o = 16; o; o >>= 1) sacc += __shfl_xor_sync(0xffffffffu, sacc, o);
-        if (lane == 0) x[i] = (S)sacc;
-    }
-}
-
-template <class S>
-static int launch_coarse(int n, const double *cinv, const double *z, double zz, const S *r, S *x, cudaStream_t s)
-{
-    const size_t smem = sizeof(double) * (size_t)n;
-    if (n <= 256) k_coarse_solve<S><<<1, 1024, smem, s>>>(n, cinv, z, zz, r, x);
-    else k_coarse_solve_wide<S><<<(n + 7) / 8, 256, smem, s>>>(n, cinv, z, zz, r, x);
+    const int w = std::min(32, (n + kSM - 1) / kSM), grid = (n + w - 1) / w;  // rows (warps) per block
+    if (sizeof(S) == 4 && w > 2 && !(n & 1))
+        k_coarse_solve<S, true><<<grid, 32 * w, sizeof(double) * (size_t)n, s>>>(n, C, r, x);
+    else
+        k_coarse_solve<S, false><<<grid, 32 * w, 0, s>>>(n, C, r, x);
     ::bd::note_launch();
     BD_LAUNCH_CHECK();
     return BD_OK;
 }
-int coarse_solve(int n, const double *cinv, const double *z, double zz, const double *r, double *x, cudaStream_t s)
-{
-    return launch_coarse(n, cinv, z, zz, r, x, s);
-}
-int coarse_solve(int n, const double *cinv, const double *z, double zz, const float *r, float *x, cudaStream_t s)
-{
-    return launch_coarse(n, cinv, z, zz, r, x, s);
-}
+int coarse_solve(int n, const double *C, const double *r, double *x, cudaStream_t s) { return launch_coarse(n, C, r, x, s); }
+int coarse_solve(int n, const double *C, const float *r, float *x, cudaStream_t s) { return launch_coarse(n, C, r, x, s); }
 
 template <class S>
 __global__ void k_copy2(int N, const v2<S> *__restrict__ a, v2<S> *__restrict__ b)
@@ -1139,7 +1112,7 @@ static int vcycle_impl(amg_hierarchy *h, const v2<S> *f0, v2<S> *u0, cudaStream_
         const S *f = (const S *)(nl == 1 ? f0 : cv.f);
         S *u = (S *)(nl == 1 ? u0 : cv.u);
         int sc = prof_begin(h, s, R_COARSE, false);
-        BD_TRY(coarse_solve(h->nc, h->cinv.p, h->zc.p, h->zz, f, u, s));
+        BD_TRY(coarse_solve(h->nc, h->cinv.p, f, u, s));
         prof_end(h, sc, 0.0, 0.0, s);
     }
     for (int l = nl - 2; l >= 0; l--) BD_TRY(up(l));

@@ -167,9 +167,7 @@ __global__ void k_st_f32(long long n, const double *__restrict__ src, float *__r
 
 // ------------------------------------------------------------------ coarsest levels
 struct StCoarseJob {
-    const double *cinv;  // n x n dense inverse of the member's rank-one-fixed coarsest operator
-    const double *z;     // its null vector
-    double zz;           // z . z
+    const double *C;     // n x n projected inverse of the member's coarsest operator
     int n;               // unknowns
     int level;           // stack level holding the member's coarsest level
     long long off;       // first unknown of the member on that level
@@ -179,39 +177,27 @@ template <class S> struct StLevelPtrs {
     S *u[kMaxLevels];
 };
 
-// x = Cinv (r - (z.r / z.z) z) in FP64 for every member at once (block k:
-// member k's coarsest level), as the single-hierarchy coarsest solve.
+// x = C r in FP64 for every member at once (blockIdx.y: the member), a warp per
+// row, as the single-hierarchy coarsest solve.
 template <class S>
-__global__ void __launch_bounds__(512) k_st_coarse(const StCoarseJob *__restrict__ jobs, StLevelPtrs<S> lp)
+__global__ void __launch_bounds__(128) k_st_coarse(const StCoarseJob *__restrict__ jobs, StLevelPtrs<S> lp)
 {
-    extern __shared__ double rs[];
-    __shared__ double red[32];
-    const StCoarseJob J = jobs[blockIdx.x];
-    const S *r = lp.f[J.level] + J.off;
-    S *x = lp.u[J.level] + J.off;
-    const int n = J.n;
-    double part = 0.0;
-    for (int i = threadIdx.x; i < n; i += blockDim.x) part += J.z[i] * (double)r[i];
-    for (int o = 16; o; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = part;
-    __syncthreads();
-    if (threadIdx.x < 32) {
-        double v = threadIdx.x < (blockDim.x >> 5) ? red[threadIdx.x] : 0.0;
-        for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-        if (threadIdx.x == 0) red[0] = v;
+    const StCoarseJob J = jobs[blockIdx.y];
+    const int lane = threadIdx.x & 31, i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    if (i >= J.n) return;
+    const v2<S> *r = (const v2<S> *)(lp.f[J.level] + J.off);
+    const double2 *row = (const double2 *)(J.C + (size_t)i * J.n);
+    double s0 = 0.0, s1 = 0.0;
+#pragma unroll 4
+    for (int j = lane; j < J.n / 2; j += 32) {
+        const double2 c = row[j];
+        const v2<S> v = r[j];
+        s0 = fma(c.x, (double)v.x, s0);
+        s1 = fma(c.y, (double)v.y, s1);
     }
-    __syncthreads();
-    const double a = J.zz > 0.0 ? red[0] / J.zz : 0.0;
-    for (int i = threadIdx.x; i < n; i += blockDim.x) rs[i] = (double)r[i] - a * J.z[i];
-    __syncthreads();
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    for (int i = warp; i < n; i += nw) {
-        const double *row = J.cinv + (size_t)i * n;
-        double s = 0.0;
-        for (int j = lane; j < n; j += 32) s += row[j] * rs[j];
-        for (int o = 16; o; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-        if (lane == 0) x[i] = (S)s;
-    }
+    s0 += s1;
+    for (int o = 16; o; o >>= 1) s0 += __shfl_xor_sync(0xffffffffu, s0, o);
+    if (lane == 0) lp.u[J.level][J.off + i] = (S)s0;
 }
 
 // ------------------------------------------------------------------ PCG reductions
@@ -848,7 +834,7 @@ int st_create(amg_stack *b, cudaStream_t s)
     for (int k = 0; k < count; k++) {
         const amg_hierarchy *hk = b->h[k];
         const int c = b->nlev[k] - 1;
-        jobs[k] = {hk->cinv.p, hk->zc.p, hk->zz, hk->nc, c, 2 * off[c][k]};
+        jobs[k] = {hk->cinv.p, hk->nc, c, 2 * off[c][k]};
         b->max_nc = std::max(b->max_nc, hk->nc);
     }
     BD_TRY(b->jobs.alloc(count));
@@ -989,10 +975,8 @@ int st_vcycle(amg_stack *b, cudaStream_t s)
         lp.f[l] = (S *)v.f;
         lp.u[l] = (S *)v.u;
     }
-    const size_t smem = sizeof(double) * (size_t)std::max(b->max_nc, 1);
-    if (smem > 48 * 1024) BD_CUDA(cudaFuncSetAttribute(k_st_coarse<S>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                       (int)smem));
-    k_st_coarse<S><<<b->count, 512, smem, s>>>(b->jobs.p, lp); ::bd::note_launch();
+    const dim3 grid((std::max(b->max_nc, 1) + 3) / 4, b->count);
+    k_st_coarse<S><<<grid, 128, 0, s>>>(b->jobs.p, lp); ::bd::note_launch();
     BD_LAUNCH_CHECK();
     for (int l = L - 2; l >= 0; l--) {
         StLevel &Lv = b->lev[l];

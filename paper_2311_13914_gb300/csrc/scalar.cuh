@@ -22,9 +22,9 @@ bool solve_graph_off();             // BD_SOLVE_GRAPH=0
 // report of a graph-form solve from its scalar block; returns the status
 int info_from_scal(const double *scal, float ms, solve_info *info);
 
-// x = Cinv (r - (z.r / z.z) z), n unknowns
-int coarse_solve(int n, const double *cinv, const double *z, double zz, const double *r, double *x, cudaStream_t s);
-int coarse_solve(int n, const double *cinv, const double *z, double zz, const float *r, float *x, cudaStream_t s);
+// x = C r with the projected coarsest inverse, n unknowns
+int coarse_solve(int n, const double *C, const double *r, double *x, cudaStream_t s);
+int coarse_solve(int n, const double *C, const float *r, float *x, cudaStream_t s);
 
 // Elliptic hierarchies (bd_elliptic_setup): the scalar form of the V-cycle.
 int scalar_build(amg_hierarchy *h, const bd_system *sys, cudaStream_t s);
