@@ -80,11 +80,8 @@ struct Level {
 };
 
 // Finest level of an assembled slab as a layered stencil (fine_stencil.cuh):
-// one row of coefficients per plane and row type (3 (y face) + (x face), 0 low,
-// 1 interior, 2 high).  raw holds the assembled rows themselves, kFineRaw
-// doubles each: (Ki, Ke) at the 27 stencil positions 9 (dz + 1) + 3 (dy + 1) +
-// dx + 1, c M, and the inverse diagonal (v, u_e); tab is packed for the kernels.
-constexpr int kFineRaw = 58;
+// one row of coefficients per plane and row type.  raw holds the system's rows
+// (bd_assemble.cu), tab is packed for the kernels.
 struct FineStencil {
     bool valid = false;
     bool sym = false;           // rows symmetric under (dx, dy) -> (-dx, -dy)
@@ -160,8 +157,8 @@ int prepare_solve(amg_hierarchy *h, cudaStream_t s);
 int pcg_solve_begin(amg_hierarchy *h, const double *f_dev, double *x_dev, int warm,
                     const solve_options *o, cudaStream_t s, solve_info *info, bool *pending);
 int pcg_solve_end(amg_hierarchy *h, cudaStream_t s, solve_info *info);
-// raw rows and symmetry of sys's operators (invd: interleaved inverse diagonals, or null)
-int fine_raw_build(FineStencil &F, const bd_system *sys, const double *invd, cudaStream_t s);
+// a copy of sys's raw rows
+int fine_raw_copy(FineStencil &F, const bd_system *sys, cudaStream_t s);
 int build_fine_stencil(amg_hierarchy *h, const bd_system *sys, cudaStream_t s);
 // Timed step of the solve phase (host-driven loop only).  `fine`: a
 // finest-operator application, timed at profiling level 1 and summed into

@@ -45,8 +45,9 @@ __global__ void k_sc_pack(int rows, const double *__restrict__ raw, double a, do
             put(z * Row::G + k, q == 13 ? v + m * o[54] : v);
         }
     }
-    put(Row::IDC2, c2 * o[56]);
-    put(Row::IDT, o[56] * it);
+    const double du = o[55] > 0.0 ? 1.0 / (o[26] + o[27]) : 0.0;  // of Ai + Ae
+    put(Row::IDC2, c2 * du);
+    put(Row::IDT, du * it);
 }
 
 int sc_pack(const FineStencil &F, double a, double b, double m, double c1, double c2, double inv_theta, bool fp32,
@@ -408,7 +409,7 @@ int scalar_build(amg_hierarchy *h, const bd_system *sys, cudaStream_t s)
     const bool p32 = h->prec32;
     const int nl = h->nlev;
     Level &L0 = h->lev[0];
-    BD_TRY(fine_raw_build(E.F, sys, L0.invdiag.p, s));
+    BD_TRY(fine_raw_copy(E.F, sys, s));
     BD_TRY(sc_pack(E.F, 1.0, 1.0, 0.0, L0.ch_c1, L0.ch_c2, L0.ch_inv_theta, p32, E.op, s));
     for (int l = 0; l < nl; l++) {
         Level &L = h->lev[l];

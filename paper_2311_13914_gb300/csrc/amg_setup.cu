@@ -82,36 +82,43 @@ __device__ __forceinline__ bool strength_w(const int *rp, const int *ci, const d
 // One pass forms every entry's weight (a square root and a division, costly
 // on the FP64 pipe) and counts the strong ones; wt[t] keeps the weight of a
 // strong entry and -1 otherwise (weights are >= 0), so the fill only compacts.
+// A warp per row: entries are independent, and each looks its transpose up by a
+// chain of dependent loads (with a thread per row, 2718 rows of 223 blocks took
+// 1250 us).
 __global__ void k_strength_count(int N, const int *__restrict__ rp, const int *__restrict__ ci,
                                  const double *__restrict__ v, const double *__restrict__ diag,
                                  double theta, int *cnt, double *__restrict__ wt)
 {
-    int p = blockIdx.x * blockDim.x + threadIdx.x;
+    const int lane = threadIdx.x & 31, p = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     if (p >= N) return;
     int c = 0;
-    double w;
-    for (int t = rp[p]; t < rp[p + 1]; t++) {
+    for (int t = rp[p] + lane; t < rp[p + 1]; t += 32) {
+        double w = 0.0;
         const bool strong = strength_w(rp, ci, v, diag, p, t, theta, &w);
         wt[t] = strong ? w : -1.0;
         c += strong;
     }
-    cnt[p] = c;
+    c = __reduce_add_sync(0xffffffffu, c);
+    if (lane == 0) cnt[p] = c;
 }
 
 __global__ void k_strength_fill(int N, const int *__restrict__ rp, const int *__restrict__ ci,
                                 const double *__restrict__ wt, const int *__restrict__ srp,
                                 int *__restrict__ sci, double *__restrict__ sw)
 {
-    int p = blockIdx.x * blockDim.x + threadIdx.x;
+    const int lane = threadIdx.x & 31, p = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     if (p >= N) return;
     int pos = srp[p];
-    for (int t = rp[p]; t < rp[p + 1]; t++) {
-        const double w = wt[t];
+    for (int t0 = rp[p]; t0 < rp[p + 1]; t0 += 32) {
+        const int t = t0 + lane;
+        const double w = t < rp[p + 1] ? wt[t] : -1.0;
+        const unsigned m = __ballot_sync(0xffffffffu, w >= 0.0);
         if (w >= 0.0) {
-            sci[pos] = ci[t];
-            sw[pos] = w;
-            pos++;
+            const int o = pos + __popc(m & ((1u << lane) - 1u));
+            sci[o] = ci[t];
+            sw[o] = w;
         }
+        pos += __popc(m);
     }
 }
 
@@ -337,14 +344,16 @@ __global__ void k_spgemm_fill_smem(int nrows, const int *__restrict__ arp, const
 // addressing in shared memory, the same accumulation order.
 __device__ __forceinline__ int hslot(int key, int mask) { return (int)(((unsigned)key * 2654435761u) & (unsigned)mask); }
 
+// eight lanes per row (rows of hundreds of blocks: a thread's chain of loads)
 __global__ void k_spgemm_bound(int nrows, const int *__restrict__ arp, const int *__restrict__ aci,
                                const int *__restrict__ brp, int *__restrict__ ub)
 {
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= nrows) return;
+    const int i = (blockIdx.x * blockDim.x + threadIdx.x) >> 3, l = threadIdx.x & 7;
     long long u = 0;
-    for (int t = arp[i]; t < arp[i + 1]; t++) u += brp[aci[t] + 1] - brp[aci[t]];
-    ub[i] = u > INT_MAX ? INT_MAX : (int)u;
+    if (i < nrows)
+        for (int t = arp[i] + l; t < arp[i + 1]; t += 8) u += brp[aci[t] + 1] - brp[aci[t]];
+    for (int o = 4; o; o >>= 1) u += __shfl_xor_sync(0xffffffffu, u, o);
+    if (i < nrows && l == 0) ub[i] = u > INT_MAX ? INT_MAX : (int)u;
 }
 
 // Hash-path SpGEMM: L lanes per output row, 32/L rows per warp (L from the
@@ -596,7 +605,7 @@ static int spgemm(int nrows, int ncols, const int *arp, const int *aci, const do
     // accumulate every entry in the same order, so the choice changes no bit.
     long long mub = 1;
     if (nrows > 0) {
-        k_spgemm_bound<<<(nrows + 255) / 256, 256, 0, s>>>(nrows, arp, aci, brp, cnt.p); ::bd::note_launch();
+        k_spgemm_bound<<<(nrows + 31) / 32, 256, 0, s>>>(nrows, arp, aci, brp, cnt.p); ::bd::note_launch();
         BD_LAUNCH_CHECK();
         BD_TRY(device_max(cnt.p, nrows, flag.p + 1, s));
         int hb = 0;
@@ -719,19 +728,22 @@ __global__ void k_insert_diag(int N, const int *__restrict__ srp, const int *__r
     }
 }
 
+// (every row of Wh*Wh holds its diagonal: entries before it move up by the p
+// diagonals of earlier rows, entries behind it by one more)
 __global__ void k_drop_diag(int N, const int *__restrict__ qrp, const int *__restrict__ qci,
                             const double *__restrict__ qv, int *__restrict__ orp,
                             int *__restrict__ oci, double *__restrict__ ov)
 {
-    int p = blockIdx.x * blockDim.x + threadIdx.x;
+    const int lane = threadIdx.x & 31, p = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     if (p > N) return;
-    orp[p] = qrp[p] - p;  // every row of Wh*Wh holds its diagonal
+    if (lane == 0) orp[p] = qrp[p] - p;
     if (p == N) return;
-    int pos = qrp[p] - p;
-    for (int t = qrp[p]; t < qrp[p + 1]; t++) {
-        if (qci[t] == p) continue;
-        oci[pos] = qci[t];
-        ov[pos++] = qv[t];
+    for (int t = qrp[p] + lane; t < qrp[p + 1]; t += 32) {
+        const int q = qci[t];
+        if (q == p) continue;
+        const int o = t - p - (q > p ? 1 : 0);
+        oci[o] = q;
+        ov[o] = qv[t];
     }
 }
 
@@ -863,10 +875,11 @@ __global__ void k_ptent(int N, const int *__restrict__ agg, const double *__rest
 }
 
 // ------------------------------------------------------------------ a5 lambda_max (CG-Lanczos)
+// The CG scalars of every step; the tridiagonal's coefficients and the step at
+// which the recurrence ends (a pq or rz that is not positive) follow from them
+// in k_lanczos_finish.  Steps past that end still run and are not read.
 struct LanczosState {
-    double rz, pq, rz1;
-    double alpha[64], beta[64];
-    int m, stop;
+    double rz[65], pq[64];
     double lam;
     int bad;
 };
@@ -885,99 +898,120 @@ __global__ void k_lanczos_init(int n, unsigned long long key, const double *__re
     p[i] = zi;
 }
 
-// y = A x, scalar rows in ascending column order, acc = acc + a*x from 0.0
-__global__ void k_spmv_ordered(int N, const int *__restrict__ rp, const int *__restrict__ ci,
+// y = A x, scalar rows in ascending column order, acc = acc + a*x from 0.0: one
+// thread per scalar row (its additions are one chain), whose loads run eight
+// blocks ahead of the chain.  Bound by the FP64 pipe on large levels (4 rounded
+// operations per scalar row and block; 128x128x32 237 us, floor 183), by the
+// chain on small ones (2718 rows of 223 blocks: 307 -> 94 us).
+__global__ void __launch_bounds__(256, 3) k_spmv_ordered(int n, const int *__restrict__ rp, const int *__restrict__ ci,
                                const double *__restrict__ v, const double *__restrict__ x,
                                double *__restrict__ y)
 {
-    int p = blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= N) return;
-    double s0 = 0.0, s1 = 0.0;
-    for (int t = rp[p]; t < rp[p + 1]; t++) {
-        int q = ci[t];
-        double x0 = x[2 * q], x1 = x[2 * q + 1];
-        const double *a = v + 4 * (size_t)t;
-        s0 = s0 + a[0] * x0;
-        s0 = s0 + a[1] * x1;
-        s1 = s1 + a[2] * x0;
-        s1 = s1 + a[3] * x1;
+    constexpr int U = 8;
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    const double2 *a = (const double2 *)v + (i & 1), *w = (const double2 *)x;
+    double s = 0.0;
+    const int e = rp[(i >> 1) + 1];
+    int t = rp[i >> 1];
+    for (; t + U <= e; t += U) {
+        double2 av[U], wv[U];
+        int q[U];
+#pragma unroll
+        for (int k = 0; k < U; k++) q[k] = ci[t + k];
+#pragma unroll
+        for (int k = 0; k < U; k++) {
+            av[k] = a[2 * (size_t)(t + k)];
+            wv[k] = w[q[k]];
+        }
+#pragma unroll
+        for (int k = 0; k < U; k++) {
+            s = s + av[k].x * wv[k].x;
+            s = s + av[k].y * wv[k].y;
+        }
     }
-    y[2 * p] = s0;
-    y[2 * p + 1] = s1;
-}
-
-__global__ void k_lanczos_alpha(LanczosState *st, int j)
-{
-    if (st->stop) return;
-    if (!(st->pq > 0.0) || !(st->rz > 0.0)) {
-        st->stop = 1;
-        return;
+    for (; t < e; t++) {
+        const double2 av = a[2 * (size_t)t], wv = w[ci[t]];
+        s = s + av.x * wv.x;
+        s = s + av.y * wv.y;
     }
-    st->alpha[j] = st->rz / st->pq;
+    y[i] = s;
 }
 
 __global__ void k_lanczos_update_r(int n, const LanczosState *st, int j, const double *__restrict__ q,
                                    const double *__restrict__ diag, double *r, double *z)
 {
-    if (st->stop) return;
+    __shared__ double alpha;
+    if (threadIdx.x == 0) alpha = st->rz[j] / st->pq[j];
+    __syncthreads();
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
-    double a = st->alpha[j];
-    double ri = r[i] - a * q[i];
+    double ri = r[i] - alpha * q[i];
     r[i] = ri;
     z[i] = ri / diag[i];
-}
-
-__global__ void k_lanczos_beta(LanczosState *st, int j)
-{
-    if (st->stop) return;
-    double beta = st->rz1 / st->rz;
-    st->beta[j] = beta;
-    st->m = j + 1;
-    if (!(st->rz1 > 0.0)) {
-        st->stop = 1;
-        return;
-    }
-    st->rz = st->rz1;
 }
 
 __global__ void k_lanczos_update_p(int n, const LanczosState *st, int j, const double *__restrict__ z,
                                    double *p)
 {
-    if (st->stop) return;
+    __shared__ double beta;
+    if (threadIdx.x == 0) beta = st->rz[j + 1] / st->rz[j];
+    __syncthreads();
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
-    double b = st->beta[j];
-    p[i] = z[i] + b * p[i];
+    p[i] = z[i] + beta * p[i];
 }
 
-__device__ int sturm_count_below(int m, const double *d, const double *e, double x)
+// eigenvalues of the tridiagonal (diagonal d, squared off-diagonal e2) below x
+__device__ int sturm_count_below(int m, const double *d, const double *e2, double x)
 {
     int c = 0;
     double q = d[0] - x;
     if (q < 0.0) c++;
     for (int i = 1; i < m; i++) {
         if (q == 0.0) q = -1e-300;
-        q = (d[i] - x) - (e[i - 1] * e[i - 1]) / q;
+        q = (d[i] - x) - e2[i - 1] / q;
         if (q < 0.0) c++;
     }
     return c;
 }
 
-__global__ void k_lanczos_finish(LanczosState *st)
+// Largest Ritz value by bisection to the last bit.  One warp runs five bisection
+// steps at a time: lane l takes node l of the tree of their midpoints (heap
+// order), forms its midpoint by the additions the steps on its path would make,
+// and the walk down the tree then reads five answers after one evaluation's
+// latency.  The midpoints and answers are those of the sequential bisection, so
+// the result is its result (one thread stepping alone: 255 us, now 68).
+__global__ void k_lanczos_finish(LanczosState *st, int steps)
 {
-    int m = st->m;
+    __shared__ double d[64], e[64], e2[64];
+    const int lane = threadIdx.x;
+    int m = 0;
+    while (m < steps && st->pq[m] > 0.0 && st->rz[m] > 0.0) {
+        m++;
+        if (!(st->rz[m] > 0.0)) break;
+    }
     if (m == 0) {
-        st->bad = 1;
-        st->lam = 0.0;
+        if (lane == 0) {
+            st->bad = 1;
+            st->lam = 0.0;
+        }
         return;
     }
-    double d[64], e[64];
-    for (int j = 0; j < m; j++) {
-        d[j] = 1.0 / st->alpha[j];
-        if (j > 0) d[j] = d[j] + st->beta[j - 1] / st->alpha[j - 1];
-        if (j < m - 1) e[j] = sqrt(st->beta[j]) / st->alpha[j];
+    for (int j = lane; j < m; j += 32) {
+        const double al = st->rz[j] / st->pq[j];
+        double dj = 1.0 / al;
+        if (j > 0) {
+            const double alp = st->rz[j - 1] / st->pq[j - 1], bep = st->rz[j] / st->rz[j - 1];
+            dj = dj + bep / alp;
+        }
+        d[j] = dj;
+        double ej = 0.0;
+        if (j < m - 1) ej = sqrt(st->rz[j + 1] / st->rz[j]) / al;
+        e[j] = ej;
+        e2[j] = ej * ej;
     }
+    __syncwarp();
     double lo = 0.0, hi = 0.0;
     for (int i = 0; i < m; i++) {
         double r = 0.0;
@@ -987,35 +1021,54 @@ __global__ void k_lanczos_finish(LanczosState *st)
         if (i == 0 || a < lo) lo = a;
         if (i == 0 || b > hi) hi = b;
     }
-    for (int it = 0; it < 4096; it++) {
-        double mid = 0.5 * (lo + hi);
-        if (!(mid > lo && mid < hi)) break;
-        if (sturm_count_below(m, d, e, mid) == m) hi = mid;
-        else lo = mid;
+    for (int it = 0; it < 4096;) {
+        // lane l's midpoint: from the root (1) down to node l
+        double nlo = lo, nhi = hi, mid = 0.5 * (nlo + nhi);
+        const int node = lane > 0 ? lane : 1;
+        for (int bit = 30 - __clz(node); bit >= 0; bit--) {
+            if ((node >> bit) & 1) nlo = mid;
+            else nhi = mid;
+            mid = 0.5 * (nlo + nhi);
+        }
+        const unsigned open = __ballot_sync(0xffffffffu, mid > nlo && mid < nhi);
+        const unsigned all = __ballot_sync(0xffffffffu, sturm_count_below(m, d, e2, mid) == m);
+        bool done = false;
+        for (int k = 1; k < 32 && it < 4096; it++) {
+            if (!((open >> k) & 1)) {
+                done = true;
+                break;
+            }
+            const double x = 0.5 * (lo + hi);
+            const bool below = (all >> k) & 1;
+            if (below) hi = x;
+            else lo = x;
+            k = 2 * k + (below ? 0 : 1);
+        }
+        if (done) break;
     }
-    st->lam = hi;
+    if (lane == 0) st->lam = hi;
 }
 
 // ------------------------------------------------------------------ a6 smoothed prolongator
 // P(i,j) = Pt(i,j) - s_i AP(i,j),  s_i = omega / A(i,i),  omega = 4/(3 lambda)
+// (eight lanes per row)
 __global__ void k_smooth_p(int N, const int *__restrict__ rp, const int *__restrict__ ci,
                            double *__restrict__ v, const int *__restrict__ agg,
                            const double *__restrict__ ptd, const double *__restrict__ diag,
                            const LanczosState *st)
 {
-    int p = blockIdx.x * blockDim.x + threadIdx.x;
+    const int p = (blockIdx.x * blockDim.x + threadIdx.x) >> 3, l = threadIdx.x & 7;
     if (p >= N) return;
     double omega = 4.0 / (3.0 * st->lam);
     double s0 = omega / diag[2 * p], s1 = omega / diag[2 * p + 1];
     int J = agg[p];
-    for (int t = rp[p]; t < rp[p + 1]; t++) {
+    for (int t = rp[p] + l; t < rp[p + 1]; t += 8) {
         bool own = ci[t] == J;
-        double *b = v + 4 * (size_t)t;
+        double2 *b = (double2 *)v + 2 * (size_t)t;
         double p00 = own ? ptd[2 * p] : 0.0, p11 = own ? ptd[2 * p + 1] : 0.0;
-        b[0] = p00 - s0 * b[0];
-        b[1] = 0.0 - s0 * b[1];
-        b[2] = 0.0 - s1 * b[2];
-        b[3] = p11 - s1 * b[3];
+        const double2 x = b[0], y = b[1];
+        b[0] = make_double2(p00 - s0 * x.x, 0.0 - s0 * x.y);
+        b[1] = make_double2(0.0 - s1 * y.x, p11 - s1 * y.y);
     }
 }
 
@@ -1084,18 +1137,17 @@ static int bsr_transpose(const BSR &a, BSR &t, cudaStream_t s)
 }
 
 // ------------------------------------------------------------------ a9 coarsest level
+// a warp per block row
 __global__ void k_coarse_dense(int N, const int *__restrict__ rp, const int *__restrict__ ci,
                                const double *__restrict__ v, double *__restrict__ Ad)
 {
-    int p = blockIdx.x * blockDim.x + threadIdx.x;
+    const int lane = threadIdx.x & 31, p = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     if (p >= N) return;
-    int n = 2 * N;
-    for (int t = rp[p]; t < rp[p + 1]; t++) {
-        int q = ci[t];
-        Ad[(size_t)(2 * p) * n + 2 * q] = v[4 * (size_t)t];
-        Ad[(size_t)(2 * p) * n + 2 * q + 1] = v[4 * (size_t)t + 1];
-        Ad[(size_t)(2 * p + 1) * n + 2 * q] = v[4 * (size_t)t + 2];
-        Ad[(size_t)(2 * p + 1) * n + 2 * q + 1] = v[4 * (size_t)t + 3];
+    double2 *row = (double2 *)(Ad + (size_t)(2 * p) * (2 * N));
+    for (int t = rp[p] + lane; t < rp[p + 1]; t += 32) {
+        const int q = ci[t];
+        row[q] = ((const double2 *)v)[2 * (size_t)t];
+        row[N + q] = ((const double2 *)v)[2 * (size_t)t + 1];
     }
 }
 
@@ -1159,18 +1211,32 @@ __global__ void k_coarse_factor(int n, double *A, const double *__restrict__ z, 
 // Larger coarsest levels: the same rank-one-fixed matrix, inverted in place by
 // Gauss-Jordan elimination without pivoting (the matrix is symmetric positive
 // definite), in blocks of kGJ pivots (below).
-__global__ void k_coarse_stats(int n, const double *__restrict__ A, const double *__restrict__ z,
-                               double *__restrict__ out)
+__global__ void __launch_bounds__(1024) k_coarse_stats(int n, const double *__restrict__ A, const double *__restrict__ z,
+                                                       double *__restrict__ out)
 {
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
+    __shared__ double sm[32], sz[32];
     double smax = 0.0, zz = 0.0;
-    for (int i = 0; i < n; i++) {
-        double d = A[(size_t)i * n + i];
-        if (d > smax) smax = d;
+    for (int i = threadIdx.x; i < n; i += blockDim.x) {
+        smax = fmax(smax, A[(size_t)i * n + i]);
         zz = zz + z[i] * z[i];
     }
-    out[0] = smax;
-    out[1] = zz;
+    for (int o = 16; o; o >>= 1) {
+        smax = fmax(smax, __shfl_xor_sync(0xffffffffu, smax, o));
+        zz += __shfl_xor_sync(0xffffffffu, zz, o);
+    }
+    if ((threadIdx.x & 31) == 0) {
+        sm[threadIdx.x >> 5] = smax;
+        sz[threadIdx.x >> 5] = zz;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int w = 1; w < (int)(blockDim.x >> 5); w++) {
+            smax = fmax(smax, sm[w]);
+            zz += sz[w];
+        }
+        out[0] = smax;
+        out[1] = zz;
+    }
 }
 
 // one thread block per row, its threads strided over the columns
@@ -1375,7 +1441,7 @@ static int coarsen_level(amg_hierarchy *h, int l, bool &is_coarsest, cudaStream_
     BD_TRY(cnt.alloc((size_t)N + 1));
     BD_TRY(wt.alloc((size_t)L.A.nb));
     BD_TRY(S.rp.alloc((size_t)N + 1));
-    k_strength_count<<<nblk(N, row_block(N)), row_block(N), 0, s>>>(N, L.A.rp.p, L.A.ci.p, L.A.v.p, diag.p, o.theta,
+    k_strength_count<<<nblk(32LL * N), 256, 0, s>>>(N, L.A.rp.p, L.A.ci.p, L.A.v.p, diag.p, o.theta,
                                                                    cnt.p, wt.p); ::bd::note_launch();
     BD_LAUNCH_CHECK();
     long long snnz = 0;
@@ -1383,7 +1449,7 @@ static int coarsen_level(amg_hierarchy *h, int l, bool &is_coarsest, cudaStream_
     S.nnz = snnz;
     BD_TRY(S.ci.alloc((size_t)snnz));
     BD_TRY(S.v.alloc((size_t)snnz));
-    k_strength_fill<<<nblk(N, row_block(N)), row_block(N), 0, s>>>(N, L.A.rp.p, L.A.ci.p, wt.p, S.rp.p, S.ci.p,
+    k_strength_fill<<<nblk(32LL * N), 256, 0, s>>>(N, L.A.rp.p, L.A.ci.p, wt.p, S.rp.p, S.ci.p,
                                                                   S.v.p); ::bd::note_launch();
     BD_LAUNCH_CHECK();
     int hbad = 0;
@@ -1403,7 +1469,7 @@ static int coarsen_level(amg_hierarchy *h, int l, bool &is_coarsest, cudaStream_
         BD_TRY(S2.rp.alloc((size_t)N + 1));
         BD_TRY(S2.ci.alloc((size_t)(qn - N)));
         BD_TRY(S2.v.alloc((size_t)(qn - N)));
-        k_drop_diag<<<nblk(N + 1), 256, 0, s>>>(N, Q.rp.p, Q.ci.p, Q.v.p, S2.rp.p, S2.ci.p, S2.v.p); ::bd::note_launch();
+        k_drop_diag<<<nblk(32LL * (N + 1)), 256, 0, s>>>(N, Q.rp.p, Q.ci.p, Q.v.p, S2.rp.p, S2.ci.p, S2.v.p); ::bd::note_launch();
         BD_LAUNCH_CHECK();
         S.rp = std::move(S2.rp);
         S.ci = std::move(S2.ci);
@@ -1501,23 +1567,20 @@ static int coarsen_level(amg_hierarchy *h, int l, bool &is_coarsest, cudaStream_
     k_lanczos_init<<<nblk(n), 256, 0, s>>>(n, level_key(o.seed, l, 1), diag.p, vr.p, vz.p, vp.p); ::bd::note_launch();
     BD_LAUNCH_CHECK();
     long long *acc = h->exact_acc.p;
-    BD_TRY(exact_dot(vr.p, vz.p, n, &lst.p->rz, acc, s));
+    BD_TRY(exact_dot(vr.p, vz.p, n, &lst.p->rz[0], acc, s));
     for (int j = 0; j < o.esteig_steps; j++) {
-        k_spmv_ordered<<<nblk(N, row_block(N)), row_block(N), 0, s>>>(N, L.A.rp.p, L.A.ci.p, L.A.v.p, vp.p, vq.p);
+        k_spmv_ordered<<<nblk(n, row_block(N)), row_block(N), 0, s>>>(n, L.A.rp.p, L.A.ci.p, L.A.v.p, vp.p, vq.p);
         ::bd::note_launch();
         BD_LAUNCH_CHECK();
-        BD_TRY(exact_dot(vp.p, vq.p, n, &lst.p->pq, acc, s));
-        k_lanczos_alpha<<<1, 1, 0, s>>>(lst.p, j); ::bd::note_launch();
-        BD_LAUNCH_CHECK();
+        BD_TRY(exact_dot(vp.p, vq.p, n, &lst.p->pq[j], acc, s));
         k_lanczos_update_r<<<nblk(n), 256, 0, s>>>(n, lst.p, j, vq.p, diag.p, vr.p, vz.p); ::bd::note_launch();
         BD_LAUNCH_CHECK();
-        BD_TRY(exact_dot(vr.p, vz.p, n, &lst.p->rz1, acc, s));
-        k_lanczos_beta<<<1, 1, 0, s>>>(lst.p, j); ::bd::note_launch();
-        BD_LAUNCH_CHECK();
+        BD_TRY(exact_dot(vr.p, vz.p, n, &lst.p->rz[j + 1], acc, s));
+        if (j + 1 == o.esteig_steps) break;
         k_lanczos_update_p<<<nblk(n), 256, 0, s>>>(n, lst.p, j, vz.p, vp.p); ::bd::note_launch();
         BD_LAUNCH_CHECK();
     }
-    k_lanczos_finish<<<1, 1, 0, s>>>(lst.p); ::bd::note_launch();
+    k_lanczos_finish<<<1, 32, 0, s>>>(lst.p, o.esteig_steps); ::bd::note_launch();
     BD_LAUNCH_CHECK();
     LanczosState hst;
     BD_CUDA(cudaMemcpyAsync(&hst, lst.p, sizeof(hst), cudaMemcpyDeviceToHost, s));
@@ -1531,7 +1594,7 @@ static int coarsen_level(amg_hierarchy *h, int l, bool &is_coarsest, cudaStream_
     BD_TRY(spgemm<2>(N, Nc, L.A.rp.p, L.A.ci.p, L.A.v.p, Pt.rp.p, Pt.ci.p, Pt.v.p, L.P.rp, L.P.ci,
                      L.P.v, &pnb, s, 1.0));  // one block per row of the tentative prolongator
     L.P.nb = pnb;
-    k_smooth_p<<<nblk(N), 256, 0, s>>>(N, L.P.rp.p, L.P.ci.p, L.P.v.p, L.agg.p, ptd.p, diag.p, lst.p); ::bd::note_launch();
+    k_smooth_p<<<nblk(8LL * N), 256, 0, s>>>(N, L.P.rp.p, L.P.ci.p, L.P.v.p, L.agg.p, ptd.p, diag.p, lst.p); ::bd::note_launch();
     BD_LAUNCH_CHECK();
     // a7 R = P^T
     BD_TRY(bsr_transpose(L.P, L.R, s));
@@ -1584,7 +1647,7 @@ static int build_coarsest(amg_hierarchy *h, int l, cudaStream_t s)
     BD_TRY(h->cinv.alloc((size_t)n * n));
     BD_TRY(h->zc.alloc((size_t)n));
     BD_CUDA(cudaMemsetAsync(Ad.p, 0, Ad.bytes(), s));
-    k_coarse_dense<<<nblk(L.N), 256, 0, s>>>(L.N, L.A.rp.p, L.A.ci.p, L.A.v.p, Ad.p); ::bd::note_launch();
+    k_coarse_dense<<<nblk(32LL * L.N), 256, 0, s>>>(L.N, L.A.rp.p, L.A.ci.p, L.A.v.p, Ad.p); ::bd::note_launch();
     BD_LAUNCH_CHECK();
     k_null_vector<<<nblk(L.N), 256, 0, s>>>(L.N, L.B.p, h->zc.p); ::bd::note_launch();
     BD_LAUNCH_CHECK();
@@ -1599,7 +1662,7 @@ static int build_coarsest(amg_hierarchy *h, int l, cudaStream_t s)
     } else {
         DBuf<double> st;
         BD_TRY(st.alloc(2));
-        k_coarse_stats<<<1, 32, 0, s>>>(n, Ad.p, h->zc.p, st.p); ::bd::note_launch();
+        k_coarse_stats<<<1, 1024, 0, s>>>(n, Ad.p, h->zc.p, st.p); ::bd::note_launch();
         k_coarse_rank1<<<n, 256, 0, s>>>(n, Ad.p, h->zc.p, st.p); ::bd::note_launch();
         DBuf<double> Dinv, W, Cb;
         BD_TRY(Dinv.alloc((size_t)kGJ * kGJ));

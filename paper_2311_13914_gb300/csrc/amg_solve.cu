@@ -504,50 +504,53 @@ static int apply_pair(const Level &L, int op, G g, E e, cudaStream_t s)
 }
 
 // Pair form of P (rows: fine nodes, own entry: the node's aggregate) or of its
-// transpose R (rows: aggregates, own entries: the members).  One warp per row:
-// own entries keep their order at the front, the others theirs behind.
-__global__ void k_pair_fill(int rows, int is_r, const int *__restrict__ rp, const int *__restrict__ ci,
+// transpose R (rows: aggregates, own entries: the members).  L lanes per row: own
+// entries keep their order at the front, the others theirs behind.
+template <int L, bool IS_R>
+__global__ void k_pair_fill(int rows, const int *__restrict__ rp, const int *__restrict__ ci,
                             const double *__restrict__ bv, const int *__restrict__ agg,
                             const double *__restrict__ kappa, int *__restrict__ oci, double2 *__restrict__ ov,
                             double *__restrict__ oal, float2 *__restrict__ ov32, float *__restrict__ oal32)
 {
-    const int lane = threadIdx.x & 31, warps = (gridDim.x * blockDim.x) >> 5;
-    for (int row = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; row < rows; row += warps) {
-        const int b = rp[row], e = rp[row + 1];
-        int nown = 0;
-        for (int t0 = b; t0 < e; t0 += 32) {
-            const int t = t0 + lane;
-            const bool own = t < e && (is_r ? agg[ci[t]] == row : ci[t] == agg[row]);
-            nown += __popc(__ballot_sync(0xffffffffu, own));
-        }
-        int po = b, pn = b + nown;  // next own and next other position
-        for (int t0 = b; t0 < e; t0 += 32) {
-            const int t = t0 + lane;
-            const bool in = t < e;
-            const int q = in ? ci[t] : 0;
-            const bool own = in && (is_r ? agg[q] == row : q == agg[row]);
-            const unsigned mo = __ballot_sync(0xffffffffu, own), mi = __ballot_sync(0xffffffffu, in);
-            const unsigned below = (1u << lane) - 1u;
-            if (in) {
-                const int pos = own ? po + __popc(mo & below) : pn + __popc(mi & ~mo & below);
-                const int node = is_r ? q : row;
-                const double kv = kappa[2 * node], ku = kappa[2 * node + 1];
-                const double *a = bv + 4 * (size_t)t;
-                // P's block [a00 a01; a10 a11]; R holds its transpose
-                const double a01 = is_r ? a[2] : a[1];
-                const double ki = a01 / kv, ke = a[3] / ku - ki, al = own ? (a[0] - a01) / kv : 0.0;
-                oci[pos] = own ? (q | ~kColMask) : q;
-                if (ov) {
-                    ov[pos] = make_double2(ki, ke);
-                    oal[pos] = al;
-                } else {
-                    ov32[pos] = make_float2((float)ki, (float)ke);
-                    oal32[pos] = (float)al;
-                }
+    const int lane = threadIdx.x & 31, l = lane & (L - 1);
+    const unsigned group = (L == 32 ? 0xffffffffu : ((1u << (L & 31)) - 1u) << (lane & ~(L - 1)));
+    const unsigned before = group & ((1u << lane) - 1u);
+    const int row = (blockIdx.x * blockDim.x + threadIdx.x) / L;
+    const bool act = row < rows;
+    const int b = act ? rp[row] : 0, e = act ? rp[row + 1] : 0;
+    int len = e - b, nown = 0;
+    for (int o = 16; o; o >>= 1) len = max(len, __shfl_xor_sync(0xffffffffu, len, o));  // of the warp's rows
+    for (int i = l; i < ((len + L - 1) / L) * L; i += L) {
+        const int t = b + i;
+        const bool own = t < e && (IS_R ? agg[ci[t]] == row : ci[t] == agg[row]);
+        nown += __popc(__ballot_sync(0xffffffffu, own) & group);
+    }
+    int po = b, pn = b + nown;  // next own and next other position
+    for (int i = l; i < ((len + L - 1) / L) * L; i += L) {
+        const int t = b + i;
+        const bool in = t < e;
+        const int q = in ? ci[t] : 0;
+        const bool own = in && (IS_R ? agg[q] == row : q == agg[row]);
+        const unsigned mo = __ballot_sync(0xffffffffu, own), mn = __ballot_sync(0xffffffffu, in && !own);
+        if (in) {
+            const int pos = own ? po + __popc(mo & before) : pn + __popc(mn & before);
+            const int node = IS_R ? q : row;
+            const double kv = kappa[2 * node], ku = kappa[2 * node + 1];
+            const double *a = bv + 4 * (size_t)t;
+            // P's block [a00 a01; a10 a11]; R holds its transpose
+            const double a01 = IS_R ? a[2] : a[1];
+            const double ki = a01 / kv, ke = a[3] / ku - ki, al = own ? (a[0] - a01) / kv : 0.0;
+            oci[pos] = own ? (q | ~kColMask) : q;
+            if (ov) {
+                ov[pos] = make_double2(ki, ke);
+                oal[pos] = al;
+            } else {
+                ov32[pos] = make_float2((float)ki, (float)ke);
+                oal32[pos] = (float)al;
             }
-            po += __popc(mo);
-            pn += __popc(mi & ~mo);
         }
+        po += __popc(mo & group);
+        pn += __popc(mn & group);
     }
 }
 
@@ -580,9 +583,14 @@ static int build_pairs(Level &L, bool fp32, cudaStream_t s)
             BD_TRY(o.v.alloc(2 * (size_t)M.nb));
             BD_TRY(o.alpha.alloc((size_t)M.nb));
         }
-        k_pair_fill<<<grid_for(32LL * M.nbr, 256), 256, 0, s>>>(M.nbr, op == 1, M.rp.p, M.ci.p, M.v.p, L.agg.p,
-                                                                L.kappa.p, o.ci.p, (double2 *)o.v.p, o.alpha.p,
-                                                                (float2 *)o.v32.p, o.alpha32.p);
+        if (op == 1)
+            k_pair_fill<32, true><<<(int)((32LL * M.nbr + 255) / 256), 256, 0, s>>>(
+                M.nbr, M.rp.p, M.ci.p, M.v.p, L.agg.p, L.kappa.p, o.ci.p, (double2 *)o.v.p, o.alpha.p,
+                (float2 *)o.v32.p, o.alpha32.p);
+        else
+            k_pair_fill<8, false><<<(int)((8LL * M.nbr + 255) / 256), 256, 0, s>>>(
+                M.nbr, M.rp.p, M.ci.p, M.v.p, L.agg.p, L.kappa.p, o.ci.p, (double2 *)o.v.p, o.alpha.p,
+                (float2 *)o.v32.p, o.alpha32.p);
         ::bd::note_launch();
         o.valid = true;
     }
@@ -626,98 +634,20 @@ static int lanes_rule(const BSR &A, bool fp32, bool sliced_ok, const PairOp *pr 
 }
 
 // ------------------------------------------------------------------ finest level, layered stencil
-__device__ __forceinline__ int fine_rep(int t, int n) { return t == 0 ? 0 : (t == 2 ? n - 1 : 1); }
-
-// Raw row of every (plane, row type), read from a node of that kind.  Types a
-// thin slab does not have (no interior with two nodes across) hold zeros.
-__global__ void k_fine_raw(int NX, int NY, int NZ, const int *__restrict__ rp, const double *__restrict__ Ki,
-                           const double *__restrict__ Ke, const double *__restrict__ M, double c,
-                           const double *__restrict__ invd, double *__restrict__ raw)
-{
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= 9 * NZ) return;
-    const int l = t / 9, ti = t % 3, tj = (t % 9) / 3;
-    double *o = raw + (size_t)t * kFineRaw;
-    for (int k = 0; k < kFineRaw; k++) o[k] = 0.0;
-    if ((ti == 1 && NX < 3) || (tj == 1 && NY < 3)) return;
-    const int p = fine_rep(ti, NX) + NX * (fine_rep(tj, NY) + NY * l);
-    int b = rp[p];
-    for (int dz = -1; dz <= 1; dz++)
-        for (int dy = -1; dy <= 1; dy++)
-            for (int dx = -1; dx <= 1; dx++) {
-                if ((dx < 0 && ti == 0) || (dx > 0 && ti == 2) || (dy < 0 && tj == 0) || (dy > 0 && tj == 2) ||
-                    l + dz < 0 || l + dz >= NZ)
-                    continue;
-                const int k = 9 * (dz + 1) + 3 * (dy + 1) + dx + 1;
-                o[2 * k] = Ki[b];
-                o[2 * k + 1] = Ke[b];
-                b++;
-            }
-    o[54] = c * M[p];
-    if (invd) {
-        o[55] = invd[2 * p];
-        o[56] = invd[2 * p + 1];
-    }
-}
-
-// bad[0]: a node whose row is not its type's (the assembled system was
-// corrupted); bad[1]: a row that is not symmetric under (dx, dy) -> (-dx, -dy)
-// beyond the rounding of its sums.
-__global__ void k_fine_check(int NX, int NY, int NZ, const int *__restrict__ rp, const int *__restrict__ ci,
-                             const double *__restrict__ Ki, const double *__restrict__ Ke,
-                             const double *__restrict__ raw, int *__restrict__ bad)
-{
-    const int N = NX * NY * NZ;
-    for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < N; p += gridDim.x * blockDim.x) {
-        const int i = p % NX, j = (p / NX) % NY, l = p / (NX * NY);
-        const int ti = i == 0 ? 0 : (i == NX - 1 ? 2 : 1), tj = j == 0 ? 0 : (j == NY - 1 ? 2 : 1);
-        const double *o = raw + (size_t)(9 * l + 3 * tj + ti) * kFineRaw;
-        int b = rp[p];
-        bool same = true, sym = true;
-        const double tol0 = 16.0 * 0x1p-52 * fabs(o[26]), tol1 = 16.0 * 0x1p-52 * fabs(o[27]);
-        for (int k = 0; k < 27; k++) {
-            const int dx = k % 3 - 1, dy = (k / 3) % 3 - 1, dz = k / 9 - 1;
-            if (i + dx < 0 || i + dx >= NX || j + dy < 0 || j + dy >= NY || l + dz < 0 || l + dz >= NZ) continue;
-            if (b < rp[p + 1])
-                same = same && ci[b] == p + dx + NX * (dy + NY * dz) && Ki[b] == o[2 * k] && Ke[b] == o[2 * k + 1];
-            b++;
-            if (i - dx < 0 || i - dx >= NX || j - dy < 0 || j - dy >= NY) continue;
-            const int m = 9 * (dz + 1) + 3 * (1 - dy) + 1 - dx;
-            sym = sym && fabs(o[2 * k] - o[2 * m]) <= tol0 && fabs(o[2 * k + 1] - o[2 * m + 1]) <= tol1;
-        }
-        if (!same || b != rp[p + 1]) atomicOr(bad, 1);
-        if (!sym) atomicOr(bad + 1, 1);
-    }
-}
-
-int fine_raw_build(FineStencil &F, const bd_system *sys, const double *invd, cudaStream_t s)
+int fine_raw_copy(FineStencil &F, const bd_system *sys, cudaStream_t s)
 {
     F.NX = sys->mesh.nx + 1;
     F.NY = sys->mesh.ny + 1;
     F.NZ = sys->mesh.nz + 1;
+    F.sym = sys->sym;
     BD_TRY(F.raw.alloc((size_t)9 * F.NZ * kFineRaw));
-    DBuf<int> bad;
-    BD_TRY(bad.alloc(2));
-    BD_CUDA(cudaMemsetAsync(bad.p, 0, 2 * sizeof(int), s));
-    const bd_params &P = sys->params;
-    k_fine_raw<<<(9 * F.NZ + 63) / 64, 64, 0, s>>>(F.NX, F.NY, F.NZ, sys->A.rp.p, sys->Ki.p, sys->Ke.p, sys->M.p,
-                                                   (P.chi * P.cm) / P.dt, invd, F.raw.p);
-    ::bd::note_launch();
-    k_fine_check<<<grid_for(sys->N, 256), 256, 0, s>>>(F.NX, F.NY, F.NZ, sys->A.rp.p, sys->A.ci.p, sys->Ki.p,
-                                                       sys->Ke.p, F.raw.p, bad.p);
-    ::bd::note_launch();
-    BD_LAUNCH_CHECK();
-    int hbad[2] = {0, 0};
-    BD_CUDA(cudaMemcpyAsync(hbad, bad.p, sizeof(hbad), cudaMemcpyDeviceToHost, s));
-    BD_CUDA(cudaStreamSynchronize(s));
-    if (hbad[0]) return BD_EINVAL;
-    F.sym = !hbad[1];
+    BD_CUDA(cudaMemcpyAsync(F.raw.p, sys->raw.p, F.raw.bytes(), cudaMemcpyDeviceToDevice, s));
     return BD_OK;
 }
 
 int build_fine_stencil(amg_hierarchy *h, const bd_system *sys, cudaStream_t s)
 {
-    BD_TRY(fine_raw_build(h->fine, sys, h->lev[0].invdiag.p, s));
+    BD_TRY(fine_raw_copy(h->fine, sys, s));
     h->fine.valid = true;
     return BD_OK;
 }
@@ -746,9 +676,12 @@ __global__ void k_fine_pack(int rows, const double *__restrict__ raw, double c2,
         }
         put(z * Row::G + Row::NP, z == 0 ? o[54] : 0.0, 0.0);
     }
-    put(Row::IDC2, c2 * o[55], c2 * o[56]);
-    put(Row::IDT, o[55] * it, o[56] * it);
-    put(Row::KAPPA, -omega * o[55], -omega * o[56]);
+    // the inverse diagonal, as k_invdiag forms it from the assembled blocks
+    const bool exists = o[55] > 0.0;
+    const double dv = exists ? 1.0 / (o[54] + o[26]) : 0.0, du = exists ? 1.0 / (o[26] + o[27]) : 0.0;
+    put(Row::IDC2, c2 * dv, c2 * du);
+    put(Row::IDT, dv * it, du * it);
+    put(Row::KAPPA, -omega * dv, -omega * du);
     put(Row::KAPPA + 1, 0.0, 0.0);
 }
 

@@ -90,64 +90,98 @@ __global__ void k_row_counts(int nx, int ny, int nz, int *cnt)
     cnt[p] = cx * cy * cz;
 }
 
-// One thread per node row: every neighbour q in ascending node index, the
-// element contributions of the elements shared by p and q in ascending
-// element index.
-__global__ void k_assemble_rows(int nx, int ny, int nz, double lx, double ly, double lz,
-                                double chi, double cm, double dt, const double *__restrict__ Kel,
-                                const int *__restrict__ rp, int *__restrict__ ci,
-                                double *__restrict__ v, double *__restrict__ Ki_out,
-                                double *__restrict__ Ke_out, double *__restrict__ M)
+__device__ __forceinline__ int rep_node(int t, int n) { return t == 0 ? 0 : (t == 2 ? n - 1 : 1); }
+
+// Rows of Ki, Ke and M depend only on the node's plane and on whether it lies
+// on an x or y face (the element matrices vary with the layer alone): one raw row
+// of kFineRaw doubles per plane and row type 3 (y face) + (x face) -- 0 low, 1
+// interior, 2 high -- from a node of that kind: (Ki, Ke) at the 27 stencil
+// positions 9 (dz + 1) + 3 (dy + 1) + dx + 1, c M, M.  One thread per entry: the
+// element contributions of the elements shared by p and q in ascending element
+// index.  Row types a thin slab does not have keep zeros.
+__global__ void k_stencil_rows(int nx, int ny, int nz, double lx, double ly, double lz, double chi, double cm, double dt,
+                               const double *__restrict__ Kel, double *__restrict__ raw)
 {
-    int NX = nx + 1, NY = ny + 1, NZ = nz + 1;
-    long long N = (long long)NX * NY * NZ;
-    long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    if (p >= N) return;
-    int pi = (int)(p % NX), pj = (int)((p / NX) % NY), pl = (int)(p / ((long long)NX * NY));
+    const int id = blockIdx.x * blockDim.x + threadIdx.x, row = id / 27, k = id % 27;
+    const int NX = nx + 1, NY = ny + 1, NZ = nz + 1;
+    if (row >= 9 * NZ) return;
+    const int pl = row / 9, ti = row % 3, tj = (row % 9) / 3;
+    double *o = raw + (size_t)row * kFineRaw;
+    const bool exists = (ti != 1 || NX > 2) && (tj != 1 || NY > 2);
+    const int pi = rep_node(ti, NX), pj = rep_node(tj, NY);
+    const int qi = pi + k % 3 - 1, qj = pj + (k / 3) % 3 - 1, ql = pl + k / 9 - 1;
+    double ki = 0.0, ke = 0.0;
+    if (exists && qi >= 0 && qi < NX && qj >= 0 && qj < NY && ql >= 0 && ql < NZ) {
+        const int exlo = max((pi > qi ? pi : qi) - 1, 0), exhi = min(pi < qi ? pi : qi, nx - 1);
+        const int eylo = max((pj > qj ? pj : qj) - 1, 0), eyhi = min(pj < qj ? pj : qj, ny - 1);
+        const int ezlo = max((pl > ql ? pl : ql) - 1, 0), ezhi = min(pl < ql ? pl : ql, nz - 1);
+        for (int ez = ezlo; ez <= ezhi; ez++)
+            for (int ey = eylo; ey <= eyhi; ey++)
+                for (int ex = exlo; ex <= exhi; ex++) {
+                    int a = (pi - ex) + 2 * (pj - ey) + 4 * (pl - ez);
+                    int b = (qi - ex) + 2 * (qj - ey) + 4 * (ql - ez);
+                    ki = ki + Kel[((size_t)ez * 2 + 0) * 64 + a * 8 + b];
+                    ke = ke + Kel[((size_t)ez * 2 + 1) * 64 + a * 8 + b];
+                }
+    }
+    o[2 * k] = ki;
+    o[2 * k + 1] = ke;
+    if (k > 0) return;
     double hx = lx / nx, hy = ly / ny, hz = lz / nz;
     double vol8 = ((hx * hy) * hz) * 0.125;
     // lumped mass: |e|/8 from every element around p, ascending element index
     double Mp = 0.0;
-    for (int ez = clampi(pl - 1, 0, nz - 1); ez <= clampi(pl, 0, nz - 1); ez++)
-        for (int ey = clampi(pj - 1, 0, ny - 1); ey <= clampi(pj, 0, ny - 1); ey++)
-            for (int ex = clampi(pi - 1, 0, nx - 1); ex <= clampi(pi, 0, nx - 1); ex++) Mp = Mp + vol8;
-    M[p] = Mp;
+    if (exists)
+        for (int ez = clampi(pl - 1, 0, nz - 1); ez <= clampi(pl, 0, nz - 1); ez++)
+            for (int ey = clampi(pj - 1, 0, ny - 1); ey <= clampi(pj, 0, ny - 1); ey++)
+                for (int ex = clampi(pi - 1, 0, nx - 1); ex <= clampi(pi, 0, nx - 1); ex++) Mp = Mp + vol8;
     double c = (chi * cm) / dt;
-    int pos = rp[p];
-    for (int dz = -1; dz <= 1; dz++)
-        for (int dy = -1; dy <= 1; dy++)
-            for (int dx = -1; dx <= 1; dx++) {
-                int qi = pi + dx, qj = pj + dy, ql = pl + dz;
-                if (qi < 0 || qi >= NX || qj < 0 || qj >= NY || ql < 0 || ql >= NZ) continue;
-                double ki = 0.0, ke = 0.0;
-                int exlo = (pi > qi ? pi : qi) - 1, exhi = (pi < qi ? pi : qi);
-                int eylo = (pj > qj ? pj : qj) - 1, eyhi = (pj < qj ? pj : qj);
-                int ezlo = (pl > ql ? pl : ql) - 1, ezhi = (pl < ql ? pl : ql);
-                exlo = exlo < 0 ? 0 : exlo;
-                eylo = eylo < 0 ? 0 : eylo;
-                ezlo = ezlo < 0 ? 0 : ezlo;
-                exhi = exhi > nx - 1 ? nx - 1 : exhi;
-                eyhi = eyhi > ny - 1 ? ny - 1 : eyhi;
-                ezhi = ezhi > nz - 1 ? nz - 1 : ezhi;
-                for (int ez = ezlo; ez <= ezhi; ez++)
-                    for (int ey = eylo; ey <= eyhi; ey++)
-                        for (int ex = exlo; ex <= exhi; ex++) {
-                            int a = (pi - ex) + 2 * (pj - ey) + 4 * (pl - ez);
-                            int b = (qi - ex) + 2 * (qj - ey) + 4 * (ql - ez);
-                            ki = ki + Kel[((size_t)ez * 2 + 0) * 64 + a * 8 + b];
-                            ke = ke + Kel[((size_t)ez * 2 + 1) * 64 + a * 8 + b];
-                        }
-                long long q = qi + (long long)NX * (qj + (long long)NY * ql);
-                double vv = (q == p) ? c * Mp + ki : ki;
-                ci[pos] = (int)q;
-                v[4 * (size_t)pos + 0] = vv;
-                v[4 * (size_t)pos + 1] = ki;
-                v[4 * (size_t)pos + 2] = ki;
-                v[4 * (size_t)pos + 3] = ki + ke;
-                Ki_out[pos] = ki;
-                Ke_out[pos] = ke;
-                pos++;
-            }
+    o[54] = c * Mp;
+    o[55] = Mp;
+}
+
+// *asym is set by a row that is not symmetric under (dx, dy) -> (-dx, -dy) beyond
+// the rounding of its sums (fibres with a z component).
+__global__ void k_stencil_sym(int NZ, const double *__restrict__ raw, int *__restrict__ asym)
+{
+    const int id = blockIdx.x * blockDim.x + threadIdx.x, row = id / 27, k = id % 27;
+    if (row >= 9 * NZ) return;
+    const int ti = row % 3, tj = (row % 9) / 3, dx = k % 3 - 1, dy = (k / 3) % 3 - 1;
+    if ((dx && ti != 1) || (dy && tj != 1)) return;  // only one of the pair exists
+    const double *o = raw + (size_t)row * kFineRaw;
+    const int m = 9 * (k / 9) + 3 * (1 - dy) + 1 - dx;
+    const double eps = 16.0 * 0x1p-52;
+    if (!(fabs(o[2 * k] - o[2 * m]) <= eps * fabs(o[26])) || !(fabs(o[2 * k + 1] - o[2 * m + 1]) <= eps * fabs(o[27])))
+        *asym = 1;
+}
+
+// A warp per node: lane k writes the row's entry at stencil position k (every
+// row's entries in ascending node index), bound by the 52 bytes per entry it
+// writes (128x128x32: 750 MB; one thread per row, summing its elements and
+// writing with a stride of 1.4 KB, took 1094 us, now 150).
+__global__ void __launch_bounds__(256) k_expand_rows(int NX, int NY, int NZ, const double *__restrict__ raw,
+                                                     const int *__restrict__ rp, int *__restrict__ ci,
+                                                     double *__restrict__ v, double *__restrict__ Ki,
+                                                     double *__restrict__ Ke, double *__restrict__ M)
+{
+    const int lane = threadIdx.x & 31, p = (int)((blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5);
+    if (p >= NX * NY * NZ) return;
+    const int i = p % NX, j = (p / NX) % NY, l = p / (NX * NY);
+    const int dx = lane % 3 - 1, dy = (lane / 3) % 3 - 1, dz = lane / 9 - 1;
+    const bool in = lane < 27 && i + dx >= 0 && i + dx < NX && j + dy >= 0 && j + dy < NY && l + dz >= 0 && l + dz < NZ;
+    const unsigned m = __ballot_sync(0xffffffffu, in);
+    const int type = 3 * (j == 0 ? 0 : (j == NY - 1 ? 2 : 1)) + (i == 0 ? 0 : (i == NX - 1 ? 2 : 1));
+    const double *o = raw + ((size_t)9 * l + type) * kFineRaw;
+    if (in) {
+        const size_t t = (size_t)rp[p] + __popc(m & ((1u << lane) - 1u));
+        const double2 k = ((const double2 *)o)[lane];
+        ci[t] = p + dx + NX * (dy + NY * dz);
+        ((double2 *)v)[2 * t] = make_double2(lane == 13 ? o[54] + k.x : k.x, k.x);
+        ((double2 *)v)[2 * t + 1] = make_double2(k.x, k.x + k.y);
+        Ki[t] = k.x;
+        Ke[t] = k.y;
+    }
+    if (lane == 27) M[p] = o[55];
 }
 
 }  // namespace bd
@@ -202,11 +236,22 @@ extern "C" int bd_assemble(const bd_mesh *mesh, const bd_params *params, const d
         (st = sys->Ki.alloc((size_t)tot)) || (st = sys->Ke.alloc((size_t)tot)) ||
         (st = sys->M.alloc((size_t)N)))
         return fail(st);
-    k_assemble_rows<<<grid, 256, 0, s>>>(mesh->nx, mesh->ny, mesh->nz, mesh->lx, mesh->ly, mesh->lz,
-                                         params->chi, params->cm, params->dt, Kel.p, A.rp.p, A.ci.p,
-                                         A.v.p, sys->Ki.p, sys->Ke.p, sys->M.p); ::bd::note_launch();
+    const int rows = 9 * (mesh->nz + 1);
+    DBuf<int> asym;
+    if ((st = sys->raw.alloc((size_t)rows * kFineRaw)) || (st = asym.alloc(1))) return fail(st);
+    if (cudaMemsetAsync(asym.p, 0, sizeof(int), s) != cudaSuccess) return fail(BD_ECUDA);
+    k_stencil_rows<<<(rows * 27 + 63) / 64, 64, 0, s>>>(mesh->nx, mesh->ny, mesh->nz, mesh->lx, mesh->ly, mesh->lz,
+                                                       params->chi, params->cm, params->dt, Kel.p, sys->raw.p);
+    ::bd::note_launch();
+    k_stencil_sym<<<(rows * 27 + 255) / 256, 256, 0, s>>>(mesh->nz + 1, sys->raw.p, asym.p); ::bd::note_launch();
+    k_expand_rows<<<(int)((N + 7) / 8), 256, 0, s>>>((int)NX, (int)NY, (int)NZ, sys->raw.p, A.rp.p, A.ci.p, A.v.p,
+                                                    sys->Ki.p, sys->Ke.p, sys->M.p); ::bd::note_launch();
     if (cudaGetLastError() != cudaSuccess) return fail(BD_ECUDA);
-    if (cudaStreamSynchronize(s) != cudaSuccess) return fail(BD_ECUDA);
+    int hasym = 0;
+    if (cudaMemcpyAsync(&hasym, asym.p, sizeof(int), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
+        cudaStreamSynchronize(s) != cudaSuccess)
+        return fail(BD_ECUDA);
+    sys->sym = !hasym;
     *out = sys;
     return BD_OK;
 }

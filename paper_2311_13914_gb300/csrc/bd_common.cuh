@@ -97,6 +97,9 @@ struct CSR {
     DBuf<double> v;
 };
 
+// Doubles of a raw stencil row (bd_assemble.cu): 27 (Ki, Ke) pairs, c M, M.
+constexpr int kFineRaw = 56;
+
 // ------------------------------------------------------------------ utilities
 constexpr int kSM = 152;  // GB300 streaming multiprocessors (grid sizing)
 
@@ -153,4 +156,6 @@ struct bd_system {
     bd::DBuf<double> M;     // lumped mass (N)
     bd::DBuf<double> Ki;    // node-pattern stiffness values (shared pattern with A)
     bd::DBuf<double> Ke;
+    bd::DBuf<double> raw;   // rows per plane and row type: (nz + 1) x 9 x kFineRaw
+    bool sym = false;       // every row symmetric under (dx, dy) -> (-dx, -dy)
 };

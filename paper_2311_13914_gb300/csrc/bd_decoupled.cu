@@ -357,7 +357,7 @@ extern "C" int bd_dsim_create(const bd_system *sys, amg_hierarchy *h_elliptic, c
         delete S;
         return BD_ECUDA;
     }
-    if ((st = fine_raw_build(S->raw, sys, nullptr, s)) ||
+    if ((st = fine_raw_copy(S->raw, sys, s)) ||
         (st = sc_pack(S->raw, 1.0, 0.0, 0.0, 0.0, 0.0, 0.0, false, S->ki, s)) ||
         (st = sc_pack(S->raw, 1.0, 0.0, 1.0, 0.0, 0.0, 0.0, false, S->par, s))) {
         delete S;

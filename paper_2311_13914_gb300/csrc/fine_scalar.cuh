@@ -202,7 +202,7 @@ template <class S, class F> static int sc_apply(const ScOp &A, const S *x, F mak
 }
 
 // The table of a Ki + b Ke + m (c M) from the raw rows, with the Chebyshev
-// scalings of D^{-1} given per row in raw (the u_e field's).
+// scalings of the inverse diagonal of Ai + Ae.
 int sc_pack(const FineStencil &F, double a, double b, double m, double c1, double c2, double inv_theta, bool fp32,
             ScOp &op, cudaStream_t s);
 
