@@ -1137,17 +1137,17 @@ static int bsr_transpose(const BSR &a, BSR &t, cudaStream_t s)
 }
 
 // ------------------------------------------------------------------ a9 coarsest level
-// a warp per block row
+// a warp per block row; ld: row stride of Ad
 __global__ void k_coarse_dense(int N, const int *__restrict__ rp, const int *__restrict__ ci,
-                               const double *__restrict__ v, double *__restrict__ Ad)
+                               const double *__restrict__ v, int ld, double *__restrict__ Ad)
 {
     const int lane = threadIdx.x & 31, p = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     if (p >= N) return;
-    double2 *row = (double2 *)(Ad + (size_t)(2 * p) * (2 * N));
+    double2 *r0 = (double2 *)(Ad + (size_t)(2 * p) * ld), *r1 = (double2 *)(Ad + (size_t)(2 * p + 1) * ld);
     for (int t = rp[p] + lane; t < rp[p + 1]; t += 32) {
         const int q = ci[t];
-        row[q] = ((const double2 *)v)[2 * (size_t)t];
-        row[N + q] = ((const double2 *)v)[2 * (size_t)t + 1];
+        r0[q] = ((const double2 *)v)[2 * (size_t)t];
+        r1[q] = ((const double2 *)v)[2 * (size_t)t + 1];
     }
 }
 
@@ -1209,15 +1209,19 @@ __global__ void k_coarse_factor(int n, double *A, const double *__restrict__ z, 
 }
 
 // Larger coarsest levels: the same rank-one-fixed matrix, inverted in place by
-// Gauss-Jordan elimination without pivoting (the matrix is symmetric positive
-// definite), in blocks of kGJ pivots (below).
-__global__ void __launch_bounds__(1024) k_coarse_stats(int n, const double *__restrict__ A, const double *__restrict__ z,
-                                                       double *__restrict__ out)
+// symmetric block elimination without pivoting (the matrix is symmetric positive
+// definite), kGJ pivots at a time on a copy padded to whole blocks.  With M = A at
+// first, the step of pivot block P is D = M[P,P]^-1, W = M[:,P] D and
+//     M[i,j] -= W[i,:] M[j,P]^T,   M[i,P] = W[i,:],   M[P,P] = -D,
+// which keeps M symmetric and ends with M = -A^-1, so only the block-lower half
+// is formed: half the FP64 work of Gauss-Jordan, which bounds the update.
+__global__ void __launch_bounds__(1024) k_coarse_stats(int n, int ld, const double *__restrict__ A,
+                                                       const double *__restrict__ z, double *__restrict__ out)
 {
     __shared__ double sm[32], sz[32];
     double smax = 0.0, zz = 0.0;
     for (int i = threadIdx.x; i < n; i += blockDim.x) {
-        smax = fmax(smax, A[(size_t)i * n + i]);
+        smax = fmax(smax, A[(size_t)i * ld + i]);
         zz = zz + z[i] * z[i];
     }
     for (int o = 16; o; o >>= 1) {
@@ -1239,134 +1243,180 @@ __global__ void __launch_bounds__(1024) k_coarse_stats(int n, const double *__re
     }
 }
 
-// one thread block per row, its threads strided over the columns
-__global__ void k_coarse_rank1(int n, double *__restrict__ A, const double *__restrict__ z,
+// one thread block per row; rows past n (the padding) get a unit diagonal
+__global__ void k_coarse_rank1(int n, int ld, double *__restrict__ A, const double *__restrict__ z,
                                const double *__restrict__ st)
 {
     const double smax = st[0], zz = st[1];
     const int i = blockIdx.x;
+    if (i >= n) {
+        if (threadIdx.x == 0) A[(size_t)i * ld + i] = 1.0;
+        return;
+    }
     for (int j = threadIdx.x; j < n; j += blockDim.x) {
-        const size_t e = (size_t)i * n + j;
+        const size_t e = (size_t)i * ld + j;
         A[e] = A[e] + (smax * z[i]) * z[j] / zz;
     }
 }
 
-// Blocked Gauss-Jordan with pivot blocks of kGJ: for the pivot rows P,
-// D = A[P,P] is inverted in shared memory, W = D^-1 A[P,:], and every other row
-// i takes A[i,j] -= A[i,P] W[:,j] (a rank-kGJ update, FP64-bound, 32 rows per
-// thread block so each W value is reused 32 times), A[i,P] = -A[i,P] D^-1,
-// while the pivot rows become W with D^-1 in the pivot columns.
-constexpr int kGJ = 32;
+constexpr int kGJ = 32;        // pivots per step, and the tile of the update
+constexpr int kGJThreads = 64;
 
-__global__ void k_gj_pivot(int n, int K, int bb, const double *__restrict__ A, double *__restrict__ Dinv,
-                           int *__restrict__ bad)
+// Inverse of the kGJ x kGJ block in S (row stride kGJ + 1) by kGJThreads threads:
+// thread t holds half a row in registers; a step costs one barrier (the pivot
+// row's owners scale it and publish it) and 16 multiply-adds per thread.
+__device__ void gj_invert(const double (*S)[kGJ + 1], double *__restrict__ Dinv, int *__restrict__ bad)
 {
-    __shared__ double D[kGJ][kGJ + 1];
-    __shared__ double prow[kGJ], pcol[kGJ];
-    __shared__ double srp;
-    for (int e = threadIdx.x; e < bb * bb; e += blockDim.x) D[e / bb][e % bb] = A[(size_t)(K + e / bb) * n + K + e % bb];
-    __syncthreads();
-    for (int k = 0; k < bb; k++) {
-        // one division per pivot, by one thread: the pivot row is scaled by its
-        // reciprocal (FP64 division is a long sequence on the FP64 pipe, and one
-        // thread block does all of this)
-        if (threadIdx.x == 0) {
-            const double piv = D[k][k];
-            srp = 1.0 / piv;
-            if (!(piv > 0.0)) *bad = 1;
-        }
-        __syncthreads();
-        const double rpiv = srp;
-        if (threadIdx.x < bb) {
-            prow[threadIdx.x] = D[k][threadIdx.x] * rpiv;
-            pcol[threadIdx.x] = D[threadIdx.x][k];
-        }
-        __syncthreads();
-        for (int e = threadIdx.x; e < bb * bb; e += blockDim.x) {
-            const int i = e / bb, j = e % bb;
-            double a;
-            if (i == k && j == k) a = rpiv;
-            else if (i == k) a = prow[j];
-            else if (j == k) a = -pcol[i] * rpiv;
-            else a = D[i][j] - pcol[i] * prow[j];
-            D[i][j] = a;
-        }
-        __syncthreads();
-    }
-    for (int e = threadIdx.x; e < bb * bb; e += blockDim.x) Dinv[e] = D[e / bb][e % bb];
-}
-
-// W[k][j] = sum_m Dinv[k][m] A[K+m][j] for every column j (bb x n), and a copy
-// Cb of the pivot columns A[:, P] (the update overwrites them).  blockIdx.y
-// takes kGJ / kGJPanelK rows k of W, so the panel spreads over the GPU.
-constexpr int kGJPanelK = 4;
-__global__ void k_gj_panel(int n, int K, int bb, const double *__restrict__ A, const double *__restrict__ Dinv,
-                           double *__restrict__ W, double *__restrict__ Cb)
-{
-    __shared__ double Di[kGJPanelK][kGJ];
-    const int k0 = blockIdx.y * kGJPanelK;
-    for (int e = threadIdx.x; e < kGJPanelK * kGJ; e += blockDim.x) {
-        const int k = k0 + e / kGJ, m = e % kGJ;
-        Di[e / kGJ][m] = k < bb && m < bb ? Dinv[k * bb + m] : 0.0;
-    }
-    __syncthreads();
-    const int j = blockIdx.x * blockDim.x + threadIdx.x;
-    if (j >= n || k0 >= bb) return;
-    if (blockIdx.y == 0)
-        for (int m = 0; m < kGJ; m++) Cb[(size_t)j * kGJ + m] = m < bb ? A[(size_t)j * n + K + m] : 0.0;
-    double col[kGJ];
+    __shared__ double prow[2][kGJ + 1];  // scaled pivot row, its reciprocal pivot
+    const int i = threadIdx.x >> 1, half = threadIdx.x & 1;
+    double a[kGJ / 2];
 #pragma unroll
-    for (int m = 0; m < kGJ; m++) col[m] = m < bb ? A[(size_t)(K + m) * n + j] : 0.0;
+    for (int c = 0; c < kGJ / 2; c++) a[c] = S[i][half * (kGJ / 2) + c];
 #pragma unroll
-    for (int kk = 0; kk < kGJPanelK; kk++) {
-        const int k = k0 + kk;
-        if (k >= bb) break;
-        double w = 0.0;
+    for (int k = 0; k < kGJ; k++) {
+        constexpr int H = kGJ / 2;
+        const int hk = k / H, ck = k % H;
+        double *pr = prow[k & 1];
+        // the row's entry in the pivot column, from the thread that holds it
+        const double f = __shfl_sync(0xffffffffu, a[ck], (threadIdx.x & 30) | hk);
+        if (i == k) {
+            if (!(f > 0.0)) *bad = 1;
+            const double rp = 1.0 / f;
 #pragma unroll
-        for (int m = 0; m < kGJ; m++) w = fma(Di[kk][m], col[m], w);
-        W[(size_t)k * n + j] = w;
-    }
-}
-
-// Column chunk blockIdx.x * blockDim.x + threadIdx.x, rows [r0, r1): an equal
-// share of the n rows for each of the gridDim.y blocks of a column chunk (the
-// grid is one resident wave), taken kGJ rows at a time through shared memory.
-__global__ void k_gj_update(int n, int K, int bb, double *__restrict__ A, const double *__restrict__ Dinv,
-                            const double *__restrict__ W, const double *__restrict__ Cb)
-{
-    __shared__ double C[kGJ][kGJ];  // A[i, P] of kGJ rows, from the copy
-    const int r0 = (int)((long long)n * blockIdx.y / gridDim.y);
-    const int r1 = (int)((long long)n * (blockIdx.y + 1) / gridDim.y);
-    const int j = blockIdx.x * blockDim.x + threadIdx.x;
-    const bool act = j < n;
-    const bool jp = j >= K && j < K + bb;
-    double w[kGJ];
-#pragma unroll
-    for (int m = 0; m < kGJ; m++)
-        w[m] = act && m < bb ? (jp ? Dinv[m * bb + (j - K)] : W[(size_t)m * n + j]) : 0.0;
-    for (int rb = r0; rb < r1; rb += kGJ) {
-        const int nr = min(kGJ, r1 - rb);
-        __syncthreads();
-        for (int e = threadIdx.x; e < kGJ * kGJ; e += blockDim.x) {
-            const int r = e / kGJ, m = e % kGJ;
-            C[r][m] = r < nr ? Cb[(size_t)(rb + r) * kGJ + m] : 0.0;
-        }
-        __syncthreads();
-        if (!act) continue;
-        for (int r = 0; r < nr; r++) {
-            const int i = rb + r;
-            const size_t e = (size_t)i * n + j;
-            if (i >= K && i < K + bb) {  // pivot row: W, with D^-1 in the pivot columns
-                // (read from W and D^-1 again: a dynamic index into w would put w in
-                // local memory for every multiply-add of the update)
-                A[e] = jp ? Dinv[(i - K) * bb + (j - K)] : W[(size_t)(i - K) * n + j];
-                continue;
+            for (int c = 0; c < H; c++) {
+                a[c] = half == hk && c == ck ? rp : a[c] * rp;
+                pr[half * H + c] = a[c];
             }
-            double a = jp ? 0.0 : A[e];
-#pragma unroll
-            for (int m = 0; m < kGJ; m++) a = fma(-C[r][m], w[m], a);
-            A[e] = a;
+            if (half == 0) pr[kGJ] = rp;
         }
+        __syncthreads();
+        if (i != k) {
+            const double rp = pr[kGJ];
+#pragma unroll
+            for (int c = 0; c < H; c++)
+                a[c] = half == hk && c == ck ? -f * rp : fma(-f, pr[half * H + c], a[c]);
+        }
+    }
+#pragma unroll
+    for (int c = 0; c < kGJ / 2; c++) Dinv[i * kGJ + half * (kGJ / 2) + c] = a[c];
+}
+
+__global__ void __launch_bounds__(kGJThreads) k_gj_first(int ld, const double *__restrict__ M, double *__restrict__ Dinv,
+                                                         int *__restrict__ bad)
+{
+    __shared__ double S[kGJ][kGJ + 1];
+    for (int e = threadIdx.x; e < kGJ * kGJ; e += kGJThreads) S[e / kGJ][e % kGJ] = M[(size_t)(e / kGJ) * ld + e % kGJ];
+    __syncthreads();
+    gj_invert(S, Dinv, bad);
+}
+
+// Rows of the panel C = M[:,P] (the block-lower half read by rows below the
+// pivots, by columns above them) and of W = C D, eight rows per block.
+constexpr int kGJPanelRows = 8;
+__global__ void __launch_bounds__(kGJPanelRows * kGJ) k_gj_panel(int ld, int K, const double *__restrict__ M,
+                                                                 const double *__restrict__ Dinv,
+                                                                 double *__restrict__ C, double *__restrict__ W)
+{
+    __shared__ double c[kGJPanelRows][kGJ + 1], D[kGJ][kGJ + 1];
+    const int i0 = blockIdx.x * kGJPanelRows, t = threadIdx.x;
+    for (int e = t; e < kGJ * kGJ; e += kGJPanelRows * kGJ) D[e / kGJ][e % kGJ] = Dinv[e];
+    if (i0 >= K) c[t / kGJ][t % kGJ] = M[(size_t)(i0 + t / kGJ) * ld + K + t % kGJ];
+    else c[t % kGJPanelRows][t / kGJPanelRows] = M[(size_t)(K + t / kGJPanelRows) * ld + i0 + t % kGJPanelRows];
+    __syncthreads();
+    const int r = t / kGJ, k = t % kGJ;
+    double w = 0.0;
+#pragma unroll
+    for (int m = 0; m < kGJ; m++) w = fma(c[r][m], D[m][k], w);
+    C[(size_t)(i0 + r) * kGJ + k] = c[r][k];
+    W[(size_t)(i0 + r) * kGJ + k] = w;
+}
+
+// One kGJ x kGJ tile of the block-lower half per block (two thousand of them at
+// 1942 unknowns, so the SMs finish within a tile or two of each other), a thread
+// 4 x 4 of it.  The next pivot block's tile goes first and its block inverts it
+// while the others update.  FP64-bound: n^2 / 2 x 32 multiply-adds a step, 1942
+// unknowns 95 us against 148 measured (the full Gauss-Jordan step took 215 us and
+// 54 more to invert its pivot block).
+__global__ void __launch_bounds__(kGJThreads) k_gj_update(int ld, int K, double *__restrict__ M,
+                                                          const double *__restrict__ Dinv,
+                                                          const double *__restrict__ C, const double *__restrict__ W,
+                                                          double *__restrict__ Dnext, int *__restrict__ bad)
+{
+    __shared__ double Ws[kGJ][kGJ + 2], Cs[kGJ][kGJ + 2];  // [m][row]
+    const int nt = ld / kGJ, kp = K / kGJ, t = threadIdx.x;
+    int idx = blockIdx.x;
+    if (kp + 1 < nt) {
+        const int first = (kp + 1) * (kp + 2) / 2 + kp + 1;  // tile (kp + 1, kp + 1)
+        idx = idx == 0 ? first : (idx == first ? 0 : idx);
+    }
+    int ti = (int)((sqrtf(8.0f * (float)idx + 1.0f) - 1.0f) * 0.5f);
+    while (ti * (ti + 1) / 2 > idx) ti--;
+    while ((ti + 1) * (ti + 2) / 2 <= idx) ti++;
+    const int tj = idx - ti * (ti + 1) / 2;
+    double *tile = M + (size_t)ti * kGJ * ld + (size_t)tj * kGJ;
+    if (ti == kp || tj == kp) {
+        for (int e = t; e < kGJ * kGJ; e += kGJThreads) {
+            const int r = e / kGJ, c = e % kGJ;
+            double v;
+            if (ti == tj) v = -Dinv[e];
+            else if (tj == kp) v = W[(size_t)(ti * kGJ + r) * kGJ + c];
+            else v = W[(size_t)(tj * kGJ + c) * kGJ + r];
+            tile[(size_t)r * ld + c] = v;
+        }
+        return;
+    }
+    for (int e = t; e < kGJ * kGJ; e += kGJThreads) {
+        Ws[e % kGJ][e / kGJ] = W[(size_t)ti * kGJ * kGJ + e];
+        Cs[e % kGJ][e / kGJ] = C[(size_t)tj * kGJ * kGJ + e];
+    }
+    const int r0 = (t >> 3) * 4, c0 = (t & 7) * 4;
+    double a[4][4];
+#pragma unroll
+    for (int r = 0; r < 4; r++) {
+        const double2 x = *(const double2 *)(tile + (size_t)(r0 + r) * ld + c0);
+        const double2 y = *(const double2 *)(tile + (size_t)(r0 + r) * ld + c0 + 2);
+        a[r][0] = x.x;
+        a[r][1] = x.y;
+        a[r][2] = y.x;
+        a[r][3] = y.y;
+    }
+    __syncthreads();
+#pragma unroll 4
+    for (int m = 0; m < kGJ; m++) {
+        double w[4], c[4];
+#pragma unroll
+        for (int k = 0; k < 4; k++) {
+            w[k] = -Ws[m][r0 + k];
+            c[k] = Cs[m][c0 + k];
+        }
+#pragma unroll
+        for (int r = 0; r < 4; r++)
+#pragma unroll
+            for (int k = 0; k < 4; k++) a[r][k] = fma(w[r], c[k], a[r][k]);
+    }
+#pragma unroll
+    for (int r = 0; r < 4; r++) {
+        *(double2 *)(tile + (size_t)(r0 + r) * ld + c0) = make_double2(a[r][0], a[r][1]);
+        *(double2 *)(tile + (size_t)(r0 + r) * ld + c0 + 2) = make_double2(a[r][2], a[r][3]);
+    }
+    if (ti != kp + 1 || tj != kp + 1) return;
+    __syncthreads();
+    double (*S)[kGJ + 1] = (double (*)[kGJ + 1])&Ws[0][0];
+#pragma unroll
+    for (int r = 0; r < 4; r++)
+#pragma unroll
+        for (int k = 0; k < 4; k++) S[r0 + r][c0 + k] = a[r][k];
+    __syncthreads();
+    gj_invert(S, Dnext, bad);
+}
+
+// the inverse, both halves, from -M's block-lower half
+__global__ void k_gj_inverse(int n, int ld, const double *__restrict__ M, double *__restrict__ Cinv)
+{
+    const int i = blockIdx.x;
+    for (int j = threadIdx.x; j < n; j += blockDim.x) {
+        const bool low = j / kGJ <= i / kGJ;
+        Cinv[(size_t)i * n + j] = -(low ? M[(size_t)i * ld + j] : M[(size_t)j * ld + i]);
     }
 }
 
@@ -1642,12 +1692,14 @@ static int build_coarsest(amg_hierarchy *h, int l, cudaStream_t s)
     int n = 2 * L.N;
     if (n > kMaxCoarse) return BD_ERANGE;
     h->nc = n;
+    const bool single = n <= kCoarseSingleBlock;
+    const int ld = single ? n : (n + kGJ - 1) / kGJ * kGJ;  // padded to whole pivot blocks
     DBuf<double> Ad;
-    BD_TRY(Ad.alloc((size_t)n * n));
+    BD_TRY(Ad.alloc((size_t)ld * ld));
     BD_TRY(h->cinv.alloc((size_t)n * n));
     BD_TRY(h->zc.alloc((size_t)n));
     BD_CUDA(cudaMemsetAsync(Ad.p, 0, Ad.bytes(), s));
-    k_coarse_dense<<<nblk(32LL * L.N), 256, 0, s>>>(L.N, L.A.rp.p, L.A.ci.p, L.A.v.p, Ad.p); ::bd::note_launch();
+    k_coarse_dense<<<nblk(32LL * L.N), 256, 0, s>>>(L.N, L.A.rp.p, L.A.ci.p, L.A.v.p, ld, Ad.p); ::bd::note_launch();
     BD_LAUNCH_CHECK();
     k_null_vector<<<nblk(L.N), 256, 0, s>>>(L.N, L.B.p, h->zc.p); ::bd::note_launch();
     BD_LAUNCH_CHECK();
@@ -1656,34 +1708,29 @@ static int build_coarsest(amg_hierarchy *h, int l, cudaStream_t s)
     BD_TRY(zz.alloc(1));
     BD_TRY(bad.alloc(1));
     BD_CUDA(cudaMemsetAsync(bad.p, 0, sizeof(int), s));
-    if (n <= kCoarseSingleBlock) {
+    DBuf<double> st, Dinv, W, C;
+    if (single) {
         k_coarse_factor<<<1, 256, 0, s>>>(n, Ad.p, h->zc.p, h->cinv.p, zz.p, bad.p); ::bd::note_launch();
         BD_LAUNCH_CHECK();
     } else {
-        DBuf<double> st;
         BD_TRY(st.alloc(2));
-        k_coarse_stats<<<1, 1024, 0, s>>>(n, Ad.p, h->zc.p, st.p); ::bd::note_launch();
-        k_coarse_rank1<<<n, 256, 0, s>>>(n, Ad.p, h->zc.p, st.p); ::bd::note_launch();
-        DBuf<double> Dinv, W, Cb;
-        BD_TRY(Dinv.alloc((size_t)kGJ * kGJ));
-        BD_TRY(W.alloc((size_t)kGJ * n));
-        BD_TRY(Cb.alloc((size_t)kGJ * n));
-        // the update as one resident wave: column chunks x equal row shares
-        int occ = 0;
-        BD_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_gj_update, 128, 0));
-        const int gx = (n + 127) / 128;
-        const int gy = std::max(1, std::min((kSM * std::max(occ, 1)) / gx, (n + kGJ - 1) / kGJ));
-        const dim3 gu(gx, gy), gp(gx, kGJ / kGJPanelK);
-        for (int K = 0; K < n; K += kGJ) {
-            const int bb = std::min(kGJ, n - K);
-            k_gj_pivot<<<1, 256, 0, s>>>(n, K, bb, Ad.p, Dinv.p, bad.p); ::bd::note_launch();
-            k_gj_panel<<<gp, 128, 0, s>>>(n, K, bb, Ad.p, Dinv.p, W.p, Cb.p); ::bd::note_launch();
-            k_gj_update<<<gu, 128, 0, s>>>(n, K, bb, Ad.p, Dinv.p, W.p, Cb.p); ::bd::note_launch();
+        BD_TRY(Dinv.alloc((size_t)2 * kGJ * kGJ));
+        BD_TRY(W.alloc((size_t)kGJ * ld));
+        BD_TRY(C.alloc((size_t)kGJ * ld));
+        k_coarse_stats<<<1, 1024, 0, s>>>(n, ld, Ad.p, h->zc.p, st.p); ::bd::note_launch();
+        k_coarse_rank1<<<ld, 256, 0, s>>>(n, ld, Ad.p, h->zc.p, st.p); ::bd::note_launch();
+        k_gj_first<<<1, kGJThreads, 0, s>>>(ld, Ad.p, Dinv.p, bad.p); ::bd::note_launch();
+        const int nt = ld / kGJ;
+        for (int k = 0; k < nt; k++) {
+            double *D = Dinv.p + (k & 1) * kGJ * kGJ, *Dn = Dinv.p + (1 - (k & 1)) * kGJ * kGJ;
+            k_gj_panel<<<ld / kGJPanelRows, kGJPanelRows * kGJ, 0, s>>>(ld, k * kGJ, Ad.p, D, C.p, W.p);
+            ::bd::note_launch();
+            k_gj_update<<<nt * (nt + 1) / 2, kGJThreads, 0, s>>>(ld, k * kGJ, Ad.p, D, C.p, W.p, Dn, bad.p);
+            ::bd::note_launch();
         }
+        k_gj_inverse<<<n, 256, 0, s>>>(n, ld, Ad.p, h->cinv.p); ::bd::note_launch();
         BD_LAUNCH_CHECK();
-        BD_CUDA(cudaMemcpyAsync(h->cinv.p, Ad.p, Ad.bytes(), cudaMemcpyDeviceToDevice, s));
         BD_CUDA(cudaMemcpyAsync(zz.p, st.p + 1, sizeof(double), cudaMemcpyDeviceToDevice, s));
-        BD_CUDA(cudaStreamSynchronize(s));  // the scratch buffers are freed on return
     }
     k_coarse_project<<<n, 128, 0, s>>>(n, h->cinv.p, h->zc.p, zz.p); ::bd::note_launch();
     BD_LAUNCH_CHECK();
