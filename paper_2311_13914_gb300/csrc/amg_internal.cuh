@@ -60,7 +60,8 @@ struct Level {
     int nagg = 0;
     double lam = 0.0;          // lambda_max(D^{-1} A) estimate
     BSR P, R;                  // prolongator / restriction (not on the coarsest)
-    // solve workspace (double2 per node)
+    // solve workspace (double2 per node), parts of one allocation
+    DBuf<char> work;
     DBuf<double> f, u, r, d, w;
     // FP32 V-cycle: value copies and workspace (float2 per node)
     DBuf<float> A32, P32, R32, invdiag32;
@@ -108,7 +109,8 @@ struct amg_hierarchy {
     // the projection orthogonal to z
     int nc = 0;
     bd::DBuf<double> cinv, zc;
-    // PCG workspace on the finest level
+    // PCG workspace on the finest level, parts of one allocation
+    bd::DBuf<char> work;
     bd::DBuf<double> x, r, z, p, q, fp, zold, fin;
     // whole-solve CUDA graph: pre-loop, a device-controlled WHILE node over one
     // PCG iteration, post-loop (built on first use, reused by every solve)

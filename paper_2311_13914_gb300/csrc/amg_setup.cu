@@ -576,16 +576,17 @@ static int launch_fill_hash(int nrows, int HCn, const int *arp, const int *aci, 
     return BD_OK;
 }
 
-// b_per_row: average blocks per row of B (sets the lanes per row of the hash path)
+// b_per_row: average blocks per row of B (sets the lanes per row of the hash path);
+// scratch: C is scratch of the setup call
 template <int BS>
 static int spgemm(int nrows, int ncols, const int *arp, const int *aci, const double *av,
                   const int *brp, const int *bci, const double *bv, DBuf<int> &crp, DBuf<int> &cci,
-                  DBuf<double> &cv, long long *cnnz, cudaStream_t s, double b_per_row)
+                  DBuf<double> &cv, long long *cnnz, cudaStream_t s, double b_per_row, bool scratch)
 {
     constexpr int BB = BS * BS;
-    BD_TRY(crp.alloc((size_t)nrows + 1));
+    BD_TRY(scratch ? crp.scratch((size_t)nrows + 1, s) : crp.alloc((size_t)nrows + 1));
     DBuf<int> cnt;
-    BD_TRY(cnt.alloc((size_t)nrows + 1));
+    BD_TRY(cnt.scratch((size_t)nrows + 1, s));
     size_t per_block = (size_t)ncols * (sizeof(int) + BB * sizeof(double));
     long long g = kSM * 4;
     long long cap = (2LL << 30) / (long long)(per_block ? per_block : 1);
@@ -597,7 +598,7 @@ static int spgemm(int nrows, int ncols, const int *arp, const int *aci, const do
     DBuf<int> mark;
     DBuf<double> acc;
     DBuf<int> flag;  // [0] hash-table overflow, [1] largest product bound, [2] longest output row
-    BD_TRY(flag.alloc(3));
+    BD_TRY(flag.scratch(3, s));
     BD_CUDA(cudaMemsetAsync(flag.p, 0, 3 * sizeof(int), s));
     // Rows with few products (the fine levels' many short rows) go to the
     // warp-per-row hash path: the dense path's thread block per row then idles
@@ -632,8 +633,8 @@ static int spgemm(int nrows, int ncols, const int *arp, const int *aci, const do
         ::bd::note_launch();
         BD_LAUNCH_CHECK();
     } else if (dense) {
-        BD_TRY(mark.alloc((size_t)grid * ncols));
-        BD_TRY(acc.alloc((size_t)grid * ncols * BB));
+        BD_TRY(mark.scratch((size_t)grid * ncols, s));
+        BD_TRY(acc.scratch((size_t)grid * ncols * BB, s));
         BD_CUDA(cudaMemsetAsync(mark.p, 0xff, mark.bytes(), s));
         k_spgemm_count<BS><<<grid, 128, 0, s>>>(nrows, arp, aci, brp, bci, ncols, mark.p, cnt.p); ::bd::note_launch();
         BD_LAUNCH_CHECK();
@@ -661,8 +662,8 @@ static int spgemm(int nrows, int ncols, const int *arp, const int *aci, const do
     if (hf[0]) return BD_ERANGE;
     const int maxrow = hf[2];
     if (maxrow > kMaxSortSeg) return BD_ERANGE;
-    BD_TRY(cci.alloc((size_t)total));
-    BD_TRY(cv.alloc((size_t)total * BB));
+    BD_TRY(scratch ? cci.scratch((size_t)total, s) : cci.alloc((size_t)total));
+    BD_TRY(scratch ? cv.scratch((size_t)total * BB, s) : cv.alloc((size_t)total * BB));
     if (dense_in_smem) {
         BD_CUDA(cudaFuncSetAttribute(k_spgemm_fill_smem<BS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      (int)dense_smem));
@@ -1111,9 +1112,9 @@ static int bsr_transpose(const BSR &a, BSR &t, cudaStream_t s)
     t.nbc = a.nbr;
     t.nb = a.nb;
     DBuf<int> cnt, fill, perm;
-    BD_TRY(cnt.alloc((size_t)a.nbc + 2));  // counts, then the largest at [a.nbc + 1]
-    BD_TRY(fill.alloc((size_t)a.nbc + 1));
-    BD_TRY(perm.alloc((size_t)a.nb));
+    BD_TRY(cnt.scratch((size_t)a.nbc + 2, s));  // counts, then the largest at [a.nbc + 1]
+    BD_TRY(fill.scratch((size_t)a.nbc + 1, s));
+    BD_TRY(perm.scratch((size_t)a.nb, s));
     BD_TRY(t.rp.alloc((size_t)a.nbc + 1));
     BD_TRY(t.ci.alloc((size_t)a.nb));
     BD_TRY(t.v.alloc(4 * (size_t)a.nb));
@@ -1478,9 +1479,9 @@ static int coarsen_level(amg_hierarchy *h, int l, bool &is_coarsest, cudaStream_
     }
     // a1 strength
     DBuf<double> diag;
-    BD_TRY(diag.alloc((size_t)n));
+    BD_TRY(diag.scratch((size_t)n, s));
     DBuf<int> bad;
-    BD_TRY(bad.alloc(1));
+    BD_TRY(bad.scratch(1, s));
     BD_CUDA(cudaMemsetAsync(bad.p, 0, sizeof(int), s));
     k_diag<<<nblk(N), 256, 0, s>>>(N, L.A.rp.p, L.A.ci.p, L.A.v.p, diag.p, bad.p); ::bd::note_launch();
     BD_LAUNCH_CHECK();
@@ -1488,17 +1489,17 @@ static int coarsen_level(amg_hierarchy *h, int l, bool &is_coarsest, cudaStream_
     S.nr = S.nc = N;
     DBuf<int> cnt;
     DBuf<double> wt;
-    BD_TRY(cnt.alloc((size_t)N + 1));
-    BD_TRY(wt.alloc((size_t)L.A.nb));
-    BD_TRY(S.rp.alloc((size_t)N + 1));
+    BD_TRY(cnt.scratch((size_t)N + 1, s));
+    BD_TRY(wt.scratch((size_t)L.A.nb, s));
+    BD_TRY(S.rp.scratch((size_t)N + 1, s));
     k_strength_count<<<nblk(32LL * N), 256, 0, s>>>(N, L.A.rp.p, L.A.ci.p, L.A.v.p, diag.p, o.theta,
                                                                    cnt.p, wt.p); ::bd::note_launch();
     BD_LAUNCH_CHECK();
     long long snnz = 0;
     BD_TRY(exclusive_scan(cnt.p, S.rp.p, N, &snnz, s));
     S.nnz = snnz;
-    BD_TRY(S.ci.alloc((size_t)snnz));
-    BD_TRY(S.v.alloc((size_t)snnz));
+    BD_TRY(S.ci.scratch((size_t)snnz, s));
+    BD_TRY(S.v.scratch((size_t)snnz, s));
     k_strength_fill<<<nblk(32LL * N), 256, 0, s>>>(N, L.A.rp.p, L.A.ci.p, wt.p, S.rp.p, S.ci.p,
                                                                   S.v.p); ::bd::note_launch();
     BD_LAUNCH_CHECK();
@@ -1508,17 +1509,17 @@ static int coarsen_level(amg_hierarchy *h, int l, bool &is_coarsest, cudaStream_
     if (hbad) return BD_EINVAL;  // non-positive diagonal: not a semi-definite operator
     if (l < o.square_levels) {
         CSR W, Q, S2;
-        BD_TRY(W.rp.alloc((size_t)N + 1));
-        BD_TRY(W.ci.alloc((size_t)snnz + N));
-        BD_TRY(W.v.alloc((size_t)snnz + N));
+        BD_TRY(W.rp.scratch((size_t)N + 1, s));
+        BD_TRY(W.ci.scratch((size_t)snnz + N, s));
+        BD_TRY(W.v.scratch((size_t)snnz + N, s));
         k_insert_diag<<<nblk(N + 1), 256, 0, s>>>(N, S.rp.p, S.ci.p, S.v.p, W.rp.p, W.ci.p, W.v.p); ::bd::note_launch();
         BD_LAUNCH_CHECK();
         long long qn = 0;
         BD_TRY(spgemm<1>(N, N, W.rp.p, W.ci.p, W.v.p, W.rp.p, W.ci.p, W.v.p, Q.rp, Q.ci, Q.v, &qn, s,
-                         (double)(snnz + N) / std::max(N, 1)));
-        BD_TRY(S2.rp.alloc((size_t)N + 1));
-        BD_TRY(S2.ci.alloc((size_t)(qn - N)));
-        BD_TRY(S2.v.alloc((size_t)(qn - N)));
+                         (double)(snnz + N) / std::max(N, 1), true));
+        BD_TRY(S2.rp.scratch((size_t)N + 1, s));
+        BD_TRY(S2.ci.scratch((size_t)(qn - N), s));
+        BD_TRY(S2.v.scratch((size_t)(qn - N), s));
         k_drop_diag<<<nblk(32LL * (N + 1)), 256, 0, s>>>(N, Q.rp.p, Q.ci.p, Q.v.p, S2.rp.p, S2.ci.p, S2.v.p); ::bd::note_launch();
         BD_LAUNCH_CHECK();
         S.rp = std::move(S2.rp);
@@ -1528,10 +1529,10 @@ static int coarsen_level(amg_hierarchy *h, int l, bool &is_coarsest, cudaStream_
     }
     // a2 MIS
     DBuf<unsigned char> state;
-    BD_TRY(state.alloc((size_t)N));
+    BD_TRY(state.scratch((size_t)N, s));
     BD_CUDA(cudaMemsetAsync(state.p, 0, (size_t)N, s));
     DBuf<int> und;
-    BD_TRY(und.alloc(1));
+    BD_TRY(und.scratch(1, s));
     unsigned long long key = level_key(o.seed, l, 0);
     int rounds = 0;
     for (;;) {
@@ -1550,8 +1551,8 @@ static int coarsen_level(amg_hierarchy *h, int l, bool &is_coarsest, cudaStream_
     BD_TRY(L.mis.alloc((size_t)N));
     BD_TRY(L.agg.alloc((size_t)N));
     DBuf<int> flag, rid;
-    BD_TRY(flag.alloc((size_t)N + 1));
-    BD_TRY(rid.alloc((size_t)N + 1));
+    BD_TRY(flag.scratch((size_t)N + 1, s));
+    BD_TRY(rid.scratch((size_t)N + 1, s));
     k_root_flags<<<nblk(N), 256, 0, s>>>(N, state.p, L.mis.p, flag.p); ::bd::note_launch();
     BD_LAUNCH_CHECK();
     long long nagg = 0;
@@ -1573,9 +1574,9 @@ static int coarsen_level(amg_hierarchy *h, int l, bool &is_coarsest, cudaStream_
     int Nc = (int)nagg;
     // a4 tentative prolongator and coarse near-null coefficients
     DBuf<int> moff, mfill, members;
-    BD_TRY(moff.alloc((size_t)Nc + 1));
-    BD_TRY(mfill.alloc((size_t)Nc + 2));  // counts, then the largest at [Nc + 1]
-    BD_TRY(members.alloc((size_t)N));
+    BD_TRY(moff.scratch((size_t)Nc + 1, s));
+    BD_TRY(mfill.scratch((size_t)Nc + 2, s));  // counts, then the largest at [Nc + 1]
+    BD_TRY(members.scratch((size_t)N, s));
     BD_CUDA(cudaMemsetAsync(mfill.p, 0, mfill.bytes(), s));
     k_count_members<<<nblk(N), 256, 0, s>>>(N, L.agg.p, mfill.p); ::bd::note_launch();
     BD_LAUNCH_CHECK();
@@ -1599,21 +1600,21 @@ static int coarsen_level(amg_hierarchy *h, int l, bool &is_coarsest, cudaStream_
     Pt.nbc = Nc;
     Pt.nb = N;
     DBuf<double> ptd;
-    BD_TRY(Pt.rp.alloc((size_t)N + 1));
-    BD_TRY(Pt.ci.alloc((size_t)N));
-    BD_TRY(Pt.v.alloc(4 * (size_t)N));
-    BD_TRY(ptd.alloc((size_t)n));
+    BD_TRY(Pt.rp.scratch((size_t)N + 1, s));
+    BD_TRY(Pt.ci.scratch((size_t)N, s));
+    BD_TRY(Pt.v.scratch(4 * (size_t)N, s));
+    BD_TRY(ptd.scratch((size_t)n, s));
     k_ptent<<<nblk(N + 1), 256, 0, s>>>(N, L.agg.p, L.B.p, C.B.p, Pt.rp.p, Pt.ci.p, Pt.v.p, ptd.p); ::bd::note_launch();
     BD_LAUNCH_CHECK();
     // a5 lambda_max of D^{-1}A
     DBuf<LanczosState> lst;
-    BD_TRY(lst.alloc(1));
+    BD_TRY(lst.scratch(1, s));
     BD_CUDA(cudaMemsetAsync(lst.p, 0, sizeof(LanczosState), s));
     DBuf<double> vr, vz, vp, vq;
-    BD_TRY(vr.alloc((size_t)n));
-    BD_TRY(vz.alloc((size_t)n));
-    BD_TRY(vp.alloc((size_t)n));
-    BD_TRY(vq.alloc((size_t)n));
+    BD_TRY(vr.scratch((size_t)n, s));
+    BD_TRY(vz.scratch((size_t)n, s));
+    BD_TRY(vp.scratch((size_t)n, s));
+    BD_TRY(vq.scratch((size_t)n, s));
     k_lanczos_init<<<nblk(n), 256, 0, s>>>(n, level_key(o.seed, l, 1), diag.p, vr.p, vz.p, vp.p); ::bd::note_launch();
     BD_LAUNCH_CHECK();
     long long *acc = h->exact_acc.p;
@@ -1642,7 +1643,7 @@ static int coarsen_level(amg_hierarchy *h, int l, bool &is_coarsest, cudaStream_
     L.P.nbr = N;
     L.P.nbc = Nc;
     BD_TRY(spgemm<2>(N, Nc, L.A.rp.p, L.A.ci.p, L.A.v.p, Pt.rp.p, Pt.ci.p, Pt.v.p, L.P.rp, L.P.ci,
-                     L.P.v, &pnb, s, 1.0));  // one block per row of the tentative prolongator
+                     L.P.v, &pnb, s, 1.0, false));  // one block per row of the tentative prolongator
     L.P.nb = pnb;
     k_smooth_p<<<nblk(8LL * N), 256, 0, s>>>(N, L.P.rp.p, L.P.ci.p, L.P.v.p, L.agg.p, ptd.p, diag.p, lst.p); ::bd::note_launch();
     BD_LAUNCH_CHECK();
@@ -1652,14 +1653,14 @@ static int coarsen_level(amg_hierarchy *h, int l, bool &is_coarsest, cudaStream_
     BSR AP;
     long long apnb = 0;
     BD_TRY(spgemm<2>(N, Nc, L.A.rp.p, L.A.ci.p, L.A.v.p, L.P.rp.p, L.P.ci.p, L.P.v.p, AP.rp, AP.ci,
-                     AP.v, &apnb, s, (double)L.P.nb / std::max(N, 1)));
+                     AP.v, &apnb, s, (double)L.P.nb / std::max(N, 1), true));
     AP.nbr = N;
     AP.nbc = Nc;
     AP.nb = apnb;
     long long cnb = 0;
     C.A.nbr = C.A.nbc = Nc;
     BD_TRY(spgemm<2>(Nc, Nc, L.R.rp.p, L.R.ci.p, L.R.v.p, AP.rp.p, AP.ci.p, AP.v.p, C.A.rp, C.A.ci,
-                     C.A.v, &cnb, s, (double)apnb / std::max(N, 1)));
+                     C.A.v, &cnb, s, (double)apnb / std::max(N, 1), false));
     C.A.nb = cnb;
     BD_CUDA(cudaStreamSynchronize(s));
     return BD_OK;
@@ -1670,8 +1671,8 @@ static int finish_level_common(Level &L, cudaStream_t s)
     int n = 2 * L.N;
     DBuf<double> diag;
     DBuf<int> bad;
-    BD_TRY(diag.alloc((size_t)n));
-    BD_TRY(bad.alloc(1));
+    BD_TRY(diag.scratch((size_t)n, s));
+    BD_TRY(bad.scratch(1, s));
     BD_CUDA(cudaMemsetAsync(bad.p, 0, sizeof(int), s));
     k_diag<<<nblk(L.N), 256, 0, s>>>(L.N, L.A.rp.p, L.A.ci.p, L.A.v.p, diag.p, bad.p); ::bd::note_launch();
     BD_LAUNCH_CHECK();
@@ -1695,7 +1696,7 @@ static int build_coarsest(amg_hierarchy *h, int l, cudaStream_t s)
     const bool single = n <= kCoarseSingleBlock;
     const int ld = single ? n : (n + kGJ - 1) / kGJ * kGJ;  // padded to whole pivot blocks
     DBuf<double> Ad;
-    BD_TRY(Ad.alloc((size_t)ld * ld));
+    BD_TRY(Ad.scratch((size_t)ld * ld, s));
     BD_TRY(h->cinv.alloc((size_t)n * n));
     BD_TRY(h->zc.alloc((size_t)n));
     BD_CUDA(cudaMemsetAsync(Ad.p, 0, Ad.bytes(), s));
@@ -1705,18 +1706,18 @@ static int build_coarsest(amg_hierarchy *h, int l, cudaStream_t s)
     BD_LAUNCH_CHECK();
     DBuf<double> zz;
     DBuf<int> bad;
-    BD_TRY(zz.alloc(1));
-    BD_TRY(bad.alloc(1));
+    BD_TRY(zz.scratch(1, s));
+    BD_TRY(bad.scratch(1, s));
     BD_CUDA(cudaMemsetAsync(bad.p, 0, sizeof(int), s));
     DBuf<double> st, Dinv, W, C;
     if (single) {
         k_coarse_factor<<<1, 256, 0, s>>>(n, Ad.p, h->zc.p, h->cinv.p, zz.p, bad.p); ::bd::note_launch();
         BD_LAUNCH_CHECK();
     } else {
-        BD_TRY(st.alloc(2));
-        BD_TRY(Dinv.alloc((size_t)2 * kGJ * kGJ));
-        BD_TRY(W.alloc((size_t)kGJ * ld));
-        BD_TRY(C.alloc((size_t)kGJ * ld));
+        BD_TRY(st.scratch(2, s));
+        BD_TRY(Dinv.scratch((size_t)2 * kGJ * kGJ, s));
+        BD_TRY(W.scratch((size_t)kGJ * ld, s));
+        BD_TRY(C.scratch((size_t)kGJ * ld, s));
         k_coarse_stats<<<1, 1024, 0, s>>>(n, ld, Ad.p, h->zc.p, st.p); ::bd::note_launch();
         k_coarse_rank1<<<ld, 256, 0, s>>>(n, ld, Ad.p, h->zc.p, st.p); ::bd::note_launch();
         k_gj_first<<<1, kGJThreads, 0, s>>>(ld, Ad.p, Dinv.p, bad.p); ::bd::note_launch();
@@ -1785,6 +1786,7 @@ extern "C" int amg_setup(const bd_system *sys, const amg_options *opts, void *st
     if (opts) o = *opts;
     BD_TRY(check_opts(&o));
     cudaStream_t s = (cudaStream_t)stream;
+    ScratchPool pool;
     amg_hierarchy *h = new (std::nothrow) amg_hierarchy();
     if (!h) return BD_ENOMEM;
     h->opts = o;
@@ -1840,6 +1842,7 @@ extern "C" int bd_elliptic_setup(const bd_system *sys, const amg_options *opts, 
     if (opts) o = *opts;
     BD_TRY(check_opts(&o));
     cudaStream_t s = (cudaStream_t)stream;
+    ScratchPool pool;
     amg_hierarchy *h = new (std::nothrow) amg_hierarchy();
     if (!h) return BD_ENOMEM;
     h->opts = o;
@@ -1884,6 +1887,7 @@ extern "C" int amg_setup_from_csr(int n, const int *row_ptr, const int *col, con
     if (opts) o = *opts;
     BD_TRY(check_opts(&o));
     cudaStream_t s = (cudaStream_t)stream;
+    ScratchPool pool;
     DBuf<int> drp, dci;
     DBuf<double> dv;
     const int *prp = row_ptr, *pci = col;

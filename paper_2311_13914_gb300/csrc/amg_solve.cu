@@ -1585,6 +1585,16 @@ static int autotune_lanes(amg_hierarchy *h, cudaStream_t s)
 }
 
 // ------------------------------------------------------------------ workspace
+// vectors of n entries each as parts of one allocation (256-byte aligned)
+template <class T> static int carve(DBuf<char> &work, size_t n, std::initializer_list<DBuf<T> *> parts)
+{
+    const size_t step = (n * sizeof(T) + 255) / 256 * 256;
+    BD_TRY(work.alloc(step * parts.size()));
+    size_t k = 0;
+    for (DBuf<T> *d : parts) d->view((T *)(work.p + step * k++), n);
+    return BD_OK;
+}
+
 int prepare_solve(amg_hierarchy *h, cudaStream_t s)
 {
     const bool p32 = h->prec32;
@@ -1592,11 +1602,7 @@ int prepare_solve(amg_hierarchy *h, cudaStream_t s)
         Level &L = h->lev[l];
         size_t n = 2 * (size_t)L.N;
         if (p32) {
-            BD_TRY(L.f32.alloc(n));
-            BD_TRY(L.u32.alloc(n));
-            BD_TRY(L.r32.alloc(n));
-            BD_TRY(L.d32.alloc(n));
-            BD_TRY(L.w32.alloc(n));
+            BD_TRY(carve(L.work, n, {&L.f32, &L.u32, &L.r32, &L.d32, &L.w32}));
             BD_TRY(L.invdiag32.alloc(n));
             const bool a32 = l > 0 || !h->fine.valid;  // the stencil has its own FP32 table
             if (a32) BD_TRY(L.A32.alloc(4 * (size_t)L.A.nb));
@@ -1612,11 +1618,7 @@ int prepare_solve(amg_hierarchy *h, cudaStream_t s)
             }
             BD_LAUNCH_CHECK();
         } else {
-            BD_TRY(L.f.alloc(n));
-            BD_TRY(L.u.alloc(n));
-            BD_TRY(L.r.alloc(n));
-            BD_TRY(L.d.alloc(n));
-            BD_TRY(L.w.alloc(n));
+            BD_TRY(carve(L.work, n, {&L.f, &L.u, &L.r, &L.d, &L.w}));
         }
         if (l < h->nlev - 1) {
             double lo = h->opts.eig_lo * L.lam, hi = h->opts.eig_hi * L.lam;
@@ -1638,13 +1640,7 @@ int prepare_solve(amg_hierarchy *h, cudaStream_t s)
     }
     if (h->fine.valid && h->nlev > 1) BD_TRY(build_pairs(h->lev[0], p32, s));
     size_t n0 = 2 * (size_t)h->lev[0].N;
-    BD_TRY(h->x.alloc(n0));
-    BD_TRY(h->r.alloc(n0));
-    BD_TRY(h->z.alloc(n0));
-    BD_TRY(h->p.alloc(n0));
-    BD_TRY(h->q.alloc(n0));
-    BD_TRY(h->fp.alloc(n0));
-    BD_TRY(h->fin.alloc(n0));
+    BD_TRY(carve(h->work, n0, {&h->x, &h->r, &h->z, &h->p, &h->q, &h->fp, &h->fin}));
     if (p32) {
         BD_TRY(h->zold.alloc(n0));
         BD_CUDA(cudaMemsetAsync(h->zold.p, 0, h->zold.bytes(), s));

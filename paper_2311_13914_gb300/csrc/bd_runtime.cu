@@ -27,6 +27,42 @@ void record_cuda_error(cudaError_t e, const char *what, const char *file, int li
              cudaGetErrorString(e), file, line);
 }
 
+// ------------------------------------------------------------------ scratch pool
+static thread_local cudaMemPool_t g_scratch = nullptr;
+
+ScratchPool::ScratchPool() : outer_(g_scratch)
+{
+    int dev = 0;
+    cudaMemPoolProps props = {};
+    props.allocType = cudaMemAllocationTypePinned;
+    props.location.type = cudaMemLocationTypeDevice;
+    if (cudaGetDevice(&dev) != cudaSuccess) return;
+    props.location.id = dev;
+    unsigned long long keep = ~0ULL;  // nothing goes back before the pool does
+    if (cudaMemPoolCreate(&pool_, &props) != cudaSuccess) {
+        pool_ = nullptr;
+        cudaGetLastError();
+        return;
+    }
+    cudaMemPoolSetAttribute(pool_, cudaMemPoolAttrReleaseThreshold, &keep);
+    g_scratch = pool_;
+}
+
+ScratchPool::~ScratchPool()
+{
+    g_scratch = outer_;
+    if (pool_) cudaMemPoolDestroy(pool_);
+}
+
+cudaMemPool_t ScratchPool::current() { return g_scratch; }
+
+bool ScratchPool::trim(cudaError_t e)
+{
+    if (e != cudaErrorMemoryAllocation || !g_scratch) return false;
+    cudaGetLastError();
+    return cudaDeviceSynchronize() == cudaSuccess && cudaMemPoolTrimTo(g_scratch, 0) == cudaSuccess;
+}
+
 // ------------------------------------------------------------------ prefix scan
 constexpr int kScanThreads = 1024;
 constexpr int kScanTile = 2 * kScanThreads;
@@ -117,8 +153,8 @@ int exclusive_scan(const int *in, int *out, int n, long long *total, cudaStream_
     if (ntiles < 1) ntiles = 1;
     DBuf<long long> sums;
     DBuf<int> flag;
-    BD_TRY(sums.alloc((size_t)ntiles + 1));
-    BD_TRY(flag.alloc(1));
+    BD_TRY(sums.scratch((size_t)ntiles + 1, s));
+    BD_TRY(flag.scratch(1, s));
     BD_CUDA(cudaMemsetAsync(flag.p, 0, sizeof(int), s));
     k_scan_tiles<<<ntiles, kScanThreads, 0, s>>>(in, out, n, sums.p); ::bd::note_launch();
     BD_LAUNCH_CHECK();
