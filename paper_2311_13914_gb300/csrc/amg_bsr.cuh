@@ -7,6 +7,7 @@
 #include <algorithm>
 
 #include "amg_internal.cuh"
+#include "fp_convert.h"
 
 namespace bd {
 

@@ -111,7 +111,8 @@ struct amg_hierarchy {
     bd::DBuf<double> cinv, zc;
     // PCG workspace on the finest level, parts of one allocation
     bd::DBuf<char> work;
-    bd::DBuf<double> x, r, z, p, q, fp, zold, fin;
+    bd::DBuf<double> x, r, z, p, q, fp, fin;
+    bd::DBuf<float> uold;       // FP32 V-cycle: its previous output (flexible beta)
     // whole-solve CUDA graph: pre-loop, a device-controlled WHILE node over one
     // PCG iteration, post-loop (built on first use, reused by every solve)
     cudaGraph_t graph = nullptr;

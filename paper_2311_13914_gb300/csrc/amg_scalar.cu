@@ -240,12 +240,14 @@ template <class S> struct S1In {
     S *__restrict__ d;
     const S *__restrict__ invd;
     S it;
-    __device__ __forceinline__ void operator()(int p, double r) const
+    __device__ __forceinline__ S load(int p) const { return d ? invd[p] : (S)0; }
+    __device__ __forceinline__ void operator()(int p, double r, S b) const
     {
-        const S v = (S)r;
+        const S v = narrow_to<S>(r);
         if (sizeof(S) == 4) f[p] = v;
-        if (d) d[p] = v * invd[p] * it;
+        if (d) d[p] = v * b * it;
     }
+    __device__ __forceinline__ void operator()(int p, double r) const { (*this)(p, r, load(p)); }
 };
 // MODE 0: q = A p and p.q; 1: r = f - A x (stored if out), ||r||^2 and sum x
 template <int MODE, class S> struct S1Reduce {
@@ -309,14 +311,18 @@ template <class S>
 __global__ void k1_z_from(int N, const S *u, const double *__restrict__ r, const double *__restrict__ zold, double *z, Fin fin)
 {
     double a = 0.0, b = 0.0, c = 0.0, d = 0.0;
-    for (int i = share_lo(N) + threadIdx.x, e = share_hi(N); i < e; i += blockDim.x) {
-        const double zi = (double)u[i], ri = r[i];
+    struct In {
+        S u;
+        double r, o;
+    };
+    share_stream(N, [&](int i) { return In{u[i], r[i], zold ? zold[i] : 0.0}; }, [&](int i, const In &q) {
+        const double zi = widen(q.u);
         z[i] = zi;
         a += zi;
-        b += ri;
-        c += ri * zi;
-        if (zold) d += ri * zold[i];
-    }
+        b += q.r;
+        c += q.r * zi;
+        d += q.r * q.o;
+    });
     block_finish<4>(a, b, c, d, fin);
 }
 __global__ void k1_p_update(int N, double *__restrict__ z, double *__restrict__ p, double *__restrict__ zold,
@@ -324,11 +330,14 @@ __global__ void k1_p_update(int N, double *__restrict__ z, double *__restrict__ 
 {
     const double mz = scal[S_MEANZ], beta = scal[S_BETA];
     const bool first = scal[S_IT] == 0.0;
-    for (int i = share_lo(N) + threadIdx.x, e = share_hi(N); i < e; i += blockDim.x) {
-        const double zi = z[i] - mz;
+    struct In {
+        double z, p;
+    };
+    share_stream(N, [&](int i) { return In{z[i], p[i]}; }, [&](int i, const In &q) {
+        const double zi = q.z - mz;
         if (zold) zold[i] = zi;
-        p[i] = first ? zi : zi + beta * p[i];
-    }
+        p[i] = first ? zi : zi + beta * q.p;
+    });
 }
 template <class S>
 __global__ void k1_xr_update(int N, double *__restrict__ x, double *__restrict__ r, const double *__restrict__ p,
@@ -336,13 +345,17 @@ __global__ void k1_xr_update(int N, double *__restrict__ x, double *__restrict__
 {
     const double alpha = fin.scal[S_ALPHA];
     double acc = 0.0;
-    for (int i = share_lo(N) + threadIdx.x, e = share_hi(N); i < e; i += blockDim.x) {
-        const double ri = r[i] - alpha * q[i];
-        x[i] += alpha * p[i];
+    struct In {
+        double x, r, p, q;
+        S b;
+    };
+    share_stream(N, [&](int i) { return In{x[i], r[i], p[i], q[i], in.load(i)}; }, [&](int i, const In &v) {
+        const double ri = v.r - alpha * v.q;
+        x[i] = v.x + alpha * v.p;
         r[i] = ri;
-        in(i, ri);
+        in(i, ri, v.b);
         acc += ri * ri;
-    }
+    });
     block_finish<1>(acc, 0.0, 0.0, 0.0, fin);
 }
 // x to mean zero, or zero for a zero right-hand side

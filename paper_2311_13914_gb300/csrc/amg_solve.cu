@@ -828,7 +828,7 @@ __global__ void __launch_bounds__(1024, 1) k_coarse_solve(int n, const double *_
     if constexpr (STAGE) {
         for (int j = threadIdx.x; j < n / 2; j += blockDim.x) {
             const v2<S> v = ((const v2<S> *)r)[j];
-            rs[j] = make_double2((double)v.x, (double)v.y);
+            rs[j] = make_double2(widen(v.x), widen(v.y));
         }
         __syncthreads();
     }
@@ -837,7 +837,7 @@ __global__ void __launch_bounds__(1024, 1) k_coarse_solve(int n, const double *_
     const double *row = C + (size_t)i * n;
     double s0 = 0.0, s1 = 0.0;
     if (n & 1) {
-        for (int j = lane; j < n; j += 32) s0 = fma(row[j], (double)r[j], s0);
+        for (int j = lane; j < n; j += 32) s0 = fma(row[j], widen(r[j]), s0);
     } else {  // even rows start on 16 bytes
 #pragma unroll 8
         for (int j = lane; j < n / 2; j += 32) {
@@ -847,7 +847,7 @@ __global__ void __launch_bounds__(1024, 1) k_coarse_solve(int n, const double *_
                 v = rs[j];
             } else {
                 const v2<S> t = ((const v2<S> *)r)[j];
-                v = make_double2((double)t.x, (double)t.y);
+                v = make_double2(widen(t.x), widen(t.y));
             }
             s0 = fma(c.x, v.x, s0);
             s1 = fma(c.y, v.y, s1);
@@ -895,7 +895,7 @@ __global__ void k_in32(int N, const double2 *__restrict__ r, const float2 *__res
     for (int i = share_lo(N) + threadIdx.x, e = share_hi(N); i < e; i += blockDim.x) {
         const double2 a = r[i];
         const float2 b = invd[i];
-        const float f0 = (float)a.x, f1 = (float)a.y;
+        const float f0 = narrow(a.x), f1 = narrow(a.y);
         f[i] = make_float2(f0, f1);
         d0[i] = make_float2(f0 * b.x * it, f1 * b.y * it);
     }
@@ -905,7 +905,7 @@ __global__ void k_out64(int N, const float2 *__restrict__ u, double2 *__restrict
 {
     for (int i = share_lo(N) + threadIdx.x, e = share_hi(N); i < e; i += blockDim.x) {
         const float2 a = u[i];
-        z[i] = make_double2((double)a.x, (double)a.y);
+        z[i] = make_double2(widen(a.x), widen(a.y));
     }
 }
 
@@ -920,7 +920,7 @@ __global__ void k_to_f32(long long n, const double *__restrict__ a, float *__res
 // (defined with the PCG reductions below).
 struct ZOut;
 static int launch_fine_z(amg_hierarchy *h, const LV<double> &lv, const double2 *u, const ZOut &zo, cudaStream_t s);
-// FP32 V-cycle output to the PCG's z (FP64) with the z statistics in one pass
+// the z statistics of the FP32 V-cycle's output
 static int launch_z_from32(amg_hierarchy *h, const float2 *u, const ZOut &zo, cudaStream_t s);
 
 // One V-cycle in precision S; f0/u0 are the finest level's right-hand side and
@@ -1005,9 +1005,8 @@ static int vcycle_impl(amg_hierarchy *h, const v2<S> *f0, v2<S> *u0, cudaStream_
         if (deg2) {
             int s2 = prof_begin(h, s, 16 * l + R_POST2, l == 0);
             double bytes = l == 0 ? fine_bytes<S>(h, L, fine ? 4 : 5) : 0.0;
-            // FP64: the post-smoother's last kernel carries the PCG's z statistics;
-            // FP32: the plain kernel, then one pass that converts u to z and sums
-            // the statistics
+            // FP64: the post-smoother's last kernel carries the PCG's z statistics
+            // (FP32: a pass of their own over u, vcycle_run)
             const bool fuse_z = fine && zo && sizeof(S) == 8;
             if (fuse_z) {
                 if constexpr (SU) BD_TRY(launch_fine_z(h, lv, u, *zo, s));
@@ -1025,12 +1024,6 @@ static int vcycle_impl(amg_hierarchy *h, const v2<S> *f0, v2<S> *u0, cudaStream_
                                    EpiPost2<S>{lv.r, lv.d, lv.invd, lv.w, u, (S)L.ch_c1, (S)L.ch_c2}, s));
             }
             prof_end(h, s2, bytes, fine_flops(h, L), s, fine_ops<S>(h, L, fuse_z ? FR_POST2Z : FR_POST2));
-            if (l == 0 && zo && sizeof(S) == 4) {
-                int sz = prof_begin(h, s, R_ZSTATS, false);
-                BD_TRY(launch_z_from32(h, (const float2 *)u, *zo, s));
-                prof_end(h, sz, 0.0, 0.0, s);
-                if (zdone) *zdone = true;
-            }
         } else {
             int s2 = prof_begin(h, s, 16 * l + R_POST2, false);
             k_copy2<S><<<grid_for(L.N, 256), 256, 0, s>>>(L.N, lv.w, u); ::bd::note_launch();
@@ -1054,7 +1047,9 @@ static int vcycle_impl(amg_hierarchy *h, const v2<S> *f0, v2<S> *u0, cudaStream_
 
 // z = B r with FP64 vectors at the boundary, in the hierarchy's precision.
 // d0_ready: the producer of r already wrote the finest level's input (D0Out);
-// zo, zdone: as vcycle_impl (z is written to z_dev either way).
+// zo, zdone (PCG): the z statistics are taken as well; an FP32 V-cycle then
+// leaves its output in the finest level's u (the PCG widens it where it reads it)
+// and z_dev unwritten.
 static int vcycle_run(amg_hierarchy *h, const double *r_dev, double *z_dev, cudaStream_t s, bool d0_ready,
                       const ZOut *zo, bool *zdone)
 {
@@ -1069,15 +1064,18 @@ static int vcycle_run(amg_hierarchy *h, const double *r_dev, double *z_dev, cuda
             BD_LAUNCH_CHECK();
             prof_end(h, si, 0.0, 0.0, s);
         }
-        bool zd = false;
-        BD_TRY((vcycle_impl<float>(h, v0.f, v0.u, s, zo, &zd)));
-        if (!zd) {
+        BD_TRY((vcycle_impl<float>(h, v0.f, v0.u, s)));
+        if (zo) {
+            int sz = prof_begin(h, s, R_ZSTATS, false);
+            BD_TRY(launch_z_from32(h, v0.u, *zo, s));
+            prof_end(h, sz, 0.0, 0.0, s);
+            if (zdone) *zdone = true;
+        } else {
             int so = prof_begin(h, s, R_VOUT, false);
             k_out64<<<grid_for(L0.N, 256), 256, 0, s>>>(L0.N, v0.u, (double2 *)z_dev); ::bd::note_launch();
             BD_LAUNCH_CHECK();
             prof_end(h, so, 0.0, 0.0, s);
         }
-        if (zdone) *zdone = zd;
         return BD_OK;
     }
     // FP64 stencil: the finest level's gathered vectors in (v + u, u) form
@@ -1106,11 +1104,10 @@ int vcycle_device(amg_hierarchy *h, const double *r_dev, double *z_dev, cudaStre
 __global__ void k_f_stats(int N, const double2 *__restrict__ f, Fin fin)
 {
     double a = 0.0, b = 0.0;
-    for (int i = share_lo(N) + threadIdx.x, e = share_hi(N); i < e; i += blockDim.x) {
-        double2 v = f[i];
+    share_stream(N, [&](int i) { return f[i]; }, [&](int, const double2 &v) {
         a += v.y;
-        b += v.x * v.x + v.y * v.y;
-    }
+        b = fma(v.x, v.x, fma(v.y, v.y, b));
+    });
     block_finish<2>(a, b, 0.0, 0.0, fin);
 }
 
@@ -1118,12 +1115,11 @@ __global__ void k_project_f(int N, const double2 *__restrict__ f, double2 *__res
 {
     const double m = fin.scal[S_MEANF];
     double a = 0.0;
-    for (int i = share_lo(N) + threadIdx.x, e = share_hi(N); i < e; i += blockDim.x) {
-        double2 v = f[i];
+    share_stream(N, [&](int i) { return f[i]; }, [&](int i, double2 v) {
         v.y -= m;
         fp[i] = v;
-        a += v.x * v.x + v.y * v.y;
-    }
+        a = fma(v.x, v.x, fma(v.y, v.y, a));
+    });
     block_finish<1>(a, 0.0, 0.0, 0.0, fin);
 }
 
@@ -1156,19 +1152,30 @@ struct D0Out {
     float2 *f32 = nullptr, *d32 = nullptr;
     const float2 *invd32 = nullptr;
     float it32 = 0.0f;
-    __device__ __forceinline__ void operator()(int p, double r0, double r1) const
+    // D^{-1} of a row (FP64 or FP32 by the mode)
+    struct Pre {
+        double2 b64;
+        float2 b32;
+    };
+    __device__ __forceinline__ Pre load(int p) const
+    {
+        Pre q{};
+        if (mode == 1 || mode == 2) q.b64 = invd64[p];
+        else if (mode == 3) q.b32 = invd32[p];
+        return q;
+    }
+    __device__ __forceinline__ void operator()(int p, double r0, double r1, const Pre &q) const
     {
         if (mode == 1 || mode == 2) {
-            const double2 b = invd64[p];
-            const double v = r0 * b.x * it, u = r1 * b.y * it;
+            const double v = r0 * q.b64.x * it, u = r1 * q.b64.y * it;
             d64[p] = mode == 1 ? make_double2(v + u, u) : make_double2(v, u);
         } else if (mode == 3) {
-            const float2 b = invd32[p];
-            const float f0 = (float)r0, f1 = (float)r1;
+            const float f0 = narrow(r0), f1 = narrow(r1);
             f32[p] = make_float2(f0, f1);
-            d32[p] = make_float2(f0 * b.x * it32, f1 * b.y * it32);
+            d32[p] = make_float2(f0 * q.b32.x * it32, f1 * q.b32.y * it32);
         }
     }
+    __device__ __forceinline__ void operator()(int p, double r0, double r1) const { (*this)(p, r0, r1, load(p)); }
 };
 
 // FP64 finest-level operator with a reduction epilogue (block CSR form, T lanes).
@@ -1285,22 +1292,19 @@ static void fine_reduce(const amg_hierarchy *h, const double2 *x, const double2 
     }
 }
 
-// sums of z_u and r_u, r.z and (flexible form) r.z_old
-__global__ void k_z_stats(int N, const double2 *__restrict__ z, const double2 *__restrict__ r,
-                          const double2 *__restrict__ zold, Fin fin)
+// sums of z_u and r_u, and r.z (FP64 V-cycle)
+__global__ void k_z_stats(int N, const double2 *__restrict__ z, const double2 *__restrict__ r, Fin fin)
 {
-    double a = 0.0, b = 0.0, c = 0.0, d = 0.0;
-    for (int i = share_lo(N) + threadIdx.x, e = share_hi(N); i < e; i += blockDim.x) {
-        const double2 zi = z[i], ri = r[i];
-        a += zi.y;
-        b += ri.y;
-        c += ri.x * zi.x + ri.y * zi.y;
-        if (zold) {
-            const double2 oi = zold[i];
-            d += ri.x * oi.x + ri.y * oi.y;
-        }
-    }
-    block_finish<4>(a, b, c, d, fin);
+    double a = 0.0, b = 0.0, c = 0.0;
+    struct In {
+        double2 z, r;
+    };
+    share_stream(N, [&](int i) { return In{z[i], r[i]}; }, [&](int, const In &q) {
+        a += q.z.y;
+        b += q.r.y;
+        c = fma(q.r.x, q.z.x, fma(q.r.y, q.z.y, c));
+    });
+    block_finish<3>(a, b, c, 0.0, fin);
 }
 
 // The V-cycle's last finest-level kernel with the z statistics fused in: the
@@ -1310,7 +1314,7 @@ __global__ void k_z_stats(int N, const double2 *__restrict__ z, const double2 *_
 struct ZOut {
     double2 *z;
     const double2 *r;
-    const double2 *zold;  // flexible CG's previous projected z, or null
+    const float2 *uold;  // FP32 V-cycle: its previous output
     Fin fin;
 };
 
@@ -1357,23 +1361,29 @@ static int launch_fine_z(amg_hierarchy *h, const LV<double> &lv, const double2 *
     return BD_OK;
 }
 
-// z = (double) u of the FP32 V-cycle, and its statistics (z_u, r_u, r.z,
-// r.z_old) in FP64 (stage 3), in one pass
-__global__ void k_z_from32(int N, const float2 *__restrict__ u, ZOut zo)
+// Statistics (z_u, r_u, r.z, r.z_old) of z = (double) u, the FP32 V-cycle's
+// output, in FP64 (stage 3).  z and the previous projected z are not stored:
+// both are the FP32 outputs, widened exactly, less their mean (S_MEANZ still holds
+// the previous one here), so the PCG reads 32 bytes per node instead of moving
+// 56 here and 48 instead of 80 in the direction's update.  Bound by the FP64
+// operations, seven a node once the conversions are integer work (256x256x64:
+// 93 + 55 -> 69 + 41 us, 128x128x32: 24.3 + 10.4 -> 20.2 + 10.2).
+__global__ void __launch_bounds__(kVecThreads, 4)
+    k_z_from32(int N, const float2 *__restrict__ u, ZOut zo)
 {
+    const double mo = zo.fin.scal[S_MEANZ];
     double a = 0.0, b = 0.0, c = 0.0, d = 0.0;
-    for (int i = share_lo(N) + threadIdx.x, e = share_hi(N); i < e; i += blockDim.x) {
-        const float2 v = u[i];
-        const double2 z = make_double2((double)v.x, (double)v.y), r = zo.r[i];
-        zo.z[i] = z;
-        a += z.y;
-        b += r.y;
-        c += r.x * z.x + r.y * z.y;
-        if (zo.zold) {
-            const double2 o = zo.zold[i];
-            d += r.x * o.x + r.y * o.y;
-        }
-    }
+    struct In {
+        float2 v, w;
+        double2 r;
+    };
+    share_stream(N, [&](int i) { return In{u[i], zo.uold[i], zo.r[i]}; }, [&](int, const In &q) {
+        const double zx = widen(q.v.x), zy = widen(q.v.y);
+        a += zy;
+        b += q.r.y;
+        c = fma(q.r.x, zx, fma(q.r.y, zy, c));
+        d = fma(q.r.x, widen(q.w.x), fma(q.r.y, widen(q.w.y) - mo, d));
+    });
     block_finish<4>(a, b, c, d, zo.fin);
 }
 
@@ -1385,39 +1395,42 @@ static int launch_z_from32(amg_hierarchy *h, const float2 *u, const ZOut &zo, cu
     return BD_OK;
 }
 
-// z <- z - mean(z_u) e_u; p = z (first iteration) or z + beta p, stored in
-// (v+u, u) form when SU; keeps the projected z for the next flexible beta
-// when zold is given.
-template <bool SU>
-__global__ void k_p_update(int N, double2 *__restrict__ z, double2 *__restrict__ p,
-                           double2 *__restrict__ zold, const double *__restrict__ scal, int first)
+// p = z - mean(z_u) e_u (first iteration) or that + beta p, stored in (v+u, u)
+// form when SU; z as the V-cycle left it (FP64, or its FP32 output, which is
+// kept for the next flexible beta).
+template <bool SU, class Z>
+__global__ void __launch_bounds__(kVecThreads, 4)
+    k_p_update(int N, const Z *__restrict__ z, double2 *__restrict__ p, Z *__restrict__ zold,
+                           const double *__restrict__ scal, int first)
 {
     const double mz = scal[S_MEANZ], beta = scal[S_BETA];
     if (first < 0) first = scal[S_IT] == 0.0;
-    for (int i = share_lo(N) + threadIdx.x, e = share_hi(N); i < e; i += blockDim.x) {
-        double2 zi = z[i];
-        zi.y -= mz;
-        z[i] = zi;
-        if (zold) zold[i] = zi;
-        const double2 zs = SU ? make_double2(zi.x + zi.y, zi.y) : zi;
-        if (first) {
-            p[i] = zs;
-        } else {
-            const double2 pi = p[i];
-            p[i] = make_double2(zs.x + beta * pi.x, zs.y + beta * pi.y);
-        }
-    }
+    struct In {
+        Z z;
+        double2 p;
+    };
+    share_stream(N, [&](int i) { return In{z[i], p[i]}; }, [&](int i, const In &q) {
+        if (zold) zold[i] = q.z;
+        const double zx = widen(q.z.x), zy = widen(q.z.y) - mz;
+        const double2 zs = make_double2(SU ? zx + zy : zx, zy);
+        p[i] = first ? zs : make_double2(zs.x + beta * q.p.x, zs.y + beta * q.p.y);
+    });
 }
 
 template <bool SU>
-__global__ void k_xr_update(int N, double2 *__restrict__ x, double2 *__restrict__ r,
+__global__ void __launch_bounds__(kVecThreads, 4)
+    k_xr_update(int N, double2 *__restrict__ x, double2 *__restrict__ r,
                             const double2 *__restrict__ p, const double2 *__restrict__ q, Fin fin, D0Out d0)
 {
     const double alpha = fin.scal[S_ALPHA];
     double acc = 0.0;
-    for (int i = share_lo(N) + threadIdx.x, e = share_hi(N); i < e; i += blockDim.x) {
-        double2 xi = x[i], ri = r[i];
-        const double2 pi = p[i], qi = q[i];
+    struct In {
+        double2 x, r, p, q;
+        D0Out::Pre b;
+    };
+    share_stream(N, [&](int i) { return In{x[i], r[i], p[i], q[i], d0.load(i)}; }, [&](int i, const In &in) {
+        double2 xi = in.x, ri = in.r;
+        const double2 pi = in.p, qi = in.q;
         const double pv = SU ? pi.x - pi.y : pi.x;
         xi.x += alpha * pv;
         xi.y += alpha * pi.y;
@@ -1425,9 +1438,9 @@ __global__ void k_xr_update(int N, double2 *__restrict__ x, double2 *__restrict_
         ri.y -= alpha * qi.y;
         x[i] = xi;
         r[i] = ri;
-        d0(i, ri.x, ri.y);
-        acc += ri.x * ri.x + ri.y * ri.y;
-    }
+        d0(i, ri.x, ri.y, in.b);
+        acc = fma(ri.x, ri.x, fma(ri.y, ri.y, acc));
+    });
     block_finish<1>(acc, 0.0, 0.0, 0.0, fin);
 }
 
@@ -1437,11 +1450,19 @@ __global__ void k_project_x(int N, double2 *__restrict__ x, const double *__rest
     for (int i = share_lo(N) + threadIdx.x, e = share_hi(N); i < e; i += blockDim.x) x[i].y -= m;
 }
 
-static void p_update(const amg_hierarchy *h, int N, double2 *z, double2 *p, double2 *zold, double *scal,
-                     int first, cudaStream_t s)
+static void p_update(amg_hierarchy *h, int N, double2 *p, double *scal, int first, cudaStream_t s)
 {
-    if (h->fine.valid) k_p_update<true><<<kVecBlocks, kVecThreads, 0, s>>>(N, z, p, zold, scal, first);
-    else k_p_update<false><<<kVecBlocks, kVecThreads, 0, s>>>(N, z, p, zold, scal, first);
+    auto run = [&](auto su) {
+        constexpr bool SU = decltype(su)::value;
+        if (h->prec32)
+            k_p_update<SU><<<kVecBlocks, kVecThreads, 0, s>>>(N, (const float2 *)h->lev[0].u32.p, p, (float2 *)h->uold.p,
+                                                             scal, first);
+        else
+            k_p_update<SU><<<kVecBlocks, kVecThreads, 0, s>>>(N, (const double2 *)h->z.p, p, (double2 *)nullptr, scal,
+                                                             first);
+    };
+    if (h->fine.valid) run(std::true_type{});
+    else run(std::false_type{});
     note_launch();
 }
 
@@ -1642,8 +1663,8 @@ int prepare_solve(amg_hierarchy *h, cudaStream_t s)
     size_t n0 = 2 * (size_t)h->lev[0].N;
     BD_TRY(carve(h->work, n0, {&h->x, &h->r, &h->z, &h->p, &h->q, &h->fp, &h->fin}));
     if (p32) {
-        BD_TRY(h->zold.alloc(n0));
-        BD_CUDA(cudaMemsetAsync(h->zold.p, 0, h->zold.bytes(), s));
+        BD_TRY(h->uold.alloc(n0));
+        BD_CUDA(cudaMemsetAsync(h->uold.p, 0, h->uold.bytes(), s));
     }
     BD_TRY(h->partial.alloc(kPart * (size_t)kRedBlocks));
     BD_TRY(h->counter.alloc(1));
@@ -1702,10 +1723,8 @@ static int pcg_solve_loop(amg_hierarchy *h, const double *f_dev, double *x_dev, 
 {
     Level &L0 = h->lev[0];
     const int N = L0.N;
-    const bool flex = h->prec32;
     double2 *x = (double2 *)x_dev, *r = (double2 *)h->r.p, *z = (double2 *)h->z.p;
     double2 *p = (double2 *)h->p.p, *q = (double2 *)h->q.p, *fp = (double2 *)h->fp.p;
-    double2 *zold = flex ? (double2 *)h->zold.p : nullptr;
     double *scal = h->scal.p;
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     BD_CUDA(cudaEventCreate(&e0));
@@ -1736,16 +1755,16 @@ static int pcg_solve_loop(amg_hierarchy *h, const double *f_dev, double *x_dev, 
     } else if (status == BD_OK && !(rr <= o->rtol * nf)) {
         status = BD_ENOTCONV;
         while (it < o->max_it) {
-            const ZOut zo{z, r, it == 0 ? nullptr : zold, make_fin(h, 3, it == 0)};
+            const ZOut zo{z, r, (const float2 *)h->uold.p, make_fin(h, 3, it == 0)};
             bool zd = false;
             BD_TRY(vcycle_run(h, (const double *)r, (double *)z, s, true, &zo, &zd));
             if (!zd) {
                 int sz = prof_begin(h, s, R_ZSTATS, false);
-                k_z_stats<<<kVecBlocks, kVecThreads, 0, s>>>(N, z, r, zo.zold, zo.fin); ::bd::note_launch();
+                k_z_stats<<<kVecBlocks, kVecThreads, 0, s>>>(N, z, r, zo.fin); ::bd::note_launch();
                 prof_end(h, sz, 0.0, 0.0, s);
             }
             int su = prof_begin(h, s, R_PUPDATE, false);
-            p_update(h, N, z, p, zold, scal, it == 0, s);
+            p_update(h, N, p, scal, it == 0, s);
             prof_end(h, su, 0.0, 0.0, s);
             // the FP64 PCG operator counts among the finest-operator launches
             // when the V-cycle is FP64 too (one kernel family per profile)
@@ -1858,10 +1877,8 @@ static int capture_solve(amg_hierarchy *h, cudaStream_t s, cudaStream_t s2)
 {
     Level &L0 = h->lev[0];
     const int N = L0.N;
-    const bool flex = h->prec32;
     double2 *x = (double2 *)h->x.p, *r = (double2 *)h->r.p, *z = (double2 *)h->z.p;
     double2 *p = (double2 *)h->p.p, *q = (double2 *)h->q.p, *fp = (double2 *)h->fp.p;
-    double2 *zold = flex ? (double2 *)h->zold.p : nullptr;
     const double2 *fin = (const double2 *)h->fin.p;
     double *scal = h->scal.p;
     // kernel-node counts per section (the launch counter counts executions, so
@@ -1878,13 +1895,13 @@ static int capture_solve(amg_hierarchy *h, cudaStream_t s, cudaStream_t s2)
     BD_LAUNCH_CHECK();
     BD_TRY(while_begin(s, s2, &w));
     const long long c1 = launch_count();
-    const ZOut zo{z, r, zold, make_fin(h, 3, -1)};
+    const ZOut zo{z, r, (const float2 *)h->uold.p, make_fin(h, 3, -1)};
     bool zd = false;
     BD_TRY(vcycle_run(h, (const double *)r, (double *)z, s2, true, &zo, &zd));
     if (!zd) {
-        k_z_stats<<<kVecBlocks, kVecThreads, 0, s2>>>(N, z, r, zold, zo.fin); ::bd::note_launch();
+        k_z_stats<<<kVecBlocks, kVecThreads, 0, s2>>>(N, z, r, zo.fin); ::bd::note_launch();
     }
-    p_update(h, N, z, p, zold, scal, -1, s2);
+    p_update(h, N, p, scal, -1, s2);
     fine_reduce<0>(h, p, nullptr, q, make_fin(h, 4, 0), s2);
     xr_update(h, N, x, r, p, q, make_fin(h, 7, 0, w.cond), s2, d0);
     BD_LAUNCH_CHECK();

@@ -58,7 +58,7 @@ template <class S> struct StPre {  // from zero: u = d0 + (c1 d0 + c2 D^{-1} (f 
     __device__ __forceinline__ void operator()(int p, S y0, S y1) const
     {
         const double *k = c.at(p);
-        const S c1 = (S)k[1], c2 = (S)k[2];
+        const S c1 = narrow_to<S>(k[1]), c2 = narrow_to<S>(k[2]);
         const v2<S> fp = f[p], id = invd[p], dp = d0[p];
         const S r0 = fp.x - y0, r1 = fp.y - y1;
         u[p] = V2<S>::mk(dp.x + (c1 * dp.x + c2 * id.x * r0), dp.y + (c1 * dp.y + c2 * id.y * r1));
@@ -80,7 +80,7 @@ template <class S> struct StStoreD0 {  // f_c = R r and d0_c = D_c^{-1} f_c / th
     StCoef c;
     __device__ __forceinline__ void operator()(int p, S y0, S y1) const
     {
-        const S it = (S)c.at(p)[0];
+        const S it = narrow_to<S>(c.at(p)[0]);
         const v2<S> id = invd[p];
         f[p] = V2<S>::mk(y0, y1);
         d0[p] = V2<S>::mk(y0 * id.x * it, y1 * id.y * it);
@@ -104,7 +104,7 @@ template <class S> struct StPost1 {  // r = f - A u, d = D^{-1} r / theta, w = u
     StCoef c;
     __device__ __forceinline__ void operator()(int p, S y0, S y1) const
     {
-        const S it = (S)c.at(p)[0];
+        const S it = narrow_to<S>(c.at(p)[0]);
         const v2<S> fp = f[p], id = invd[p], up = u[p];
         const S r0 = fp.x - y0, r1 = fp.y - y1;
         const S d0 = r0 * id.x * it, d1 = r1 * id.y * it;
@@ -123,7 +123,7 @@ template <class S> struct StPost2 {  // u = w + (c1 d + c2 D^{-1} (r - A d))
     __device__ __forceinline__ void operator()(int p, S y0, S y1) const
     {
         const double *k = c.at(p);
-        const S c1 = (S)k[1], c2 = (S)k[2];
+        const S c1 = narrow_to<S>(k[1]), c2 = narrow_to<S>(k[2]);
         const v2<S> rp_ = r[p], dp = d[p], id = invd[p], wp = w[p];
         const S r0 = rp_.x - y0, r1 = rp_.y - y1;
         u[p] = V2<S>::mk(wp.x + (c1 * dp.x + c2 * id.x * r0), wp.y + (c1 * dp.y + c2 * id.y * r1));
@@ -192,8 +192,8 @@ __global__ void __launch_bounds__(128) k_st_coarse(const StCoarseJob *__restrict
     for (int j = lane; j < J.n / 2; j += 32) {
         const double2 c = row[j];
         const v2<S> v = r[j];
-        s0 = fma(c.x, (double)v.x, s0);
-        s1 = fma(c.y, (double)v.y, s1);
+        s0 = fma(c.x, widen(v.x), s0);
+        s1 = fma(c.y, widen(v.y), s1);
     }
     s0 += s1;
     for (int o = 16; o; o >>= 1) s0 += __shfl_xor_sync(0xffffffffu, s0, o);
@@ -217,8 +217,9 @@ struct StRed {
 // input f0, d0 and output u0 in its precision S).
 template <class S> struct StPcg {
     const double2 *fin;
-    double2 *fp, *x, *r, *z, *p, *q, *zold;
+    double2 *fp, *x, *r, *p, *q;
     v2<S> *f0, *d0;
+    v2<S> *uold;                   // FP32 V-cycle: its previous output (flexible beta)
     const v2<S> *u0, *invd0;
     StCoef c0;
     const int *mem;                // finest-level node -> member
@@ -234,10 +235,10 @@ template <class S>
 __device__ __forceinline__ void st_vin(const StPcg<S> &v, int i, double2 ri)
 {
     const double it = v.c0.at(i)[0];
-    if (sizeof(S) == 4) v.f0[i] = V2<S>::mk((S)ri.x, (S)ri.y);
+    const S rv = narrow_to<S>(ri.x), ru = narrow_to<S>(ri.y), itS = narrow_to<S>(it);
+    if (sizeof(S) == 4) v.f0[i] = V2<S>::mk(rv, ru);
     const v2<S> id = v.invd0[i];
-    const S itS = (S)it;
-    const S dv = (S)ri.x * id.x * itS, du = (S)ri.y * id.y * itS;
+    const S dv = rv * id.x * itS, du = ru * id.y * itS;
     v.d0[i] = V2<S>::mk(v.dsu ? dv + du : dv, du);
 }
 
@@ -345,16 +346,17 @@ __global__ void __launch_bounds__(kStThreads) k_st_red(StRed R, StPcg<S> v)
         }
     } else if (MODE == R_ZSTATS) {
         if (sc[T_ACTIVE] != 0.0) {
+            const double mzo = sc[T_MEANZ];
             for (int i = b + threadIdx.x; i < e; i += blockDim.x) {
                 const v2<S> u = v.u0[i];
-                const double2 zi = make_double2((double)u.x, (double)u.y), ri = v.r[i];
-                v.z[i] = zi;
+                const double2 zi = make_double2(widen(u.x), widen(u.y)), ri = v.r[i];
                 acc[0] += zi.y;
                 acc[1] += ri.y;
-                acc[2] += ri.x * zi.x + ri.y * zi.y;
+                acc[2] = fma(ri.x, zi.x, fma(ri.y, zi.y, acc[2]));
                 if (R.flex) {
-                    const double2 o = v.zold[i];
-                    acc[3] += ri.x * o.x + ri.y * o.y;
+                    // the previous z: its FP32 values less their mean (still in T_MEANZ)
+                    const v2<S> o = v.uold[i];
+                    acc[3] = fma(ri.x, widen(o.x), fma(ri.y, widen(o.y) - mzo, acc[3]));
                 }
             }
         }
@@ -363,7 +365,7 @@ __global__ void __launch_bounds__(kStThreads) k_st_red(StRed R, StPcg<S> v)
             for (int i = b + threadIdx.x; i < e; i += blockDim.x) {
                 const double2 p = v.p[i], q = v.q[i];
                 const double pv = v.psu ? p.x - p.y : p.x;
-                acc[0] += pv * q.x + p.y * q.y;
+                acc[0] = fma(pv, q.x, fma(p.y, q.y, acc[0]));
             }
     } else if (MODE == R_XR) {
         if (sc[T_ACTIVE] != 0.0) {
@@ -378,7 +380,7 @@ __global__ void __launch_bounds__(kStThreads) k_st_red(StRed R, StPcg<S> v)
                 v.x[i] = xi;
                 v.r[i] = ri;
                 st_vin<S>(v, i, ri);
-                acc[0] += ri.x * ri.x + ri.y * ri.y;
+                acc[0] = fma(ri.x, ri.x, fma(ri.y, ri.y, acc[0]));
             }
         }
     } else if (MODE == R_TRUE) {  // q = A x of the final iterate
@@ -431,9 +433,9 @@ __global__ void __launch_bounds__(kStThreads) k_st_red(StRed R, StPcg<S> v)
     }
 }
 
-// z <- z - mean(z_u) e_u; p = z (first iteration) or z + beta p, stored in
-// (v + u, u) form when psu; the projected z kept for the next flexible beta.
-// Members no longer iterating keep p.
+// p = z - mean(z_u) e_u (first iteration) or that + beta p, stored in (v + u, u)
+// form when psu; z is the V-cycle's output, kept in FP32 for the next flexible
+// beta.  Members no longer iterating keep p.
 template <class S>
 __global__ void k_st_p(int N, StPcg<S> v, const double *__restrict__ scal)
 {
@@ -442,11 +444,10 @@ __global__ void k_st_p(int N, StPcg<S> v, const double *__restrict__ scal)
         if (m < 0) continue;  // padding after a member's last node
         const double *sc = scal + (size_t)m * T_NSLOTS;
         if (sc[T_ACTIVE] == 0.0) continue;
-        double2 zi = v.z[i];
-        zi.y -= sc[T_MEANZ];
-        v.z[i] = zi;
-        if (v.zold) v.zold[i] = zi;
-        const double2 zs = v.psu ? make_double2(zi.x + zi.y, zi.y) : zi;
+        const v2<S> u = v.u0[i];
+        if (v.uold) v.uold[i] = u;
+        const double zx = widen(u.x), zy = widen(u.y) - sc[T_MEANZ];
+        const double2 zs = make_double2(v.psu ? zx + zy : zx, zy);
         if (sc[T_IT] == 0.0) {
             v.p[i] = zs;
         } else {
@@ -519,7 +520,8 @@ struct amg_stack {
     DBuf<StCoarseJob> jobs;
     int max_nc = 0;
     // PCG on the finest level
-    DBuf<double> fin, x, r, z, p, q, fp, zold;
+    DBuf<double> fin, x, r, p, q, fp;
+    DBuf<float> uold;
     DBuf<int> cmem, cbeg, cend, mc0, mc1, nn;
     int nchunks = 0;
     DBuf<double> part, scal;
@@ -844,11 +846,10 @@ int st_create(amg_stack *b, cudaStream_t s)
     BD_TRY(st_vec(b->fin, n2, s));
     BD_TRY(st_vec(b->x, n2, s));
     BD_TRY(st_vec(b->r, n2, s));
-    BD_TRY(st_vec(b->z, n2, s));
     BD_TRY(st_vec(b->p, n2, s));
     BD_TRY(st_vec(b->q, n2, s));
     BD_TRY(st_vec(b->fp, n2, s));
-    if (p32) BD_TRY(st_vec(b->zold, n2, s));
+    if (p32) BD_TRY(st_vec(b->uold, n2, s));
     b->off0.assign(count, 0);
     b->n0.assign(count, 0);
     std::vector<int> cm, cb, ce, m0(count, 0), m1(count, 0), nn(count, 0);
@@ -1011,10 +1012,9 @@ StPcg<S> st_pcg(amg_stack *b)
     v.fp = (double2 *)b->fp.p;
     v.x = (double2 *)b->x.p;
     v.r = (double2 *)b->r.p;
-    v.z = (double2 *)b->z.p;
     v.p = (double2 *)b->p.p;
     v.q = (double2 *)b->q.p;
-    v.zold = b->p32 ? (double2 *)b->zold.p : nullptr;
+    v.uold = b->p32 ? (v2<S> *)b->uold.p : nullptr;
     v.f0 = v0.f;
     v.d0 = v0.d;
     v.u0 = v0.u;

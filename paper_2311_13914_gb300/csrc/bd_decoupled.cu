@@ -106,10 +106,13 @@ __global__ void k_par_direction(int N, const double *__restrict__ dinv, const do
 {
     const double beta = scal[S_BETA];
     const bool first = scal[S_IT] == 0.0;
-    for (int i = share_lo(N) + threadIdx.x, e = share_hi(N); i < e; i += blockDim.x) {
-        const double z = dinv[i] * r[i];
-        p[i] = first ? z : fma(beta, p[i], z);
-    }
+    struct In {
+        double d, r, p;
+    };
+    share_stream(N, [&](int i) { return In{dinv[i], r[i], p[i]}; }, [&](int i, const In &q) {
+        const double z = q.d * q.r;
+        p[i] = first ? z : fma(beta, q.p, z);
+    });
 }
 
 // v += alpha p, r -= alpha q; partials r.r, r.D^{-1}r
@@ -117,15 +120,18 @@ __global__ void k_par_update(int N, const double *__restrict__ p, const double *
                              const double *__restrict__ dinv, double *__restrict__ v, double *__restrict__ r, Fin fin)
 {
     const double alpha = fin.scal[S_ALPHA];
+    struct In {
+        double p, q, d, v, r;
+    };
     double rr = 0.0, rz = 0.0;
     if (fin.scal[S_BREAK] == 0.0)
-        for (int i = share_lo(N) + threadIdx.x, e = share_hi(N); i < e; i += blockDim.x) {
-            v[i] = fma(alpha, p[i], v[i]);
-            const double rv = fma(-alpha, q[i], r[i]);
+        share_stream(N, [&](int i) { return In{p[i], q[i], dinv[i], v[i], r[i]}; }, [&](int i, const In &k) {
+            v[i] = fma(alpha, k.p, k.v);
+            const double rv = fma(-alpha, k.q, k.r);
             r[i] = rv;
             rr += rv * rv;
-            rz += rv * (dinv[i] * rv);
-        }
+            rz += rv * (k.d * rv);
+        });
     block_finish<2>(rr, rz, 0.0, 0.0, fin);
 }
 
