@@ -132,9 +132,10 @@ __global__ void k_strength_fill(int N, const int *__restrict__ rp, const int *__
 template <int BS>
 __global__ void k_spgemm_count(int nrows, const int *__restrict__ arp, const int *__restrict__ aci,
                                const int *__restrict__ brp, const int *__restrict__ bci, int ncols,
-                               int *__restrict__ mark_all, int *__restrict__ cnt)
+                               int *__restrict__ mark_all, int *__restrict__ cnt, int *longest)
 {
     __shared__ int count;
+    int most = 0;
     int *mark = mark_all + (size_t)blockIdx.x * ncols;
     for (int i = blockIdx.x; i < nrows; i += gridDim.x) {
         if (threadIdx.x == 0) count = 0;
@@ -148,8 +149,10 @@ __global__ void k_spgemm_count(int nrows, const int *__restrict__ arp, const int
         }
         __syncthreads();
         if (threadIdx.x == 0) cnt[i] = count;
+        most = max(most, count);
         __syncthreads();
     }
+    if (threadIdx.x == 0 && most > 0) atomicMax(longest, most);
 }
 
 template <int BS>
@@ -231,6 +234,135 @@ __global__ void k_spgemm_fill(int nrows, const int *__restrict__ arp, const int 
     (void)P2;
 }
 
+// The middles [t, te) of an output row, one at a time: the block a of A and the
+// entry of B's row that a thread of offset `off` takes first, with the loads of
+// the following middles in flight (column of the third, range of the second,
+// entry of the next): three dependent loads from L2 would otherwise stand between
+// a middle's products and the next's.
+template <int BS> struct MidWalk {
+    static constexpr int BB = BS * BS;
+    const int *__restrict__ aci;
+    const double *__restrict__ av;
+    const int *__restrict__ brp;
+    const int *__restrict__ bci;
+    const double *__restrict__ bv;
+    int t, te, off;
+    int s0, s1, j;          // this middle
+    double a[BB], b[BB];
+    int n0, n1, jn;         // the next one
+    double an[BB], bn[BB];
+    int m0, m1, k3;         // range of the second, column of the third
+
+    static __device__ __forceinline__ void load(const double *__restrict__ v, size_t at, double (&o)[BB])
+    {
+        if constexpr (BS == 2) {
+            const double2 x = ((const double2 *)v)[2 * at], y = ((const double2 *)v)[2 * at + 1];
+            o[0] = x.x;
+            o[1] = x.y;
+            o[2] = y.x;
+            o[3] = y.y;
+        } else {
+            o[0] = v[at];
+        }
+    }
+    __device__ __forceinline__ int column(int q) const { return q < te ? aci[q] : -1; }
+    __device__ __forceinline__ void range(int k, int &b0, int &b1) const
+    {
+        b0 = k >= 0 ? brp[k] : 0;
+        b1 = k >= 0 ? brp[k + 1] : 0;
+    }
+    __device__ __forceinline__ void entry(int q, int b0, int b1, int &jj, double (&aa)[BB], double (&bb)[BB]) const
+    {
+        if (q < te) load(av, (size_t)q, aa);
+        if (b0 + off < b1) {
+            jj = bci[b0 + off];
+            load(bv, (size_t)(b0 + off), bb);
+        }
+    }
+    __device__ __forceinline__ void start(int t_, int te_, int off_)
+    {
+        t = t_;
+        te = te_;
+        off = off_;
+        const int k0 = column(t), k1 = column(t + 1), k2 = column(t + 2);
+        k3 = column(t + 3);
+        range(k0, s0, s1);
+        range(k1, n0, n1);
+        range(k2, m0, m1);
+        j = jn = 0;
+        entry(t, s0, s1, j, a, b);
+        entry(t + 1, n0, n1, jn, an, bn);
+    }
+    __device__ __forceinline__ void next()
+    {
+        t++;
+        s0 = n0;
+        s1 = n1;
+        j = jn;
+#pragma unroll
+        for (int e = 0; e < BB; e++) {
+            a[e] = an[e];
+            b[e] = bn[e];
+        }
+        n0 = m0;
+        n1 = m1;
+        range(k3, m0, m1);
+        k3 = column(t + 3);
+        entry(t + 1, n0, n1, jn, an, bn);
+    }
+    // f(column, block of B) for this middle's entries off, off + stride, ...
+    template <class F> __device__ __forceinline__ void entries(int stride, F &&f) const
+    {
+        int q = s0 + off, jc = j;
+        if (q >= s1) return;
+        double bc[BB];
+#pragma unroll
+        for (int e = 0; e < BB; e++) bc[e] = b[e];
+        for (;;) {
+            const int q2 = q + stride;
+            const bool more = q2 < s1;
+            int j2 = 0;
+            double b2[BB];
+            if (more) {
+                j2 = bci[q2];
+                load(bv, (size_t)q2, b2);
+            }
+            f(jc, bc);
+            if (!more) break;
+            jc = j2;
+#pragma unroll
+            for (int e = 0; e < BB; e++) bc[e] = b2[e];
+            q = q2;
+        }
+    }
+};
+
+// c (+)= a b in the order of the scalar middle index (2k, then 2k + 1); fresh:
+// from zero.  c's elements are `plane` apart.
+template <int BS>
+__device__ __forceinline__ void block_mac(double *c, int plane, const double (&a)[BS * BS], const double (&b)[BS * BS],
+                                          bool fresh)
+{
+    constexpr int BB = BS * BS;
+    double v[BB];
+#pragma unroll
+    for (int e = 0; e < BB; e++) v[e] = fresh ? 0.0 : c[(size_t)e * plane];
+    if (BS == 1) {
+        v[0] = v[0] + a[0] * b[0];
+    } else {
+        v[0] = v[0] + a[0] * b[0];
+        v[1] = v[1] + a[0] * b[1];
+        v[2] = v[2] + a[2] * b[0];
+        v[3] = v[3] + a[2] * b[1];
+        v[0] = v[0] + a[1] * b[2];
+        v[1] = v[1] + a[1] * b[3];
+        v[2] = v[2] + a[3] * b[2];
+        v[3] = v[3] + a[3] * b[3];
+    }
+#pragma unroll
+    for (int e = 0; e < BB; e++) c[(size_t)e * plane] = v[e];
+}
+
 // Dense path with the row's accumulators and column marks in shared memory
 // (coarse levels: few columns), otherwise identical to k_spgemm_count /
 // k_spgemm_fill: a block per output row, every entry accumulated in ascending
@@ -239,8 +371,9 @@ __global__ void k_spgemm_fill(int nrows, const int *__restrict__ arp, const int 
 // the fill.
 __global__ void k_spgemm_count_smem(int nrows, const int *__restrict__ arp, const int *__restrict__ aci,
                                     const int *__restrict__ brp, const int *__restrict__ bci, int ncols,
-                                    int *__restrict__ cnt)
+                                    int *__restrict__ cnt, int *longest)
 {
+    int most = 0;
     extern __shared__ int smark[];
     __shared__ int count;
     for (int j = threadIdx.x; j < ncols; j += blockDim.x) smark[j] = -1;
@@ -257,8 +390,10 @@ __global__ void k_spgemm_count_smem(int nrows, const int *__restrict__ arp, cons
         }
         __syncthreads();
         if (threadIdx.x == 0) cnt[i] = count;
+        most = max(most, count);
         __syncthreads();
     }
+    if (threadIdx.x == 0 && most > 0) atomicMax(longest, most);
 }
 
 template <int BS>
@@ -277,35 +412,16 @@ __global__ void k_spgemm_fill_smem(int nrows, const int *__restrict__ arp, const
     for (int i = blockIdx.x; i < nrows; i += gridDim.x) {
         if (threadIdx.x == 0) count = 0;
         __syncthreads();
-        for (int t = arp[i]; t < arp[i + 1]; t++) {
-            int k = aci[t];
-            double a[BB];
-#pragma unroll
-            for (int e = 0; e < BB; e++) a[e] = av[(size_t)t * BB + e];
-            for (int s2 = brp[k] + threadIdx.x; s2 < brp[k + 1]; s2 += blockDim.x) {
-                int j = bci[s2];
-                double *c = sacc + (size_t)j * BB;
-                if (mark[j] != i) {
+        MidWalk<BS> w{aci, av, brp, bci, bv};
+        for (w.start(arp[i], arp[i + 1], threadIdx.x); w.t < w.te; w.next()) {
+            w.entries(blockDim.x, [&](int j, const double (&b)[BB]) {
+                const bool fresh = mark[j] != i;
+                if (fresh) {
                     mark[j] = i;
-#pragma unroll
-                    for (int e = 0; e < BB; e++) c[e] = 0.0;
                     cols[atomicAdd(&count, 1)] = j;
                 }
-                const double *b = bv + (size_t)s2 * BB;
-                if (BS == 1) {
-                    c[0] = c[0] + a[0] * b[0];
-                } else {
-                    // scalar middle index 2k then 2k+1
-                    c[0] = c[0] + a[0] * b[0];
-                    c[0] = c[0] + a[1] * b[2];
-                    c[1] = c[1] + a[0] * b[1];
-                    c[1] = c[1] + a[1] * b[3];
-                    c[2] = c[2] + a[2] * b[0];
-                    c[2] = c[2] + a[3] * b[2];
-                    c[3] = c[3] + a[2] * b[1];
-                    c[3] = c[3] + a[3] * b[3];
-                }
-            }
+                block_mac<BS>(sacc + j, ncols, w.a, b, fresh);
+            });
             __syncthreads();
         }
         int n = count;
@@ -333,7 +449,7 @@ __global__ void k_spgemm_fill_smem(int nrows, const int *__restrict__ arp, const
             int j = cols[x];
             cci[base + x] = j;
 #pragma unroll
-            for (int e = 0; e < BB; e++) cv[(size_t)(base + x) * BB + e] = sacc[(size_t)j * BB + e];
+            for (int e = 0; e < BB; e++) cv[(size_t)(base + x) * BB + e] = sacc[(size_t)e * ncols + j];
         }
         __syncthreads();
     }
@@ -344,7 +460,8 @@ __global__ void k_spgemm_fill_smem(int nrows, const int *__restrict__ arp, const
 // addressing in shared memory, the same accumulation order.
 __device__ __forceinline__ int hslot(int key, int mask) { return (int)(((unsigned)key * 2654435761u) & (unsigned)mask); }
 
-// eight lanes per row (rows of hundreds of blocks: a thread's chain of loads)
+// Largest number of products of a row; eight lanes per row (rows of hundreds of
+// blocks: a thread's chain of loads).
 __global__ void k_spgemm_bound(int nrows, const int *__restrict__ arp, const int *__restrict__ aci,
                                const int *__restrict__ brp, int *__restrict__ ub)
 {
@@ -353,7 +470,8 @@ __global__ void k_spgemm_bound(int nrows, const int *__restrict__ arp, const int
     if (i < nrows)
         for (int t = arp[i] + l; t < arp[i + 1]; t += 8) u += brp[aci[t] + 1] - brp[aci[t]];
     for (int o = 4; o; o >>= 1) u += __shfl_xor_sync(0xffffffffu, u, o);
-    if (i < nrows && l == 0) ub[i] = u > INT_MAX ? INT_MAX : (int)u;
+    const int m = __reduce_max_sync(0xffffffffu, u > INT_MAX ? INT_MAX : (int)u);
+    if ((threadIdx.x & 31) == 0 && m > 0) atomicMax(ub, m);
 }
 
 // Hash-path SpGEMM: L lanes per output row, 32/L rows per warp (L from the
@@ -370,38 +488,65 @@ __device__ __forceinline__ unsigned sub_mask(int lane)
 template <int L>
 __global__ void k_spgemm_count_hash(int nrows, const int *__restrict__ arp, const int *__restrict__ aci,
                                     const int *__restrict__ brp, const int *__restrict__ bci, int HC,
-                                    int *__restrict__ cnt, int *overflow)
+                                    int *__restrict__ cnt, int *overflow, int *longest)
 {
     constexpr int R = 32 / L;
     extern __shared__ int hk[];
     const int warps = blockDim.x >> 5, wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int sub = lane / L, sl = lane % L;
+    int most = 0;
     int *keys = hk + ((size_t)wid * R + sub) * HC;
     for (int base = (blockIdx.x * warps + wid) * R; base < nrows; base += gridDim.x * warps * R) {
         const int i = base + sub;
         for (int x = sl; x < HC; x += L) keys[x] = -1;
         __syncwarp();
         int c = 0;
+        bool full = false;
         if (i < nrows) {
-            for (int t = arp[i]; t < arp[i + 1]; t++) {
-                int k = aci[t];
-                for (int s2 = brp[k] + sl; s2 < brp[k + 1]; s2 += L) {
-                    int j = bci[s2], h = hslot(j, HC - 1), probe = 0;
+            // the columns of the middles after this one, as MidWalk
+            const int te = arp[i + 1];
+            int t = arp[i];
+            auto column = [&](int q) { return q < te ? aci[q] : -1; };
+            auto first = [&](int b0, int b1) { return b0 + sl < b1 ? bci[b0 + sl] : 0; };
+            const int k0 = column(t), k1 = column(t + 1), k2 = column(t + 2);
+            int k3 = column(t + 3);
+            int s0 = k0 >= 0 ? brp[k0] : 0, s1 = k0 >= 0 ? brp[k0 + 1] : 0;
+            int n0 = k1 >= 0 ? brp[k1] : 0, n1 = k1 >= 0 ? brp[k1 + 1] : 0;
+            int m0 = k2 >= 0 ? brp[k2] : 0, m1 = k2 >= 0 ? brp[k2 + 1] : 0;
+            int j = first(s0, s1), jn = first(n0, n1);
+            for (; t < te; t++) {
+                for (int q = s0 + sl; q < s1 && !full; q += L) {
+                    const int j2 = q + L < s1 ? bci[q + L] : 0;
+                    int h = hslot(j, HC - 1), probe = 0;
                     for (; probe < HC; probe++) {
                         int old = atomicCAS(&keys[h], -1, j);
                         if (old == -1) { c++; break; }
                         if (old == j) break;
                         h = (h + 1) & (HC - 1);
                     }
-                    if (probe == HC) atomicOr(overflow, 1);
+                    full = probe == HC;
+                    j = j2;
                 }
+                s0 = n0;
+                s1 = n1;
+                j = jn;
+                n0 = m0;
+                n1 = m1;
+                m0 = k3 >= 0 ? brp[k3] : 0;
+                m1 = k3 >= 0 ? brp[k3 + 1] : 0;
+                k3 = column(t + 4);
+                jn = first(n0, n1);
             }
+            if (full) atomicOr(overflow, 1);
         }
 #pragma unroll
         for (int o = L / 2; o; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o, L);
         if (i < nrows && sl == 0) cnt[i] = c;
+        most = max(most, c);
         __syncwarp();
     }
+    most = __reduce_max_sync(0xffffffffu, most);
+    if (lane == 0 && most > 0) atomicMax(longest, most);
 }
 
 template <int BS, int L>
@@ -431,41 +576,20 @@ __global__ void k_spgemm_fill_hash(int nrows, const int *__restrict__ arp, const
         int tmax = tn;
 #pragma unroll
         for (int o = 16; o; o >>= 1) tmax = max(tmax, __shfl_xor_sync(0xffffffffu, tmax, o));
-        for (int tt = 0; tt < tmax; tt++) {
-            if (tt < tn) {
-                const int t = t0 + tt;
-                const int k = aci[t];
-                double a[BB];
-#pragma unroll
-                for (int e = 0; e < BB; e++) a[e] = av[(size_t)t * BB + e];
-                for (int s2 = brp[k] + sl; s2 < brp[k + 1]; s2 += L) {
-                    int j = bci[s2], h = hslot(j, HC - 1);
-                    for (int probe = 0; probe < HC; probe++) {
-                        int old = atomicCAS(&keys[h], -1, j);
-                        if (old == -1) {
-#pragma unroll
-                            for (int e = 0; e < BB; e++) acc[(size_t)h * BB + e] = 0.0;
-                            break;
-                        }
-                        if (old == j) break;
-                        h = (h + 1) & (HC - 1);
-                    }
-                    double *c = acc + (size_t)h * BB;
-                    const double *b = bv + (size_t)s2 * BB;
-                    if (BS == 1) {
-                        c[0] = c[0] + a[0] * b[0];
-                    } else {
-                        c[0] = c[0] + a[0] * b[0];
-                        c[0] = c[0] + a[1] * b[2];
-                        c[1] = c[1] + a[0] * b[1];
-                        c[1] = c[1] + a[1] * b[3];
-                        c[2] = c[2] + a[2] * b[0];
-                        c[2] = c[2] + a[3] * b[2];
-                        c[3] = c[3] + a[2] * b[1];
-                        c[3] = c[3] + a[3] * b[3];
-                    }
+        MidWalk<BS> w{aci, av, brp, bci, bv};
+        w.start(t0, t0 + tn, sl);
+        for (int tt = 0; tt < tmax; tt++, w.next()) {
+            w.entries(L, [&](int j, const double (&b)[BB]) {
+                int h = hslot(j, HC - 1);
+                bool fresh = false;
+                for (int probe = 0; probe < HC; probe++) {
+                    const int old = atomicCAS(&keys[h], -1, j);
+                    fresh = old == -1;
+                    if (fresh || old == j) break;
+                    h = (h + 1) & (HC - 1);
                 }
-            }
+                block_mac<BS>(acc + h, HC, w.a, b, fresh);
+            });
             __syncwarp();
         }
         // compact the occupied slots, sort them by column, emit
@@ -515,8 +639,55 @@ __global__ void k_spgemm_fill_hash(int nrows, const int *__restrict__ arp, const
             for (int x = sl; x < n; x += L) {
                 cci[cb + x] = sk[x];
 #pragma unroll
-                for (int e = 0; e < BB; e++) cv[(size_t)(cb + x) * BB + e] = acc[(size_t)sp[x] * BB + e];
+                for (int e = 0; e < BB; e++) cv[(size_t)(cb + x) * BB + e] = acc[(size_t)e * HC + sp[x]];
             }
+        }
+        __syncwarp();
+    }
+}
+
+// Dense path by warps: a warp per output row with its own accumulators for all
+// ncols columns and a bit per column that is in use, no barrier between middles and
+// no sort.  For products of many rows onto few columns: two rows and more for every
+// warp the SMs hold, or the slowest row's chain of middles sets the time and a
+// thread block per row is faster (128x128x32's levels: 2718 rows by 971 columns, 402
+// blocks a row, 4.0 ms by blocks, 2.9 by warps; 971 by 971 5.3 by blocks, 7.1 by
+// warps; the FP64 operations take 1.8 and 3.3).
+template <int BS>
+__global__ void k_spgemm_fill_warp(int nrows, const int *__restrict__ arp, const int *__restrict__ aci,
+                                   const double *__restrict__ av, const int *__restrict__ brp,
+                                   const int *__restrict__ bci, const double *__restrict__ bv, int ncols,
+                                   const int *__restrict__ crp, int *__restrict__ cci, double *__restrict__ cv)
+{
+    constexpr int BB = BS * BS;
+    extern __shared__ double wacc[];
+    const int lane = threadIdx.x;
+    const int words = (ncols + 31) >> 5;
+    unsigned *used = (unsigned *)(wacc + (size_t)ncols * BB);
+    for (int x = lane; x < words; x += 32) used[x] = 0u;
+    __syncwarp();
+    for (int i = blockIdx.x; i < nrows; i += gridDim.x) {
+        MidWalk<BS> w{aci, av, brp, bci, bv};
+        for (w.start(arp[i], arp[i + 1], lane); w.t < w.te; w.next()) {
+            w.entries(32, [&](int j, const double (&b)[BB]) {
+                const unsigned bit = 1u << (j & 31);
+                const bool fresh = !(atomicOr(&used[j >> 5], bit) & bit);
+                block_mac<BS>(wacc + j, ncols, w.a, b, fresh);
+            });
+            __syncwarp();
+        }
+        int at = crp[i];
+        for (int x = 0; x < words; x++) {
+            const unsigned m = used[x];
+            __syncwarp();
+            if (m >> lane & 1u) {
+                const int pos = at + __popc(m & ((1u << lane) - 1u)), j = 32 * x + lane;
+                cci[pos] = j;
+#pragma unroll
+                for (int e = 0; e < BB; e++) cv[(size_t)pos * BB + e] = wacc[(size_t)e * ncols + j];
+            }
+            if (lane == 0) used[x] = 0u;
+            at += __popc(m);
         }
         __syncwarp();
     }
@@ -529,6 +700,9 @@ static int pow2_at_least(long long v)
     return p;
 }
 
+// Shared memory of an SM, and how much of it a warp's rows may take: four warps, one
+// per scheduler, keep the FP64 pipe about two thirds busy.
+constexpr size_t kSmemSM = 227u << 10, kWarpRowBytes = 55u << 10;
 constexpr long long kHashProducts = 4096;  // products per row up to which the hash path is used
 
 // Lanes per output row of the hash path: the power of two nearest above the
@@ -540,21 +714,57 @@ static int hash_lanes(double b_per_row)
     return L;
 }
 
+// Warps of a block: as many as fit, unless the rows would then leave SMs without a
+// block (all products of a 48x48x12 slab, 1463 rows on the second level: setup 9.2 -> 8.7 ms,
+// with the launches saved in the scans and maxima).
+static int hash_warps(int nrows, int rows_per_warp, size_t fit)
+{
+    const long long spread = ((long long)nrows + rows_per_warp * kSM - 1) / (rows_per_warp * kSM);
+    return (int)std::max<long long>(1, std::min<long long>({8, (long long)fit, spread}));
+}
+
 template <int L>
 static int launch_count_hash(int nrows, int HCs, const int *arp, const int *aci, const int *brp, const int *bci,
                              int *cnt, int *flag, cudaStream_t s)
 {
     constexpr int R = 32 / L;
     const size_t per_warp = (size_t)R * HCs * 4;
-    const int warps = std::max(1, std::min(8, (int)((192u << 10) / per_warp)));
+    const int warps = hash_warps(nrows, R, (192u << 10) / per_warp);
     const size_t smem = (size_t)warps * per_warp;
     if (smem > (227u << 10)) return BD_ERANGE;
     BD_CUDA(cudaFuncSetAttribute(k_spgemm_count_hash<L>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     const long long rows_per_block = (long long)warps * R;
     const int gb = (int)std::min<long long>(kSM * 8, std::max<long long>(1, (nrows + rows_per_block - 1) / rows_per_block));
-    k_spgemm_count_hash<L><<<gb, 32 * warps, smem, s>>>(nrows, arp, aci, brp, bci, HCs, cnt, flag); ::bd::note_launch();
+    k_spgemm_count_hash<L><<<gb, 32 * warps, smem, s>>>(nrows, arp, aci, brp, bci, HCs, cnt, flag, flag + 2);
+    ::bd::note_launch();
     BD_LAUNCH_CHECK();
     return BD_OK;
+}
+
+// Table of the count pass: half full at most for rows of n columns.
+static int count_table(long long n)
+{
+    return std::max(32, pow2_at_least(2 * std::min<long long>(n, kMaxSortSeg)));
+}
+
+// Row lengths by hashing.  The bound on a row's products is several times its length
+// (the products of A P meet four to a column, those of R (A P) tens), and tables of
+// that size leave room for a few rows per SM only, so the first attempt takes
+// tables for a quarter of it; flag[0] tells that some row did not fit.
+static int count_hash_rows(int nrows, int HCs, int lanes, const int *arp, const int *aci, const int *brp,
+                           const int *bci, int *cnt, int *flag, cudaStream_t s)
+{
+    // rows whose tables do not fit 32/lanes to a warp take more lanes each
+    int Lc = lanes;
+    while (Lc < 32 && (size_t)(32 / Lc) * HCs * 4 > (192u << 10)) Lc <<= 1;
+    switch (Lc) {
+    case 1: return launch_count_hash<1>(nrows, HCs, arp, aci, brp, bci, cnt, flag, s);
+    case 2: return launch_count_hash<2>(nrows, HCs, arp, aci, brp, bci, cnt, flag, s);
+    case 4: return launch_count_hash<4>(nrows, HCs, arp, aci, brp, bci, cnt, flag, s);
+    case 8: return launch_count_hash<8>(nrows, HCs, arp, aci, brp, bci, cnt, flag, s);
+    case 16: return launch_count_hash<16>(nrows, HCs, arp, aci, brp, bci, cnt, flag, s);
+    default: return launch_count_hash<32>(nrows, HCs, arp, aci, brp, bci, cnt, flag, s);
+    }
 }
 
 template <int BS, int L>
@@ -565,7 +775,7 @@ static int launch_fill_hash(int nrows, int HCn, const int *arp, const int *aci, 
     const size_t per = ((size_t)HCn * BS * BS + (size_t)(3 * HCn + 1) / 2) * sizeof(double);
     const size_t per_warp = (size_t)R * per;
     if (per_warp > (200u << 10)) return BD_ERANGE;
-    const int warps = std::max(1, std::min(8, (int)((200u << 10) / per_warp)));
+    const int warps = hash_warps(nrows, R, (200u << 10) / per_warp);
     const size_t smem = per_warp * warps;
     BD_CUDA(cudaFuncSetAttribute(k_spgemm_fill_hash<BS, L>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     const long long rows_per_block = (long long)warps * R;
@@ -606,16 +816,14 @@ static int spgemm(int nrows, int ncols, const int *arp, const int *aci, const do
     // accumulate every entry in the same order, so the choice changes no bit.
     long long mub = 1;
     if (nrows > 0) {
-        k_spgemm_bound<<<(nrows + 31) / 32, 256, 0, s>>>(nrows, arp, aci, brp, cnt.p); ::bd::note_launch();
+        k_spgemm_bound<<<(nrows + 31) / 32, 256, 0, s>>>(nrows, arp, aci, brp, flag.p + 1); ::bd::note_launch();
         BD_LAUNCH_CHECK();
-        BD_TRY(device_max(cnt.p, nrows, flag.p + 1, s));
         int hb = 0;
         BD_CUDA(cudaMemcpyAsync(&hb, flag.p + 1, sizeof(int), cudaMemcpyDeviceToHost, s));
         BD_CUDA(cudaStreamSynchronize(s));
         mub = std::max<long long>(mub, hb);
         if (mub <= kHashProducts) dense = false;
     }
-    int HCn = 0;
     const int lanes = hash_lanes(b_per_row);
     ::bd::note_spgemm_path(dense);
     // the dense path keeps a row's accumulators in shared memory when they
@@ -629,42 +837,47 @@ static int spgemm(int nrows, int ncols, const int *arp, const int *aci, const do
                                      (int)std::max<size_t>(cs, 4)));
         const int gc = (int)std::min<long long>(nrows, (long long)kSM * 8);
         k_spgemm_count_smem<<<std::max(gc, 1), 128, std::max<size_t>(cs, 4), s>>>(nrows, arp, aci, brp, bci, ncols,
-                                                                                   cnt.p);
+                                                                                   cnt.p, flag.p + 2);
         ::bd::note_launch();
         BD_LAUNCH_CHECK();
     } else if (dense) {
         BD_TRY(mark.scratch((size_t)grid * ncols, s));
         BD_TRY(acc.scratch((size_t)grid * ncols * BB, s));
         BD_CUDA(cudaMemsetAsync(mark.p, 0xff, mark.bytes(), s));
-        k_spgemm_count<BS><<<grid, 128, 0, s>>>(nrows, arp, aci, brp, bci, ncols, mark.p, cnt.p); ::bd::note_launch();
+        k_spgemm_count<BS><<<grid, 128, 0, s>>>(nrows, arp, aci, brp, bci, ncols, mark.p, cnt.p, flag.p + 2);
+        ::bd::note_launch();
         BD_LAUNCH_CHECK();
     } else {
-        int HCs = pow2_at_least(2 * std::min<long long>(mub, kMaxSortSeg));
-        if (HCs < 32) HCs = 32;
-        // rows whose tables do not fit 32/lanes to a warp take more lanes each
-        int Lc = lanes;
-        while (Lc < 32 && (size_t)(32 / Lc) * HCs * 4 > (192u << 10)) Lc <<= 1;
-        switch (Lc) {
-        case 1: BD_TRY(launch_count_hash<1>(nrows, HCs, arp, aci, brp, bci, cnt.p, flag.p, s)); break;
-        case 2: BD_TRY(launch_count_hash<2>(nrows, HCs, arp, aci, brp, bci, cnt.p, flag.p, s)); break;
-        case 4: BD_TRY(launch_count_hash<4>(nrows, HCs, arp, aci, brp, bci, cnt.p, flag.p, s)); break;
-        case 8: BD_TRY(launch_count_hash<8>(nrows, HCs, arp, aci, brp, bci, cnt.p, flag.p, s)); break;
-        case 16: BD_TRY(launch_count_hash<16>(nrows, HCs, arp, aci, brp, bci, cnt.p, flag.p, s)); break;
-        default: BD_TRY(launch_count_hash<32>(nrows, HCs, arp, aci, brp, bci, cnt.p, flag.p, s)); break;
-        }
+        BD_TRY(count_hash_rows(nrows, count_table(mub / 4), lanes, arp, aci, brp, bci, cnt.p, flag.p, s));
     }
-    BD_TRY(device_max(cnt.p, nrows, flag.p + 2, s));  // cnt: the output row lengths
     long long total = 0;
     BD_TRY(exclusive_scan(cnt.p, crp.p, nrows, &total, s));
     int hf[3] = {0, 0, 0};
     BD_CUDA(cudaMemcpyAsync(hf, flag.p, sizeof(hf), cudaMemcpyDeviceToHost, s));
     BD_CUDA(cudaStreamSynchronize(s));
+    if (hf[0]) {  // a row outgrew the count's first table: once more with one that holds all products
+        BD_CUDA(cudaMemsetAsync(flag.p, 0, 3 * sizeof(int), s));
+        BD_TRY(count_hash_rows(nrows, count_table(mub), lanes, arp, aci, brp, bci, cnt.p, flag.p, s));
+        BD_TRY(exclusive_scan(cnt.p, crp.p, nrows, &total, s));
+        BD_CUDA(cudaMemcpyAsync(hf, flag.p, sizeof(hf), cudaMemcpyDeviceToHost, s));
+        BD_CUDA(cudaStreamSynchronize(s));
+    }
     if (hf[0]) return BD_ERANGE;
     const int maxrow = hf[2];
     if (maxrow > kMaxSortSeg) return BD_ERANGE;
     BD_TRY(scratch ? cci.scratch((size_t)total, s) : cci.alloc((size_t)total));
     BD_TRY(scratch ? cv.scratch((size_t)total * BB, s) : cv.alloc((size_t)total * BB));
-    if (dense_in_smem) {
+    // tables at most three quarters full
+    const int HCn = pow2_at_least(std::max(16LL, 4LL * maxrow / 3 + 1));
+    const size_t hash_row = ((size_t)HCn * BB + (size_t)(3 * HCn + 1) / 2) * sizeof(double);
+    const size_t warp_row = (size_t)ncols * BB * sizeof(double) + (size_t)((ncols + 31) / 32) * sizeof(int);
+    if (dense && warp_row <= kWarpRowBytes && nrows >= 2 * kSM * (long long)(kSmemSM / (warp_row + 1024))) {
+        BD_CUDA(cudaFuncSetAttribute(k_spgemm_fill_warp<BS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)warp_row));
+        const int gw = (int)std::min<long long>(nrows, kSM * 32LL);
+        k_spgemm_fill_warp<BS><<<gw, 32, warp_row, s>>>(nrows, arp, aci, av, brp, bci, bv, ncols, crp.p, cci.p, cv.p);
+        ::bd::note_launch();
+        BD_LAUNCH_CHECK();
+    } else if (dense_in_smem) {
         BD_CUDA(cudaFuncSetAttribute(k_spgemm_fill_smem<BS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      (int)dense_smem));
         const int per_sm = std::max(1, (int)((227u << 10) / (dense_smem + 1024)));
@@ -683,12 +896,9 @@ static int spgemm(int nrows, int ncols, const int *arp, const int *aci, const do
                                                   acc.p, crp.p, cci.p, cv.p, P2); ::bd::note_launch();
         BD_LAUNCH_CHECK();
     } else {
-        HCn = pow2_at_least(2LL * std::max(maxrow, 16));
         // rows whose tables do not fit 32/lanes to a warp take more lanes each
         int Lf = lanes;
-        while (Lf < 32 && (size_t)(32 / Lf) * (((size_t)HCn * BB + (size_t)(3 * HCn + 1) / 2) * sizeof(double)) >
-                              (200u << 10))
-            Lf <<= 1;
+        while (Lf < 32 && (size_t)(32 / Lf) * hash_row > kWarpRowBytes) Lf <<= 1;
         switch (Lf) {
         case 1: BD_TRY((launch_fill_hash<BS, 1>(nrows, HCn, arp, aci, av, brp, bci, bv, crp.p, cci.p, cv.p, s))); break;
         case 2: BD_TRY((launch_fill_hash<BS, 2>(nrows, HCn, arp, aci, av, brp, bci, bv, crp.p, cci.p, cv.p, s))); break;

@@ -127,47 +127,54 @@ __global__ void k_scan_sums(long long *sums, int ntiles, long long *total)
     if (threadIdx.x == 0) *total = carry;
 }
 
-__global__ void k_scan_add(int *out, int n, const long long *tile_off, const long long *total,
-                           int *overflow)
+// Adds a tile's offset: the sum of the tiles before it, which every block forms
+// itself (scanned: sums already holds the offsets).
+__global__ void k_scan_add(int *out, int n, const long long *sums, bool scanned, long long *total)
 {
-    long long base = (long long)blockIdx.x * kScanTile;
-    long long off = tile_off[blockIdx.x];
-    for (int k = 0; k < 2; k++) {
-        long long i = base + 2 * threadIdx.x + k;
-        if (i < n) {
-            long long v = off + out[i];
-            if (v > INT_MAX) *overflow = 1;
-            out[i] = (int)v;
-        }
+    __shared__ long long wt[32];
+    __shared__ long long tot;
+    const int b = blockIdx.x;
+    long long off = 0;
+    if (scanned) {
+        off = sums[b];
+    } else {
+        for (int i = threadIdx.x; i < b; i += blockDim.x) off += sums[i];
+        block_exclusive_scan(off, wt, &tot);
+        off = tot;
     }
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-        long long t = *total;
-        if (t > INT_MAX) *overflow = 1;
+    const long long base = (long long)b * kScanTile;
+    for (int k = 0; k < 2; k++) {
+        const long long i = base + 2 * threadIdx.x + k;
+        if (i < n) out[i] = (int)(off + out[i]);
+    }
+    if (b == (int)gridDim.x - 1 && threadIdx.x == 0) {
+        const long long t = scanned ? *total : off + sums[b];
+        *total = t;
         out[n] = (int)(t > INT_MAX ? INT_MAX : t);
     }
 }
+
+constexpr int kScanDirect = 4096;  // tiles up to which every block adds up its own offset
 
 int exclusive_scan(const int *in, int *out, int n, long long *total, cudaStream_t s)
 {
     int ntiles = (n + kScanTile - 1) / kScanTile;
     if (ntiles < 1) ntiles = 1;
     DBuf<long long> sums;
-    DBuf<int> flag;
     BD_TRY(sums.scratch((size_t)ntiles + 1, s));
-    BD_TRY(flag.scratch(1, s));
-    BD_CUDA(cudaMemsetAsync(flag.p, 0, sizeof(int), s));
     k_scan_tiles<<<ntiles, kScanThreads, 0, s>>>(in, out, n, sums.p); ::bd::note_launch();
     BD_LAUNCH_CHECK();
-    k_scan_sums<<<1, kScanThreads, 0, s>>>(sums.p, ntiles, sums.p + ntiles); ::bd::note_launch();
-    BD_LAUNCH_CHECK();
-    k_scan_add<<<ntiles, kScanThreads, 0, s>>>(out, n, sums.p, sums.p + ntiles, flag.p); ::bd::note_launch();
+    const bool scanned = ntiles > kScanDirect;
+    if (scanned) {
+        k_scan_sums<<<1, kScanThreads, 0, s>>>(sums.p, ntiles, sums.p + ntiles); ::bd::note_launch();
+        BD_LAUNCH_CHECK();
+    }
+    k_scan_add<<<ntiles, kScanThreads, 0, s>>>(out, n, sums.p, scanned, sums.p + ntiles); ::bd::note_launch();
     BD_LAUNCH_CHECK();
     long long t = 0;
-    int of = 0;
     BD_CUDA(cudaMemcpyAsync(&t, sums.p + ntiles, sizeof(t), cudaMemcpyDeviceToHost, s));
-    BD_CUDA(cudaMemcpyAsync(&of, flag.p, sizeof(int), cudaMemcpyDeviceToHost, s));
     BD_CUDA(cudaStreamSynchronize(s));
-    if (of) return BD_ERANGE;
+    if (t > INT_MAX) return BD_ERANGE;  // (counts are not negative, so no offset exceeds the total)
     if (total) *total = t;
     return BD_OK;
 }
