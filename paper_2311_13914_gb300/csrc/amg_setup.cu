@@ -337,6 +337,100 @@ template <int BS> struct MidWalk {
     }
 };
 
+// The same for 2x2 blocks by groups of four lanes, lane e of a group forming element e
+// of its entry's product: group `grp` of the row's G takes entries grp, grp + G, ...
+struct MidWalkElem {
+    const int *__restrict__ aci;
+    const double *__restrict__ av;
+    const int *__restrict__ brp;
+    const int *__restrict__ bci;
+    const double *__restrict__ bv;
+    int t, te, grp, e;
+    int s0, s1, j;
+    double2 a;              // the row of a that element e needs
+    double b0, b1;          // and the column of b
+    int n0, n1, jn;
+    double2 an;
+    double bn0, bn1;
+    int m0, m1, k3;
+
+    __device__ __forceinline__ int column(int q) const { return q < te ? aci[q] : -1; }
+    __device__ __forceinline__ void range(int k, int &r0, int &r1) const
+    {
+        r0 = k >= 0 ? brp[k] : 0;
+        r1 = k >= 0 ? brp[k + 1] : 0;
+    }
+    __device__ __forceinline__ void block(int q, int &jj, double &x, double &y) const
+    {
+        jj = bci[q];
+        const double *b = bv + 4 * (size_t)q + (e & 1);
+        x = b[0];
+        y = b[2];
+    }
+    __device__ __forceinline__ void entry(int q, int r0, int r1, int &jj, double2 &aa, double &x, double &y) const
+    {
+        if (q < te) aa = ((const double2 *)av)[2 * (size_t)q + (e >> 1)];
+        if (r0 + grp < r1) block(r0 + grp, jj, x, y);
+    }
+    __device__ __forceinline__ void start(int t_, int te_, int grp_, int e_)
+    {
+        t = t_;
+        te = te_;
+        grp = grp_;
+        e = e_;
+        const int k0 = column(t), k1 = column(t + 1), k2 = column(t + 2);
+        k3 = column(t + 3);
+        range(k0, s0, s1);
+        range(k1, n0, n1);
+        range(k2, m0, m1);
+        j = jn = 0;
+        a = an = make_double2(0.0, 0.0);
+        b0 = b1 = bn0 = bn1 = 0.0;
+        entry(t, s0, s1, j, a, b0, b1);
+        entry(t + 1, n0, n1, jn, an, bn0, bn1);
+    }
+    __device__ __forceinline__ void next()
+    {
+        t++;
+        s0 = n0;
+        s1 = n1;
+        j = jn;
+        a = an;
+        b0 = bn0;
+        b1 = bn1;
+        n0 = m0;
+        n1 = m1;
+        range(k3, m0, m1);
+        k3 = column(t + 3);
+        entry(t + 1, n0, n1, jn, an, bn0, bn1);
+    }
+    // f(has an entry, column, b) by all lanes together
+    template <class F> __device__ __forceinline__ void entries(int G, F &&f) const
+    {
+        int q = s0 + grp, jc = j;
+        double x = b0, y = b1;
+        for (int base = s0; base < s1; base += G) {
+            const int q2 = q + G;
+            int j2 = 0;
+            double x2 = 0.0, y2 = 0.0;
+            if (q2 < s1) block(q2, j2, x2, y2);
+            f(q < s1, jc, x, y);
+            q = q2;
+            jc = j2;
+            x = x2;
+            y = y2;
+        }
+    }
+    // element e of c + a b, or of a b (fresh), in the order of block_mac
+    __device__ __forceinline__ double mac(double c, bool fresh, double x, double y) const
+    {
+        double v = fresh ? 0.0 : c;
+        v = v + a.x * x;
+        v = v + a.y * y;
+        return v;
+    }
+};
+
 // c (+)= a b in the order of the scalar middle index (2k, then 2k + 1); fresh:
 // from zero.  c's elements are `plane` apart.
 template <int BS>
@@ -412,17 +506,38 @@ __global__ void k_spgemm_fill_smem(int nrows, const int *__restrict__ arp, const
     for (int i = blockIdx.x; i < nrows; i += gridDim.x) {
         if (threadIdx.x == 0) count = 0;
         __syncthreads();
-        MidWalk<BS> w{aci, av, brp, bci, bv};
-        for (w.start(arp[i], arp[i + 1], threadIdx.x); w.t < w.te; w.next()) {
-            w.entries(blockDim.x, [&](int j, const double (&b)[BB]) {
-                const bool fresh = mark[j] != i;
-                if (fresh) {
-                    mark[j] = i;
-                    cols[atomicAdd(&count, 1)] = j;
-                }
-                block_mac<BS>(sacc + j, ncols, w.a, b, fresh);
-            });
-            __syncthreads();
+        if constexpr (BS == 2) {
+            MidWalkElem w{aci, av, brp, bci, bv};
+            const int lane = threadIdx.x & 31, e = threadIdx.x & 3;
+            for (w.start(arp[i], arp[i + 1], threadIdx.x >> 2, e); w.t < w.te; w.next()) {
+                w.entries(blockDim.x >> 2, [&](bool on, int j, double x, double y) {
+                    bool fresh = false;
+                    if (on && e == 0) {
+                        fresh = mark[j] != i;
+                        if (fresh) {
+                            mark[j] = i;
+                            cols[atomicAdd(&count, 1)] = j;
+                        }
+                    }
+                    fresh = __shfl_sync(0xffffffffu, (int)fresh, lane & ~3);
+                    double *c = sacc + 4 * (size_t)j + e;
+                    if (on) *c = w.mac(*c, fresh, x, y);
+                });
+                __syncthreads();
+            }
+        } else {
+            MidWalk<BS> w{aci, av, brp, bci, bv};
+            for (w.start(arp[i], arp[i + 1], threadIdx.x); w.t < w.te; w.next()) {
+                w.entries(blockDim.x, [&](int j, const double (&b)[BB]) {
+                    const bool fresh = mark[j] != i;
+                    if (fresh) {
+                        mark[j] = i;
+                        cols[atomicAdd(&count, 1)] = j;
+                    }
+                    block_mac<BS>(sacc + j, 1, w.a, b, fresh);
+                });
+                __syncthreads();
+            }
         }
         int n = count;
         int p2 = 1;
@@ -449,7 +564,7 @@ __global__ void k_spgemm_fill_smem(int nrows, const int *__restrict__ arp, const
             int j = cols[x];
             cci[base + x] = j;
 #pragma unroll
-            for (int e = 0; e < BB; e++) cv[(size_t)(base + x) * BB + e] = sacc[(size_t)e * ncols + j];
+            for (int e = 0; e < BB; e++) cv[(size_t)(base + x) * BB + e] = sacc[(size_t)j * BB + e];
         }
         __syncthreads();
     }
@@ -646,6 +761,98 @@ __global__ void k_spgemm_fill_hash(int nrows, const int *__restrict__ arp, const
     }
 }
 
+// Hash path with a warp per row and four lanes per product (MidWalkElem): eight
+// products at a time in four FP64 instructions, where a lane per product takes
+// sixteen for up to 32 and leaves most lanes idle on rows of B of 7 to 20 blocks, and
+// half of one row's chain of middles.  128x128x32: the finest A P (rows of B of 6.8
+// blocks) 6.6 -> 5.2 ms, R (A P) 4.9 -> 4.0, the next level's 3.1 -> 2.4 (the FP64
+// operations at full lanes take 2.5, 2.0 and 1.2); 48x48x12, 1463 rows of 120
+// middles: 0.76 -> 0.48.  A thread block per row gains the same way (39.5 M products of
+// 2718 rows 2.6 -> 2.1).
+__global__ void __launch_bounds__(256, 3) k_spgemm_fill_elem(int nrows, const int *__restrict__ arp,
+                                                          const int *__restrict__ aci, const double *__restrict__ av,
+                                                          const int *__restrict__ brp, const int *__restrict__ bci,
+                                                          const double *__restrict__ bv, int HC,
+                                                          const int *__restrict__ crp, int *__restrict__ cci,
+                                                          double *__restrict__ cv)
+{
+    extern __shared__ double hs[];
+    const int warps = blockDim.x >> 5, wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int grp = lane >> 2, e = lane & 3;
+    const size_t per = (size_t)HC * 4 + (size_t)(3 * HC + 1) / 2;  // in doubles
+    double *acc = hs + (size_t)wid * per;
+    int *keys = (int *)(acc + (size_t)HC * 4);
+    int *sk = keys + HC, *sp = sk + HC;
+    for (int i = blockIdx.x * warps + wid; i < nrows; i += gridDim.x * warps) {
+        for (int x = lane; x < HC; x += 32) keys[x] = -1;
+        __syncwarp();
+        MidWalkElem w{aci, av, brp, bci, bv};
+        for (w.start(arp[i], arp[i + 1], grp, e); w.t < w.te; w.next()) {
+            w.entries(8, [&](bool on, int j, double x, double y) {
+                int h = 0;
+                if (on && e == 0) {
+                    h = hslot(j, HC - 1);
+                    for (int probe = 0; probe < HC; probe++) {
+                        const int old = atomicCAS(&keys[h], -1, j);
+                        if (old == -1) {
+                            h |= 1 << 30;
+                            break;
+                        }
+                        if (old == j) break;
+                        h = (h + 1) & (HC - 1);
+                    }
+                }
+                h = __shfl_sync(0xffffffffu, h, lane & ~3);
+                const bool fresh = h >> 30;
+                double *c = acc + 4 * (size_t)(h & (HC - 1)) + e;
+                if (on) *c = w.mac(*c, fresh, x, y);
+            });
+            __syncwarp();
+        }
+        // compact the occupied slots, sort them by column, emit
+        int n = 0;
+        for (int x0 = 0; x0 < HC; x0 += 32) {
+            const int x = x0 + lane;
+            const bool has = x < HC && keys[x] != -1;
+            const unsigned m = __ballot_sync(0xffffffffu, has);
+            if (has) {
+                const int pos = n + __popc(m & ((1u << lane) - 1u));
+                sk[pos] = keys[x];
+                sp[pos] = x;
+            }
+            n += __popc(m);
+        }
+        int p2 = 1;
+        while (p2 < n) p2 <<= 1;
+        for (int x = n + lane; x < p2; x += 32) {
+            sk[x] = INT_MAX;
+            sp[x] = 0;
+        }
+        __syncwarp();
+        for (int kk = 2; kk <= p2; kk <<= 1)
+            for (int jj = kk >> 1; jj > 0; jj >>= 1) {
+                for (int x = lane; x < p2; x += 32) {
+                    const int y = x ^ jj;
+                    if (y > x) {
+                        const int cx = sk[x], cy = sk[y];
+                        if ((cx > cy) == ((x & kk) == 0)) {
+                            sk[x] = cy;
+                            sk[y] = cx;
+                            const int tp = sp[x];
+                            sp[x] = sp[y];
+                            sp[y] = tp;
+                        }
+                    }
+                }
+                __syncwarp();
+            }
+        const int cb = crp[i];
+        for (int x = lane; x < n; x += 32) cci[cb + x] = sk[x];
+        for (int x = lane; x < 4 * n; x += 32) cv[4 * (size_t)cb + x] = acc[4 * (size_t)sp[x >> 2] + (x & 3)];
+        __syncwarp();
+    }
+}
+
 // Dense path by warps: a warp per output row with its own accumulators for all
 // ncols columns and a bit per column that is in use, no barrier between middles and
 // no sort.  For products of many rows onto few columns: two rows and more for every
@@ -786,6 +993,27 @@ static int launch_fill_hash(int nrows, int HCn, const int *arp, const int *aci, 
     return BD_OK;
 }
 
+// 2x2 blocks: rows of B of one or two blocks (a tentative prolongator) keep a lane or two
+// per row, which fills every FP64 instruction (549153 rows 1.8 ms; four lanes per
+// product would take 3.0 for the FP64 operations alone), unless that leaves
+// schedulers without a warp (1463 rows: 0.21 -> 0.08 ms by elements).
+constexpr int kLaneRows = 32 * 4 * kSM;
+
+static int launch_fill_elem(int nrows, int HCn, const int *arp, const int *aci, const double *av, const int *brp,
+                            const int *bci, const double *bv, const int *crp, int *cci, double *cv, cudaStream_t s)
+{
+    const size_t per_warp = ((size_t)HCn * 4 + (size_t)(3 * HCn + 1) / 2) * sizeof(double);
+    if (per_warp > (200u << 10)) return BD_ERANGE;
+    const int warps = hash_warps(nrows, 1, (200u << 10) / per_warp);
+    const size_t smem = per_warp * warps;
+    BD_CUDA(cudaFuncSetAttribute(k_spgemm_fill_elem, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    const int gb = (int)std::min<long long>(kSM * 32, std::max<long long>(1, (nrows + warps - 1) / warps));
+    k_spgemm_fill_elem<<<gb, 32 * warps, smem, s>>>(nrows, arp, aci, av, brp, bci, bv, HCn, crp, cci, cv);
+    ::bd::note_launch();
+    BD_LAUNCH_CHECK();
+    return BD_OK;
+}
+
 // b_per_row: average blocks per row of B (sets the lanes per row of the hash path);
 // scratch: C is scratch of the setup call
 template <int BS>
@@ -896,10 +1124,17 @@ static int spgemm(int nrows, int ncols, const int *arp, const int *aci, const do
                                                   acc.p, crp.p, cci.p, cv.p, P2); ::bd::note_launch();
         BD_LAUNCH_CHECK();
     } else {
+        bool done = false;
+        if constexpr (BS == 2) {
+            if (lanes >= 4 || nrows < kLaneRows) {
+                BD_TRY(launch_fill_elem(nrows, HCn, arp, aci, av, brp, bci, bv, crp.p, cci.p, cv.p, s));
+                done = true;
+            }
+        }
         // rows whose tables do not fit 32/lanes to a warp take more lanes each
         int Lf = lanes;
         while (Lf < 32 && (size_t)(32 / Lf) * hash_row > kWarpRowBytes) Lf <<= 1;
-        switch (Lf) {
+        if (!done) switch (Lf) {
         case 1: BD_TRY((launch_fill_hash<BS, 1>(nrows, HCn, arp, aci, av, brp, bci, bv, crp.p, cci.p, cv.p, s))); break;
         case 2: BD_TRY((launch_fill_hash<BS, 2>(nrows, HCn, arp, aci, av, brp, bci, bv, crp.p, cci.p, cv.p, s))); break;
         case 4: BD_TRY((launch_fill_hash<BS, 4>(nrows, HCn, arp, aci, av, brp, bci, bv, crp.p, cci.p, cv.p, s))); break;
