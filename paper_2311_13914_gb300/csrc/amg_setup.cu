@@ -1202,32 +1202,53 @@ __device__ __forceinline__ bool beats(unsigned long long hp, int p, unsigned lon
     return hp > hq || (hp == hq && p < q);
 }
 
+// Eight lanes per node here and in k_assign (rows of the squared graph hold some 125
+// entries; a thread's walk is a chain of loads: 31213 nodes, select 16.5 -> 6.7 us,
+// exclude 10.6 -> 7.2, assign 28 -> 8).
+struct NodeLanes {
+    int p, l;           // node, lane of the node's eight
+    unsigned mask;      // the node's lanes in the warp
+    __device__ __forceinline__ NodeLanes()
+        : p((int)((blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 3)), l(threadIdx.x & 7),
+          mask(0xffu << (threadIdx.x & 24)) {}
+    // whether f(t) holds for an entry t of [b, e), by all lanes of the warp together
+    template <class F> __device__ __forceinline__ bool any(int b, int e, F &&f) const
+    {
+        bool found = false;
+        for (int t = b + l;; t += 8) {
+            const bool go = !found && t < e;
+            if (!__any_sync(0xffffffffu, go)) break;
+            found = (__ballot_sync(0xffffffffu, go ? f(t) : found) & mask) != 0;
+        }
+        return found;
+    }
+};
+
 __global__ void k_mis_select(int N, const int *__restrict__ srp, const int *__restrict__ sci,
                              unsigned char *state, unsigned long long key)
 {
-    int p = blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= N || state[p] != 0) return;
-    unsigned long long hp = mix64((unsigned long long)p ^ key);
-    for (int t = srp[p]; t < srp[p + 1]; t++) {
-        int q = sci[t];
-        unsigned char sq = ((volatile unsigned char *)state)[q];
-        if (sq == 1) return;
-        if (sq == 0 && beats(mix64((unsigned long long)q ^ key), q, hp, p)) return;
-    }
-    state[p] = 1;
+    const NodeLanes n;
+    const bool act = n.p < N && state[n.p] == 0;
+    const unsigned long long hp = mix64((unsigned long long)n.p ^ key);
+    const bool lost = n.any(act ? srp[n.p] : 0, act ? srp[n.p + 1] : 0, [&](int t) {
+        const int q = sci[t];
+        const unsigned char sq = ((volatile unsigned char *)state)[q];
+        return sq == 1 || (sq == 0 && beats(mix64((unsigned long long)q ^ key), q, hp, n.p));
+    });
+    if (act && n.l == 0 && !lost) state[n.p] = 1;
 }
 
 __global__ void k_mis_exclude(int N, const int *__restrict__ srp, const int *__restrict__ sci,
                               unsigned char *state, int *undecided)
 {
-    int p = blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= N || state[p] != 0) return;
-    for (int t = srp[p]; t < srp[p + 1]; t++)
-        if (state[sci[t]] == 1) {
-            state[p] = 2;
-            return;
-        }
-    atomicAdd(undecided, 1);
+    const NodeLanes n;
+    const bool act = n.p < N && state[n.p] == 0;
+    const bool out = n.any(act ? srp[n.p] : 0, act ? srp[n.p + 1] : 0,
+                           [&](int t) { return ((volatile unsigned char *)state)[sci[t]] == 1; });
+    const bool left = act && n.l == 0 && !out;
+    if (act && n.l == 0 && out) state[n.p] = 2;
+    const unsigned m = __ballot_sync(0xffffffffu, left);
+    if ((threadIdx.x & 31) == 0 && m) atomicAdd(undecided, __popc(m));
 }
 
 // ------------------------------------------------------------------ a3 aggregation
@@ -1244,27 +1265,33 @@ __global__ void k_assign(int N, const int *__restrict__ srp, const int *__restri
                          const double *__restrict__ sw, const unsigned char *__restrict__ mis,
                          const int *__restrict__ root_id, int *__restrict__ agg, int *bad)
 {
-    int p = blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= N) return;
-    if (mis[p]) {
-        agg[p] = root_id[p];
-        return;
-    }
-    int best = -1;
+    const NodeLanes n;
+    const int p = n.p;
+    const bool act = p < N, root = act && mis[p];
+    int best = -1;  // the first entry of the largest weight
     double bw = -1.0;
-    for (int t = srp[p]; t < srp[p + 1]; t++) {
-        int q = sci[t];
-        if (mis[q] && sw[t] > bw) {
+    for (int t = act && !root ? srp[p] + n.l : 0, e = act && !root ? srp[p + 1] : 0; t < e; t += 8)
+        if (mis[sci[t]] && sw[t] > bw) {
             bw = sw[t];
-            best = q;
+            best = t;
+        }
+    for (int o = 4; o; o >>= 1) {
+        const double w2 = __shfl_xor_sync(0xffffffffu, bw, o);
+        const int t2 = __shfl_xor_sync(0xffffffffu, best, o);
+        if (t2 >= 0 && (best < 0 || w2 > bw || (w2 == bw && t2 < best))) {
+            bw = w2;
+            best = t2;
         }
     }
-    if (best < 0) {
+    if (!act || n.l) return;
+    if (root) {
+        agg[p] = root_id[p];
+    } else if (best < 0) {
         *bad = 1;
         agg[p] = 0;
-        return;
+    } else {
+        agg[p] = root_id[sci[best]];
     }
-    agg[p] = root_id[best];
 }
 
 // ------------------------------------------------------------------ a4 tentative prolongator
@@ -1982,9 +2009,9 @@ static int coarsen_level(amg_hierarchy *h, int l, bool &is_coarsest, cudaStream_
     int rounds = 0;
     for (;;) {
         BD_CUDA(cudaMemsetAsync(und.p, 0, sizeof(int), s));
-        k_mis_select<<<nblk(N), 256, 0, s>>>(N, S.rp.p, S.ci.p, state.p, key); ::bd::note_launch();
+        k_mis_select<<<nblk(8LL * N), 256, 0, s>>>(N, S.rp.p, S.ci.p, state.p, key); ::bd::note_launch();
         BD_LAUNCH_CHECK();
-        k_mis_exclude<<<nblk(N), 256, 0, s>>>(N, S.rp.p, S.ci.p, state.p, und.p); ::bd::note_launch();
+        k_mis_exclude<<<nblk(8LL * N), 256, 0, s>>>(N, S.rp.p, S.ci.p, state.p, und.p); ::bd::note_launch();
         BD_LAUNCH_CHECK();
         int hu = 0;
         BD_CUDA(cudaMemcpyAsync(&hu, und.p, sizeof(int), cudaMemcpyDeviceToHost, s));
@@ -2003,7 +2030,7 @@ static int coarsen_level(amg_hierarchy *h, int l, bool &is_coarsest, cudaStream_
     long long nagg = 0;
     BD_TRY(exclusive_scan(flag.p, rid.p, N, &nagg, s));
     BD_CUDA(cudaMemsetAsync(bad.p, 0, sizeof(int), s));
-    k_assign<<<nblk(N), 256, 0, s>>>(N, S.rp.p, S.ci.p, S.v.p, L.mis.p, rid.p, L.agg.p, bad.p); ::bd::note_launch();
+    k_assign<<<nblk(8LL * N), 256, 0, s>>>(N, S.rp.p, S.ci.p, S.v.p, L.mis.p, rid.p, L.agg.p, bad.p); ::bd::note_launch();
     BD_LAUNCH_CHECK();
     BD_CUDA(cudaMemcpyAsync(&hbad, bad.p, sizeof(int), cudaMemcpyDeviceToHost, s));
     BD_CUDA(cudaStreamSynchronize(s));
@@ -2063,15 +2090,21 @@ static int coarsen_level(amg_hierarchy *h, int l, bool &is_coarsest, cudaStream_
     k_lanczos_init<<<nblk(n), 256, 0, s>>>(n, level_key(o.seed, l, 1), diag.p, vr.p, vz.p, vp.p); ::bd::note_launch();
     BD_LAUNCH_CHECK();
     long long *acc = h->exact_acc.p;
-    BD_TRY(exact_dot(vr.p, vz.p, n, &lst.p->rz[0], acc, s));
+    BD_CUDA(cudaMemsetAsync(acc, 0, h->exact_acc.bytes(), s));
+    BD_TRY(exact_dot(vr.p, vz.p, n, &lst.p->rz[0], acc, s, true));
     for (int j = 0; j < o.esteig_steps; j++) {
         k_spmv_ordered<<<nblk(n, row_block(N)), row_block(N), 0, s>>>(n, L.A.rp.p, L.A.ci.p, L.A.v.p, vp.p, vq.p);
         ::bd::note_launch();
         BD_LAUNCH_CHECK();
-        BD_TRY(exact_dot(vp.p, vq.p, n, &lst.p->pq[j], acc, s));
-        k_lanczos_update_r<<<nblk(n), 256, 0, s>>>(n, lst.p, j, vq.p, diag.p, vr.p, vz.p); ::bd::note_launch();
-        BD_LAUNCH_CHECK();
-        BD_TRY(exact_dot(vr.p, vz.p, n, &lst.p->rz[j + 1], acc, s));
+        BD_TRY(exact_dot(vp.p, vq.p, n, &lst.p->pq[j], acc, s, true));
+        if (n <= kDotUpdateMax) {
+            BD_TRY(exact_dot_update(&lst.p->rz[j], &lst.p->pq[j], vq.p, diag.p, vr.p, vz.p, n, &lst.p->rz[j + 1], acc,
+                                    s));
+        } else {
+            k_lanczos_update_r<<<nblk(n), 256, 0, s>>>(n, lst.p, j, vq.p, diag.p, vr.p, vz.p); ::bd::note_launch();
+            BD_LAUNCH_CHECK();
+            BD_TRY(exact_dot(vr.p, vz.p, n, &lst.p->rz[j + 1], acc, s, true));
+        }
         if (j + 1 == o.esteig_steps) break;
         k_lanczos_update_p<<<nblk(n), 256, 0, s>>>(n, lst.p, j, vz.p, vp.p); ::bd::note_launch();
         BD_LAUNCH_CHECK();

@@ -1140,7 +1140,7 @@ __global__ void k_zero_if(int N, double2 *__restrict__ x, const double *__restri
 
 // The next V-cycle's finest-level input, written by the kernel that forms the
 // PCG residual r, so that the V-cycle needs no pass of its own over r.  FP64:
-// d0 = D^{-1} r / theta, in (v + u, u) form for a sliced-ELL finest level
+// d0 = D^{-1} r / theta, in (v + u, u) form for a stencil finest level
 // (mode 1) or in (v, u) form (mode 2); FP32 V-cycle (mode 3): f = (float) r
 // and d0 = D^{-1} f / theta in FP32.  The same arithmetic as k_scale_d0 and
 // k_in32.
@@ -1571,7 +1571,7 @@ static int tune_operator(Level &L, int op, bool sliced_ok, const v2<S> *x, const
 }
 
 // Time the candidate forms of every block operator the V-cycle applies (A
-// below the finest level, or on it where it is not sliced ELL; R and P) on
+// below the finest level, or on it where it is not a stencil; R and P) on
 // this GPU and keep the fastest.  The workspace vectors serve as operands;
 // their contents do not matter.  The form changes the order of a row's sum,
 // so the choice is fixed per hierarchy: every solve with it is reproducible.
@@ -1674,7 +1674,7 @@ int prepare_solve(amg_hierarchy *h, cudaStream_t s)
     if (!h->host_init) BD_CUDA(cudaMallocHost((void **)&h->host_init, sizeof(double) * S_NSLOTS));
     // lanes per block row of the V-cycle's block-CSR operators
     // (the sliced form for A only below the finest level: the PCG's fused
-    // A p and residual reductions on a non-sliced-ELL finest level use
+    // A p and residual reductions on a block-CSR finest level use
     // block-CSR; nothing on the coarsest level, which is solved densely)
     for (int l = 0; l < h->nlev; l++) {
         Level &L = h->lev[l];

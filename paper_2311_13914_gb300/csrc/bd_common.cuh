@@ -195,8 +195,14 @@ int sort_segments(int *keys, int *payload, const int *seg, int nseg, int max_len
 // blocks' arrival counter.
 constexpr int kExactLimbs = 68;
 constexpr int kExactScratch = kExactLimbs + 2;
-int exact_dot(const double *x, const double *y, int n, double *out, long long *acc,
-              cudaStream_t s);
+int exact_dot(const double *x, const double *y, int n, double *out, long long *acc, cudaStream_t s,
+              bool clean = false);
+// r -= (*num / *den) q, z = r / diag (entry by entry), out = r . z, with a clean
+// accumulator; one launch less for vectors of one product per thread (up to
+// kDotUpdateMax), where longer ones would take their divisions on few warps
+constexpr int kDotUpdateMax = 2 * kSM * 512;
+int exact_dot_update(const double *num, const double *den, const double *q, const double *diag, double *r, double *z,
+                     int n, double *out, long long *acc, cudaStream_t s);
 
 // Copy helpers between caller arrays (host or device) and device buffers.
 int copy_in(void *dst_dev, const void *src, size_t bytes, int src_on_device, cudaStream_t s);

@@ -407,9 +407,37 @@ __device__ double exact_round(long long *l, int flags)
 // step, shared by three launches with a one-thread rounding, took 57 us for 1.1 M
 // products (now 16, the call included; reading them takes 2.6 us of HBM).
 constexpr int kDotThreads = 512, kDotUnroll = 4;
-__global__ void __launch_bounds__(kDotThreads) k_exact_dot(const double *__restrict__ x, const double *__restrict__ y,
-                                                           int n, long long *gacc, double *__restrict__ out)
+// Products of two vectors.
+struct DotProducts {
+    const double *__restrict__ x;
+    const double *__restrict__ y;
+    __device__ __forceinline__ void start() {}
+    __device__ __forceinline__ double operator()(long long j) const { return __dmul_rn(x[j], y[j]); }
+};
+// Products r_j z_j of the vectors it forms in passing: r -= (num / den) q, z = r / diag.
+struct DotUpdate {
+    const double *num, *den;
+    const double *__restrict__ q;
+    const double *__restrict__ diag;
+    double *__restrict__ r;
+    double *__restrict__ z;
+    double alpha;
+    __device__ __forceinline__ void start() { alpha = __ddiv_rn(*num, *den); }
+    __device__ __forceinline__ double operator()(long long j) const
+    {
+        const double rj = __dsub_rn(r[j], __dmul_rn(alpha, q[j])), zj = __ddiv_rn(rj, diag[j]);
+        r[j] = rj;
+        z[j] = zj;
+        return __dmul_rn(rj, zj);
+    }
+};
+// clean: the accumulator is zero and is left so (no clear between the calls of a
+// sequence).
+template <class F>
+__global__ void __launch_bounds__(kDotThreads) k_exact_dot(F product, int n, long long *gacc, double *__restrict__ out,
+                                                           int clean)
 {
+    product.start();
     __shared__ long long acc[kExactLimbs];
     __shared__ int flags, emax;
     __shared__ bool last;
@@ -426,7 +454,7 @@ __global__ void __launch_bounds__(kDotThreads) k_exact_dot(const double *__restr
 #pragma unroll
         for (int k = 0; k < kDotUnroll; k++) {
             const long long j = i + k * stride;
-            p[k] = j < n ? __dmul_rn(x[j], y[j]) : 0.0;
+            p[k] = j < n ? product(j) : 0.0;
         }
     };
     fetch(i0);
@@ -495,14 +523,31 @@ __global__ void __launch_bounds__(kDotThreads) k_exact_dot(const double *__restr
     __syncwarp();
     const double r = exact_round(acc, (int)__ldcg(gacc + kExactLimbs));
     if (threadIdx.x == 0) *out = r;
+    __syncwarp();
+    if (clean)
+        for (int i = threadIdx.x; i < kExactScratch; i += 32) gacc[i] = 0;
 }
 
-int exact_dot(const double *x, const double *y, int n, double *out, long long *acc, cudaStream_t s)
+// Two blocks per SM at most; a product per thread before a second one (62426
+// products in 31 blocks of four 9.2 us, in 122 blocks 8.4).
+static int dot_blocks(int n)
 {
-    BD_CUDA(cudaMemsetAsync(acc, 0, sizeof(long long) * kExactScratch, s));
-    const long long per = (long long)kDotThreads * kDotUnroll;
-    const int grid = (int)std::max<long long>(1, std::min<long long>(2 * kSM, (n + per - 1) / per));
-    k_exact_dot<<<grid, kDotThreads, 0, s>>>(x, y, n, acc, out); ::bd::note_launch();
+    return (int)std::max<long long>(1, std::min<long long>(2 * kSM, ((long long)n + kDotThreads - 1) / kDotThreads));
+}
+
+int exact_dot(const double *x, const double *y, int n, double *out, long long *acc, cudaStream_t s, bool clean)
+{
+    if (!clean) BD_CUDA(cudaMemsetAsync(acc, 0, sizeof(long long) * kExactScratch, s));
+    k_exact_dot<<<dot_blocks(n), kDotThreads, 0, s>>>(DotProducts{x, y}, n, acc, out, clean); ::bd::note_launch();
+    BD_LAUNCH_CHECK();
+    return BD_OK;
+}
+
+int exact_dot_update(const double *num, const double *den, const double *q, const double *diag, double *r, double *z,
+                     int n, double *out, long long *acc, cudaStream_t s)
+{
+    k_exact_dot<<<dot_blocks(n), kDotThreads, 0, s>>>(DotUpdate{num, den, q, diag, r, z, 0.0}, n, acc, out, 1);
+    ::bd::note_launch();
     BD_LAUNCH_CHECK();
     return BD_OK;
 }
