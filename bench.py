@@ -199,7 +199,8 @@ def source_digest() -> str:
     removed (a comment edit leaves the compiled kernels, and so the recorded
     traffic, valid)."""
     h = hashlib.sha256()
-    for f in ("amg_solve.cu", "amg_internal.cuh", "bd_common.cuh"):
+    for f in ("amg_solve.cu", "amg_internal.cuh", "bd_common.cuh", "fine_stencil.cuh", "amg_bsr.cuh",
+              "pcg_reduce.cuh", "fp_convert.h"):
         text = open(os.path.join(ROOT, "paper_2311_13914_gb300", "csrc", f)).read()
         text = re.sub(r"/\*.*?\*/", " ", text, flags=re.S)
         text = re.sub(r"//[^\n]*", " ", text)
@@ -245,13 +246,14 @@ def csr_equivalent(info, launch_s, hbm_peak, fp32):
             "csr_equivalent_frac": nbytes / launch_s / 1e9 / hbm_peak}
 
 
-def coarse_levels_roofline(B, h, bd_, its, hbm_peak, fp32):
+def coarse_levels_roofline(B, h, bd_, its, hbm_peak, fp32, pairs=False):
     """Roofline entries of the coarse-level operators (block CSR or sliced
     block form; levels >= 1 for A, every level for R and P): algorithmic bytes
     per launch (per 2x2 block 4 values and a 4-byte column, 4 bytes of row
     offset per row, the V-cycle step's vector streams), FP64 operations per
     launch (4 FMA per block; the epilogues' few per row not counted; none in
-    the FP32 V-cycle) and the event-timed mean per launch from the per-step
+    the FP32 V-cycle; pairs: the finest R and P of an assembled slab hold 2 values
+    and issue 2 FMA per block) and the event-timed mean per launch from the per-step
     breakdown (one launch per step and PCG iteration)."""
     val = 4 if fp32 else 8
     vec = 2 * val
@@ -259,8 +261,8 @@ def coarse_levels_roofline(B, h, bd_, its, hbm_peak, fp32):
     info = [B.amg_level_info(h, l) for l in range(nl)]
     out = []
 
-    def entry(name, us, rows, blocks, nbytes):
-        ops = 0.0 if fp32 else 4.0 * blocks
+    def entry(name, us, rows, blocks, nbytes, fma=4.0):
+        ops = 0.0 if fp32 else fma * blocks
         t_hbm = nbytes / (hbm_peak * 1e9)
         t_alu = ops / FP64_OPS_PEAK
         bound = "alu" if t_alu > t_hbm else "hbm"
@@ -273,7 +275,8 @@ def coarse_levels_roofline(B, h, bd_, its, hbm_peak, fp32):
     for l in range(nl - 1):
         rows, rows_c = info[l]["n"] // 2, info[l + 1]["n"] // 2
         pb = info[l]["p_nnz"] // 4
-        mat_p = (4 * val + 4) * pb
+        fma = 2.0 if pairs and l == 0 else 4.0
+        mat_p = (fma * val + 4) * pb
         if l >= 1:
             nb = info[l]["nnz"] // 4
             mat = (4 * val + 4) * nb + 4 * (rows + 1)
@@ -285,11 +288,11 @@ def coarse_levels_roofline(B, h, bd_, its, hbm_peak, fp32):
         r = bd_.get(f"L{l}_restrict")
         if r:
             out.append(entry(f"R{l}", 1e3 * r[0] / its, rows_c, pb,
-                             mat_p + 4 * (rows_c + 1) + vec * rows + 3 * vec * rows_c))
+                             mat_p + 4 * (rows_c + 1) + vec * rows + 3 * vec * rows_c, fma))
         pp = bd_.get(f"L{l}_prolong")
         if pp:
             out.append(entry(f"P{l}", 1e3 * pp[0] / its, rows, pb,
-                             mat_p + 4 * (rows + 1) + vec * rows_c + 2 * vec * rows))
+                             mat_p + 4 * (rows + 1) + vec * rows_c + 2 * vec * rows, fma))
     return out
 
 
@@ -478,7 +481,7 @@ def run_ours(args):
                      sorted(bd_.items(), key=lambda kv: -kv[1][0])}
         pk = measured_peaks()
         coarse_roof = coarse_levels_roofline(B, h, bd_, its, pk["hbm_gbs"] if pk else 6800.0,
-                                             args.precision == "fp32")
+                                             args.precision == "fp32", pairs=True)
         fine_info = B.amg_level_info(h, 0)
         sim.close()
         h.close()
@@ -529,8 +532,8 @@ def run_ours(args):
     achieved_tops = rec["prof_fp64_ops"] / prof_s / 1e12 if prof_s > 0 else None
     fp32 = rec["prof_precision"] == 1
     t_hbm = rec["prof_bytes"] / (hbm_peak * 1e9)
-    # FP64: every operation the fused launches issue to the FP64 pipe (the 2
-    # FMA per stored node pair and the epilogues), against its issue rate;
+    # FP64: every operation the fused launches issue to the FP64 pipe (the
+    # stencil's adds and FMAs and the epilogues), against its issue rate;
     # the FP32 V-cycle's launches issue almost none
     t_alu = rec["prof_fp64_ops"] / FP64_OPS_PEAK
     per_launch = rec["prof_bytes"] / rec["prof_launches"] if rec["prof_launches"] else None
@@ -547,8 +550,8 @@ def run_ours(args):
     # measured HBM peak, or the FP64 operations at the FP64 pipe's issue rate
     roof = dict(alu if t_alu > t_hbm else hbm)
     roof.update({"traffic": traffic,
-                 "kernel": ("finest-level operator, sliced ELL, FP32 V-cycle (fused epilogues)" if fp32
-                            else "finest-level operator, sliced ELL, FP64 (fused epilogues) and PCG A p"),
+                 "kernel": ("finest-level operator, layered stencil, FP32 V-cycle (fused epilogues)" if fp32
+                            else "finest-level operator, layered stencil, FP64 (fused epilogues) and PCG A p"),
                  "algorithmic_bytes_per_launch": per_launch, "launches": rec["prof_launches"],
                  "fp64_ops_per_launch": rec["prof_fp64_ops"] / nl,
                  "hbm_gbs": achieved_gbs, "hbm_frac": hbm["frac"],
@@ -568,7 +571,8 @@ def run_ours(args):
         "dtype": "f64 (FP32 V-cycle)" if args.precision == "fp32" else "f64", "data": "synthetic",
         "config": {"workload": desc.format(T=T), "time_steps_per_step": T,
                    "parallelism": f"replicas x{world}",
-                   "l2": "inputs larger than L2 (finest operator 0.52 GB > 129 MB)",
+                   "l2": ("inputs larger than L2 (operators and vectors of a PCG iteration, 0.44 GB at "
+                          "128x128x32, 0.27 GB with the FP32 V-cycle, > 129 MB)"),
                    "setup_ms": statistics.mean(rec["setup_ms"]),
                    "solve_only_solves_per_s": T / (statistics.mean(rec["solve_ms"]) / 1e3),
                    "mean_pcg_iters": statistics.mean(rec["iters"]),

@@ -217,8 +217,8 @@ int amg_level_info(const amg_hierarchy *h, int level, int *n, long long *nnz, in
  *                   stable) within windows of 1024 rows, 32/K rows per warp,
  *                   K lanes per row, entries stored group-major so every load
  *                   of a warp is contiguous; it gives the same bits as T = K;
- *   0               not applied in block form (A on a sliced-ELL finest level,
- *                   everything on the coarsest level, solved densely).
+ *   0               not applied in block form (A on a finest level applied as a
+ *                   stencil, everything on the coarsest level, solved densely).
  * The sliced form is never used for A on the finest level. */
 int amg_level_lanes(const amg_hierarchy *h, int level, int lanes[3]);
 
@@ -325,13 +325,12 @@ void amg_stack_destroy(amg_stack *b);
  * SpMV launches of the V-cycle, and of PCG when the V-cycle is FP64) is
  * bracketed by CUDA events on the launching stream; the durations, the
  * algorithmic bytes (matrix values and indices once, each vector stream once)
- * and the flops the kernels execute (an FMA counts 2; the sliced-ELL form of
- * the finest level needs 2 FMA per stored node pair with its gathered vector
- * in (v + u, u) form, 2 FMA and an add otherwise, where the 2x2-block operator
- * would take 8 flops per block) are summed; the last post-smoothing launch
- * with the PCG's z statistics counts its FP64 streams (r read, z written, and
- * z_old read in the flexible form) too.  Switching it on resets the sums, switching it off keeps them
- * for amg_profile_read; reading requires no pending work.  enable: 0 off,
+ * and the flops the kernels execute (an FMA counts 2; the stencil form of the
+ * finest level takes 68 per node, 108 for fields whose fibres leave the plane,
+ * where the 2x2-block operator would take 8 per block) are summed; the last
+ * post-smoothing launch with the PCG's z statistics counts its FP64 streams (r
+ * read, z written) too.  Switching it on resets the sums, switching it off keeps
+ * them for amg_profile_read; reading requires no pending work.  enable: 0 off,
  * 1 on, 2 on with the per-step breakdown below.  While it is on,
  * solves run the host-driven loop (one launch at a time) instead of the
  * whole-solve CUDA graph. */
@@ -358,7 +357,7 @@ int amg_profile_read(const amg_hierarchy *h, amg_kernel_profile *out);
  * solve, 1 V-cycle input, 2 V-cycle output, 3 preconditioned-residual
  * statistics, 4 search-direction update, 5 A p with p.Ap, 6 iterate and
  * residual update).  Steps fused into others have no entry of their own: on a
- * sliced-ELL finest level the statistics ride on the last post-smoothing step
+ * stencil finest level the FP64 statistics ride on the last post-smoothing step
  * (16 * 0 + 5), and in the PCG the V-cycle input is written by the residual
  * update (so k = 1, 2, 3 appear only for amg_vcycle or a finest level in
  * block-CSR form).  Steps shorter than the host's launch rate read high.

@@ -24,7 +24,7 @@ def _operators(h):
     for level in range(nl - 1):
         for op in (0, 1, 2):
             if op == 0 and level == 0:
-                continue  # the finest A: sliced ELL, or block-CSR fused with the PCG
+                continue  # the finest A: a stencil, or block-CSR fused with the PCG
             yield level, op
 
 
