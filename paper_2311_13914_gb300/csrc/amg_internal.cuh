@@ -85,7 +85,7 @@ struct Level {
 // (bd_assemble.cu), tab is packed for the kernels.
 struct FineStencil {
     bool valid = false;
-    bool sym = false;           // rows symmetric under (dx, dy) -> (-dx, -dy)
+    bool sym = false;           // the symmetric form holds (bd_assemble.cu)
     int NX = 0, NY = 0, NZ = 0; // nodes
     DBuf<double> raw;           // NZ x 9 x kFineRaw
     DBuf<double> tab;           // packed rows, FP64 (always: the PCG's A p)

@@ -140,19 +140,26 @@ __global__ void k_stencil_rows(int nx, int ny, int nz, double lx, double ly, dou
     o[55] = Mp;
 }
 
-// *asym is set by a row that is not symmetric under (dx, dy) -> (-dx, -dy) beyond
-// the rounding of its sums (fibres with a z component).
+// *asym is set where the symmetric stencil form does not hold beyond the rounding
+// of the rows' sums (fibres with a z component).  That form adds opposite in-plane
+// neighbours first, so a row must be symmetric under (dx, dy) -> (-dx, -dy) where
+// both neighbours exist, and it applies the dz = +1 coefficients of the plane below
+// for dz = -1, so the two must be equal for every row type and position.  Neither
+// implies the other: a slab one element wide in x (or y) has no row with both
+// members of an x (y) pair, and only the coupling between its planes tells.
 __global__ void k_stencil_sym(int NZ, const double *__restrict__ raw, int *__restrict__ asym)
 {
     const int id = blockIdx.x * blockDim.x + threadIdx.x, row = id / 27, k = id % 27;
     if (row >= 9 * NZ) return;
     const int ti = row % 3, tj = (row % 9) / 3, dx = k % 3 - 1, dy = (k / 3) % 3 - 1;
-    if ((dx && ti != 1) || (dy && tj != 1)) return;  // only one of the pair exists
     const double *o = raw + (size_t)row * kFineRaw;
-    const int m = 9 * (k / 9) + 3 * (1 - dy) + 1 - dx;
     const double eps = 16.0 * 0x1p-52;
-    if (!(fabs(o[2 * k] - o[2 * m]) <= eps * fabs(o[26])) || !(fabs(o[2 * k + 1] - o[2 * m + 1]) <= eps * fabs(o[27])))
-        *asym = 1;
+    auto differ = [&](const double *p, int m) {  // entry k of this row from entry m of row p
+        return !(fabs(o[2 * k] - p[2 * m]) <= eps * fabs(o[26])) ||
+               !(fabs(o[2 * k + 1] - p[2 * m + 1]) <= eps * fabs(o[27]));
+    };
+    if ((!dx || ti == 1) && (!dy || tj == 1) && differ(o, 9 * (k / 9) + 3 * (1 - dy) + 1 - dx)) *asym = 1;
+    if (k < 9 && row >= 9 && differ(o - 9 * kFineRaw, k + 18)) *asym = 1;
 }
 
 // A warp per node: lane k writes the row's entry at stencil position k (every

@@ -225,5 +225,5 @@ struct bd_system {
     bd::DBuf<double> Ki;    // node-pattern stiffness values (shared pattern with A)
     bd::DBuf<double> Ke;
     bd::DBuf<double> raw;   // rows per plane and row type: (nz + 1) x 9 x kFineRaw
-    bool sym = false;       // every row symmetric under (dx, dy) -> (-dx, -dy)
+    bool sym = false;       // the symmetric stencil form holds for every row (bd_assemble.cu)
 };
