@@ -15,6 +15,7 @@
 #include <cmath>
 
 #include "amg_internal.cuh"
+#include "grid_index.h"
 #include "scalar.cuh"
 
 namespace bd {
@@ -89,7 +90,7 @@ __global__ void k_strength_count(int N, const int *__restrict__ rp, const int *_
                                  const double *__restrict__ v, const double *__restrict__ diag,
                                  double theta, int *cnt, double *__restrict__ wt)
 {
-    const int lane = threadIdx.x & 31, p = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int lane = threadIdx.x & 31, p = grid_row<5>(blockIdx.x, blockDim.x, threadIdx.x);
     if (p >= N) return;
     int c = 0;
     for (int t = rp[p] + lane; t < rp[p + 1]; t += 32) {
@@ -106,7 +107,7 @@ __global__ void k_strength_fill(int N, const int *__restrict__ rp, const int *__
                                 const double *__restrict__ wt, const int *__restrict__ srp,
                                 int *__restrict__ sci, double *__restrict__ sw)
 {
-    const int lane = threadIdx.x & 31, p = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int lane = threadIdx.x & 31, p = grid_row<5>(blockIdx.x, blockDim.x, threadIdx.x);
     if (p >= N) return;
     int pos = srp[p];
     for (int t0 = rp[p]; t0 < rp[p + 1]; t0 += 32) {
@@ -580,7 +581,7 @@ __device__ __forceinline__ int hslot(int key, int mask) { return (int)(((unsigne
 __global__ void k_spgemm_bound(int nrows, const int *__restrict__ arp, const int *__restrict__ aci,
                                const int *__restrict__ brp, int *__restrict__ ub)
 {
-    const int i = (blockIdx.x * blockDim.x + threadIdx.x) >> 3, l = threadIdx.x & 7;
+    const int i = grid_row<3>(blockIdx.x, blockDim.x, threadIdx.x), l = threadIdx.x & 7;
     long long u = 0;
     if (i < nrows)
         for (int t = arp[i] + l; t < arp[i + 1]; t += 8) u += brp[aci[t] + 1] - brp[aci[t]];
@@ -1180,7 +1181,7 @@ __global__ void k_drop_diag(int N, const int *__restrict__ qrp, const int *__res
                             const double *__restrict__ qv, int *__restrict__ orp,
                             int *__restrict__ oci, double *__restrict__ ov)
 {
-    const int lane = threadIdx.x & 31, p = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int lane = threadIdx.x & 31, p = grid_row<5>(blockIdx.x, blockDim.x, threadIdx.x);
     if (p > N) return;
     if (lane == 0) orp[p] = qrp[p] - p;
     if (p == N) return;
@@ -1209,7 +1210,7 @@ struct NodeLanes {
     int p, l;           // node, lane of the node's eight
     unsigned mask;      // the node's lanes in the warp
     __device__ __forceinline__ NodeLanes()
-        : p((int)((blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 3)), l(threadIdx.x & 7),
+        : p(grid_row<3>(blockIdx.x, blockDim.x, threadIdx.x)), l(threadIdx.x & 7),
           mask(0xffu << (threadIdx.x & 24)) {}
     // whether f(t) holds for an entry t of [b, e), by all lanes of the warp together
     template <class F> __device__ __forceinline__ bool any(int b, int e, F &&f) const
@@ -1530,7 +1531,7 @@ __global__ void k_smooth_p(int N, const int *__restrict__ rp, const int *__restr
                            const double *__restrict__ ptd, const double *__restrict__ diag,
                            const LanczosState *st)
 {
-    const int p = (blockIdx.x * blockDim.x + threadIdx.x) >> 3, l = threadIdx.x & 7;
+    const int p = grid_row<3>(blockIdx.x, blockDim.x, threadIdx.x), l = threadIdx.x & 7;
     if (p >= N) return;
     double omega = 4.0 / (3.0 * st->lam);
     double s0 = omega / diag[2 * p], s1 = omega / diag[2 * p + 1];
@@ -1614,7 +1615,7 @@ static int bsr_transpose(const BSR &a, BSR &t, cudaStream_t s)
 __global__ void k_coarse_dense(int N, const int *__restrict__ rp, const int *__restrict__ ci,
                                const double *__restrict__ v, int ld, double *__restrict__ Ad)
 {
-    const int lane = threadIdx.x & 31, p = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int lane = threadIdx.x & 31, p = grid_row<5>(blockIdx.x, blockDim.x, threadIdx.x);
     if (p >= N) return;
     double2 *r0 = (double2 *)(Ad + (size_t)(2 * p) * ld), *r1 = (double2 *)(Ad + (size_t)(2 * p + 1) * ld);
     for (int t = rp[p] + lane; t < rp[p + 1]; t += 32) {

@@ -19,6 +19,7 @@
 #include "amg_bsr.cuh"
 #include "amg_internal.cuh"
 #include "fine_stencil.cuh"
+#include "grid_index.h"
 #include "pcg_reduce.cuh"
 #include "scalar.cuh"
 
@@ -515,7 +516,7 @@ __global__ void k_pair_fill(int rows, const int *__restrict__ rp, const int *__r
     const int lane = threadIdx.x & 31, l = lane & (L - 1);
     const unsigned group = (L == 32 ? 0xffffffffu : ((1u << (L & 31)) - 1u) << (lane & ~(L - 1)));
     const unsigned before = group & ((1u << lane) - 1u);
-    const int row = (blockIdx.x * blockDim.x + threadIdx.x) / L;
+    const int row = (int)(grid_index(blockIdx.x, blockDim.x, threadIdx.x) / L);
     const bool act = row < rows;
     const int b = act ? rp[row] : 0, e = act ? rp[row + 1] : 0;
     int len = e - b, nown = 0;

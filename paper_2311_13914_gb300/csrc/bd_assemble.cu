@@ -8,6 +8,7 @@
 // in ascending element index), so the operator is bit-reproducible and
 // bit-symmetric.
 #include "bd_common.cuh"
+#include "grid_index.h"
 
 namespace bd {
 
@@ -171,7 +172,7 @@ __global__ void __launch_bounds__(256) k_expand_rows(int NX, int NY, int NZ, con
                                                      double *__restrict__ v, double *__restrict__ Ki,
                                                      double *__restrict__ Ke, double *__restrict__ M)
 {
-    const int lane = threadIdx.x & 31, p = (int)((blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5);
+    const int lane = threadIdx.x & 31, p = grid_row<5>(blockIdx.x, blockDim.x, threadIdx.x);
     if (p >= NX * NY * NZ) return;
     const int i = p % NX, j = (p / NX) % NY, l = p / (NX * NY);
     const int dx = lane % 3 - 1, dy = (lane / 3) % 3 - 1, dz = lane / 9 - 1;
