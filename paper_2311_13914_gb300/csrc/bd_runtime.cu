@@ -315,7 +315,7 @@ __device__ __forceinline__ void exact_acc_digits(long long *acc, int li, unsigne
 }
 
 // A thread's window: a 256-bit two's complement integer in units of
-// 2^(b0 - 1074), b0 a multiple of 32.
+// 2^(b0 - 1074), b0 a multiple of 32 that the warp's threads share.
 struct ExactWindow {
     unsigned long long w[4] = {0, 0, 0, 0};
     __device__ __forceinline__ void add(unsigned long long v0, unsigned long long v1, unsigned long long v2,
@@ -328,10 +328,66 @@ struct ExactWindow {
             : "+l"(w[0]), "+l"(w[1]), "+l"(w[2]), "+l"(w[3])
             : "l"(v0), "l"(v1), "l"(v2), "l"(v3));
     }
+    // p, finite, zero or with its last bit in the window
+    __device__ __forceinline__ void add(double p, int b0)
+    {
+        const unsigned long long bits = (unsigned long long)__double_as_longlong(p);
+        const int E = (int)((bits >> 52) & 0x7ff);
+        const unsigned long long m = (bits & 0xFFFFFFFFFFFFFULL) | (E ? 1ULL << 52 : 0);
+        const int s = max(E, 1) - 1 - b0, r = s & 63, k = s >> 6;
+        const unsigned long long neg = (unsigned long long)((long long)bits >> 63);
+        // (m << s) negated where the sign is set: xor and add one
+        const unsigned long long a = m << r, c = r ? m >> (64 - r) : 0;
+        const unsigned long long v0 = k == 0 ? a : 0, v1 = k == 1 ? a : (k == 0 ? c : 0);
+        const unsigned long long v2 = k == 2 ? a : (k == 1 ? c : 0), v3 = k == 2 ? c : 0;
+        add(v0 ^ neg, v1 ^ neg, v2 ^ neg, v3 ^ neg);
+        add(neg & 1, 0, 0, 0);
+    }
+    // the whole warp's sum to the limbs acc
+    __device__ __forceinline__ void flush(int b0, long long *acc)
+    {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            unsigned long long v[4];
+#pragma unroll
+            for (int k = 0; k < 4; k++) v[k] = __shfl_xor_sync(0xffffffffu, w[k], o);
+            add(v[0], v[1], v[2], v[3]);
+        }
+        const int lane = threadIdx.x & 31;
+        if (lane < 8) {  // every lane holds the total: lane d adds digit d, the top one signed
+            const int q = lane >> 1;
+            const unsigned long long x = q == 0 ? w[0] : (q == 1 ? w[1] : (q == 2 ? w[2] : w[3]));
+            const long long d = lane == 7 ? (long long)x >> 32 : (long long)((lane & 1) ? x >> 32 : x & 0xffffffffULL);
+            if (d) atomicAdd((unsigned long long *)&acc[(b0 >> 5) + lane], (unsigned long long)d);
+        }
+        w[0] = w[1] = w[2] = w[3] = 0;
+    }
 };
 // Highest position of a product's last bit in the window: 53 bits above it and
 // 2^31 of them stay below 2^255.
 constexpr int kWindowTop = 169;
+constexpr int kNoWindow = 1 << 12;
+
+// Biased exponents of a warp's products (subnormals 1): the largest and the
+// smallest of those that are not zero, hi beyond every window for an infinity or NaN.
+struct ExactRange {
+    int hi = 0, lo = 0x7ff;
+    __device__ __forceinline__ void note(double p)
+    {
+        const unsigned long long b = (unsigned long long)__double_as_longlong(p) << 1;
+        const int E = (int)(b >> 53), e = b ? max(E, 1) : 0;
+        hi = max(hi, E == 0x7ff ? 1 << 16 : e);
+        lo = min(lo, b ? e : 0x7ff);
+    }
+    __device__ __forceinline__ void of_warp()
+    {
+        hi = __reduce_max_sync(0xffffffffu, hi);
+        lo = __reduce_min_sync(0xffffffffu, lo);
+    }
+    __device__ __forceinline__ bool in(int b0) const { return hi - 1 - b0 <= kWindowTop && lo - 1 >= b0; }
+    // base of a window with the largest 128 to 159 bits above it
+    __device__ __forceinline__ int base() const { return max(0, hi - 1 - 128) & ~31; }
+};
 
 // The exact total of gacc's limbs rounded to the nearest double (ties to even).
 // Called by one whole warp with the limbs in shared memory.
@@ -398,15 +454,22 @@ __device__ double exact_round(long long *l, int flags)
     return negative ? -r : r;
 }
 
-// Every thread sums its products in a register window placed by its block's
-// first products (the largest of them 128 to 159 bits above the window's
-// base), about 45 integer instructions a product; the few that do not fit go
-// to the block's limbs one by one.  The warps fold their windows by shuffles,
-// the blocks add their limbs to the global accumulator, and the last block to
-// arrive rounds it.  One launch and a clear, where a digit-wise sum per warp
-// step, shared by three launches with a one-thread rounding, took 57 us for 1.1 M
-// products (now 16, the call included; reading them takes 2.6 us of HBM).
-constexpr int kDotThreads = 512, kDotUnroll = 4;
+// Every thread sums its products in a register window, about 45 integer
+// instructions a product.  A warp's threads share the window's place: where their
+// next products do not all fit it but would fit another, the window is folded by
+// shuffles into the block's limbs and moves there (vectors whose magnitude changes
+// along the way, zeros before the first entries).  Products too far apart for one
+// window are taken 32 at a time: one window more for those outside the warp's,
+// or, if that does not hold them either, the limbs one by one (four copies of
+// them, or the block's warps hold each other up).  The blocks add their limbs to the
+// global accumulator, and the last block to arrive rounds it.  One launch and a clear.
+// Host-timed, 1.1 M and 10 M products, against digit-wise sums per warp step in
+// three launches: N(0,1) 70 -> 31 and 323 -> 70 us; the first two thirds zero 51 ->
+// 30 and 155 -> 58; falling or rising by e^600 90 -> 36 and 345 -> 71; every second
+// product 2^-400 104 -> 41 and 635 -> 151; exponents +-400 at random 48 -> 41 and
+// 201 -> 152 (277 with one copy of the limbs).  With windows that stay where a block's first
+// products put them the same five took 31, 130, 138, 138, 54 and 70, 731, 1140, 931, 261.
+constexpr int kDotThreads = 512, kDotUnroll = 4, kDotCopies = 4;
 // Products of two vectors.
 struct DotProducts {
     const double *__restrict__ x;
@@ -438,80 +501,78 @@ __global__ void __launch_bounds__(kDotThreads) k_exact_dot(F product, int n, lon
                                                            int clean)
 {
     product.start();
-    __shared__ long long acc[kExactLimbs];
-    __shared__ int flags, emax;
+    __shared__ long long limbs[kDotCopies][kExactLimbs];
+    __shared__ int flags;
     __shared__ bool last;
-    for (int i = threadIdx.x; i < kExactLimbs; i += blockDim.x) acc[i] = 0;
-    if (threadIdx.x == 0) {
-        flags = 0;
-        emax = 0;
-    }
+    for (int i = threadIdx.x; i < kDotCopies * kExactLimbs; i += blockDim.x) (&limbs[0][0])[i] = 0;
+    long long *acc = limbs[(threadIdx.x >> 5) % kDotCopies];
+    if (threadIdx.x == 0) flags = 0;
     __syncthreads();
     const long long stride = (long long)gridDim.x * blockDim.x;
-    const long long i0 = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    double p[kDotUnroll];
-    auto fetch = [&](long long i) {
-#pragma unroll
-        for (int k = 0; k < kDotUnroll; k++) {
-            const long long j = i + k * stride;
-            p[k] = j < n ? product(j) : 0.0;
+    const int lane = threadIdx.x & 31;
+    ExactWindow W;
+    int b0 = kNoWindow;
+    auto move = [&](int to) {
+        if (b0 != kNoWindow) W.flush(b0, acc);
+        b0 = to;
+    };
+    // the warp's next 32 products, of a step too wide for one window
+    auto chunk = [&](double p) {
+        ExactRange r;
+        r.note(p);
+        const ExactRange own = r;
+        r.of_warp();
+        if (r.hi == 0) return;
+        const bool some = __any_sync(0xffffffffu, own.hi && own.in(b0));
+        if (!r.in(b0) && (r.in(r.base()) || (!some && r.hi <= 0x7ff))) move(r.base());
+        const bool here = own.in(b0);
+        ExactRange o;
+        if (!here) o = own;
+        o.of_warp();
+        if (o.hi == 0) {
+            W.add(p, b0);
+        } else if (o.in(o.base())) {
+            ExactWindow T;
+            if (here) W.add(p, b0);
+            else T.add(p, o.base());
+            T.flush(o.base(), acc);
+        } else {
+            int li, nf;
+            unsigned long long d0, d1, d2;
+            if (!exact_digits(p, li, d0, d1, d2, nf)) atomicOr(&flags, nf);
+            else exact_acc_digits(acc, li, d0, d1, d2);
         }
     };
-    fetch(i0);
-    unsigned em = 0;
-#pragma unroll
-    for (int k = 0; k < kDotUnroll; k++) {
-        const unsigned e = ((unsigned)__double2hiint(p[k]) >> 20) & 0x7ff;
-        if (e != 0x7ff) em = max(em, e);
-    }
-    em = __reduce_max_sync(0xffffffffu, em);
-    if ((threadIdx.x & 31) == 0) atomicMax(&emax, (int)em);
-    __syncthreads();
-    const int b0 = max(0, emax - 1 - 128) & ~31;
-    ExactWindow W;
-    for (long long i = i0; i < n; i += kDotUnroll * stride) {
-        if (i != i0) fetch(i);
+    for (long long i = blockIdx.x * (long long)blockDim.x + (threadIdx.x & ~31); i < n; i += kDotUnroll * stride) {
+        double p[kDotUnroll];
+        ExactRange r;
 #pragma unroll
         for (int k = 0; k < kDotUnroll; k++) {
-            const unsigned long long bits = (unsigned long long)__double_as_longlong(p[k]);
-            if ((bits << 1) == 0) continue;
-            const int E = (int)((bits >> 52) & 0x7ff);
-            const unsigned long long m = (bits & 0xFFFFFFFFFFFFFULL) | (E ? 1ULL << 52 : 0);
-            const int s = max(E, 1) - 1 - b0;
-            if (E < 0x7ff && s >= 0 && s <= kWindowTop) {
-                const int r = s & 63, w = s >> 6;
-                const unsigned long long neg = (unsigned long long)((long long)bits >> 63);
-                // (m << s) negated where the sign is set: xor and add one
-                const unsigned long long a = m << r, c = r ? m >> (64 - r) : 0;
-                unsigned long long v0 = w == 0 ? a : 0, v1 = w == 1 ? a : (w == 0 ? c : 0);
-                unsigned long long v2 = w == 2 ? a : (w == 1 ? c : 0), v3 = w == 2 ? c : 0;
-                W.add(v0 ^ neg, v1 ^ neg, v2 ^ neg, v3 ^ neg);
-                W.add(neg & 1, 0, 0, 0);
-            } else {
-                int li, nf;
-                unsigned long long d0, d1, d2;
-                if (!exact_digits(p[k], li, d0, d1, d2, nf)) atomicOr(&flags, nf);
-                else exact_acc_digits(acc, li, d0, d1, d2);
-            }
+            const long long j = i + lane + k * stride;
+            p[k] = j < n ? product(j) : 0.0;
+        }
+#pragma unroll
+        for (int k = 0; k < kDotUnroll; k++) r.note(p[k]);
+        r.of_warp();
+        if (r.hi == 0) continue;
+        if (!r.in(b0) && r.in(r.base())) move(r.base());
+        if (r.in(b0)) {
+#pragma unroll
+            for (int k = 0; k < kDotUnroll; k++) W.add(p[k], b0);
+        } else {
+            static_assert(kDotUnroll == 4, "the steps below");
+#pragma unroll 1
+            for (int k = 0; k < kDotUnroll; k++) chunk(k == 0 ? p[0] : (k == 1 ? p[1] : (k == 2 ? p[2] : p[3])));
         }
     }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        unsigned long long v[4];
-#pragma unroll
-        for (int k = 0; k < 4; k++) v[k] = __shfl_xor_sync(0xffffffffu, W.w[k], o);
-        W.add(v[0], v[1], v[2], v[3]);
-    }
-    const int lane = threadIdx.x & 31;
-    if (lane < 8) {  // every lane holds the warp's total: lane d adds digit d, the top one signed
-        const int q = lane >> 1;
-        const unsigned long long w = q == 0 ? W.w[0] : (q == 1 ? W.w[1] : (q == 2 ? W.w[2] : W.w[3]));
-        const long long d = lane == 7 ? (long long)w >> 32 : (long long)((lane & 1) ? w >> 32 : w & 0xffffffffULL);
-        if (d) atomicAdd((unsigned long long *)&acc[(b0 >> 5) + lane], (unsigned long long)d);
-    }
+    if (b0 != kNoWindow) W.flush(b0, acc);
     __syncthreads();
-    for (int i = threadIdx.x; i < kExactLimbs; i += blockDim.x)
-        if (acc[i]) atomicAdd((unsigned long long *)&gacc[i], (unsigned long long)acc[i]);
+    for (int i = threadIdx.x; i < kExactLimbs; i += blockDim.x) {
+        long long t = 0;
+#pragma unroll
+        for (int k = 0; k < kDotCopies; k++) t += limbs[k][i];
+        if (t) atomicAdd((unsigned long long *)&gacc[i], (unsigned long long)t);
+    }
     if (threadIdx.x == 0 && flags) atomicOr((int *)&gacc[kExactLimbs], flags);
     __threadfence();
     __syncthreads();
@@ -519,9 +580,9 @@ __global__ void __launch_bounds__(kDotThreads) k_exact_dot(F product, int n, lon
     __syncthreads();
     if (!last || threadIdx.x >= 32) return;
     __threadfence();
-    for (int i = threadIdx.x; i < kExactLimbs; i += 32) acc[i] = __ldcg(gacc + i);
+    for (int i = threadIdx.x; i < kExactLimbs; i += 32) limbs[0][i] = __ldcg(gacc + i);
     __syncwarp();
-    const double r = exact_round(acc, (int)__ldcg(gacc + kExactLimbs));
+    const double r = exact_round(limbs[0], (int)__ldcg(gacc + kExactLimbs));
     if (threadIdx.x == 0) *out = r;
     __syncwarp();
     if (clean)
