@@ -219,14 +219,21 @@ int amg_level_info(const amg_hierarchy *h, int level, int *n, long long *nnz, in
  *                   of a warp is contiguous; it gives the same bits as T = K;
  *   0               not applied in block form (A on a finest level applied as a
  *                   stencil, everything on the coarsest level, solved densely).
- * The sliced form is never used for A on the finest level. */
+ * The sliced form is never used for A on the finest level.  On a hierarchy of
+ * bd_elliptic_setup these are the forms of its block operators; bd_dsim_step
+ * solves on the u_e field, with block-CSR lanes of its own choice for the coarse
+ * operators' (u_e, u_e) entries. */
 int amg_level_lanes(const amg_hierarchy *h, int level, int lanes[3]);
 
 /* Override the forms chosen by amg_setup (values as amg_level_lanes returns
  * them; 0 keeps an operator's current form).  Builds the sliced forms it
  * needs in the V-cycle's precision and drops the hierarchy's captured solve
  * graph (the next solve captures it anew).  No solve with h may be in flight
- * on any stream; synchronises `stream`.  Errors: BD_EINVAL (NULL, level out
+ * on any stream; synchronises `stream`.  On a hierarchy of
+ * bd_elliptic_setup the forms hold for the one-field operators of bd_dsim_step as
+ * well: T lanes for T, K for -K (they have no sliced form), and the form
+ * amg_level_lanes gave after setup brings back the one setup chose for
+ * them.  Errors: BD_EINVAL (NULL, level out
  * of range, a value not listed above, a nonzero value for an operator the
  * level does not apply in block form, or a sliced form for A on the finest
  * level), BD_ESTATE (a batch of amg_batch_create holds h), BD_ENOMEM, BD_ECUDA. */

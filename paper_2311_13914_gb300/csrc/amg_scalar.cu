@@ -12,6 +12,7 @@
 // (amg_solve.cu).
 #include <algorithm>
 #include <cmath>
+#include <cstdlib>
 #include <new>
 #include <type_traits>
 
@@ -383,6 +384,8 @@ struct Arr {
 struct ScLevel {
     Arr A, P, R, invd, f, u, r, d;
     int lanes[3] = {1, 1, 1};
+    // the forms setup chose, here and for the block operators (amg_set_level_lanes)
+    int chosen[3] = {1, 1, 1}, block[3] = {0, 0, 0};
 };
 
 }  // namespace
@@ -401,10 +404,17 @@ struct ScalarEll {
     double *host = nullptr;  // pinned: initial scalars, then results
     bool failed = false;
     long long pre = 0, body = 0, post = 0;
-    ~ScalarEll()
+    void drop_graph()
     {
         if (exec) cudaGraphExecDestroy(exec);
         if (graph) cudaGraphDestroy(graph);
+        exec = nullptr;
+        graph = nullptr;
+        failed = false;
+    }
+    ~ScalarEll()
+    {
+        drop_graph();
         if (cap) cudaStreamDestroy(cap);
         if (cap2) cudaStreamDestroy(cap2);
         if (ev[0]) cudaEventDestroy(ev[0]);
@@ -443,6 +453,11 @@ int scalar_build(amg_hierarchy *h, const bd_system *sys, cudaStream_t s)
         C.lanes[1] = lanes_for(L.R, true);
         C.lanes[2] = lanes_for(L.P, true);
     }
+    for (int l = 0; l < nl - 1; l++)
+        for (int op = 0; op < 3; op++) {
+            E.lev[l].chosen[op] = E.lev[l].lanes[op];
+            E.lev[l].block[op] = h->lev[l].lanes[op];
+        }
     const int n = h->nc / 2;
     BD_TRY(E.cinv.alloc((size_t)n * n));
     k_uu_dense<<<grid_for((long long)n * n, 256), 256, 0, s>>>(n, h->cinv.p, E.cinv.p); ::bd::note_launch();
@@ -465,6 +480,14 @@ int scalar_build(amg_hierarchy *h, const bd_system *sys, cudaStream_t s)
     BD_CUDA(cudaStreamSynchronize(s));
     h->scalar = up;
     return BD_OK;
+}
+
+void scalar_set_lanes(amg_hierarchy *h, int level, int op, int T)
+{
+    if (!h->scalar) return;
+    h->scalar->drop_graph();
+    ScLevel &C = h->scalar->lev[level];
+    C.lanes[op] = T == C.block[op] ? C.chosen[op] : std::abs(T);
 }
 
 namespace {
@@ -596,9 +619,7 @@ bool scalar_ready(amg_hierarchy *h, const solve_options *o)
         if (st != BD_OK) {
             drop_capture(E.cap2);
             drop_capture(E.cap);
-            if (E.graph) cudaGraphDestroy(E.graph);
-            E.graph = nullptr;
-            E.exec = nullptr;
+            E.drop_graph();
             E.failed = true;
         }
     }

@@ -2269,6 +2269,7 @@ extern "C" int amg_set_level_lanes(amg_hierarchy *h, int level, const int lanes[
             drop_sliced(L.sl[op]);
         }
         L.lanes[op] = T;
+        scalar_set_lanes(h, level, op, T);
     }
     return BD_OK;
 }

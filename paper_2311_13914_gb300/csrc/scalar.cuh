@@ -31,6 +31,10 @@ int scalar_build(amg_hierarchy *h, const bd_system *sys, cudaStream_t s);
 // whether the scalar solve runs (not with live timing, strict mode, graphs off or
 // a degree-1 smoother: the block solve serves those)
 bool scalar_ready(amg_hierarchy *h, const solve_options *o);
+// amg_set_level_lanes' form T for a one-field operator: as many lanes a row (a
+// sliced form stands for its lanes, with the same bits), and for the form setup chose
+// for the block operator the one it chose here
+void scalar_set_lanes(amg_hierarchy *h, int level, int op, int T);
 // (Ai + Ae) x = f from the x given; f, x: N doubles on the device
 int scalar_solve(amg_hierarchy *h, const double *f, double *x, const solve_options *o, cudaStream_t s, solve_info *info);
 
