@@ -89,7 +89,9 @@ typedef struct {
                               fastest unless the rule's form is within 3 %.
                               Either way the choice is fixed per hierarchy, so its
                               solves are reproducible; the two choices differ in
-                              the summation order of row sums (last bits) (0)       */
+                              the summation order of row sums (last bits).
+                              bd_elliptic_setup times the one-field operators of
+                              bd_dsim_step (their block-CSR lanes) as well (0)      */
 } amg_options;
 
 typedef struct {

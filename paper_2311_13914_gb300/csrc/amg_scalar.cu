@@ -423,6 +423,38 @@ struct ScalarEll {
     }
 };
 
+namespace {
+
+template <class S, class E>
+int csr(const BSR &M, Arr &v, int T, const S *x, E e, cudaStream_t s)
+{
+    return launch_bsr_rows(M.nbr, M.rp.p, M.ci.p, MatOne<S>{Buf<S>::p(v)}, T, GatherOne<S>{x}, e, s);
+}
+
+// Time the lanes of every coarse operator (amg_options.autotune).  The workspace
+// vectors serve as operands; their contents do not matter.
+template <class S> int tune(amg_hierarchy *h, ScalarEll &E, cudaStream_t s)
+{
+    auto P = [&](Arr &a) { return Buf<S>::p(a); };
+    for (int l = 0; l < h->nlev - 1; l++) {
+        Level &L = h->lev[l];
+        ScLevel &C = E.lev[l], &D = E.lev[l + 1];
+        if (l > 0)
+            BD_TRY(tune_csr_lanes(L.A, [&](int T) {
+                return csr<S>(L.A, C.A, T, (const S *)P(C.u), E1Resid<S>{P(C.f), P(C.r)}, s);
+            }, s, &C.lanes[0]));
+        BD_TRY(tune_csr_lanes(L.R, [&](int T) {
+            return csr<S>(L.R, C.R, T, (const S *)P(C.r), E1Resid<S>{P(D.f), P(D.r)}, s);
+        }, s, &C.lanes[1]));
+        BD_TRY(tune_csr_lanes(L.P, [&](int T) {
+            return csr<S>(L.P, C.P, T, (const S *)P(D.u), E1Resid<S>{P(C.f), P(C.d)}, s);
+        }, s, &C.lanes[2]));
+    }
+    return BD_OK;
+}
+
+}  // namespace
+
 int scalar_build(amg_hierarchy *h, const bd_system *sys, cudaStream_t s)
 {
     h->scalar.reset();
@@ -453,6 +485,7 @@ int scalar_build(amg_hierarchy *h, const bd_system *sys, cudaStream_t s)
         C.lanes[1] = lanes_for(L.R, true);
         C.lanes[2] = lanes_for(L.P, true);
     }
+    if (h->opts.autotune) BD_TRY(p32 ? tune<float>(h, E, s) : tune<double>(h, E, s));
     for (int l = 0; l < nl - 1; l++)
         for (int op = 0; op < 3; op++) {
             E.lev[l].chosen[op] = E.lev[l].lanes[op];
@@ -491,12 +524,6 @@ void scalar_set_lanes(amg_hierarchy *h, int level, int op, int T)
 }
 
 namespace {
-
-template <class S, class E>
-int csr(const BSR &M, Arr &v, int T, const S *x, E e, cudaStream_t s)
-{
-    return launch_bsr_rows(M.nbr, M.rp.p, M.ci.p, MatOne<S>{Buf<S>::p(v)}, T, GatherOne<S>{x}, e, s);
-}
 
 // One V-cycle on the u_e field; the finest level's input is in lev[0].d and f0.
 // FP64: the last step writes z and its statistics (zf) unless there is one level.

@@ -1514,21 +1514,90 @@ static D0Out d0_out(amg_hierarchy *h)
 constexpr int kLaneCands = 13, kLaneReps = 3;
 constexpr long long kTuneMinBlocks = 20000;  // smaller operators keep the rule
 
-template <class S>
-static int tune_operator(Level &L, int op, bool sliced_ok, const v2<S> *x, const v2<S> *f, v2<S> *out,
-                         const S *vals, cudaEvent_t (*ev)[kLaneReps][2], cudaStream_t s)
+struct TuneEvents {
+    cudaEvent_t e[kLaneCands][kLaneReps][2] = {};
+    int create()
+    {
+        for (auto &c : e)
+            for (auto &r : c)
+                for (cudaEvent_t &v : r) BD_CUDA(cudaEventCreate(&v));
+        return BD_OK;
+    }
+    ~TuneEvents()
+    {
+        for (auto &c : e)
+            for (auto &r : c)
+                for (cudaEvent_t v : r)
+                    if (v) cudaEventDestroy(v);
+    }
+};
+
+// block-CSR candidates of M, at most kLaneCands - 4
+static int csr_candidates(const BSR &M, int *cand)
 {
-    const BSR &M = op == 0 ? L.A : (op == 1 ? L.R : L.P);
-    const bool fp32 = sizeof(S) == 4;
     const double avg = M.nbr > 0 ? (double)M.nb / M.nbr : 1.0;
-    const EpiResid<S> epi{f, out};
-    int Tlo = 1, Thi = 256;
+    int Tlo = 1, Thi = 256, nc = 0;
     while (Tlo * 16 < avg && Tlo < 32) Tlo <<= 1;
     while (Thi > 1 && Thi > 4.0 * avg) Thi >>= 1;
     if (avg < 32.0) Thi = std::min(Thi, 32);
     Thi = std::max(Thi, Tlo);
-    int cand[kLaneCands], nc = 0;
     for (int T = Tlo; T <= Thi && nc < kLaneCands - 4; T <<= 1) cand[nc++] = T;
+    return nc;
+}
+
+// candidate c, once untimed and then kLaneReps times between events
+template <class F> static int time_candidate(F run, cudaEvent_t (*ev)[2], cudaStream_t s)
+{
+    BD_TRY(run());
+    for (int k = 0; k < kLaneReps; k++) {
+        BD_CUDA(cudaEventRecord(ev[k][0], s));
+        BD_TRY(run());
+        BD_CUDA(cudaEventRecord(ev[k][1], s));
+    }
+    return BD_OK;
+}
+
+// the fastest median wins unless the rule's choice (when among the
+// candidates) is within 3 % of it: near-ties then resolve the same way
+// on every run
+static int pick_candidate(const int *cand, int nc, int rule, const TuneEvents &ev, int *pick)
+{
+    float best = 0.0f, t_rule = -1.0f;
+    int bestT = rule;
+    for (int c = 0; c < nc; c++) {
+        float t[kLaneReps];
+        for (int k = 0; k < kLaneReps; k++) BD_CUDA(cudaEventElapsedTime(&t[k], ev.e[c][k][0], ev.e[c][k][1]));
+        const float med = std::max(std::min(t[0], t[1]), std::min(std::max(t[0], t[1]), t[2]));
+        if (cand[c] == rule) t_rule = med;
+        if (c == 0 || med < best) {
+            best = med;
+            bestT = cand[c];
+        }
+    }
+    *pick = (t_rule >= 0.0f && t_rule <= 1.03f * best) ? rule : bestT;
+    return BD_OK;
+}
+
+int tune_csr_lanes(const BSR &M, const std::function<int(int)> &run, cudaStream_t s, int *lanes)
+{
+    if (M.nb < kTuneMinBlocks) return BD_OK;
+    int cand[kLaneCands];
+    const int nc = csr_candidates(M, cand);
+    TuneEvents ev;
+    BD_TRY(ev.create());
+    for (int c = 0; c < nc; c++) BD_TRY(time_candidate([&] { return run(cand[c]); }, ev.e[c], s));
+    BD_CUDA(cudaStreamSynchronize(s));
+    return pick_candidate(cand, nc, *lanes, ev, lanes);
+}
+
+template <class S>
+static int tune_operator(Level &L, int op, bool sliced_ok, const v2<S> *x, const v2<S> *f, v2<S> *out,
+                         const S *vals, TuneEvents &ev, cudaStream_t s)
+{
+    const BSR &M = op == 0 ? L.A : (op == 1 ? L.R : L.P);
+    const bool fp32 = sizeof(S) == 4;
+    const EpiResid<S> epi{f, out};
+    int cand[kLaneCands], nc = csr_candidates(M, cand);
     const int ncsr = nc;
     if (sliced_ok && !fp32 && M.nbr >= kSlicedMinRows)
         for (int K = 1; K <= 8; K <<= 1) cand[nc++] = -K;
@@ -1540,31 +1609,12 @@ static int tune_operator(Level &L, int op, bool sliced_ok, const v2<S> *x, const
     for (int c = 0; c < nc; c++) {
         if (cand[c] < 0) BD_TRY(build_op(L, op, -cand[c], fp32, s));
         L.lanes[op] = cand[c];
-        BD_TRY(run());
-        for (int k = 0; k < kLaneReps; k++) {
-            BD_CUDA(cudaEventRecord(ev[c][k][0], s));
-            BD_TRY(run());
-            BD_CUDA(cudaEventRecord(ev[c][k][1], s));
-        }
+        BD_TRY(time_candidate(run, ev.e[c], s));
         if (cand[c] < 0 || c + 1 == ncsr) BD_CUDA(cudaStreamSynchronize(s));
     }
     BD_CUDA(cudaStreamSynchronize(s));
-    // the fastest median wins unless the rule's choice (when among the
-    // candidates) is within 3 % of it: near-ties then resolve the same way
-    // on every run
-    float best = 0.0f, t_rule = -1.0f;
-    int bestT = rule;
-    for (int c = 0; c < nc; c++) {
-        float t[kLaneReps];
-        for (int k = 0; k < kLaneReps; k++) BD_CUDA(cudaEventElapsedTime(&t[k], ev[c][k][0], ev[c][k][1]));
-        const float med = std::max(std::min(t[0], t[1]), std::min(std::max(t[0], t[1]), t[2]));
-        if (cand[c] == rule) t_rule = med;
-        if (c == 0 || med < best) {
-            best = med;
-            bestT = cand[c];
-        }
-    }
-    const int pick = (t_rule >= 0.0f && t_rule <= 1.03f * best) ? rule : bestT;
+    int pick = rule;
+    BD_TRY(pick_candidate(cand, nc, rule, ev, &pick));
     L.lanes[op] = pick;
     if (pick > 0) drop_sliced(L.sl[op]);
     else if (L.sl[op].K != -pick) BD_TRY(build_op(L, op, -pick, fp32, s));
@@ -1579,16 +1629,12 @@ static int tune_operator(Level &L, int op, bool sliced_ok, const v2<S> *x, const
 template <class S>
 static int autotune_lanes(amg_hierarchy *h, cudaStream_t s)
 {
-    cudaEvent_t ev[kLaneCands][kLaneReps][2] = {};
-    int st = BD_OK;
-    for (auto &c : ev)
-        for (auto &r : c)
-            for (cudaEvent_t &e : r)
-                if (st == BD_OK && cudaEventCreate(&e) != cudaSuccess) st = BD_ECUDA;
-    for (int l = 0; l < h->nlev - 1 && st == BD_OK; l++) {
+    TuneEvents ev;
+    BD_TRY(ev.create());
+    for (int l = 0; l < h->nlev - 1; l++) {
         Level &L = h->lev[l];
         const LV<S> lv = view<S>(h, l), cv = view<S>(h, l + 1);
-        for (int op = 0; op < 3 && st == BD_OK; op++) {
+        for (int op = 0; op < 3; op++) {
             if (op == 0 && l == 0 && h->fine.valid) continue;
             const BSR &M = op == 0 ? L.A : (op == 1 ? L.R : L.P);
             if (M.nb < kTuneMinBlocks) continue;
@@ -1596,14 +1642,10 @@ static int autotune_lanes(amg_hierarchy *h, cudaStream_t s)
             const v2<S> *x = op == 0 ? lv.u : (op == 1 ? lv.r : cv.u);
             const v2<S> *f = op == 1 ? cv.f : lv.f;
             v2<S> *out = op == 0 ? lv.r : (op == 1 ? cv.r : lv.w);
-            st = tune_operator<S>(L, op, op > 0 || l > 0, x, f, out, vals, ev, s);
+            BD_TRY(tune_operator<S>(L, op, op > 0 || l > 0, x, f, out, vals, ev, s));
         }
     }
-    for (auto &c : ev)
-        for (auto &r : c)
-            for (cudaEvent_t e : r)
-                if (e) cudaEventDestroy(e);
-    return st;
+    return BD_OK;
 }
 
 // ------------------------------------------------------------------ workspace

@@ -3,6 +3,8 @@
 // one field (amg_scalar.cu).
 #pragma once
 
+#include <functional>
+
 #include "amg_internal.cuh"
 
 namespace bd {
@@ -25,6 +27,10 @@ int info_from_scal(const double *scal, float ms, solve_info *info);
 // x = C r with the projected coarsest inverse, n unknowns
 int coarse_solve(int n, const double *C, const double *r, double *x, cudaStream_t s);
 int coarse_solve(int n, const double *C, const float *r, float *x, cudaStream_t s);
+
+// amg_options.autotune for an operator in block-CSR form: *lanes, the rule's choice,
+// gives way to the candidate run(T) is fastest with (operators of few blocks keep it)
+int tune_csr_lanes(const BSR &M, const std::function<int(int)> &run, cudaStream_t s, int *lanes);
 
 // Elliptic hierarchies (bd_elliptic_setup): the scalar form of the V-cycle.
 int scalar_build(amg_hierarchy *h, const bd_system *sys, cudaStream_t s);

@@ -60,3 +60,32 @@ def test_set_lanes_reach_the_decoupled_step(B, precision):
     f[0::2] = 0.0
     forms.time_forms(h, f, candidates=(1, 8), reps=1, warm=1)
     assert np.array_equal(_step(B, sysh, h, N), first)
+
+
+def test_tuner_reaches_the_one_field_operators(B):
+    """Launches that amg_options.autotune adds to the setup: the block hierarchy of the same
+    matrix tells how many of them are the block operators'.  FP32, whose candidates are
+    block-CSR only, launches the same number every time."""
+    m = W.mesh(48, 48, 12)
+    N = W.n_nodes(m)
+    sysh = B.bd_assemble(m, W.DEFAULT_PARAMS, W.fibre_table(m, 120.0, 5.0))
+    opts = [B.amg_options_default(precision=1, autotune=a) for a in (0, 1)]
+    plain = B.bd_elliptic_setup(sysh, opts[0])
+    A = B.amg_export_level(plain, 0)["A"]
+
+    def added(setup):
+        counts = []
+        for o in opts:
+            before = B.bd_launch_count()
+            h = setup(o)
+            counts.append(B.bd_launch_count() - before)
+        return counts[1] - counts[0], h
+
+    blocks, _ = added(lambda o: B.amg_setup_from_csr(2 * N, *A, o))
+    both, tuned = added(lambda o: B.bd_elliptic_setup(sysh, o))
+    # the finest R and P and the second level's A have 20000 blocks and more, each at
+    # least four candidates of four launches
+    assert blocks > 0 and both >= blocks + 3 * 4 * 4
+    x, y = _step(B, sysh, plain, N), _step(B, sysh, tuned, N)
+    assert np.linalg.norm(x - y) <= 1e-6 * np.linalg.norm(x)
+    assert np.array_equal(_step(B, sysh, tuned, N), y)
