@@ -939,8 +939,8 @@ static int launch_count_hash(int nrows, int HCs, const int *arp, const int *aci,
     const size_t per_warp = (size_t)R * HCs * 4;
     const int warps = hash_warps(nrows, R, (192u << 10) / per_warp);
     const size_t smem = (size_t)warps * per_warp;
-    if (smem > (227u << 10)) return BD_ERANGE;
-    BD_CUDA(cudaFuncSetAttribute(k_spgemm_count_hash<L>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    if (smem > kDynamicSmem) return BD_ERANGE;
+    BD_TRY(allow_smem(k_spgemm_count_hash<L>));
     const long long rows_per_block = (long long)warps * R;
     const int gb = (int)std::min<long long>(kSM * 8, std::max<long long>(1, (nrows + rows_per_block - 1) / rows_per_block));
     k_spgemm_count_hash<L><<<gb, 32 * warps, smem, s>>>(nrows, arp, aci, brp, bci, HCs, cnt, flag, flag + 2);
@@ -982,10 +982,10 @@ static int launch_fill_hash(int nrows, int HCn, const int *arp, const int *aci, 
     constexpr int R = 32 / L;
     const size_t per = ((size_t)HCn * BS * BS + (size_t)(3 * HCn + 1) / 2) * sizeof(double);
     const size_t per_warp = (size_t)R * per;
-    if (per_warp > (200u << 10)) return BD_ERANGE;
-    const int warps = hash_warps(nrows, R, (200u << 10) / per_warp);
+    if (per_warp > kDynamicSmem) return BD_ERANGE;
+    const int warps = hash_warps(nrows, R, kDynamicSmem / per_warp);
     const size_t smem = per_warp * warps;
-    BD_CUDA(cudaFuncSetAttribute(k_spgemm_fill_hash<BS, L>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    BD_TRY(allow_smem(k_spgemm_fill_hash<BS, L>));
     const long long rows_per_block = (long long)warps * R;
     const int gb = (int)std::min<long long>(kSM * 8, std::max<long long>(1, (nrows + rows_per_block - 1) / rows_per_block));
     k_spgemm_fill_hash<BS, L><<<gb, 32 * warps, smem, s>>>(nrows, arp, aci, av, brp, bci, bv, HCn, crp, cci, cv);
@@ -1004,10 +1004,10 @@ static int launch_fill_elem(int nrows, int HCn, const int *arp, const int *aci, 
                             const int *bci, const double *bv, const int *crp, int *cci, double *cv, cudaStream_t s)
 {
     const size_t per_warp = ((size_t)HCn * 4 + (size_t)(3 * HCn + 1) / 2) * sizeof(double);
-    if (per_warp > (200u << 10)) return BD_ERANGE;
-    const int warps = hash_warps(nrows, 1, (200u << 10) / per_warp);
+    if (per_warp > kDynamicSmem) return BD_ERANGE;
+    const int warps = hash_warps(nrows, 1, kDynamicSmem / per_warp);
     const size_t smem = per_warp * warps;
-    BD_CUDA(cudaFuncSetAttribute(k_spgemm_fill_elem, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    BD_TRY(allow_smem(k_spgemm_fill_elem));
     const int gb = (int)std::min<long long>(kSM * 32, std::max<long long>(1, (nrows + warps - 1) / warps));
     k_spgemm_fill_elem<<<gb, 32 * warps, smem, s>>>(nrows, arp, aci, av, brp, bci, bv, HCn, crp, cci, cv);
     ::bd::note_launch();
@@ -1059,11 +1059,10 @@ static int spgemm(int nrows, int ncols, const int *arp, const int *aci, const do
     // fit (with the largest column list a row can have)
     const size_t dense_smem = (size_t)ncols * (BB * sizeof(double) + sizeof(int)) +
                               (size_t)pow2_at_least(std::max(ncols, 1)) * sizeof(int);
-    const bool dense_in_smem = dense && dense_smem <= (200u << 10);
+    const bool dense_in_smem = dense && dense_smem <= kDynamicSmem;
     if (dense_in_smem) {
         const size_t cs = (size_t)ncols * sizeof(int);
-        BD_CUDA(cudaFuncSetAttribute(k_spgemm_count_smem, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)std::max<size_t>(cs, 4)));
+        BD_TRY(allow_smem(k_spgemm_count_smem));
         const int gc = (int)std::min<long long>(nrows, (long long)kSM * 8);
         k_spgemm_count_smem<<<std::max(gc, 1), 128, std::max<size_t>(cs, 4), s>>>(nrows, arp, aci, brp, bci, ncols,
                                                                                    cnt.p, flag.p + 2);
@@ -1101,14 +1100,13 @@ static int spgemm(int nrows, int ncols, const int *arp, const int *aci, const do
     const size_t hash_row = ((size_t)HCn * BB + (size_t)(3 * HCn + 1) / 2) * sizeof(double);
     const size_t warp_row = (size_t)ncols * BB * sizeof(double) + (size_t)((ncols + 31) / 32) * sizeof(int);
     if (dense && warp_row <= kWarpRowBytes && nrows >= 2 * kSM * (long long)(kSmemSM / (warp_row + 1024))) {
-        BD_CUDA(cudaFuncSetAttribute(k_spgemm_fill_warp<BS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)warp_row));
+        BD_TRY(allow_smem(k_spgemm_fill_warp<BS>));
         const int gw = (int)std::min<long long>(nrows, kSM * 32LL);
         k_spgemm_fill_warp<BS><<<gw, 32, warp_row, s>>>(nrows, arp, aci, av, brp, bci, bv, ncols, crp.p, cci.p, cv.p);
         ::bd::note_launch();
         BD_LAUNCH_CHECK();
     } else if (dense_in_smem) {
-        BD_CUDA(cudaFuncSetAttribute(k_spgemm_fill_smem<BS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)dense_smem));
+        BD_TRY(allow_smem(k_spgemm_fill_smem<BS>));
         const int per_sm = std::max(1, (int)((227u << 10) / (dense_smem + 1024)));
         const int gf = (int)std::min<long long>(nrows, (long long)kSM * per_sm);
         k_spgemm_fill_smem<BS><<<std::max(gf, 1), 256, dense_smem, s>>>(nrows, arp, aci, av, brp, bci, bv, ncols,
@@ -1119,8 +1117,7 @@ static int spgemm(int nrows, int ncols, const int *arp, const int *aci, const do
         int P2 = pow2_at_least(maxrow);
         BD_CUDA(cudaMemsetAsync(mark.p, 0xff, mark.bytes(), s));
         size_t smem = (size_t)P2 * sizeof(int);
-        BD_CUDA(cudaFuncSetAttribute(k_spgemm_fill<BS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)std::max<size_t>(smem, 4)));
+        BD_TRY(allow_smem(k_spgemm_fill<BS>));
         k_spgemm_fill<BS><<<grid, 128, smem, s>>>(nrows, arp, aci, av, brp, bci, bv, ncols, mark.p,
                                                   acc.p, crp.p, cci.p, cv.p, P2); ::bd::note_launch();
         BD_LAUNCH_CHECK();

@@ -165,6 +165,18 @@ constexpr int kFineRaw = 56;
 // ------------------------------------------------------------------ utilities
 constexpr int kSM = 152;  // GB300 streaming multiprocessors (grid sizing)
 
+// Dynamic shared memory above the default 48 KB for a kernel's launches.  The limit
+// is an attribute of the function that every thread of the process shares: set to
+// each launch's size, one thread's smaller size between another's setting and its
+// launch made that launch fail.  One value for all sizes instead (the launch's own
+// size decides what a block takes).
+constexpr size_t kDynamicSmem = 200u << 10;
+template <class K> int allow_smem(K kernel)
+{
+    BD_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDynamicSmem));
+    return BD_OK;
+}
+
 inline int grid_for(long long work, int block, int per_sm_cap = 8) {
     long long g = (work + block - 1) / block;
     long long cap = (long long)kSM * per_sm_cap * 4;

@@ -251,8 +251,7 @@ int sort_segments(int *keys, int *payload, const int *seg, int nseg, int max_len
     int P = 1;
     while (P < max_len) P <<= 1;
     size_t smem = 2 * (size_t)P * sizeof(int);
-    BD_CUDA(cudaFuncSetAttribute(k_sort_segments, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)smem));
+    BD_TRY(allow_smem(k_sort_segments));
     int threads = P >= 256 ? 256 : (P < 32 ? 32 : P);
     int grid = nseg < kSM * 16 ? nseg : kSM * 16;
     k_sort_segments<<<grid, threads, smem, s>>>(keys, payload, seg, nseg, P); ::bd::note_launch();
