@@ -257,7 +257,10 @@ int amg_vcycle(amg_hierarchy *h, const double *r, double *z, int on_device, void
  * iteration loop is a WHILE node whose condition the last reduction kernel of
  * each iteration sets on the device (converged, breakdown, or max_it reached),
  * so the host synchronises once per solve.  A hierarchy serves one solve at a
- * time.  With profiling on or strict mode, a host-driven loop with the same
+ * time.  CUDA permits no device-wide synchronisation (cudaDeviceSynchronize) by
+ * any thread of the process while a graph is being captured: make none in another
+ * thread during a hierarchy's first solve, nor during the first solve of a batch,
+ * a stack or new pointers of theirs, or the first bd_dsim_step.  With profiling on or strict mode, a host-driven loop with the same
  * kernels in the same order runs instead (identical results).
  * f, x: n = 2N doubles, host or device.  f is projected orthogonal to (0,1)
  * (Euclidean mean of the u_e entries removed) unless opts->strict, in which
@@ -342,7 +345,9 @@ void amg_stack_destroy(amg_stack *b);
  * them for amg_profile_read; reading requires no pending work.  enable: 0 off,
  * 1 on, 2 on with the per-step breakdown below.  While it is on,
  * solves run the host-driven loop (one launch at a time) instead of the
- * whole-solve CUDA graph. */
+ * whole-solve CUDA graph.  On a hierarchy of bd_elliptic_setup that loop is the
+ * block form of the solve: with timing on bd_dsim_step takes it instead of the
+ * one-field solve it takes otherwise, so the sums are the block operators'. */
 typedef struct {
     long long launches;
     double total_ms;
@@ -350,9 +355,9 @@ typedef struct {
     double flops;
     int precision;     /* 0: the timed launches are FP64, 1: FP32 (V-cycle) */
     double fp64_ops;   /* FP64 pipe operations of those launches: a fused
-                          multiply-add, an add or a multiply counts one (2 FMA
-                          per stored node pair in the (v + u, u) form, and the
-                          fused epilogue's operations per node) */
+                          multiply-add, an add or a multiply counts one (the
+                          stencil's 41 per node, 57 in the general form, and
+                          the fused epilogue's) */
 } amg_kernel_profile;
 int amg_profile_enable(amg_hierarchy *h, int enable);
 int amg_profile_read(const amg_hierarchy *h, amg_kernel_profile *out);
@@ -368,8 +373,8 @@ int amg_profile_read(const amg_hierarchy *h, amg_kernel_profile *out);
  * residual update).  Steps fused into others have no entry of their own: on a
  * stencil finest level the FP64 statistics ride on the last post-smoothing step
  * (16 * 0 + 5), and in the PCG the V-cycle input is written by the residual
- * update (so k = 1, 2, 3 appear only for amg_vcycle or a finest level in
- * block-CSR form).  Steps shorter than the host's launch rate read high.
+ * update (so k = 1 and 2 appear only for amg_vcycle, k = 3 only with an FP32
+ * V-cycle or a finest level in block-CSR form).  Steps shorter than the host's launch rate read high.
  * Switching profiling on from off resets these sums too. */
 int amg_profile_breakdown(const amg_hierarchy *h, double *ms, long long *count);
 
@@ -398,6 +403,11 @@ void bd_sim_destroy(bd_sim *s);
  * + M (I_app - chi I_ion(v^n, w^{n+1})) (Eq. 7, ionic sign as in bd_step) by
  * CG from v^n, Jacobi-preconditioned (jacobi = 1) or unpreconditioned (0, the
  * paper's GPU runs).  Both solves stop at ||r||_2 <= rtol ||f||_2.
+ *
+ * The elliptic solve runs on the u_e field alone, with operators of its own beside
+ * the hierarchy's blocks; with strict, live timing (amg_profile_enable),
+ * cheb_degree 1 or without graphs it is the block solve, which agrees to the
+ * tolerance, not bit for bit.
  *
  * bd_elliptic_setup builds the hierarchy of the elliptic operator in the
  * block form the hierarchy code takes, [I, 0; 0, Ai + Ae] on the node pattern

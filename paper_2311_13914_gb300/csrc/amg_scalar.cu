@@ -480,7 +480,12 @@ int scalar_build(amg_hierarchy *h, const bd_system *sys, cudaStream_t s)
         if (l > 0) BD_TRY(uu(L.A, C.A));
         BD_TRY(uu(L.P, C.P));
         BD_TRY(uu(L.R, C.R));
-        // one value per entry: rows are bound by latency and bytes, as FP32 blocks
+        // one value per entry: rows are bound by latency and bytes, as FP32 blocks.
+        // Every power of two timed for every operator inside the elliptic iteration
+        // (48x48x12 to 160x160x40, both precisions): the rule's choice is the fastest to
+        // within 3 us of 95 to 340 an iteration, but for A2 at 128x128x32 in FP64 (2956
+        // rows of 241: 128 threads, 64 take 11 of 343 less) and R0, P0 and A1 at
+        // 160x160x40 (6, 11 and 9 of 550 with half the lanes).
         C.lanes[0] = lanes_for(L.A, true);
         C.lanes[1] = lanes_for(L.R, true);
         C.lanes[2] = lanes_for(L.P, true);

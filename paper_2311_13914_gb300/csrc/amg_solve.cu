@@ -608,7 +608,12 @@ static int build_pairs(Level &L, bool fp32, cudaStream_t s)
 // 96x96x24 block-CSR wins, 78 against 93) and, on levels of 65536 rows and more,
 // rows in between and long ones (4 lanes; 256x256x64, 249682 rows: 840 -> 743).
 // Restrictions from 96 blocks a row from 8192 rows on.  Longer rows still and
-// everything else: the block-CSR rule.
+// everything else: the block-CSR rule.  Between those slabs (80x80x20, 112x112x28,
+// 144x144x36, 160x160x40, 192x192x48, 224x224x56, A1's 7885 to 171480 rows) the rule's
+// A1 is the fastest form to within 1 %, but for 6 % at 7885 rows (8 lanes) and 8 % at
+// 63151 (sliced 4); R0 and P0 to within 4 % but for R0 at 63151 rows (8 lanes 60.3,
+// 4 lanes 66.7) and P0 at 137781 (1 lane 15.0, sliced 17.7); R1 of 9114 and 14710 rows
+// takes 41.8 and 57.7 sliced where 16 and 8 lanes take 31.2 and 46.3.
 //
 // The finest R and P in pair form have their own crossovers.  R: few lanes
 // where rows fill the GPU (T rows >= 200 K), else up to 16 (31542 rows: 8 lanes

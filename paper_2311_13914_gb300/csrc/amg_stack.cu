@@ -7,7 +7,7 @@
 // kernel launch over all members instead of one launch per member.  Within a
 // level the members that smooth there come first (rows [0, Ns)), the members
 // whose coarsest level it is follow; their dense solves run together in one
-// launch (one thread block per member).  The projected PCG of Section 2.2
+// launch (a warp per row).  The projected PCG of Section 2.2
 // keeps its scalars per member (null-space means, alpha, beta, residual norm,
 // the stopping test): every reduction runs over chunks of at most kStChunk
 // nodes that never span two members, and the last block to finish adds each
@@ -830,7 +830,6 @@ int st_create(amg_stack *b, cudaStream_t s)
             S.lanes[2] = lanes_for(S.P, p32);
         }
     }
-    // the finest A in FP64 for the PCG's products: lanes for its rows
     // coarsest-level jobs
     std::vector<StCoarseJob> jobs(count);
     for (int k = 0; k < count; k++) {

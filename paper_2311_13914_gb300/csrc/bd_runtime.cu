@@ -814,8 +814,8 @@ extern "C" int bd_dot_exact_noalloc(const double *x, const double *y, long long 
     if (n > 2147483647LL) return BD_ERANGE;
     long long *acc = nullptr;
     BD_TRY(bd::noalloc_scratch(&acc));
-    // exact_dot clears the accumulator on `stream`, then launches the partial
-    // and rounding kernels; nothing is allocated.
+    // exact_dot clears the accumulator on `stream`, then launches one kernel whose
+    // last block rounds; nothing is allocated.
     return bd::exact_dot(x, y, (int)n, out, acc, (cudaStream_t)stream);
 }
 

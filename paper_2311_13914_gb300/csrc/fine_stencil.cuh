@@ -20,7 +20,8 @@
 // the general form (27 coefficients) serves every other field.  Against the
 // operator stored in sliced ELL (20 and 9 bytes per node pair), event-timed per
 // launch: 128x128x32 FP64 67.6 -> 51 us (residual), FP32 33 -> 10.4;
-// 256x256x64 FP64 A p 462 -> 343, FP32 219 -> 37.5.
+// 256x256x64 FP64 A p 462 -> 343, FP32 219 -> 37.5.  The general form: 65.8, 13.8,
+// 458 and 65.4 (54 multiply-adds a node, as many as the sliced ELL's).
 #pragma once
 
 #include "amg_bsr.cuh"
@@ -62,7 +63,10 @@ struct FineGrid {
 // clocks, and two blocks (two warps per scheduler) hide every load; more of them
 // only shorten the walks and add halo planes (128x128x32, residual: 4 blocks
 // 61.6 us, 3 53.0, 2 51.0).  FP32: latency and L1 wavefronts; 6 blocks of 80
-// registers beat 8 of 64 (256x256x64, residual: 48 -> 37.5 us).
+// registers beat 8 of 64 (256x256x64, residual: 48 -> 37.5 us).  General form, pre-smoother
+// at 128x128x32 and 256x256x64: FP64 1 block 83.3 and 655 us, 2 68.3 and 472, 3 70.5
+// and 482; FP32 4 blocks 15.2 and 93, 5 14.6 and 75 (36 bytes of a thread's registers
+// spilled), 6 15.2 and 84.
 constexpr int kFineTPB = 128;
 template <class S, bool SYM> struct FineMinB { static constexpr int v = sizeof(S) == 8 ? 2 : (SYM ? 6 : 5); };
 
